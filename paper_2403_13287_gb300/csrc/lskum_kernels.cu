@@ -3,6 +3,7 @@
 // reductions (residue, forces). One thread per point; the neighbour loop
 // gathers q, q-derivatives and coordinates of the stencil.
 #include "lskum_device.cuh"
+#include "lskum_fixed.cuh"
 #include "lskum_kernels.h"
 
 namespace lskum {
@@ -346,23 +347,27 @@ __device__ __forceinline__ void flag_nonphysical(int *status, int64_t p)
     atomicMin(status + 1, (int)p);
 }
 
-// One member's term of E11: w_s [Gs(q~_i) - Gs(q~_0)] + w_n [Gn(q~_i) - Gn(q~_0)],
+// One member's term of E11, w_s [Gs(q~_i) - Gs(q~_0)] + w_n [Gn(q~_i) - Gn(q~_0)],
 // Gs = Gx+ or Gx- and Gn = Gy+ or Gy- by the member's sub-stencil bits m,
-// in the frame (t, n) of P_0; R in the order [mass, s-momentum, n-momentum, energy].
-__device__ __forceinline__ void edge_residual(const double qti[4], const double qt0[4], uint8_t m, double2 w,
-                                              double2 n0, double tx, double ty, const Gas &gas, double R[4],
-                                              bool &ok)
+// in the frame (t, n) of P_0: [mass, s-momentum, n-momentum, energy].
+struct EdgeTerm {
+    double R[4];
+    bool ok;
+};
+struct Vec4 {
+    double v[4];
+};
+
+// in FP64: states outside the fixed-point form's ranges, and gamma != 1.4.
+// Not inlined: it keeps its registers out of the loop that hardly ever calls it.
+__device__ __noinline__ EdgeTerm edge_term_fp64(Vec4 qi, Vec4 q0, uint32_t m, double2 w, double2 n0, Gas gas)
 {
-    // equal reconstructed states have dG = 0 exactly (compared as bit patterns,
-    // on the integer pipe; +0 against -0 only costs a flux evaluation giving dG = 0)
-    if (((__double_as_longlong(qti[0]) ^ __double_as_longlong(qt0[0])) |
-         (__double_as_longlong(qti[1]) ^ __double_as_longlong(qt0[1])) |
-         (__double_as_longlong(qti[2]) ^ __double_as_longlong(qt0[2])) |
-         (__double_as_longlong(qti[3]) ^ __double_as_longlong(qt0[3]))) == 0)
-        return;
+    const double *qti = qi.v, *qt0 = q0.v;
+    const double tx = n0.y, ty = -n0.x;
+    EdgeTerm o = {{0.0, 0.0, 0.0, 0.0}, true};
     Prim si, s0;
-    ok &= prim_from_q(qti, gas, tx, ty, n0, si);
-    ok &= prim_from_q(qt0, gas, tx, ty, n0, s0);
+    o.ok &= prim_from_q(qti, gas, tx, ty, n0, si);
+    o.ok &= prim_from_q(qt0, gas, tx, ty, n0, s0);
     const double us_i = si.us, un_i = si.un, us_0 = s0.us, un_0 = s0.un;
     // w != 0 tested on the bits (integer pipe; +-0 are the zeros)
     if ((__double_as_longlong(w.x) & ~(long long)kSignBit) != 0) {
@@ -374,7 +379,7 @@ __device__ __forceinline__ void edge_residual(const double qti[4], const double 
         // subtraction, so equal states give exactly zero (a contracted
         // fma(rho_i, m_i, -rho_0 m_0) would leave a product's rounding)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) R[k] += w.x * __dsub_rn(Gi[k], G0[k]);
+        for (int k = 0; k < 4; ++k) o.R[k] += w.x * __dsub_rn(Gi[k], G0[k]);
     }
     if ((__double_as_longlong(w.y) & ~(long long)kSignBit) != 0) {
         const unsigned long long sg = (m & M_YPOS) ? 0ull : kSignBit;
@@ -382,11 +387,57 @@ __device__ __forceinline__ void edge_residual(const double qti[4], const double 
         split_flux(sg, si, un_i, us_i, si.Sn, Gi);
         split_flux(sg, s0, un_0, us_0, s0.Sn, G0);
         // Gn components are [mass, n-momentum, s-momentum, energy]
-        R[0] += w.y * __dsub_rn(Gi[0], G0[0]);
-        R[1] += w.y * __dsub_rn(Gi[2], G0[2]);
-        R[2] += w.y * __dsub_rn(Gi[1], G0[1]);
-        R[3] += w.y * __dsub_rn(Gi[3], G0[3]);
+        o.R[0] += w.y * __dsub_rn(Gi[0], G0[0]);
+        o.R[1] += w.y * __dsub_rn(Gi[2], G0[2]);
+        o.R[2] += w.y * __dsub_rn(Gi[1], G0[1]);
+        o.R[3] += w.y * __dsub_rn(Gi[3], G0[3]);
     }
+    return o;
+}
+
+// The member's term added into R: in fixed point (lskum_fixed.cuh) where both
+// states lie in its ranges, else in FP64. nx, ny: the normal n0 in fixed point.
+__device__ __forceinline__ void edge_residual(const double qti[4], const double qt0[4], uint8_t m, double2 w,
+                                              double2 n0, FixOp nx, FixOp ny, const Gas &gas, double R[4], bool &ok)
+{
+    // equal reconstructed states have dG = 0 exactly (compared as bit patterns,
+    // on the integer pipe; +0 against -0 only costs a flux evaluation giving dG = 0)
+    if (((__double_as_longlong(qti[0]) ^ __double_as_longlong(qt0[0])) |
+         (__double_as_longlong(qti[1]) ^ __double_as_longlong(qt0[1])) |
+         (__double_as_longlong(qti[2]) ^ __double_as_longlong(qt0[2])) |
+         (__double_as_longlong(qti[3]) ^ __double_as_longlong(qt0[3]))) == 0)
+        return;
+    FixState si, s0;
+    const bool in_range = fix_state(qti, nx, ny, si) & fix_state(qt0, nx, ny, s0);
+    if (gas.g14 && in_range) {
+        FixEdge g;
+        fix_edge(si, s0, g);
+        double dG[4];
+        if ((__double_as_longlong(w.x) & ~(long long)kSignBit) != 0) {
+            const bool plus = (m & M_XPOS) != 0;
+            fix_flux_difference(g, si, s0, true, plus ? 0 : -1, dG);
+            const double ws = flip_sign(w.x, plus ? 0ull : kSignBit);
+            R[0] = fma(ws, dG[0], R[0]);
+            R[1] = fma(w.x, dG[1], R[1]);
+            R[2] = fma(ws, dG[2], R[2]);
+            R[3] = fma(ws, dG[3], R[3]);
+        }
+        if ((__double_as_longlong(w.y) & ~(long long)kSignBit) != 0) {
+            const bool plus = (m & M_YPOS) != 0;
+            fix_flux_difference(g, si, s0, false, plus ? 0 : -1, dG);
+            const double ws = flip_sign(w.y, plus ? 0ull : kSignBit);
+            R[0] = fma(ws, dG[0], R[0]);
+            R[1] = fma(ws, dG[2], R[1]);   // the s-momentum is the transverse one here
+            R[2] = fma(w.y, dG[1], R[2]);
+            R[3] = fma(ws, dG[3], R[3]);
+        }
+        return;
+    }
+    const EdgeTerm o = edge_term_fp64(Vec4{{qti[0], qti[1], qti[2], qti[3]}}, Vec4{{qt0[0], qt0[1], qt0[2], qt0[3]}}, m, w,
+                                      n0, gas);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) R[k] += o.R[k];
+    ok &= o.ok;
 }
 
 template <bool KIN>
@@ -403,6 +454,7 @@ __global__ void __launch_bounds__(128) k_flux_update(FluxParams P)
         const double2 xy0 = g.xy[p];
         const double2 n0 = g.nrm[p];
         const double tx = n0.y, ty = -n0.x;
+        const FixOp fnx = fix_op(fix_unit(n0.x)), fny = fix_op(fix_unit(n0.y));
         double q0[4], g0[8];
         load4(P.q, p, q0);
         const bool second = P.order == 2;
@@ -436,7 +488,7 @@ __global__ void __launch_bounds__(128) k_flux_update(FluxParams P)
                     qt0[k] = fma(-h.y, g0[4 + k], fma(-h.x, g0[k], qt0[k]));
                 }
             }
-            edge_residual(qti, qt0, m, w, n0, tx, ty, P.gas, R, ok);
+            edge_residual(qti, qt0, m, w, n0, fnx, fny, P.gas, R, ok);
         }
         if constexpr (KIN) {
             // kinetic boundary mode: the mirror images of the neighbours
@@ -450,7 +502,7 @@ __global__ void __launch_bounds__(128) k_flux_update(FluxParams P)
                 image_q(g, e, m, n0, qf, P.q, P.qg, hs, second, qti);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) qt0[k] = second ? fma(-hs.y, g0[4 + k], fma(-hs.x, g0[k], q0[k])) : q0[k];
-                edge_residual(qti, qt0, m, w, n0, tx, ty, P.gas, R, ok);
+                edge_residual(qti, qt0, m, w, n0, fnx, fny, P.gas, R, ok);
             }
         }
         if (!ok) flag_nonphysical(P.status, p);
