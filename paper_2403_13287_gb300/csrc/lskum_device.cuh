@@ -48,6 +48,7 @@ struct DevGeom {
     const double2 *__restrict__ fxw;
     const double2 *__restrict__ hd;  // FP64 contexts: per edge (P_i - P_0)/2, or nullptr
     const float2 *__restrict__ hd_f; // FP64 contexts: hd rounded to FP32 (the limiter's screening of d_m), or nullptr
+    const longlong2 *__restrict__ hfx; // FP64 contexts: hd in fixed point (fix_pack_pair), or nullptr
     // kinetic boundary mode (all nullptr otherwise): the mirror images of the
     // neighbours of each wall and far-field point, per point in CSR form
     // (rows are empty at interior points); an image of P_i has local offsets
@@ -322,6 +323,31 @@ __device__ __forceinline__ void store8(double *a, int64_t p, const double v[8])
     double2 *a2 = reinterpret_cast<double2 *>(a);
 #pragma unroll
     for (int k = 0; k < 4; ++k) a2[4 * p + k] = make_double2(v[2 * k], v[2 * k + 1]);
+}
+
+// row p of a read-only [n][4] or [n][8] array (32-byte aligned rows) by
+// 256-bit loads through the non-coherent path
+__device__ __forceinline__ void gather4(const double *a, int64_t p, double v[4])
+{
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(a + 4 * p));
+}
+__device__ __forceinline__ void gather8(const double *a, int64_t p, double v[8])
+{
+    gather4(a, 2 * p, v);
+    gather4(a, 2 * p + 1, v + 4);
+}
+
+// double -> float, round to nearest (ties away), on the integer pipe for
+// magnitudes of 2^-100 to 2^100 and for 0; the conversion instruction (FP64
+// pipe) elsewhere
+__device__ __forceinline__ float f64_to_f32(double x)
+{
+    const long long b = __double_as_longlong(x);
+    const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+    if (e == 0u) return 0.0f;
+    if (e - 923u > 200u) return __double2float_rn(x);
+    const unsigned long long m = ((unsigned long long)b & 0x7fffffffffffffffull) + (1ull << 28);
+    return __uint_as_float(((unsigned)(m >> 29) - ((1023u - 127u) << 23)) | ((unsigned)(b >> 32) & 0x80000000u));
 }
 
 // q-variables of a conserved state (E13), same operation order as the

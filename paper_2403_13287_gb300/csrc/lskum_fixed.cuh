@@ -8,7 +8,7 @@
 // and two adds, 3-4 cycles instead of 16, and keeps 60 bits where a double
 // keeps 53. The result is rounded to a double once per component. The flux
 // launch went from 178 to 50 FP64 warp instructions per edge and from 6.82 to
-// 2.70 ms at 2.5 million points (second order, RK4), its error against multiple
+// 2.26 ms at 2.5 million points (second order, RK4), its error against multiple
 // precision is 2-8 times below that of the FP64 chain.
 //
 // With r = beta^(-1/2), S_t = u.t sqrt(beta), S_n likewise, every flux is a
@@ -100,6 +100,8 @@ LSKUM_FIX_FN int32_t fix_mulhi32(int32_t a, int32_t b)
 }
 LSKUM_FIX_FN int fix_min(int a, int b) { return a < b ? a : b; }
 LSKUM_FIX_FN int fix_max(int a, int b) { return a > b ? a : b; }
+LSKUM_FIX_FN int64_t fix_min64(int64_t a, int64_t b) { return a < b ? a : b; }
+LSKUM_FIX_FN int64_t fix_max64(int64_t a, int64_t b) { return a > b ? a : b; }
 LSKUM_FIX_FN int64_t fix_shl(int64_t v, int s) { return (int64_t)((uint64_t)v << s); }
 
 // --- products ---------------------------------------------------------------
@@ -114,6 +116,7 @@ LSKUM_FIX_FN FixOp fix_op(int64_t a)
     const int32_t lo = (int32_t)a;
     return FixOp{(int32_t)(a >> 32) + (int32_t)((uint32_t)lo >> 31), lo};
 }
+LSKUM_FIX_FN int64_t fix_value(FixOp a) { return fix_shl((int64_t)a.hi, 32) + a.lo; }
 // a b 2^-64 within (-1.25, 0.25] (the low x low product is left out)
 LSKUM_FIX_FN int64_t fix_mul(FixOp a, FixOp b)
 {
@@ -158,9 +161,12 @@ LSKUM_FIX_FN double fix_to_double(int64_t v, int e)
 struct FixState {
     int64_t St, Sn;        // Q61, |.| < 4
     int64_t H;             // Q59, hc + (St^2 + Sn^2)/2 < 9.7
-    int64_t c0, c1, c3;    // rho r, rho r^2, rho r^3: c 2^e
-    int e0, e1, e3;
+    int64_t c0, c1, c3;    // rho r, rho r^2, rho r^3: c 2^e, e from n and k (fix_e0 ...)
+    int n, k;              // exp(q1 + s2) = M 2^n, beta = b 4^k
 };
+LSKUM_FIX_FN int fix_e0(int n, int k) { return n - 6 * k - 58; }
+LSKUM_FIX_FN int fix_e1(int n, int k) { return n - 7 * k - 57; }
+LSKUM_FIX_FN int fix_e3(int n, int k) { return n - 8 * k - 57; }
 
 // the double x times r/2 (R = r 2^61 in (0.7, 1.42), times 2^-k) as Q61; false
 // from 3.9375 on
@@ -254,23 +260,21 @@ LSKUM_FIX_FN bool fix_state(const double q[4], FixOp nx, FixOp ny, FixState &s)
     s.c0 = fix_mul_s<1>(M, r6);                                  // Q58, below 2^62 like the others
     s.c1 = fix_mul_s<1>(M, r7);                                  // Q57
     s.c3 = fix_mul_s<1>(M, r8);                                  // Q57
-    s.e0 = n - 6 * k - 58;
-    s.e1 = n - 7 * k - 57;
-    s.e3 = n - 8 * k - 57;
+    s.n = n;
+    s.k = k;
     return ok;
 }
 
-// two factors c 2^e, both below 2^62, brought to one exponent (returned), the larger in [2^61, 2^62)
-LSKUM_FIX_FN int fix_align(int64_t &ci, int ei, int64_t &c0, int e0)
+// c 2^e, c below 2^62, against another factor's exponent eo: c at the larger of
+// the two (es)
+LSKUM_FIX_FN int64_t fix_align_half(int64_t c, int e, int eo, int &es)
 {
-    const int d = ei - e0;
-    c0 >>= fix_max(fix_min(d, 63), 0);
-    ci >>= fix_max(fix_min(-d, 63), 0);
-    const int lz = fix_clz((uint32_t)((uint64_t)(ci | c0) >> 32)) - 2;
-    ci <<= lz;
-    c0 <<= lz;
-    return fix_max(ei, e0) - lz;
+    es = fix_max(e, eo);
+    return c >> fix_min(es - e, 63);
 }
+// the left shift that takes the larger of two such factors (c, and one with
+// high word hi) into [2^61, 2^62)
+LSKUM_FIX_FN int fix_top(int64_t c, uint32_t hi) { return fix_clz((uint32_t)((uint64_t)c >> 32) | hi) - 2; }
 
 // the bounded parts of one state's split flux with z = sgn S_d, So the
 // transverse S: P in Q61, Phi/2 + z P in Q58, So P in Q58, H P - E/4 in Q57
@@ -316,40 +320,149 @@ LSKUM_FIX_FN void fix_parts(int64_t Sd, int64_t sgn, int64_t So, int64_t H, int6
     F[3] = fix_mul_s<1>(fix_op(H), Po) - (E >> 7);
 }
 
-// An edge's two states with their factors at common exponents
-struct FixEdge {
-    FixOp c0i, c1i, c3i, c00, c10, c30;
-    int e0, e1, e3;
-};
-LSKUM_FIX_FN void fix_edge(const FixState &si, const FixState &s0, FixEdge &g)
+// the parts times the state's (shifted) factors: c < 2^62 and F[0] < 2^63,
+// |F[1..3]| < 2^62.4, so one, two more bits of the products fit
+LSKUM_FIX_FN void fix_scale(FixOp c0, FixOp c1, FixOp c3, int64_t F[4])
 {
-    int64_t a = si.c0, b = s0.c0;
-    g.e0 = fix_align(a, si.e0, b, s0.e0) + 2;
-    g.c0i = fix_op(a);
-    g.c00 = fix_op(b);
-    a = si.c1, b = s0.c1;
-    g.e1 = fix_align(a, si.e1, b, s0.e1) + 4;
-    g.c1i = fix_op(a);
-    g.c10 = fix_op(b);
-    a = si.c3, b = s0.c3;
-    g.e3 = fix_align(a, si.e3, b, s0.e3) + 5;
-    g.c3i = fix_op(a);
-    g.c30 = fix_op(b);
+    F[0] = fix_mul_s<1>(c0, fix_op(F[0]));
+    F[1] = fix_mul_s<2>(c1, fix_op(F[1]));
+    F[2] = fix_mul_s<2>(c1, fix_op(F[2]));
+    F[3] = fix_mul_s<2>(c3, fix_op(F[3]));
 }
 
-// G(q~_i) - G(q~_0) of one direction without the factors sgn of components
-// 0, 2 and 3: [mass, d-momentum, o-momentum, energy]. sgn = 0 for G+, -1 for G-.
-LSKUM_FIX_FN void fix_flux_difference(const FixEdge &g, const FixState &si, const FixState &s0, bool along_t,
-                                      int64_t sgn, double dG[4])
+// --- the q-derivative passes' parts ------------------------------------------
+// Two doubles with one exponent: x = X 2^(e-1084), X the op's value, |X| < 2^62.
+struct FixPair {
+    FixOp x, y;
+    int e;   // the larger biased exponent (0: both zero or subnormal, 0x7ff: not finite)
+};
+template <int Q>
+LSKUM_FIX_FN int64_t fix_mantissa(int64_t b, int drop)   // 1.xx in Q60 or Q61, signed, shifted right
 {
-    int64_t Fi[4], F0[4];
-    fix_parts(along_t ? si.St : si.Sn, sgn, along_t ? si.Sn : si.St, si.H, Fi);
-    fix_parts(along_t ? s0.St : s0.Sn, sgn, along_t ? s0.Sn : s0.St, s0.H, F0);
-    // c < 2^62 and F[0] < 2^63, |F[1..3]| < 2^62.4: one, two more bits of the products fit
-    dG[0] = fix_to_double(fix_mul_s<1>(g.c0i, fix_op(Fi[0])) - fix_mul_s<1>(g.c00, fix_op(F0[0])), g.e0);
-    dG[1] = fix_to_double(fix_mul_s<2>(g.c1i, fix_op(Fi[1])) - fix_mul_s<2>(g.c10, fix_op(F0[1])), g.e1);
-    dG[2] = fix_to_double(fix_mul_s<2>(g.c1i, fix_op(Fi[2])) - fix_mul_s<2>(g.c10, fix_op(F0[2])), g.e1);
-    dG[3] = fix_to_double(fix_mul_s<2>(g.c3i, fix_op(Fi[3])) - fix_mul_s<2>(g.c30, fix_op(F0[3])), g.e3);
+    const int64_t m = (((b & 0xfffffffffffffll) | 0x10000000000000ll) << (Q - 52)) >> fix_min(drop, 63);
+    return fix_flip(m, b >> 63);
+}
+LSKUM_FIX_FN FixPair fix_pair(double x, double y)
+{
+    const int64_t bx = fix_bits(x), by = fix_bits(y);
+    const int ex = (int)(bx >> 52) & 0x7ff, ey = (int)(by >> 52) & 0x7ff;
+    FixPair p;
+    p.e = fix_max(ex, ey);
+    // a zero beside a finite number is shifted out: its exponent field is 0
+    p.x = fix_op(ex ? fix_mantissa<61>(bx, p.e - ex) : 0);
+    p.y = fix_op(ey ? fix_mantissa<61>(by, p.e - ey) : 0);
+    return p;
+}
+// A pair with its exponent in the low bits of the two words, 4 each: e - 895
+// (1..255, |x|, |y| up to 2^127 and the larger at least 2^-127); 0 where it
+// does not fit. The bits given up are below 2^-57 of the larger.
+LSKUM_FIX_FN void fix_pack_pair(double x, double y, int64_t &wx, int64_t &wy)
+{
+    const FixPair p = fix_pair(x, y);
+    const int e = p.e - 895;
+    const bool fits = e >= 1 && e <= 255;
+    wx = fits ? (fix_value(p.x) & ~15ll) | (e & 15) : 0;
+    wy = fits ? (fix_value(p.y) & ~15ll) | (e >> 4) : 0;
+}
+LSKUM_FIX_FN FixPair fix_unpack_pair(int64_t wx, int64_t wy)
+{
+    FixPair p;
+    const int e = ((int)wx & 15) | (((int)wy & 15) << 4);
+    p.e = e ? e + 895 : 0x7ff;   // 0x7ff: fix_dot_in_range refuses it
+    p.x = fix_op(wx & ~15ll);
+    p.y = fix_op(wy & ~15ll);
+    return p;
+}
+// the exponents of h and g for which fix_dot's result is a normal number: away
+// from both ends by the 60 bits that a cancelling sum may lose
+LSKUM_FIX_FN bool fix_dot_in_range(const FixPair &h, const FixPair &g)
+{
+    return (unsigned)(h.e + g.e - 1100) < 1900u && fix_max(h.e, g.e) < 0x7ff;
+}
+// h.x g.x + h.y g.y, rounded once (2^-56 of |h||g| before the rounding; the
+// cross sum stays below 2^63: four times (2^30 - 1) 2^31)
+LSKUM_FIX_FN double fix_dot(const FixPair &h, const FixPair &g)
+{
+    int64_t m = (int64_t)h.x.hi * g.x.lo;
+    m += (int64_t)h.x.lo * g.x.hi;
+    m += (int64_t)h.y.hi * g.y.lo;
+    m += (int64_t)h.y.lo * g.y.hi;
+    int64_t c = (int64_t)h.x.hi * g.x.hi + (m >> 32);
+    c += (int64_t)h.y.hi * g.y.hi;
+    return fix_to_double(c, h.e + g.e - 2104);
+}
+
+// round(2^22 / f) within a unit or so, f the float with these bits in [1, 2)
+LSKUM_FIX_FN int32_t fix_rcp_seed(uint32_t bits)
+{
+#ifdef __CUDACC__
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(bits)));
+    return __float_as_int(y + 2.0f) - 0x40000000;   // [2, 4) has a unit of 2^-22
+#else
+    float f;
+    memcpy(&f, &bits, 4);
+    const float y = 1.0f / f + 2.0f;
+    int32_t v;
+    memcpy(&v, &y, 4);
+    return v - 0x40000000;
+#endif
+}
+
+// 1/m in Q62 (in (0.5, 1]) of m in Q61, 2^61 <= m < 2^62
+LSKUM_FIX_FN int64_t fix_rcp(int64_t m)
+{
+    const int32_t Y = fix_rcp_seed(0x3f800000u | ((uint32_t)(m >> 38) & 0x7fffffu));   // Q22
+    // e = 1 - m Y exactly to 2^-63, r = Y (1 + e + e^2), |e| < 2^-21
+    const uint64_t t = (((uint64_t)(uint32_t)m * (uint32_t)Y) >> 20) + (((uint64_t)(uint32_t)(m >> 32) * (uint32_t)Y) << 12);
+    const int64_t e = (int64_t)(0x8000000000000000ull - t);       // Q63
+    const int32_t eh = (int32_t)(e >> 11);                         // Q52
+    const int64_t c = (e >> 1) + (fix_mulhi32(eh, eh) >> 10);      // Q62
+    return ((int64_t)Y << 40) + (((int64_t)Y * c) >> 22);
+}
+
+// Venkatakrishnan's f(x, d) = N / M, N = x (x + 2d) + eps2,
+// M = x (x + d) + 2 d^2 + eps2, for 0 <= x < 2d (so that f <= 1) and exponents
+// within fix_phi_in_range. Everything is scaled by the power of two that takes
+// the larger of d and sqrt(eps2) to order 1; N keeps an exponent of its own, so
+// that a small f keeps its relative precision (2^-54 before the final rounding).
+LSKUM_FIX_FN bool fix_phi_in_range(double d, double eps2)
+{
+    const int ed = (int)(fix_bits(d) >> 52), ee = (int)(fix_bits(eps2) >> 52);
+    return (unsigned)(ed - 300) < 1400u && (unsigned)ee < 1700u;
+}
+LSKUM_FIX_FN double fix_phi(double x, double d, double eps2)
+{
+    const int64_t bx = fix_bits(x), bd = fix_bits(d), be = fix_bits(eps2);
+    const int ex = (int)(bx >> 52), ed = (int)(bd >> 52), ee = (int)(be >> 52);
+    const int p = fix_max(ed, 1023 + ((ee - 1022) >> 1));          // biased exponent of the scale
+    const int64_t X = ex ? fix_mantissa<60>(bx, 0) : 0;             // x = X 2^(ex - p), 1.xx in Q60
+    const int ux = ex ? ex - p : -4096, ue = ee ? ee + 1023 - 2 * p : -4096;   // ux <= 1, ue <= 0
+    const int64_t xs = X >> fix_min(1 - ux, 63);                    // x < 4 in Q59
+    const int64_t ds = fix_mantissa<60>(bd, p - ed + 1);            // d < 2 in Q59
+    const int64_t E = ee ? fix_mantissa<57>(be, 0) : 0;             // eps2 = E 2^ue, 1.xx in Q57
+    const int64_t T = fix_mul_s<2>(fix_op(X), fix_op(xs + 2 * ds)); // x (x + 2d) = T 2^ux, T < 16 in Q57
+    const int un = fix_max(ux, ue);
+    const int64_t N = (T >> fix_min(un - ux, 63)) + (E >> fix_min(un - ue, 63));   // Q57, times 2^un
+    // M < 34 in Q56, at least 1/4
+    const int64_t M = fix_mul_s<2>(fix_op(xs), fix_op(xs + ds)) + fix_sqr_s<3>(fix_op(ds)) + (E >> fix_min(1 - ue, 63));
+    const int lz = fix_clz((uint32_t)((uint64_t)M >> 32)) - 2;
+    const int64_t f = fix_mul_s<2>(fix_op(N), fix_op(fix_rcp(M << lz)));   // N / (M 2^(lz - 61)), Q57
+    return un < -900 ? 0.0 : fix_to_double(f, un + lz - 62);      // below 2^-890: 0
+}
+
+// a - b where sign and exponent agree (the difference is then exact), in range
+// for fix_to_double
+LSKUM_FIX_FN bool fix_same_binade(double a, double b)
+{
+    const int64_t ba = fix_bits(a), x = ba ^ fix_bits(b);
+    return ((uint64_t)x >> 52) == 0 && (unsigned)(((int)(ba >> 52) & 0x7ff) - 100) < 1900u;
+}
+LSKUM_FIX_FN double fix_difference(double a, double b)
+{
+    const int64_t ba = fix_bits(a), bb = fix_bits(b);
+    return fix_to_double(fix_flip((ba & 0xfffffffffffffll) - (bb & 0xfffffffffffffll), ba >> 63),
+                         ((int)(ba >> 52) & 0x7ff) - 1075);
 }
 
 }  // namespace lskum

@@ -66,6 +66,47 @@ __device__ __forceinline__ void image_q(const DevGeom &g, int e, uint8_t m, doub
 // 1/64 of the integer ALU rate, so the stencil extrema take this form.
 __device__ __forceinline__ long long order_key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffLL); }
 
+// C consecutive values of a row (aligned to C values): read-only load, store
+template <int C>
+__device__ __forceinline__ void gather_c(const double *a, double v[C])
+{
+    if constexpr (C == 4) {
+        gather4(a, 0, v);
+    } else if constexpr (C == 2) {
+        const double2 w = __ldg(reinterpret_cast<const double2 *>(a));
+        v[0] = w.x;
+        v[1] = w.y;
+    } else {
+        v[0] = __ldg(a);
+    }
+}
+template <int C>
+__device__ __forceinline__ void store_c(double *a, const double v[C])
+{
+    if constexpr (C == 4) {
+        store4(a, 0, v);
+    } else if constexpr (C == 2) {
+        *reinterpret_cast<double2 *>(a) = make_double2(v[0], v[1]);
+    } else {
+        *a = v[0];
+    }
+}
+// components k0 .. k0 + C - 1 (k0 a multiple of C) without an indexed array in memory
+template <int C>
+__device__ __forceinline__ void components(const double v[4], int k0, double o[C])
+{
+    if constexpr (C == 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) o[k] = v[k];
+    } else if constexpr (C == 2) {
+        o[0] = k0 ? v[2] : v[0];
+        o[1] = k0 ? v[3] : v[1];
+    } else {
+        const double a = (k0 & 1) ? v[1] : v[0], b = (k0 & 1) ? v[3] : v[2];
+        o[0] = (k0 & 2) ? b : a;
+    }
+}
+
 // Kinds of q-derivative pass (the template argument PASS): QG_INNER an inner
 // iteration, QG_LIMIT the limiter applied at its end, QG_EXTREMA a first
 // pass that also stores the limiter's extremum measure for a limited inner
@@ -86,40 +127,43 @@ enum { QG_LIMIT = 1, QG_INNER = 2, QG_EXTREMA = 4 };
 // !(fl(v + c) < L) (a NaN or an overflow marks the edge too); the marked
 // edges (one bit each: at most LSKUM_MAX_DEGREE = 25) are then evaluated in
 // FP64 exactly as the plain loop evaluates them.
-__device__ __forceinline__ void largest_shift_screened(const DevGeom &g, int e0, int e1, const double sx[4],
-                                                       const double sy[4], unsigned long long dm[4])
+template <int C>
+__device__ __forceinline__ void largest_shift_screened(const DevGeom &g, int e0, int e1, const double sx[C],
+                                                       const double sy[C], unsigned long long dm[C])
 {
     constexpr float kMargin = 9.5367431640625e-07f;  // 2^-20 = 16 u
     constexpr float kTiny = 7.52316384526264e-37f;   // 2^-120
-    float sf[4], tf[4], L[4];
+    float sf[C], tf[C], L[C];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        sf[k] = __double2float_rn(sx[k]);
-        tf[k] = __double2float_rn(sy[k]);
+    for (int k = 0; k < C; ++k) {
+        sf[k] = f64_to_f32(sx[k]);
+        tf[k] = f64_to_f32(sy[k]);
         L[k] = 0.0f;
     }
     for (int e = e0; e < e1; ++e) {
         const float2 h = g.hd_f[e];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < C; ++k) {
             const float a = h.x * sf[k], b = h.y * tf[k];
             const float c = fmaf(kMargin, fabsf(a) + fabsf(b), kTiny);
             L[k] = fmaxf(L[k], fabsf(a + b) - c);
         }
     }
-    uint32_t cand[4] = {0u, 0u, 0u, 0u};
+    uint32_t cand[C];
+#pragma unroll
+    for (int k = 0; k < C; ++k) cand[k] = 0u;
     for (int e = e0; e < e1; ++e) {
         const float2 h = g.hd_f[e];
         const uint32_t bit = 1u << (e - e0);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < C; ++k) {
             const float a = h.x * sf[k], b = h.y * tf[k];
             const float c = fmaf(kMargin, fabsf(a) + fabsf(b), kTiny);
             if (!(fabsf(a + b) + c < L[k])) cand[k] |= bit;
         }
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < C; ++k) {
         uint32_t m = cand[k];
         while (m) {
             const int j = __ffs(m) - 1;
@@ -150,30 +194,51 @@ __device__ __forceinline__ void largest_shift_screened(const DevGeom &g, int e0,
 // f(x_m, d_m): one quotient per component (a reciprocal and two Newton steps).
 // KIN: the kinetic boundary mode (mirror images in g.ioff...; a separate
 // instantiation keeps the plain kernel's registers as they are)
-template <bool KIN, int PASS>
+// The FP64 pipe bounds the pass (16 SM cycles per warp instruction). Per edge
+// and component the inner pass keeps two FP64 fused multiply-adds (s -= a c);
+// c = h . grad q_i comes from the integer pipes (fix_dot), q_i - q_0 of the
+// first pass too where it is exact, and the limiter's quotient (fix_phi): pass
+// average 0.700 -> 0.444 ms at 2.5 million points.
+// LANES lanes per point, 4 / LANES components each: every lane runs the point's
+// whole edge loop in row order, so the arithmetic of a component is the same
+// bit for bit whatever LANES is, and a small cloud spreads over more warps with
+// a shorter serial chain in each.
+template <bool KIN, int PASS, int LANES>
 __global__ void __launch_bounds__(128) k_qgrad(DevGeom g, const double *__restrict__ q,
                                                const double *__restrict__ qg_old, const double *__restrict__ g1,
                                                double *__restrict__ qg_new, double *__restrict__ ext, double limK)
 {
     constexpr bool INNER = (PASS & QG_INNER) != 0, LIMIT = (PASS & QG_LIMIT) != 0;
     constexpr bool EXTR = !INNER && (PASS & (QG_LIMIT | QG_EXTREMA)) != 0;   // extrema found here
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    constexpr int C = 4 / LANES;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t p = t / LANES;
+    const int k0 = (int)(t % LANES) * C;   // this lane's components: k0 .. k0 + C - 1
     if (p >= g.n) return;
-    double sx[4], sy[4];
+    double sx[C], sy[C];
     // order keys of the largest and smallest q_i - q_0 (P_0's own difference: +0)
-    long long kmax[4] = {0, 0, 0, 0}, kmin[4] = {0, 0, 0, 0};
+    long long kmax[C], kmin[C];
     const int e0 = g.off[p], e1 = g.off[p + 1];
     double2 xy0 = make_double2(0.0, 0.0);
     if ((INNER || LIMIT) && !g.hd) xy0 = g.xy[p];
+    auto half_offset = [&](int e, int64_t i) {
+        if (g.hd) return g.hd[e];
+        const double2 xyi = g.xy[i];
+        return make_double2(0.5 * (xyi.x - xy0.x), 0.5 * (xyi.y - xy0.y));
+    };
     if constexpr (!INNER) {
-        double q0[4];
-        load4(q, p, q0);
+        double q0[C];
+        gather_c<C>(q + 4 * p + k0, q0);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) sx[k] = sy[k] = 0.0;
-        auto add = [&](const double qi[4], double2 a) {
+        for (int k = 0; k < C; ++k) {
+            sx[k] = sy[k] = 0.0;
+            kmax[k] = kmin[k] = 0;
+        }
+        auto add = [&](const double *qi, double2 a) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const double dq = qi[k] - q0[k];
+            for (int k = 0; k < C; ++k) {
+                // on the integer pipe where that is exact (the same bits)
+                const double dq = fix_same_binade(qi[k], q0[k]) ? fix_difference(qi[k], q0[k]) : qi[k] - q0[k];
                 if constexpr (EXTR) {
                     const long long key = order_key(__double_as_longlong(dq));
                     kmax[k] = max(kmax[k], key);
@@ -184,8 +249,8 @@ __global__ void __launch_bounds__(128) k_qgrad(DevGeom g, const double *__restri
             }
         };
         for (int e = e0; e < e1; ++e) {
-            double qi[4];
-            load4(q, g.idx[e], qi);
+            double qi[C];
+            gather_c<C>(q + 4 * (int64_t)g.idx[e] + k0, qi);
             add(qi, g.lsw[e]);
         }
         if constexpr (KIN) {
@@ -195,35 +260,44 @@ __global__ void __launch_bounds__(128) k_qgrad(DevGeom g, const double *__restri
                 const double2 n0 = g.nrm[p];
                 const double *qf = g.qinf + 4 * (g.pcase ? (int)g.pcase[p] : 0);
                 for (int e = f0; e < f1; ++e) {
-                    double qi[4];
+                    double qi[4], qk[C];
                     image_q(g, e, g.imask[e], n0, qf, q, nullptr, make_double2(0.0, 0.0), false, qi);
-                    add(qi, g.ilsw[e]);
+                    components<C>(qi, k0, qk);
+                    add(qk, g.ilsw[e]);
                 }
             }
         }
     } else {
-        double t[8];
-        load8(g1, p, t);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            sx[k] = t[k];
-            sy[k] = t[4 + k];
-        }
+        gather_c<C>(g1 + 8 * p + k0, sx);
+        gather_c<C>(g1 + 8 * p + 4 + k0, sy);
         for (int e = e0; e < e1; ++e) {
-            const int i = g.idx[e];
+            const int64_t i = g.idx[e];
             const double2 a = g.lsw[e];
-            double2 h;
-            if (g.hd) {
-                h = g.hd[e];
+            double gx[C], gy[C];
+            gather_c<C>(qg_old + 8 * i + k0, gx);
+            gather_c<C>(qg_old + 8 * i + 4 + k0, gy);
+            // h . grad q_i in fixed point: half of the FP64 pipe's work moves to
+            // the integer pipes, which are idle otherwise
+            int64_t hx, hy;   // the half offset in its stored form, made here in mixed contexts
+            if (g.hfx) {
+                const longlong2 w = __ldg(g.hfx + e);
+                hx = w.x;
+                hy = w.y;
             } else {
-                const double2 xyi = g.xy[i];
-                h = make_double2(0.5 * (xyi.x - xy0.x), 0.5 * (xyi.y - xy0.y));
+                const double2 h = half_offset(e, i);
+                fix_pack_pair(h.x, h.y, hx, hy);
             }
-            double gi[8];
-            load8(qg_old, i, gi);
+            const FixPair hp = fix_unpack_pair(hx, hy);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const double c = fma(h.y, gi[4 + k], h.x * gi[k]);
+            for (int k = 0; k < C; ++k) {
+                const FixPair gp = fix_pair(gx[k], gy[k]);
+                double c = 0.0;
+                if (fix_dot_in_range(hp, gp)) {
+                    c = fix_dot(hp, gp);
+                } else if (gp.e) {
+                    const double2 h = half_offset(e, i);
+                    c = fma(h.y, gy[k], h.x * gx[k]);
+                }
                 sx[k] = fma(-a.x, c, sx[k]);
                 sy[k] = fma(-a.y, c, sy[k]);
             }
@@ -240,77 +314,81 @@ __global__ void __launch_bounds__(128) k_qgrad(DevGeom g, const double *__restri
                     const double2 a = g.ilsw[e];
                     double2 h = g.ihd[e];
                     reflect2(h.x, h.y, n0.x, n0.y);
-                    double gi[8], c[4];
+                    double gi[8], c[4], ck[C];
                     load8(qg_old, g.iidx[e], gi);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) c[k] = fma(-h.y, gi[4 + k], -h.x * gi[k]);
                     reflect2(c[1], c[2], n0.x, n0.y);
+                    components<C>(c, k0, ck);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        sx[k] = fma(a.x, c[k], sx[k]);
-                        sy[k] = fma(a.y, c[k], sy[k]);
+                    for (int k = 0; k < C; ++k) {
+                        sx[k] = fma(a.x, ck[k], sx[k]);
+                        sy[k] = fma(a.y, ck[k], sy[k]);
                     }
                 }
             }
         }
-        load8(qg_old, p, t);
+        double tx[C], ty[C];
+        gather_c<C>(qg_old + 8 * p + k0, tx);
+        gather_c<C>(qg_old + 8 * p + 4 + k0, ty);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            sx[k] = fma(0.5, t[k], sx[k]);
-            sy[k] = fma(0.5, t[4 + k], sy[k]);
+        for (int k = 0; k < C; ++k) {
+            sx[k] = fma(0.5, tx[k], sx[k]);
+            sy[k] = fma(0.5, ty[k], sy[k]);
         }
     }
     // x_m = min(D+, -D-) per component
-    double xm[4];
+    double xm[C];
     if constexpr (EXTR) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
+        for (int k = 0; k < C; ++k)
             xm[k] = __longlong_as_double((long long)min((unsigned long long)kmax[k],
                                                         abs_bits(__longlong_as_double(order_key(kmin[k])))));
     }
     if constexpr (LIMIT) {
-        if constexpr (INNER) load4(ext, p, xm);
-        unsigned long long dm[4] = {0, 0, 0, 0};   // bits of d_m (non-negative doubles order as integers)
+        if constexpr (INNER) gather_c<C>(ext + 4 * p + k0, xm);
+        unsigned long long dm[C];   // bits of d_m (non-negative doubles order as integers)
+#pragma unroll
+        for (int k = 0; k < C; ++k) dm[k] = 0;
         if (g.hd_f && e1 - e0 <= 32) {
-            largest_shift_screened(g, e0, e1, sx, sy, dm);
+            largest_shift_screened<C>(g, e0, e1, sx, sy, dm);
         } else {
             for (int e = e0; e < e1; ++e) {
-                double2 h;
-                if (g.hd) {
-                    h = g.hd[e];
-                } else {
-                    const double2 xyi = g.xy[g.idx[e]];
-                    h = make_double2(0.5 * (xyi.x - xy0.x), 0.5 * (xyi.y - xy0.y));
-                }
+                const double2 h = half_offset(e, g.idx[e]);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) dm[k] = max(dm[k], abs_bits(fma(h.x, sx[k], h.y * sy[k])));
+                for (int k = 0; k < C; ++k) dm[k] = max(dm[k], abs_bits(fma(h.x, sx[k], h.y * sy[k])));
             }
         }
         if constexpr (KIN) {
             for (int e = g.ioff[p]; e < g.ioff[p + 1]; ++e) {
                 const double2 h = g.ihd[e];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) dm[k] = max(dm[k], abs_bits(fma(h.x, sx[k], h.y * sy[k])));
+                for (int k = 0; k < C; ++k) dm[k] = max(dm[k], abs_bits(fma(h.x, sx[k], h.y * sy[k])));
             }
         }
         const double hK = g.dmin[p] * limK;
         const double eps2 = hK * hK * hK;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            // f(x, d) = N / M, N = x (x + 2d) + eps^2, M = x (x + d) + (2d^2 + eps^2),
-            // evaluated for every component (warps diverge on x < 2d anyway)
-            const double x = xm[k], d = __longlong_as_double((long long)dm[k]), d2 = 2.0 * d;
-            const double N = fma(x, x + d2, eps2);
-            const double M = fma(x, x + d, fma(d2, d, eps2));
-            const double phi = x < d2 ? N * rcp_newton(M) : 1.0;
+        for (int k = 0; k < C; ++k) {
+            // f(x, d) = N / M, N = x (x + 2d) + eps^2, M = x (x + d) + (2d^2 + eps^2):
+            // in fixed point (13 FP64 instructions fewer per component), in FP64
+            // for extreme exponents. Non-negative doubles order as their bits.
+            const double x = xm[k], d = __longlong_as_double((long long)dm[k]);
+            double phi = 1.0;
+            if (fix_phi_in_range(d, eps2)) {
+                if (__double_as_longlong(x) < (long long)dm[k] + (1ll << 52)) phi = fix_phi(x, d, eps2);
+            } else if (x < 2.0 * d) {
+                const double N = fma(x, x + 2.0 * d, eps2);
+                phi = N * rcp_newton(fma(x, x + d, fma(2.0 * d, d, eps2)));
+            }
             sx[k] *= phi;
             sy[k] *= phi;
         }
     } else if constexpr (EXTR) {
-        store4(ext, p, xm);
+        store_c<C>(ext + 4 * p + k0, xm);
     }
-    double out[8] = {sx[0], sx[1], sx[2], sx[3], sy[0], sy[1], sy[2], sy[3]};
-    store8(qg_new, p, out);
+    store_c<C>(qg_new + 8 * p + k0, sx);
+    store_c<C>(qg_new + 8 * p + 4 + k0, sy);
 }
 
 // --------------------------------------------------------------------------
@@ -347,171 +425,12 @@ __device__ __forceinline__ void flag_nonphysical(int *status, int64_t p)
     atomicMin(status + 1, (int)p);
 }
 
-// One member's term of E11, w_s [Gs(q~_i) - Gs(q~_0)] + w_n [Gn(q~_i) - Gn(q~_0)],
-// Gs = Gx+ or Gx- and Gn = Gy+ or Gy- by the member's sub-stencil bits m,
-// in the frame (t, n) of P_0: [mass, s-momentum, n-momentum, energy].
-struct EdgeTerm {
-    double R[4];
-    bool ok;
-};
-struct Vec4 {
-    double v[4];
-};
-
-// in FP64: states outside the fixed-point form's ranges, and gamma != 1.4.
-// Not inlined: it keeps its registers out of the loop that hardly ever calls it.
-__device__ __noinline__ EdgeTerm edge_term_fp64(Vec4 qi, Vec4 q0, uint32_t m, double2 w, double2 n0, Gas gas)
-{
-    const double *qti = qi.v, *qt0 = q0.v;
-    const double tx = n0.y, ty = -n0.x;
-    EdgeTerm o = {{0.0, 0.0, 0.0, 0.0}, true};
-    Prim si, s0;
-    o.ok &= prim_from_q(qti, gas, tx, ty, n0, si);
-    o.ok &= prim_from_q(qt0, gas, tx, ty, n0, s0);
-    const double us_i = si.us, un_i = si.un, us_0 = s0.us, un_0 = s0.un;
-    // w != 0 tested on the bits (integer pipe; +-0 are the zeros)
-    if ((__double_as_longlong(w.x) & ~(long long)kSignBit) != 0) {
-        const unsigned long long sg = (m & M_XPOS) ? 0ull : kSignBit;
-        double Gi[4], G0[4];
-        split_flux(sg, si, us_i, un_i, si.Ss, Gi);
-        split_flux(sg, s0, us_0, un_0, s0.Ss, G0);
-        // dG = G(q~_i) - G(q~_0) from the two rounded fluxes: an unfused
-        // subtraction, so equal states give exactly zero (a contracted
-        // fma(rho_i, m_i, -rho_0 m_0) would leave a product's rounding)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o.R[k] += w.x * __dsub_rn(Gi[k], G0[k]);
-    }
-    if ((__double_as_longlong(w.y) & ~(long long)kSignBit) != 0) {
-        const unsigned long long sg = (m & M_YPOS) ? 0ull : kSignBit;
-        double Gi[4], G0[4];
-        split_flux(sg, si, un_i, us_i, si.Sn, Gi);
-        split_flux(sg, s0, un_0, us_0, s0.Sn, G0);
-        // Gn components are [mass, n-momentum, s-momentum, energy]
-        o.R[0] += w.y * __dsub_rn(Gi[0], G0[0]);
-        o.R[1] += w.y * __dsub_rn(Gi[2], G0[2]);
-        o.R[2] += w.y * __dsub_rn(Gi[1], G0[1]);
-        o.R[3] += w.y * __dsub_rn(Gi[3], G0[3]);
-    }
-    return o;
-}
-
-// The member's term added into R: in fixed point (lskum_fixed.cuh) where both
-// states lie in its ranges, else in FP64. nx, ny: the normal n0 in fixed point.
-__device__ __forceinline__ void edge_residual(const double qti[4], const double qt0[4], uint8_t m, double2 w,
-                                              double2 n0, FixOp nx, FixOp ny, const Gas &gas, double R[4], bool &ok)
-{
-    // equal reconstructed states have dG = 0 exactly (compared as bit patterns,
-    // on the integer pipe; +0 against -0 only costs a flux evaluation giving dG = 0)
-    if (((__double_as_longlong(qti[0]) ^ __double_as_longlong(qt0[0])) |
-         (__double_as_longlong(qti[1]) ^ __double_as_longlong(qt0[1])) |
-         (__double_as_longlong(qti[2]) ^ __double_as_longlong(qt0[2])) |
-         (__double_as_longlong(qti[3]) ^ __double_as_longlong(qt0[3]))) == 0)
-        return;
-    FixState si, s0;
-    const bool in_range = fix_state(qti, nx, ny, si) & fix_state(qt0, nx, ny, s0);
-    if (gas.g14 && in_range) {
-        FixEdge g;
-        fix_edge(si, s0, g);
-        double dG[4];
-        if ((__double_as_longlong(w.x) & ~(long long)kSignBit) != 0) {
-            const bool plus = (m & M_XPOS) != 0;
-            fix_flux_difference(g, si, s0, true, plus ? 0 : -1, dG);
-            const double ws = flip_sign(w.x, plus ? 0ull : kSignBit);
-            R[0] = fma(ws, dG[0], R[0]);
-            R[1] = fma(w.x, dG[1], R[1]);
-            R[2] = fma(ws, dG[2], R[2]);
-            R[3] = fma(ws, dG[3], R[3]);
-        }
-        if ((__double_as_longlong(w.y) & ~(long long)kSignBit) != 0) {
-            const bool plus = (m & M_YPOS) != 0;
-            fix_flux_difference(g, si, s0, false, plus ? 0 : -1, dG);
-            const double ws = flip_sign(w.y, plus ? 0ull : kSignBit);
-            R[0] = fma(ws, dG[0], R[0]);
-            R[1] = fma(ws, dG[2], R[1]);   // the s-momentum is the transverse one here
-            R[2] = fma(w.y, dG[1], R[2]);
-            R[3] = fma(ws, dG[3], R[3]);
-        }
-        return;
-    }
-    const EdgeTerm o = edge_term_fp64(Vec4{{qti[0], qti[1], qti[2], qti[3]}}, Vec4{{qt0[0], qt0[1], qt0[2], qt0[3]}}, m, w,
-                                      n0, gas);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) R[k] += o.R[k];
-    ok &= o.ok;
-}
-
+// The residual R of point p (one lane per point, whole warps of consecutive
+// points): written out, or the time step, the state update and the residue partials
 template <bool KIN>
-__global__ void __launch_bounds__(128) k_flux_update(FluxParams P)
+__device__ __forceinline__ void state_update(const FluxParams &P, int64_t p, bool live, uint8_t flag, const double Rg[4])
 {
     const DevGeom &g = P.g;
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double Rg[4] = {0.0, 0.0, 0.0, 0.0};
-    const bool live = p < g.n;
-    uint8_t flag = FLAG_FARFIELD;
-    if (live) flag = g.flag[p] & 3;  // bit 7 marks FP64 closures in mixed contexts
-    // far-field points are held at the free stream, except in the kinetic boundary mode
-    if (live && (flag != FLAG_FARFIELD || KIN)) {
-        const double2 xy0 = g.xy[p];
-        const double2 n0 = g.nrm[p];
-        const double tx = n0.y, ty = -n0.x;
-        const FixOp fnx = fix_op(fix_unit(n0.x)), fny = fix_op(fix_unit(n0.y));
-        double q0[4], g0[8];
-        load4(P.q, p, q0);
-        const bool second = P.order == 2;
-        if (second) load8(P.qg, p, g0);
-        double R[4] = {0.0, 0.0, 0.0, 0.0};
-        bool ok = true;
-        const int e0 = g.off[p], e1 = g.off[p + 1];
-        for (int e = e0; e < e1; ++e) {
-            const double2 w = g.fxw[e];
-            // weights outside every needed sub-stencil are +0 exactly: tested on the bits
-            if ((__double_as_longlong(w.x) | __double_as_longlong(w.y)) == 0) continue;
-            const int i = g.idx[e];
-            const uint8_t m = g.mask[e];
-            double qti[4], qt0[4];
-            load4(P.q, i, qti);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) qt0[k] = q0[k];
-            if (second) {
-                double2 h;
-                if (g.hd) {
-                    h = g.hd[e];
-                } else {
-                    const double2 xyi = g.xy[i];
-                    h = make_double2(0.5 * (xyi.x - xy0.x), 0.5 * (xyi.y - xy0.y));
-                }
-                double gi[8];
-                load8(P.qg, i, gi);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    qti[k] = fma(-h.y, gi[4 + k], fma(-h.x, gi[k], qti[k]));
-                    qt0[k] = fma(-h.y, g0[4 + k], fma(-h.x, g0[k], qt0[k]));
-                }
-            }
-            edge_residual(qti, qt0, m, w, n0, fnx, fny, P.gas, R, ok);
-        }
-        if constexpr (KIN) {
-            // kinetic boundary mode: the mirror images of the neighbours
-            const int f0 = g.ioff[p], f1 = g.ioff[p + 1];
-            const double *qf = g.qinf + 4 * (g.pcase ? (int)g.pcase[p] : 0);
-            for (int e = f0; e < f1; ++e) {
-                const double2 w = g.ifxw[e];
-                const uint8_t m = g.imask[e];
-                const double2 hs = g.ihd[e];
-                double qti[4], qt0[4];
-                image_q(g, e, m, n0, qf, P.q, P.qg, hs, second, qti);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) qt0[k] = second ? fma(-hs.y, g0[4 + k], fma(-hs.x, g0[k], q0[k])) : q0[k];
-                edge_residual(qti, qt0, m, w, n0, fnx, fny, P.gas, R, ok);
-            }
-        }
-        if (!ok) flag_nonphysical(P.status, p);
-        Rg[0] = R[0];
-        Rg[1] = R[1] * tx + R[2] * n0.x;
-        Rg[2] = R[1] * ty + R[2] * n0.y;
-        Rg[3] = R[3];
-    }
-
     if (P.mode == 0) {
         if (live) store4(P.R, p, Rg);
         return;
@@ -578,6 +497,382 @@ __global__ void __launch_bounds__(128) k_flux_update(FluxParams P)
 
     // ---- residue partials: a pair of R_rho^2 sums per warp, at stage 0 ----
     if (P.mode == 1 || P.stage == 0) warp_residue_pair(P.pcase, p, live, Rg[0] * Rg[0], P.norm_part);
+}
+
+// One member's term of E11 is w_s [Gs(q~_i) - Gs(q~_0)] + w_n [Gn(q~_i) - Gn(q~_0)],
+// Gs = Gx+ or Gx- and Gn = Gy+ or Gy- by the member's sub-stencil bits m, in
+// the frame (t, n) of P_0.
+struct Vec4 {
+    double v[4];
+};
+struct FluxDifference {
+    double d[4];
+    bool ok;
+};
+
+// G(q~_i) - G(q~_0) along t or n, [mass, along, transverse, energy], in FP64:
+// for states outside the fixed-point form's ranges. Not inlined: it keeps its
+// registers out of the loop that hardly ever calls it. The difference is an
+// unfused subtraction of the two rounded fluxes, so equal states give exactly
+// zero (a contracted fma(rho_i, m_i, -rho_0 m_0) would leave a product's rounding).
+__device__ __noinline__ FluxDifference flux_difference_fp64(Vec4 qi, Vec4 q0, bool along_t, unsigned long long sbit,
+                                                            double2 n0, Gas gas)
+{
+    FluxDifference o = {{0.0, 0.0, 0.0, 0.0}, true};
+    Prim si, s0;
+    o.ok &= prim_from_q(qi.v, gas, n0.y, -n0.x, n0, si);
+    o.ok &= prim_from_q(q0.v, gas, n0.y, -n0.x, n0, s0);
+    double Gi[4], G0[4];
+    split_flux(sbit, si, along_t ? si.us : si.un, along_t ? si.un : si.us, along_t ? si.Ss : si.Sn, Gi);
+    split_flux(sbit, s0, along_t ? s0.us : s0.un, along_t ? s0.un : s0.us, along_t ? s0.Ss : s0.Sn, G0);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) o.d[k] = __dsub_rn(Gi[k], G0[k]);
+    return o;
+}
+
+// the member's whole term in FP64 by one lane (gamma != 1.4), R in the order
+// [mass, s-momentum, n-momentum, energy]
+__device__ __forceinline__ void edge_residual(const double qti[4], const double qt0[4], uint8_t m, double2 w,
+                                              double2 n0, double tx, double ty, const Gas &gas, double R[4],
+                                              bool &ok)
+{
+    // equal reconstructed states have dG = 0 exactly (compared as bit patterns,
+    // on the integer pipe; +0 against -0 only costs a flux evaluation giving dG = 0)
+    if (((__double_as_longlong(qti[0]) ^ __double_as_longlong(qt0[0])) |
+         (__double_as_longlong(qti[1]) ^ __double_as_longlong(qt0[1])) |
+         (__double_as_longlong(qti[2]) ^ __double_as_longlong(qt0[2])) |
+         (__double_as_longlong(qti[3]) ^ __double_as_longlong(qt0[3]))) == 0)
+        return;
+    Prim si, s0;
+    ok &= prim_from_q(qti, gas, tx, ty, n0, si);
+    ok &= prim_from_q(qt0, gas, tx, ty, n0, s0);
+    // w != 0 tested on the bits (integer pipe; +-0 are the zeros)
+    if ((__double_as_longlong(w.x) & ~(long long)kSignBit) != 0) {
+        const unsigned long long sg = (m & M_XPOS) ? 0ull : kSignBit;
+        double Gi[4], G0[4];
+        split_flux(sg, si, si.us, si.un, si.Ss, Gi);
+        split_flux(sg, s0, s0.us, s0.un, s0.Ss, G0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) R[k] += w.x * __dsub_rn(Gi[k], G0[k]);
+    }
+    if ((__double_as_longlong(w.y) & ~(long long)kSignBit) != 0) {
+        const unsigned long long sg = (m & M_YPOS) ? 0ull : kSignBit;
+        double Gi[4], G0[4];
+        split_flux(sg, si, si.un, si.us, si.Sn, Gi);
+        split_flux(sg, s0, s0.un, s0.us, s0.Sn, G0);
+        // Gn components are [mass, n-momentum, s-momentum, energy]
+        R[0] += w.y * __dsub_rn(Gi[0], G0[0]);
+        R[1] += w.y * __dsub_rn(Gi[2], G0[2]);
+        R[2] += w.y * __dsub_rn(Gi[1], G0[1]);
+        R[3] += w.y * __dsub_rn(Gi[3], G0[3]);
+    }
+}
+
+__device__ __forceinline__ uint32_t other_lane(uint32_t v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ int64_t other_lane(int64_t v)
+{
+    const uint32_t lo = other_lane((uint32_t)v), hi = other_lane((uint32_t)((uint64_t)v >> 32));
+    return (int64_t)(((uint64_t)hi << 32) | lo);
+}
+__device__ __forceinline__ double other_lane(double v)
+{
+    return __longlong_as_double(other_lane((int64_t)__double_as_longlong(v)));
+}
+
+// One member of a point's stencil, evaluated by two neighbouring lanes: lane 0
+// holds the neighbour's reconstructed state, lane 1 the point's own one (qt).
+// Each turns its state into fixed point and forms the products c F of both
+// directions; then lane 0 takes the difference of the fluxes along t, lane 1
+// that along n: d = [mass, along, transverse, energy]. Called by whole warps;
+// act is the same in both lanes of a pair, and pairs without a member
+// (act = false) take part in the shuffles only and get d = 0.
+__device__ __forceinline__ void member_difference(bool act, int l, const double qt[4], uint32_t m, double2 w, double2 n0,
+                                                  FixOp nx, FixOp ny, const Gas &gas, double d[4], bool &ok)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) d[k] = 0.0;
+    // equal reconstructed states have dG = 0 exactly (compared as bit patterns);
+    // the last component decides almost always
+    // (every lane takes part in every shuffle and vote: no && or ?: before them)
+    const int64_t other3 = other_lane((int64_t)__double_as_longlong(qt[3]));
+    bool differ = act && other3 != __double_as_longlong(qt[3]);
+    if (__any_sync(0xffffffffu, act && !differ)) {
+        bool any = false;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int64_t o = other_lane((int64_t)__double_as_longlong(qt[k]));
+            any |= o != __double_as_longlong(qt[k]);
+        }
+        differ = act && (differ || any);
+    }
+    if (!__any_sync(0xffffffffu, differ)) return;
+    const bool xp = (m & M_XPOS) != 0, yp = (m & M_YPOS) != 0;
+    const unsigned long long sbit = (l ? yp : xp) ? 0ull : kSignBit;   // of this lane's direction
+    FixState s;
+    bool fixed = fix_state(qt, nx, ny, s);
+    const uint32_t other_fixed = other_lane((uint32_t)fixed);
+    fixed = fixed && other_fixed != 0;
+    if (__any_sync(0xffffffffu, differ && fixed)) {
+        if (!fixed) s.St = s.Sn = 0;   // an index of the tables; the result is not used
+        // the two states' factors at common exponents
+        const int en = (int)other_lane((uint32_t)s.n), ek = (int)other_lane((uint32_t)s.k);
+        int e0, e1, e3;
+        const int64_t c0 = fix_align_half(s.c0, fix_e0(s.n, s.k), fix_e0(en, ek), e0);
+        const int64_t c1 = fix_align_half(s.c1, fix_e1(s.n, s.k), fix_e1(en, ek), e1);
+        const int64_t c3 = fix_align_half(s.c3, fix_e3(s.n, s.k), fix_e3(en, ek), e3);
+        const int z0 = fix_top(c0, other_lane((uint32_t)((uint64_t)c0 >> 32)));
+        const int z1 = fix_top(c1, other_lane((uint32_t)((uint64_t)c1 >> 32)));
+        const int z3 = fix_top(c3, other_lane((uint32_t)((uint64_t)c3 >> 32)));
+        const FixOp o0 = fix_op(c0 << z0), o1 = fix_op(c1 << z1), o3 = fix_op(c3 << z3);
+        int64_t Ft[4], Fn[4];
+        fix_parts(s.St, xp ? 0 : -1, s.Sn, s.H, Ft);
+        fix_scale(o0, o1, o3, Ft);
+        fix_parts(s.Sn, yp ? 0 : -1, s.St, s.H, Fn);
+        fix_scale(o0, o1, o3, Fn);
+        // lane 0: G_t(neighbour) - G_t(own), lane 1: G_n(neighbour) - G_n(own);
+        // the products lack the factor sgn of components 0, 2 and 3
+        const bool use = differ && fixed;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t r = other_lane(l ? Ft[k] : Fn[k]);
+            const double v =
+                fix_to_double(l ? r - Fn[k] : Ft[k] - r, k == 0 ? e0 - z0 + 2 : k == 3 ? e3 - z3 + 5 : e1 - z1 + 4);
+            if (use) d[k] = k == 1 ? v : flip_sign(v, sbit);
+        }
+    }
+    const bool slow = differ && !fixed;
+    if (__any_sync(0xffffffffu, slow)) {
+        Vec4 qi, q0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double r = other_lane(qt[k]);
+            qi.v[k] = l ? r : qt[k];
+            q0.v[k] = l ? qt[k] : r;
+        }
+        if (slow) {
+            const FluxDifference f = flux_difference_fp64(qi, q0, l == 0, sbit, n0, gas);
+            // (a direction of weight zero adds nothing, whatever its difference)
+            if ((__double_as_longlong(l ? w.y : w.x) & ~(long long)kSignBit) != 0) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) d[k] = f.d[k];
+            }
+            ok &= f.ok;
+        }
+    }
+}
+
+// A[k] += w d[k] of the group's members in row order: the own one (PAIRS = 1),
+// or those that the PAIRS pairs of a point hold, one each
+template <int PAIRS>
+__device__ __forceinline__ void add_members(double w, const double d[4], double A[4])
+{
+    if constexpr (PAIRS == 1) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) A[k] = fma(w, d[k], A[k]);
+    } else {
+        const int l = threadIdx.x & 1;
+#pragma unroll
+        for (int j = 0; j < PAIRS; ++j) {
+            const double wj = __shfl_sync(0xffffffffu, w, 2 * j + l, 2 * PAIRS);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) A[k] = fma(wj, __shfl_sync(0xffffffffu, d[k], 2 * j + l, 2 * PAIRS), A[k]);
+        }
+    }
+}
+
+// What bounds it: the FP64 pipe (76 % busy: the reconstruction, the sums, the
+// state update) and the integer ALUs (52 %), 62 % of the issue slots. 64
+// registers and a few spills, for 32 warps per SM, beat 80 (24 warps) and 128
+// (16): 2.30 / 2.48 / 2.67 ms at 2.5 million points. One lane per member with
+// both states took 2.58 ms and a chain twice as long.
+// Two lanes per member (member_difference), PAIRS pairs of lanes per point. With
+// one pair the members of a row follow one another; with 2 or 4 each pair takes
+// every second or fourth, and the differences are added in row order all the
+// same (add_members), so that a small cloud spreads over more warps with a
+// fraction of the serial chain and every launch gives the same bits. The state
+// update runs afterwards with one lane per point (R through shared memory).
+template <int PAIRS>
+struct FluxShape {
+    static constexpr int kThreads = PAIRS == 4 ? 256 : 128, kPoints = kThreads / (2 * PAIRS);
+    static_assert(kPoints % 32 == 0, "whole warps of points");
+};
+template <bool KIN, int PAIRS>
+__global__ void __launch_bounds__(FluxShape<PAIRS>::kThreads, PAIRS == 1 ? 8 : PAIRS == 2 ? 6 : 2) k_flux_update(FluxParams P)
+{
+    constexpr int POINTS = FluxShape<PAIRS>::kPoints;
+    __shared__ double2 s_R[POINTS][2];
+    const DevGeom &g = P.g;
+    {
+        const int l = threadIdx.x & 1, pair = (threadIdx.x >> 1) % PAIRS, pt = threadIdx.x / (2 * PAIRS);
+        const int64_t pp = (int64_t)blockIdx.x * POINTS + pt, p = pp < g.n ? pp : g.n - 1;
+        const uint8_t flag = g.flag[p] & 3;  // bit 7 marks FP64 closures in mixed contexts
+        // far-field points are held at the free stream, except in the kinetic boundary mode
+        const bool work = pp < g.n && (flag != FLAG_FARFIELD || KIN);
+        const double2 n0 = g.nrm[p];
+        const FixOp fnx = fix_op(fix_unit(n0.x)), fny = fix_op(fix_unit(n0.y));
+        const bool second = P.order == 2;
+        const int e0 = g.off[p], deg = work ? g.off[p + 1] - e0 : 0;
+        double2 xy0 = make_double2(0.0, 0.0);
+        if (second && !g.hd) xy0 = g.xy[p];
+        double A[4] = {0.0, 0.0, 0.0, 0.0};
+        bool ok = true;
+        // whole warps go through the longest row's rounds: the members exchange by shuffles
+        const int most = __reduce_max_sync(0xffffffffu, (deg + PAIRS - 1) / PAIRS);
+#pragma unroll 1
+        for (int r = 0; r < most; ++r) {
+            const int j = r * PAIRS + pair;
+            const int e = j < deg ? e0 + j : e0;
+            const double2 w = g.fxw[e];
+            // weights outside every needed sub-stencil are +0 exactly: tested on the bits
+            const bool act = j < deg && (__double_as_longlong(w.x) | __double_as_longlong(w.y)) != 0;
+            const int i = g.idx[e];
+            const int64_t row = l ? p : (int64_t)i;
+            double qt[4], d[4];
+            gather4(P.q, row, qt);
+            if (second) {
+                double2 h;
+                if (g.hd) {
+                    h = g.hd[e];
+                } else {
+                    const double2 xyi = g.xy[i];
+                    h = make_double2(0.5 * (xyi.x - xy0.x), 0.5 * (xyi.y - xy0.y));
+                }
+                double gr[8];
+                gather8(P.qg, row, gr);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) qt[k] = fma(-h.y, gr[4 + k], fma(-h.x, gr[k], qt[k]));
+            }
+            member_difference(act, l, qt, g.mask[e], w, n0, fnx, fny, P.gas, d, ok);
+            add_members<PAIRS>(l ? w.y : w.x, d, A);
+        }
+        if constexpr (KIN) {
+            // kinetic boundary mode: the mirror images of the neighbours
+            const int f0 = g.ioff[p], nim = work ? g.ioff[p + 1] - f0 : 0;
+            const int imost = __reduce_max_sync(0xffffffffu, (nim + PAIRS - 1) / PAIRS);
+            const double *qf = g.qinf + 4 * (g.pcase ? (int)g.pcase[p] : 0);
+#pragma unroll 1
+            for (int r = 0; r < imost; ++r) {
+                const int j = r * PAIRS + pair;
+                const bool act = j < nim;
+                double2 w = make_double2(0.0, 0.0);
+                uint8_t m = 0;
+                double qt[4], d[4];
+                gather4(P.q, p, qt);
+                if (act) {
+                    const int e = f0 + j;
+                    w = g.ifxw[e];
+                    m = g.imask[e];
+                    const double2 hs = g.ihd[e];
+                    if (l == 0) {
+                        image_q(g, e, m, n0, qf, P.q, P.qg, hs, second, qt);
+                    } else if (second) {
+                        double gr[8];
+                        gather8(P.qg, p, gr);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) qt[k] = fma(-hs.y, gr[4 + k], fma(-hs.x, gr[k], qt[k]));
+                    }
+                }
+                member_difference(act, l, qt, m, w, n0, fnx, fny, P.gas, d, ok);
+                add_members<PAIRS>(l ? w.y : w.x, d, A);
+            }
+        }
+        if (!ok) flag_nonphysical(P.status, p);
+        // lane 0 holds the sums along t, lane 1 those along n: R in the order
+        // [mass, s-momentum, n-momentum, energy]
+        double N[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) N[k] = other_lane(A[k]);
+        if (threadIdx.x % (2 * PAIRS) == 0) {
+            const double Rs = A[1] + N[2], Rn = A[2] + N[1];
+            const double tx = n0.y, ty = -n0.x;
+            s_R[pt][0] = make_double2(A[0] + N[0], Rs * tx + Rn * n0.x);
+            s_R[pt][1] = make_double2(Rs * ty + Rn * n0.y, A[3] + N[3]);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x >= POINTS) return;
+    const int64_t p = (int64_t)blockIdx.x * POINTS + threadIdx.x;
+    const bool live = p < g.n;
+    const uint8_t flag = live ? g.flag[p] & 3 : FLAG_FARFIELD;
+    const double2 R01 = s_R[threadIdx.x][0], R23 = s_R[threadIdx.x][1];
+    const double Rg[4] = {R01.x, R01.y, R23.x, R23.y};
+
+    state_update<KIN>(P, p, live, flag, Rg);
+}
+
+// One lane per point, all in FP64: gamma != 1.4, which the fixed-point form does
+// not cover
+template <bool KIN>
+__global__ void __launch_bounds__(128) k_flux_update_fp64(FluxParams P)
+{
+    const DevGeom &g = P.g;
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    double Rg[4] = {0.0, 0.0, 0.0, 0.0};
+    const bool live = p < g.n;
+    uint8_t flag = FLAG_FARFIELD;
+    if (live) flag = g.flag[p] & 3;  // bit 7 marks FP64 closures in mixed contexts
+    // far-field points are held at the free stream, except in the kinetic boundary mode
+    if (live && (flag != FLAG_FARFIELD || KIN)) {
+        const double2 xy0 = g.xy[p];
+        const double2 n0 = g.nrm[p];
+        const double tx = n0.y, ty = -n0.x;
+        double q0[4], g0[8];
+        load4(P.q, p, q0);
+        const bool second = P.order == 2;
+        if (second) load8(P.qg, p, g0);
+        double R[4] = {0.0, 0.0, 0.0, 0.0};
+        bool ok = true;
+        const int e0 = g.off[p], e1 = g.off[p + 1];
+        for (int e = e0; e < e1; ++e) {
+            const double2 w = g.fxw[e];
+            // weights outside every needed sub-stencil are +0 exactly: tested on the bits
+            if ((__double_as_longlong(w.x) | __double_as_longlong(w.y)) == 0) continue;
+            const int i = g.idx[e];
+            const uint8_t m = g.mask[e];
+            double qti[4], qt0[4];
+            load4(P.q, i, qti);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) qt0[k] = q0[k];
+            if (second) {
+                double2 h;
+                if (g.hd) {
+                    h = g.hd[e];
+                } else {
+                    const double2 xyi = g.xy[i];
+                    h = make_double2(0.5 * (xyi.x - xy0.x), 0.5 * (xyi.y - xy0.y));
+                }
+                double gi[8];
+                load8(P.qg, i, gi);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    qti[k] = fma(-h.y, gi[4 + k], fma(-h.x, gi[k], qti[k]));
+                    qt0[k] = fma(-h.y, g0[4 + k], fma(-h.x, g0[k], qt0[k]));
+                }
+            }
+            edge_residual(qti, qt0, m, w, n0, tx, ty, P.gas, R, ok);
+        }
+        if constexpr (KIN) {
+            // kinetic boundary mode: the mirror images of the neighbours
+            const int f0 = g.ioff[p], f1 = g.ioff[p + 1];
+            const double *qf = g.qinf + 4 * (g.pcase ? (int)g.pcase[p] : 0);
+            for (int e = f0; e < f1; ++e) {
+                const double2 w = g.ifxw[e];
+                const uint8_t m = g.imask[e];
+                const double2 hs = g.ihd[e];
+                double qti[4], qt0[4];
+                image_q(g, e, m, n0, qf, P.q, P.qg, hs, second, qti);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) qt0[k] = second ? fma(-hs.y, g0[4 + k], fma(-hs.x, g0[k], q0[k])) : q0[k];
+                edge_residual(qti, qt0, m, w, n0, tx, ty, P.gas, R, ok);
+            }
+        }
+        if (!ok) flag_nonphysical(P.status, p);
+        Rg[0] = R[0];
+        Rg[1] = R[1] * tx + R[2] * n0.x;
+        Rg[2] = R[1] * ty + R[2] * n0.y;
+        Rg[3] = R[3];
+    }
+    state_update<KIN>(P, p, live, flag, Rg);
 }
 
 // residue() of every case = sqrt(sum R_rho^2)/n_case from the per-warp
@@ -706,17 +1001,17 @@ __global__ void __launch_bounds__(256) k_forces(int64_t nwall, Gas gas, double q
 // ----------------------------------------------------------------------------
 static inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
-template <bool KIN>
+template <bool KIN, int LANES>
 static void qgrad_pass(int pass, const DevGeom &g, const double *q, const double *qg_old, const double *g1,
                        double *qg_new, double *ext, double limK, cudaStream_t s)
 {
-    const unsigned nb = blocks_for(g.n, 128);
+    const unsigned nb = blocks_for(LANES * g.n, 128);
     switch (pass) {
-    case 0: k_qgrad<KIN, 0><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
-    case QG_EXTREMA: k_qgrad<KIN, QG_EXTREMA><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
-    case QG_LIMIT: k_qgrad<KIN, QG_LIMIT><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
-    case QG_INNER: k_qgrad<KIN, QG_INNER><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
-    default: k_qgrad<KIN, QG_INNER | QG_LIMIT><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
+    case 0: k_qgrad<KIN, 0, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
+    case QG_EXTREMA: k_qgrad<KIN, QG_EXTREMA, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
+    case QG_LIMIT: k_qgrad<KIN, QG_LIMIT, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
+    case QG_INNER: k_qgrad<KIN, QG_INNER, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
+    default: k_qgrad<KIN, QG_INNER | QG_LIMIT, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
     }
 }
 
@@ -726,12 +1021,34 @@ cudaError_t launch_qgrad(const DevGeom &g, const double *q, const double *qg_old
     const bool inner = qg_old != nullptr, limit = limiter_K > 0.0;
     if (inner && (!g1 || (limit && !ext))) return cudaErrorInvalidValue;
     const int pass = inner ? (QG_INNER | (limit ? QG_LIMIT : 0)) : limit ? QG_LIMIT : ext ? QG_EXTREMA : 0;
-    if (g.ioff) qgrad_pass<true>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, s);
-    else qgrad_pass<false>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, s);
+    // Lanes per point (the same bits either way). A small cloud is bound by the
+    // serial chain of a warp and by idle SMs, and 4 lanes shorten the one and
+    // fill the other: pass average 14.8 against 18.9 us at 3k points, 18.4
+    // against 19.4 at 40k. From 64k on (23.8 against 23.3 us; 0.497 against 0.444 ms at
+    // 2.5M) the index, weight and offset work that every lane repeats counts
+    // more. One lane with all four components: 27 us at 3k, 0.450 ms at 2.5M.
+    const bool four = g.n < 60000;
+    if (g.ioff) {
+        if (four) qgrad_pass<true, 4>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, s);
+        else qgrad_pass<true, 2>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, s);
+    } else if (four) {
+        qgrad_pass<false, 4>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, s);
+    } else {
+        qgrad_pass<false, 2>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, s);
+    }
     return cudaGetLastError();
 }
 
 int64_t residue_parts(int64_t n) { return 2 * ((n + 31) / 32); }
+
+template <int PAIRS>
+static void flux_pairs(const FluxParams &P, cudaStream_t s)
+{
+    constexpr int T = FluxShape<PAIRS>::kThreads;
+    const unsigned nb = blocks_for(P.g.n, FluxShape<PAIRS>::kPoints);
+    if (P.g.ioff) k_flux_update<true, PAIRS><<<nb, T, 0, s>>>(P);
+    else k_flux_update<false, PAIRS><<<nb, T, 0, s>>>(P);
+}
 
 cudaError_t launch_flux(const DevGeom &g, const Gas &gas, const FluxLaunch &L, cudaStream_t s)
 {
@@ -742,8 +1059,21 @@ cudaError_t launch_flux(const DevGeom &g, const Gas &gas, const FluxLaunch &L, c
     P.dt = L.dt; P.R = L.R; P.norm_part = L.norm_part; P.status = L.status;
     P.pcase = L.pcase; P.case_uinf = L.case_uinf;
     P.cfl = L.cfl; P.order = L.order; P.mode = L.mode; P.stage = L.stage;
-    if (g.ioff) k_flux_update<true><<<blocks_for(g.n, 128), 128, 0, s>>>(P);
-    else k_flux_update<false><<<blocks_for(g.n, 128), 128, 0, s>>>(P);
+    // Pairs of lanes per point (the same bits whichever): more while the cloud
+    // leaves SMs idle and the launch is one warp's serial chain. 4 / 2 / 1 pairs
+    // take 31 / 42 / 69 us at 3k points, 42 / 48 / 71 at 10k, 64 / 49 / 65 at
+    // 20k, 99 / 76 / 80 at 40k and 145 / 103 / 99 at 64k, where every pair adds
+    // all members' terms again.
+    if (!gas.g14) {
+        if (g.ioff) k_flux_update_fp64<true><<<blocks_for(g.n, 128), 128, 0, s>>>(P);
+        else k_flux_update_fp64<false><<<blocks_for(g.n, 128), 128, 0, s>>>(P);
+    } else if (g.n < 14000) {
+        flux_pairs<4>(P, s);
+    } else if (g.n < 50000) {
+        flux_pairs<2>(P, s);
+    } else {
+        flux_pairs<1>(P, s);
+    }
     return cudaGetLastError();
 }
 

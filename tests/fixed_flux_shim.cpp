@@ -14,10 +14,31 @@ extern "C" void fixed_flux(long n, const double *qi, const double *q0, const dou
         const bool oi = fix_state(qi + 4 * e, a, b, si), o0 = fix_state(q0 + 4 * e, a, b, s0);
         ok[e] = oi && o0;
         if (!ok[e]) continue;
-        FixEdge g;
-        fix_edge(si, s0, g);
+        // the two states' factors at common exponents, as the two lanes of the kernel share them
+        int e0, e1, e3;
+        int64_t ci[3] = {si.c0, si.c1, si.c3}, c0[3] = {s0.c0, s0.c1, s0.c3};
+        const int ei[3] = {fix_e0(si.n, si.k), fix_e1(si.n, si.k), fix_e3(si.n, si.k)};
+        const int eo[3] = {fix_e0(s0.n, s0.k), fix_e1(s0.n, s0.k), fix_e3(s0.n, s0.k)};
+        int *ex[3] = {&e0, &e1, &e3};
+        const int up[3] = {2, 4, 5};
+        for (int j = 0; j < 3; ++j) {
+            ci[j] = fix_align_half(ci[j], ei[j], eo[j], *ex[j]);
+            c0[j] = fix_align_half(c0[j], eo[j], ei[j], *ex[j]);
+            const int z = fix_top(ci[j], (uint32_t)((uint64_t)c0[j] >> 32));
+            ci[j] <<= z;
+            c0[j] <<= z;
+            *ex[j] += up[j] - z;
+        }
+        const bool t = along[e] != 0;
+        const int64_t m = sgn[e] < 0 ? -1 : 0;
+        int64_t Fi[4], F0[4];
+        fix_parts(t ? si.St : si.Sn, m, t ? si.Sn : si.St, si.H, Fi);
+        fix_parts(t ? s0.St : s0.Sn, m, t ? s0.Sn : s0.St, s0.H, F0);
+        fix_scale(fix_op(ci[0]), fix_op(ci[1]), fix_op(ci[2]), Fi);
+        fix_scale(fix_op(c0[0]), fix_op(c0[1]), fix_op(c0[2]), F0);
+        const int es[4] = {e0, e1, e1, e3};
         double d[4];
-        fix_flux_difference(g, si, s0, along[e] != 0, sgn[e] < 0 ? -1 : 0, d);
+        for (int k = 0; k < 4; ++k) d[k] = fix_to_double(Fi[k] - F0[k], es[k]);
         const double s = sgn[e];
         dG[4 * e] = s * d[0];
         dG[4 * e + 1] = d[1];
@@ -41,14 +62,46 @@ extern "C" void fixed_exp(long n, const long long *x, long long *M, int *m)
     for (long e = 0; e < n; ++e) M[e] = fix_exp(x[e], m[e]);
 }
 
-// c F through fix_align and the last product: (ci, c0) at exponent 0 -> the aligned pair's high-word products with F
+// c F through fix_top and the last product: (ci, c0) at exponent 0 -> the aligned pair's high-word products with F
 extern "C" void fixed_scaled(long n, const long long *ci, const long long *c0, const long long *F, long long *gi,
                              long long *g0, int *ex)
 {
     for (long e = 0; e < n; ++e) {
         int64_t a = ci[e], b = c0[e];
-        ex[e] = fix_align(a, 0, b, 0);
+        const int z = fix_top(a, (uint32_t)((uint64_t)b >> 32));
+        a <<= z;
+        b <<= z;
+        ex[e] = -z;
         gi[e] = fix_mul(fix_op(a), fix_op(F[e]));
         g0[e] = fix_mul(fix_op(b), fix_op(F[e]));
+    }
+}
+
+// h . g of rows [hx, hy, gx, gy], h through its stored form; ok: in range
+extern "C" void fixed_dot(long n, const double *a, double *c, int *ok)
+{
+    for (long e = 0; e < n; ++e) {
+        int64_t wx, wy;
+        fix_pack_pair(a[4 * e], a[4 * e + 1], wx, wy);
+        const FixPair h = fix_unpack_pair(wx, wy), g = fix_pair(a[4 * e + 2], a[4 * e + 3]);
+        ok[e] = fix_dot_in_range(h, g);
+        c[e] = ok[e] ? fix_dot(h, g) : 0.0;
+    }
+}
+
+// f(x, d) of rows [x, d, eps2] where x < 2 d
+extern "C" void fixed_phi(long n, const double *a, double *f, int *ok)
+{
+    for (long e = 0; e < n; ++e) {
+        ok[e] = fix_phi_in_range(a[3 * e + 1], a[3 * e + 2]);
+        f[e] = ok[e] && a[3 * e] < 2.0 * a[3 * e + 1] ? fix_phi(a[3 * e], a[3 * e + 1], a[3 * e + 2]) : 1.0;
+    }
+}
+
+extern "C" void fixed_difference(long n, const double *a, double *d, int *ok)
+{
+    for (long e = 0; e < n; ++e) {
+        ok[e] = fix_same_binade(a[2 * e], a[2 * e + 1]);
+        d[e] = ok[e] ? fix_difference(a[2 * e], a[2 * e + 1]) : 0.0;
     }
 }

@@ -1,4 +1,6 @@
-"""The fixed-point split fluxes of the FP64 form (csrc/lskum_fixed.cuh).
+"""The fixed-point parts of the FP64 form (csrc/lskum_fixed.cuh): the split
+fluxes, and the dot products, differences and limiter quotients of the
+q-derivative passes.
 
 CPU: the header compiled for the host against multiple precision, over the
 range of states it accepts and at that range's edges, and the states it has to
@@ -17,6 +19,7 @@ import os
 import re
 import subprocess
 import sys
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -176,6 +179,74 @@ def test_words_at_the_ends_of_their_ranges(shim):
             assert abs(mp.ldexp(mp.mpf(int(got)), int(ex[e])) - mp.mpf(fac) * int(Fs[e]) / mp.mpf(2) ** 64) <= mp.ldexp(mp.mpf(1.25), int(ex[e])), e
 
 
+def _rows(shim, name, a):
+    out, ok = np.zeros(len(a)), np.zeros(len(a), dtype=np.int32)
+    a = np.ascontiguousarray(a)
+    getattr(shim.lib, name)(ctypes.c_long(len(a)), a.ctypes.data_as(ctypes.c_void_p), out.ctypes.data_as(ctypes.c_void_p),
+                            ok.ctypes.data_as(ctypes.c_void_p))
+    return out, ok.astype(bool)
+
+
+@pytest.mark.parametrize("spread", [0, 30, 120])
+def test_dot_products(shim, spread):
+    """h . g against exact rationals: the products' dropped words cost at most
+    2 units of 2^-58 |h||g| and the stored form of h 2^-57 of |h| (together
+    below 2^-55.4), then one rounding."""
+    rng = np.random.default_rng(5)
+    n = 3000
+    a = rng.standard_normal((n, 4)) * 2.0 ** rng.integers(-spread, spread + 1, (n, 4))
+    a[:50, 1], a[50:100, 2], a[100:150, 3], a[150:200, 2:] = 0.0, 0.0, 0.0, 0.0
+    a[200:400, 3] = -a[200:400, 0] * a[200:400, 2] / a[200:400, 1]     # cancelling sums
+    c, ok = _rows(shim, "fixed_dot", a)
+    assert ok[:150].all() and ok[200:].mean() > 0.9
+    for e in np.nonzero(ok)[0]:
+        h0, h1, g0, g1 = [Fraction(float(v)) for v in a[e]]
+        exact = h0 * g0 + h1 * g1
+        size = Fraction(float(np.hypot(a[e, 0], a[e, 1]))) * Fraction(float(np.hypot(a[e, 2], a[e, 3])))
+        assert abs(Fraction(float(c[e])) - exact) <= abs(exact) / 2 ** 53 + size * Fraction(1, 2 ** 55)
+
+
+def test_dot_product_range(shim):
+    # a non-finite gradient or too extreme an exponent is left to FP64
+    bad = [[1, 1, np.inf, 0], [1, 1, 0, np.nan], [1, 1, -np.inf, np.inf], [1e39, 1, 1, 1], [1e-39, 0, 1, 1],
+           [1, 1, 1e308, 0], [1, 1, 5e-324, 0], [1, 1, 1e-300, 0], [0, 0, 1, 1]]
+    assert not _rows(shim, "fixed_dot", np.array(bad, dtype=float))[1].any()
+
+
+@pytest.mark.parametrize("eps,d", [(-60, -10), (-10, -30), (-20, -10), (-500, -200)])
+def test_limiter_quotient(shim, eps, d):
+    """f(x, d) relative to exact rationals: operands within 2^-59, three
+    truncated products of order 2^-56 each over M >= 1/4, the reciprocal within
+    2^-60: below 2^-53, then one rounding."""
+    rng = np.random.default_rng(6)
+    n = 2000
+    D = rng.uniform(0.5, 2, n) * 2.0 ** rng.uniform(d - 5, d + 5, n)
+    X = 2 * D * rng.uniform(0, 1, n)
+    E = rng.uniform(0.5, 2, n) * 2.0 ** rng.uniform(eps - 10, eps + 10, n)
+    X[:100] = 0.0
+    E[100:200] = 0.0
+    X[200:300] = np.nextafter(2 * D[200:300], 0)
+    X[300:400] = D[300:400] * 2.0 ** rng.uniform(-60, -20, 100)
+    f, ok = _rows(shim, "fixed_phi", np.stack([X, D, E], axis=1))
+    assert ok.all() and np.all(f >= 0) and np.all(f <= 1)
+    for e in range(n):
+        x, dd, ep = Fraction(float(X[e])), Fraction(float(D[e])), Fraction(float(E[e]))
+        want = (x * (x + 2 * dd) + ep) / (x * (x + dd) + 2 * dd * dd + ep)
+        assert abs(Fraction(float(f[e])) - want) <= want * Fraction(2, 2 ** 53)
+
+
+def test_differences_are_exact(shim):
+    rng = np.random.default_rng(7)
+    a = rng.uniform(-4, 4, 4000)
+    b = np.concatenate([a[:2000] * (1 + 1e-3 * rng.uniform(-1, 1, 2000)), rng.uniform(-4, 4, 2000)])
+    b[:20] = a[:20]
+    d, ok = _rows(shim, "fixed_difference", np.stack([a, b], axis=1))
+    assert np.array_equal(ok, (np.signbit(a) == np.signbit(b)) & (np.frexp(a)[1] == np.frexp(b)[1]))
+    assert np.array_equal(d[ok], (a - b)[ok]) and not np.signbit(d[:20]).any()
+    special = np.array([[np.inf, np.inf], [np.nan, np.nan], [0.0, 0.0], [1e-310, 1e-310]])
+    assert not _rows(shim, "fixed_difference", special)[1].any()
+
+
 def test_tables_are_the_generator_output(tmp_path):
     pytest.importorskip("mpmath")
     work = tmp_path / "csrc"
@@ -215,3 +286,40 @@ def test_residual_across_the_range_matches_the_oracle(gamma, mach, boundary):
                             boundary=boundary, mach=0.8, aoa_deg=1.0)
     err = np.abs(R - Ro) / np.maximum(S, 1e-300)
     assert np.all(np.abs(R - Ro) <= 1e-12 * S), err.max()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("order,limiter,boundary", [(1, 0.0, 0), (2, 0.0, 0), (2, 1.0, 0), (2, 1.0, 1)])
+def test_every_launch_form_gives_the_same_bits(order, limiter, boundary):
+    """The FP64 kernels split a point over more lanes the smaller the cloud: 4,
+    2 or 1 pairs in the flux kernel, 4 or 2 lanes in the q-derivative passes.
+    A 3250-point cloud alone, beside 18k points and beside 64k points in one
+    batch (all three forms): bitwise the same states and residuals, and the
+    18k cloud's residual at the oracle's bar."""
+    import torch
+
+    import oracle
+    from paper_2403_13287_gb300.cloudgen import naca0012_cloud, smooth_state
+    from paper_2403_13287_gb300.lskum import Solver
+    a, mid, big = naca0012_cloud(130, 24, seed=11), naca0012_cloud(180, 99, seed=3, shuffle=True), naca0012_cloud(324, 197, seed=4)
+    kw = dict(order=order, inner_iters=3, time_scheme=1, limiter_K=limiter, precision=0, reorder=1, boundary=boundary)
+    U0 = {id(c): smooth_state(c, 0.85, 1.0, amp=0.05, seed=9) for c in (a, mid, big)}
+    got = []
+    for clouds in ([a], [a, mid], [a, mid, big], [mid]):
+        if len(clouds) > 1:
+            s = Solver.batch([(c, 0.85, 1.0) for c in clouds], **kw)
+        else:
+            s = Solver(clouds[0], mach=0.85, aoa_deg=1.0, **kw)
+        U = np.ascontiguousarray(np.concatenate([U0[id(c)] for c in clouds], axis=1))
+        R = s.residual(torch.from_numpy(U).cuda()).cpu().numpy()
+        s.set_state(U)
+        s.step(2)
+        got.append((R, s.get_state()))
+        s.close()
+    n, m = a["n"], mid["n"]
+    for R, V in got[1:3]:
+        assert np.array_equal(R[:, :n], got[0][0]) and np.array_equal(V[:, :n], got[0][1])
+        assert np.array_equal(R[:, n:n + m], got[3][0]) and np.array_equal(V[:, n:n + m], got[3][1])
+    Ro, S = oracle.residual(mid, oracle.split_stencils(mid), U0[id(mid)], order=order, inner=3, limiter=limiter,
+                            want_scale=True, boundary=boundary, mach=0.85, aoa_deg=1.0)
+    assert np.all(np.abs(got[3][0] - Ro) <= 1e-12 * S + 1e-300)
