@@ -386,7 +386,8 @@ typedef struct {
 
 lskum_status lskum_autotune(lskum_ctx *ctx, int reps, lskum_tuning *out);
 
-/* Select shapes directly (0 is the default of each kernel). */
+/* Select shapes directly. A context starts with a flux shape chosen by its number
+ * of points and boundary mode, and with q-derivative shape 0. */
 lskum_status lskum_set_tuning(lskum_ctx *ctx, int flux_variant, int qgrad_variant);
 
 /*

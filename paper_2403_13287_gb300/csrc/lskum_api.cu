@@ -726,6 +726,7 @@ static lskum_status create_impl(lskum_ctx *c, const double *x, const double *y, 
         c->qext = b + 8 * n * qbytes;
     }
     if (c->mixed) {
+        c->var_flux = mixed_default_flux(n, c->kinetic);
         // FP32 geometry in CSR order, then scattered into the SELL-32 layout
         CK(c, dalloc(c, &c->nrm_f, n));
         CK(c, dalloc(c, &c->dmin_f, n));

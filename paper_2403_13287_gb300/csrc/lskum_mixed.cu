@@ -934,6 +934,19 @@ void mixed_variant_shape(int kernel_class, int v, int *threads, int *min_blocks)
     *min_blocks = t[v][1];
 }
 
+// The flux shape of a context that has not been tuned, by its size: the
+// pipelined loop always (12 to 17 % of a step over shape 0), at the register
+// budget that measured best for RK4 steps: plain boundaries, below 120,000
+// points 64 x 8 (128 registers: a warp's chain counts, SMs are idle), from there
+// 64 x 12 (80 registers: resident warps count); the two cross between 93k
+// (0.1550 / 0.1566 ms a step) and 160k points (0.2404 / 0.2389), and differ by
+// 4.5 % at 2.5M. The kinetic mode, without the rows in shared memory, takes
+// 64 x 10 at every size (within 2 % of its best from 3k to 2.5M).
+int mixed_default_flux(int64_t n, bool kinetic)
+{
+    return kinetic ? 23 : n < 120000 ? 14 : 22;
+}
+
 cudaError_t launch_qgrad_mixed(const MixedGeom &g, const float *q, const float *qg_old, const float *g1,
                                float *qg_new, float *ext, double limiter_K, cudaStream_t s, int variant)
 {

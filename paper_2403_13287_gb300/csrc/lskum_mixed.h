@@ -84,6 +84,7 @@ cudaError_t launch_sell_fill(int64_t n, const int32_t *off, const int32_t *slice
 // launch-shape variants (threads per block, minimum resident blocks per SM);
 // kernel_class 0 = flux, 1 = q-derivatives; variant 0 is the default
 int mixed_variants(int kernel_class);
+int mixed_default_flux(int64_t n, bool kinetic);  // flux variant of an untuned context
 void mixed_variant_shape(int kernel_class, int variant, int *threads, int *min_blocks);
 // One q-derivative pass in FP32, with the same pass rules as launch_qgrad:
 // an inner pass (qg_old != nullptr) needs g1, the first pass's result for the
