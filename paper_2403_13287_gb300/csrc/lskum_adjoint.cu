@@ -24,6 +24,7 @@
 #include <type_traits>
 
 #include "lskum_adjoint.h"
+#include "lskum_fixed.cuh"
 
 namespace lskum {
 
@@ -388,9 +389,38 @@ __device__ __forceinline__ void state_adjoint_rev(const double qt[4], double tx,
 }
 
 // ---------------------------------------------------------------------------
-// flux adjoint, owner side
+// flux adjoint, owner side, one lane per point: the FP32 product, and FP64 with
+// gamma != 1.4. GEOM: with the cotangents of weights and offsets.
 // ---------------------------------------------------------------------------
-template <class T>
+// weights (w_s, w_n) and offset of an edge: the FP64 geometry, or its FP32 copy
+__device__ __forceinline__ void edge_geometry(const AdjParamsT<double> &P, int e, int i, double2 xy0, bool second,
+                                              double &wx, double &wy, double &dx, double &dy)
+{
+    const double2 w = P.g.fxw[e];
+    wx = w.x;
+    wy = w.y;
+    if (second) {
+        const double2 xyi = P.g.xy[i];
+        dx = xyi.x - xy0.x;
+        dy = xyi.y - xy0.y;
+    }
+}
+__device__ __forceinline__ void edge_geometry(const AdjParamsT<float> &P, int e, int, double2, bool, float &wx,
+                                              float &wy, float &dx, float &dy)
+{
+    const float4 v = __ldg(P.ef + e);
+    dx = v.x;
+    dy = v.y;
+    wx = v.z;
+    wy = v.w;
+}
+
+// an exact double of a float; the FP32 one avoids the conversion instruction
+// (FP64 pipe), subnormals become zero
+__device__ __forceinline__ double to_f64(double v) { return v; }
+__device__ __forceinline__ double to_f64(float v) { return f32_to_f64_ip(v); }
+
+template <class T, bool GEOM>
 __global__ void __launch_bounds__(128) k_adj_flux(AdjParamsT<T> P)
 {
     const DevGeom &g = P.g;
@@ -405,7 +435,7 @@ __global__ void __launch_bounds__(128) k_adj_flux(AdjParamsT<T> P)
         // R = 0 there: no cotangent flows from this point
         for (int e = e0; e < e1; ++e) {
             st4(P.ebar, e, qb0);
-            P.wbar[e] = make_double2(0.0, 0.0);
+            if constexpr (GEOM) P.wbar[e] = make_double2(0.0, 0.0);
         }
         st4(P.qbar, p, qb0);
         if (second) st8(P.gbar, p, gb0);
@@ -427,17 +457,14 @@ __global__ void __launch_bounds__(128) k_adj_flux(AdjParamsT<T> P)
         const uint8_t m = g.mask[e];
         const int ks = xsub(m), kn = ysub(m);
         const bool us_ = sub_needed(f, ks), un_ = sub_needed(f, kn);
-        const double2 wd = g.fxw[e];
-        const T wx = T(wd.x), wy = T(wd.y);
+        T wx, wy, dx = T(0), dy = T(0);
+        edge_geometry(P, e, i, xy0, second, wx, wy, dx, dy);
         T qti[4], qt0[4];
         ld4(P.q, i, qti);
-        T dx = T(0), dy = T(0), gi[8];
+        T gi[8];
 #pragma unroll
         for (int k = 0; k < 4; ++k) qt0[k] = q0[k];
         if (second) {
-            const double2 xyi = g.xy[i];
-            dx = T(xyi.x - xy0.x);
-            dy = T(xyi.y - xy0.y);
             ld8(P.qg, i, gi);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -467,41 +494,260 @@ __global__ void __launch_bounds__(128) k_adj_flux(AdjParamsT<T> P)
             for (int k = 0; k < 4; ++k) qbi[k] = qbo[k] = T(0);
         }
         // R += w (G(q~_i) - G(q~_0)): + for the neighbour, - for the owner
-        T wbx = T(0), wby = T(0);
+        if constexpr (GEOM) {
+            T wbx = T(0), wby = T(0);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            wbx += Rl[k] * (Gsi[k] - Gs0[k]);
-            wby += Rl[k] * (Gni[k] - Gn0[k]);
-            qbo[k] = -qbo[k];
+            for (int k = 0; k < 4; ++k) {
+                wbx += Rl[k] * (Gsi[k] - Gs0[k]);
+                wby += Rl[k] * (Gni[k] - Gn0[k]);
+            }
+            P.wbar[e] = make_double2(us_ ? to_f64(wbx) : 0.0, un_ ? to_f64(wby) : 0.0);
         }
-        P.wbar[e] = make_double2(us_ ? (double)wbx : 0.0, un_ ? (double)wby : 0.0);
         st4(P.ebar, e, qbi);
         T dxb = T(0), dyb = T(0);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
+            qbo[k] = -qbo[k];
             qb0[k] += qbo[k];
             if (second) {
                 // q~_0 = q_0 - (dx qx_0 + dy qy_0)/2
                 gb0[k] -= h * dx * qbo[k];
                 gb0[4 + k] -= h * dy * qbo[k];
-                dxb -= h * qbo[k] * g0[k];
-                dyb -= h * qbo[k] * g0[4 + k];
+                if constexpr (GEOM) {
+                    dxb -= h * qbo[k] * g0[k];
+                    dyb -= h * qbo[k] * g0[4 + k];
+                }
             }
         }
-        double2 db = P.dbar[e];
-        db.x += (double)dxb;
-        db.y += (double)dyb;
-        P.dbar[e] = db;
+        if constexpr (GEOM) {
+            double2 db = P.dbar[e];
+            db.x += to_f64(dxb);
+            db.y += to_f64(dyb);
+            P.dbar[e] = db;
+        }
     }
     st4(P.qbar, p, qb0);
     if (second) st8(P.gbar, p, gb0);
 }
 
 // ---------------------------------------------------------------------------
+// flux adjoint, owner side, FP64 with gamma = 1.4, two lanes per edge: lane 0
+// differentiates at the neighbour's state, lane 1 at the point's own one.
+//
+// In the variables of the fixed-point fluxes (lskum_fixed.cuh) the adjoint is
+// short: per direction with cotangent (r0, ra, ro, r3) of [mass, along,
+// transverse, energy], J = sum of r G is
+//   s0 P + a1 F1 + s2 So P + s3 F3,  s0 = sgn r0 C0, a1 = ra C1, s2 = sgn ro C1,
+//   s3 = sgn r3 C3, F1 = Phi/2 + z P, F3 = H P - E/4, z = sgn S_d,
+// and P' = Phi, F1' = 2 P, E' = -2 z E give
+//   dJ/dz = (s0 + s2 So + s3 H) Phi + 2 a1 P + s3 z E/2,
+//   dJ/dSo = s2 P, dJ/dH = s3 P, dJ/dx = J (all factors carry exp(x)),
+//   dJ/dln r = 6 s0 P + 7 (a1 F1 + s2 So P) + 8 s3 F3.
+// Then H = hc + (S_t^2 + S_n^2)/2, x = q1 + S_t^2 + S_n^2, S = (q2, q3).(t, n) r/2,
+// r = (-q4/2)^(-1/2). J itself is what the weight's cotangent needs. Phi, E, P,
+// F1, F3 and the factors come from the integer pipes: about 100 FP64
+// instructions per lane and edge instead of 400 per edge in one lane, and J's
+// rounding error is a fifth of the FP64 chain's. 40k points: 536 -> 186 us.
+// ---------------------------------------------------------------------------
+struct DirCotangent {
+    double J;                        // sum of r G, without the weight
+    double bd, bo, bH, bx, bl;       // w dJ/d(S_d, S_o, H, x, ln r)
+};
+__device__ __forceinline__ DirCotangent direction_cotangent(const FixState &s, bool along_t, unsigned long long sbit,
+                                                            double Sd, double So, double H, double C0, double C1,
+                                                            double C3, double r0, double ra, double ro, double r3,
+                                                            double w)
+{
+    int64_t Phi_, E_, P_;
+    const FixOp zo = fix_phi_e(along_t ? s.St : s.Sn, sbit ? -1 : 0, Phi_, E_, P_);
+    const FixOp Po = fix_op(P_);
+    const double Phi = fix_to_double(Phi_, -62), P = fix_to_double(P_, -61), P2 = fix_to_double(P_, -60);
+    const double Eh = fix_to_double(E_, -63);                                       // E/2
+    const double F1 = fix_to_double((Phi_ >> 5) + fix_mul(zo, Po), -58);
+    const double F3 = fix_to_double(fix_mul_s<1>(fix_op(s.H), Po) - (E_ >> 7), -57);
+    const double s0 = flip_sign(r0 * C0, sbit), a1 = ra * C1, s2 = flip_sign(ro * C1, sbit), y3 = r3 * C3, s3 = flip_sign(y3, sbit);
+    const double K = fma(s3, H, fma(s2, So, s0));
+    const double u1 = a1 * F1, u3 = s3 * F3, s2P = s2 * P, v = So * s2P, uv = u1 + v;
+    DirCotangent o;
+    o.J = fma(s0, P, uv + u3);
+    const double Jl = fma(6.0, o.J, fma(2.0, u3, uv));
+    const double Jz = fma(K, Phi, fma(a1, P2, y3 * (Sd * Eh)));    // sgn z = S_d
+    o.bd = flip_sign(w, sbit) * Jz;
+    o.bo = w * s2P;
+    o.bH = w * (s3 * P);
+    o.bx = w * o.J;
+    o.bl = w * Jl;
+    return o;
+}
+
+// a state outside the fixed-point ranges: the FP64 reverse mode
+struct StateCotangent {
+    double qb[4], Js, Jn;
+};
+__device__ __noinline__ StateCotangent state_cotangent_fp64(double q0, double q1, double q2, double q3, double2 n0,
+                                                            int flags, double wx, double wy, double R0, double Rs,
+                                                            double Rn, double R3, double inv_gm1)
+{
+    const double qt[4] = {q0, q1, q2, q3}, Rl[4] = {R0, Rs, Rn, R3};
+    const bool us_ = flags & 1, un_ = flags & 2;
+    double cs[4], cn[4], Gs[4] = {0.0, 0.0, 0.0, 0.0}, Gn[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int k = 0; k < 4; ++k) {
+        cs[k] = us_ ? wx * Rl[k] : 0.0;
+        cn[k] = un_ ? wy * Rl[k] : 0.0;
+    }
+    StateCotangent o;
+    state_adjoint_rev(qt, n0.y, -n0.x, n0.x, n0.y, us_, flags & 4 ? 1.0 : -1.0, un_, flags & 8 ? 1.0 : -1.0, cs, cn,
+                      inv_gm1, true, o.qb, Gs, Gn);
+    o.Js = o.Jn = 0.0;
+    for (int k = 0; k < 4; ++k) {
+        o.Js += Rl[k] * Gs[k];
+        o.Jn += Rl[k] * Gn[k];
+    }
+    return o;
+}
+
+template <bool GEOM>
+__global__ void __launch_bounds__(128) k_adj_flux_pair(AdjParams P)
+{
+    const DevGeom &g = P.g;
+    const int64_t pp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 1;
+    const int l = threadIdx.x & 1;
+    const int64_t p = pp < g.n ? pp : g.n - 1;
+    const uint8_t f = g.flag[p] & 3;
+    const bool second = P.order == 2, live = pp < g.n;
+    double qb0[4] = {0.0, 0.0, 0.0, 0.0}, gb0[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    const int e0 = g.off[p], e1 = g.off[p + 1];
+    if (live && l == 0 && f == FLAG_FARFIELD) {
+        // R = 0 there: no cotangent flows from this point
+        for (int e = e0; e < e1; ++e) {
+            st4(P.ebar, e, qb0);
+            if constexpr (GEOM) P.wbar[e] = make_double2(0.0, 0.0);
+        }
+    }
+    const int deg = live && f != FLAG_FARFIELD ? e1 - e0 : 0;
+    const double2 xy0 = g.xy[p];
+    const double2 n0 = g.nrm[p];
+    const FixOp fnx = fix_op(fix_unit(n0.x)), fny = fix_op(fix_unit(n0.y));
+    const double tx = n0.y, ty = -n0.x;
+    double Rb[4], g0[8];
+    ld4(P.Rbar, p, Rb);
+    // frame-order cotangent of R_local: R_global = (R0, R1 t + R2 n, R3)
+    const double Rs = Rb[1] * tx + Rb[2] * ty, Rn = Rb[1] * n0.x + Rb[2] * n0.y;
+    if (second) ld8(P.qg, p, g0);
+    // whole warps go through the longest row: the lanes exchange J by shuffles
+    const int most = __reduce_max_sync(0xffffffffu, deg);
+#pragma unroll 1
+    for (int j = 0; j < most; ++j) {
+        const bool act = j < deg;
+        const int e = act ? e0 + j : e0;
+        const int i = g.idx[e];
+        const uint8_t m = g.mask[e];
+        const bool us_ = sub_needed(f, xsub(m)), un_ = sub_needed(f, ysub(m));
+        const double2 w = g.fxw[e];   // zero where the sub-stencil is not needed
+        const int64_t row = l ? p : (int64_t)i;
+        double qt[4], qb[4], Js, Jn;
+        gather4(P.q, row, qt);
+        double2 h = make_double2(0.0, 0.0);
+        if (second) {
+            if (g.hd) {
+                h = g.hd[e];
+            } else {
+                const double2 xyi = g.xy[i];
+                h = make_double2(0.5 * (xyi.x - xy0.x), 0.5 * (xyi.y - xy0.y));
+            }
+            double gr[8];
+            gather8(P.qg, row, gr);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) qt[k] = fma(-h.y, gr[4 + k], fma(-h.x, gr[k], qt[k]));
+        }
+        FixState s;
+        if (fix_state(qt, fnx, fny, s)) {
+            const double St = fix_to_double(s.St, -61), Sn = fix_to_double(s.Sn, -61), H = fix_to_double(s.H, -59);
+            const double C0 = fix_to_double(s.c0, fix_e0(s.n, s.k)), C1 = fix_to_double(s.c1, fix_e1(s.n, s.k)),
+                         C3 = fix_to_double(s.c3, fix_e3(s.n, s.k)), hr = fix_to_double(s.r, -62 - s.k);
+            const DirCotangent a = direction_cotangent(s, true, (m & M_XPOS) ? 0ull : kSignBit, St, Sn, H, C0, C1, C3,
+                                                       Rb[0], Rs, Rn, Rb[3], w.x);
+            const DirCotangent b = direction_cotangent(s, false, (m & M_YPOS) ? 0ull : kSignBit, Sn, St, H, C0, C1, C3,
+                                                       Rb[0], Rn, Rs, Rb[3], w.y);
+            Js = a.J;
+            Jn = b.J;
+            const double bx = a.bx + b.bx, d = fma(2.0, bx, a.bH + b.bH);
+            const double bt = fma(St, d, a.bd + b.bo), bn = fma(Sn, d, a.bo + b.bd);
+            const double bl = fma(St, bt, fma(Sn, bn, a.bl + b.bl));
+            const double mt = bt * hr, mn = bn * hr;
+            qb[0] = bx;
+            qb[1] = fma(mt, tx, mn * n0.x);
+            qb[2] = fma(mt, ty, mn * n0.y);
+            qb[3] = bl * (hr * hr);
+        } else {
+            const StateCotangent o = state_cotangent_fp64(
+                qt[0], qt[1], qt[2], qt[3], n0, (us_ ? 1 : 0) | (un_ ? 2 : 0) | ((m & M_XPOS) ? 4 : 0) | ((m & M_YPOS) ? 8 : 0),
+                w.x, w.y, Rb[0], Rs, Rn, Rb[3], P.inv_gm1);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) qb[k] = o.qb[k];
+            Js = o.Js;
+            Jn = o.Jn;
+        }
+        // R += w (G(q~_i) - G(q~_0)): + for the neighbour, - for the owner
+        if constexpr (GEOM) {
+            const double Jso = __shfl_xor_sync(0xffffffffu, Js, 1), Jno = __shfl_xor_sync(0xffffffffu, Jn, 1);
+            if (act && l == 0) P.wbar[e] = make_double2(us_ ? Js - Jso : 0.0, un_ ? Jn - Jno : 0.0);
+        }
+        if (act && l == 0) st4(P.ebar, e, qb);
+        if (act && l == 1) {
+            double dxb = 0.0, dyb = 0.0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                qb0[k] -= qb[k];
+                if (second) {
+                    // q~_0 = q_0 - h.grad q_0, with the cotangent -qb; h = d/2
+                    gb0[k] = fma(h.x, qb[k], gb0[k]);
+                    gb0[4 + k] = fma(h.y, qb[k], gb0[4 + k]);
+                    if constexpr (GEOM) {
+                        dxb = fma(qb[k], g0[k], dxb);
+                        dyb = fma(qb[k], g0[4 + k], dyb);
+                    }
+                }
+            }
+            if constexpr (GEOM) {
+                if (second) {
+                    double2 db = P.dbar[e];
+                    db.x = fma(0.5, dxb, db.x);
+                    db.y = fma(0.5, dyb, db.y);
+                    P.dbar[e] = db;
+                }
+            }
+        }
+    }
+    if (live && l == 1) {
+        st4(P.qbar, p, qb0);
+        if (second) st8(P.gbar, p, gb0);
+    }
+}
+
+// half offset and full-stencil weights of incoming edge t
+__device__ __forceinline__ void incoming(const AdjParamsT<double> &P, int t, double &hx, double &hy, double &ax, double &ay)
+{
+    const double2 hh = __ldg(P.thd + t), a = __ldg(P.tlsw + t);
+    hx = hh.x;
+    hy = hh.y;
+    ax = a.x;
+    ay = a.y;
+}
+__device__ __forceinline__ void incoming(const AdjParamsT<float> &P, int t, float &hx, float &hy, float &ax, float &ay)
+{
+    const float4 v = __ldg(P.tf + t);
+    ax = v.x;
+    ay = v.y;
+    hx = 0.5f * v.z;
+    hy = 0.5f * v.w;
+}
+
+// ---------------------------------------------------------------------------
 // flux adjoint, neighbour side: point p gathers the cotangents of q~_p over
 // the edges that reach it
 // ---------------------------------------------------------------------------
-template <class T>
+template <class T, bool GEOM>
 __global__ void __launch_bounds__(128) k_adj_flux_gather(AdjParamsT<T> P)
 {
     const DevGeom &g = P.g;
@@ -513,43 +759,81 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather(AdjParamsT<T> P)
     ld4(P.qbar, p, qb);
     if (second) {
         ld8(P.gbar, p, gb);
-        ld8(P.qg, p, gp);
+        if constexpr (GEOM) ld8(P.qg, p, gp);
     }
-    const double2 xyp = g.xy[p];
-    for (int t = P.toff[p]; t < P.toff[p + 1]; ++t) {
+    const int t1 = P.toff[p + 1];
+    for (int t = P.toff[p]; t < t1; ++t) {
         const int e = P.tedge[t];
         T eb[4];
         ld4(P.ebar, e, eb);
 #pragma unroll
         for (int k = 0; k < 4; ++k) qb[k] += eb[k];
         if (second) {
-            const double2 xys = g.xy[P.tsrc[t]];
-            const T dx = T(xyp.x - xys.x), dy = T(xyp.y - xys.y);
+            T hx, hy, ax, ay;
+            incoming(P, t, hx, hy, ax, ay);
             T dxb = T(0), dyb = T(0);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 // q~_p = q_p - (dx qx_p + dy qy_p)/2 on this edge
-                gb[k] -= h * dx * eb[k];
-                gb[4 + k] -= h * dy * eb[k];
-                dxb -= h * eb[k] * gp[k];
-                dyb -= h * eb[k] * gp[4 + k];
+                gb[k] -= hx * eb[k];
+                gb[4 + k] -= hy * eb[k];
+                if constexpr (GEOM) {
+                    dxb -= h * eb[k] * gp[k];
+                    dyb -= h * eb[k] * gp[4 + k];
+                }
             }
-            double2 d = P.dbar[e];
-            d.x += (double)dxb;
-            d.y += (double)dyb;
-            P.dbar[e] = d;
+            if constexpr (GEOM) {
+                double2 d = P.dbar[e];
+                d.x += to_f64(dxb);
+                d.y += to_f64(dyb);
+                P.dbar[e] = d;
+            }
         }
     }
     st4(P.qbar, p, qb);
     if (second) st8(P.gbar, p, gb);
 }
 
+// full-stencil weights and half offset of edge e of point p (neighbour i)
+__device__ __forceinline__ void outgoing(const AdjParamsT<double> &P, int e, int i, double2 xyp, bool inner, double &hx,
+                                         double &hy, double &ax, double &ay)
+{
+    const double2 a = P.g.lsw[e];
+    ax = a.x;
+    ay = a.y;
+    if (!inner) return;
+    if (P.g.hd) {
+        const double2 hh = P.g.hd[e];
+        hx = hh.x;
+        hy = hh.y;
+    } else {
+        const double2 xyi = P.g.xy[i];
+        hx = 0.5 * (xyi.x - xyp.x);
+        hy = 0.5 * (xyi.y - xyp.y);
+    }
+}
+__device__ __forceinline__ void outgoing(const AdjParamsT<float> &P, int e, int, double2, bool inner, float &hx,
+                                         float &hy, float &ax, float &ay)
+{
+    const float2 a = __ldg(P.ea + e);
+    ax = a.x;
+    ay = a.y;
+    if (!inner) return;
+    const float4 v = __ldg(P.ef + e);
+    hx = 0.5f * v.x;
+    hy = 0.5f * v.y;
+}
+
 // ---------------------------------------------------------------------------
 // one least-squares pass of E15 in reverse. Forward (per component c):
 //   g_p = sum_e a_e s_e,  s_e = (q_i - q_p) - [dx (gx'_i - gx'_p) + dy (gy'_i - gy'_p)]/2
-// with g' the previous iterate (absent in the first-order pass).
+// with g' the previous iterate (absent in the first-order pass). GEOM: with the
+// cotangents of the weights and offsets; without them an outgoing edge only
+// gives the owner's q its share, and no neighbour value is read for it (FP32 at
+// 640k points: 228 -> 58 us a pass, half of it from the geometry's FP32 copies,
+// which spare the FP64 pipe the conversions).
 // ---------------------------------------------------------------------------
-template <class T>
+template <class T, bool GEOM>
 __global__ void __launch_bounds__(128) k_adj_grad(AdjParamsT<T> P, const T *__restrict__ gprev,
                                                   const T *__restrict__ gbar_in, T *__restrict__ gbar_out)
 {
@@ -560,8 +844,11 @@ __global__ void __launch_bounds__(128) k_adj_grad(AdjParamsT<T> P, const T *__re
     T qb[4], gb[8], qp[4], gbo[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     ld4(P.qbar, p, qb);
     ld8(gbar_in, p, gb);
-    ld4(P.q, p, qp);
-    const double2 xyp = g.xy[p];
+    double2 xyp = make_double2(0.0, 0.0);
+    if constexpr (GEOM) {
+        ld4(P.q, p, qp);
+        if (!g.hd) xyp = g.xy[p];
+    }
     // an inner pass is sum_e a_e (q_i - q_0 - h_e.grad q_i) + grad q_0 / 2
     // (h_e the half offset; the terms in grad q_0 add up to grad q_0 / 2 since
     // sum_e a_e d_e^T = I, and the forward passes take them so), so grad q_0
@@ -572,69 +859,55 @@ __global__ void __launch_bounds__(128) k_adj_grad(AdjParamsT<T> P, const T *__re
     }
     // outgoing edges: owner terms, and the cotangents of a_e and of the offsets
     for (int e = g.off[p]; e < g.off[p + 1]; ++e) {
-        const int i = g.idx[e];
-        const double2 ad = g.lsw[e];
-        const T ax = T(ad.x), ay = T(ad.y);
-        T qi[4], gi[8];
-        ld4(P.q, i, qi);
-        T hx = T(0), hy = T(0);
-        if (inner) {
-            ld8(gprev, i, gi);
-            double2 hh;
-            if (g.hd) {
-                hh = g.hd[e];
-            } else {
-                const double2 xyi = g.xy[i];
-                hh = make_double2(0.5 * (xyi.x - xyp.x), 0.5 * (xyi.y - xyp.y));
-            }
-            hx = T(hh.x);
-            hy = T(hh.y);
-        }
-        T abx = T(0), aby = T(0), dbx = T(0), dby = T(0);
+        T hx = T(0), hy = T(0), ax, ay;
+        if constexpr (!GEOM) {
+            outgoing(P, e, 0, xyp, false, hx, hy, ax, ay);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const T sb = ax * gb[k] + ay * gb[4 + k];
-            T s = qi[k] - qp[k];
-            if (inner) {
-                s = s - (hx * gi[k] + hy * gi[4 + k]);
-                // d_e = 2 h_e: d_bar = -(sb/2) grad q_i
-                dbx -= T(0.5) * sb * gi[k];
-                dby -= T(0.5) * sb * gi[4 + k];
+            for (int k = 0; k < 4; ++k) {
+                const T sb = ax * gb[k] + ay * gb[4 + k];
+                qb[k] -= sb;
             }
-            qb[k] -= sb;
-            abx += s * gb[k];
-            aby += s * gb[4 + k];
-        }
-        double2 ab = P.abar[e];
-        ab.x += (double)abx;
-        ab.y += (double)aby;
-        P.abar[e] = ab;
-        if (inner) {
-            double2 db = P.dbar[e];
-            db.x += (double)dbx;
-            db.y += (double)dby;
-            P.dbar[e] = db;
+        } else {
+            const int i = g.idx[e];
+            outgoing(P, e, i, xyp, inner, hx, hy, ax, ay);
+            T qi[4], gi[8];
+            ld4(P.q, i, qi);
+            if (inner) ld8(gprev, i, gi);
+            T abx = T(0), aby = T(0), dbx = T(0), dby = T(0);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const T sb = ax * gb[k] + ay * gb[4 + k];
+                T s = qi[k] - qp[k];
+                if (inner) {
+                    s = s - (hx * gi[k] + hy * gi[4 + k]);
+                    // d_e = 2 h_e: d_bar = -(sb/2) grad q_i
+                    dbx -= T(0.5) * sb * gi[k];
+                    dby -= T(0.5) * sb * gi[4 + k];
+                }
+                qb[k] -= sb;
+                abx += s * gb[k];
+                aby += s * gb[4 + k];
+            }
+            double2 ab = P.abar[e];
+            ab.x += to_f64(abx);
+            ab.y += to_f64(aby);
+            P.abar[e] = ab;
+            if (inner) {
+                double2 db = P.dbar[e];
+                db.x += to_f64(dbx);
+                db.y += to_f64(dby);
+                P.dbar[e] = db;
+            }
         }
     }
     // incoming edges: the terms of this point as a neighbour
-    for (int t = P.toff[p]; t < P.toff[p + 1]; ++t) {
-        const int e = P.tedge[t], src = P.tsrc[t];
-        const double2 ad = g.lsw[e];
-        const T ax = T(ad.x), ay = T(ad.y);
+    const int t1 = P.toff[p + 1];
+    for (int t = P.toff[p]; t < t1; ++t) {
+        const int src = P.tsrc[t];
+        T hx, hy, ax, ay;
+        incoming(P, t, hx, hy, ax, ay);
         T gs[8];
         ld8(gbar_in, src, gs);
-        T hx = T(0), hy = T(0);
-        if (inner) {
-            double2 hh;
-            if (g.hd) {
-                hh = g.hd[e];
-            } else {
-                const double2 xys = g.xy[src];
-                hh = make_double2(0.5 * (xyp.x - xys.x), 0.5 * (xyp.y - xys.y));
-            }
-            hx = T(hh.x);
-            hy = T(hh.y);
-        }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const T sb = ax * gs[k] + ay * gs[4 + k];
@@ -923,8 +1196,10 @@ __global__ void __launch_bounds__(256) k_adj_points(AdjParams P, const double2 *
     if (yb_out) yb_out[o] = accumulate ? yb_out[o] + yb : yb;
 }
 
-// q_bar to U_bar through E13 (duals over the four conserved variables);
-// adds into Ub_acc ([n][4], internal order)
+// q_bar to U_bar through E13, adds into Ub_acc ([n][4], internal order). With
+// p = (gamma-1) (E - m^2/(2 rho)), m^2 = m1^2 + m2^2 and g = 1/(gamma-1):
+//   q1 = ln rho + g ln(rho/(2p)) - m^2/(2 rho p), q2 = m1/p, q3 = m2/p, q4 = -rho/p,
+// in reverse by hand (40 FP64 operations and two quotients per point)
 template <class T>
 __global__ void __launch_bounds__(256) k_adj_state(AdjParamsT<T> P, const double *__restrict__ U,
                                                    double *__restrict__ Ub_acc)
@@ -932,36 +1207,28 @@ __global__ void __launch_bounds__(256) k_adj_state(AdjParamsT<T> P, const double
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t n = P.g.n;
     if (p >= n) return;
-    double u[4], qb[4];
+    double u[4], qb[4], ub[4];
     ld4(U, p, u);
     T qt[4];
     ld4(P.qbar, p, qt);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) qb[k] = (double)qt[k];
-    D4 Ud[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        Ud[k] = dconst(u[k]);
-        Ud[k].d[k] = 1.0;
-    }
-    const D4 rinv = recip(Ud[0]);
-    const D4 u1 = Ud[1] * rinv, u2 = Ud[2] * rinv;
-    const D4 pr = (1.0 / P.inv_gm1) * (Ud[3] - 0.5 * (Ud[0] * (u1 * u1 + u2 * u2)));
-    const D4 beta = 0.5 * (Ud[0] * recip(pr));
-    D4 q[4];
-    q[0] = dlog(Ud[0]) + P.inv_gm1 * dlog(beta) - beta * (u1 * u1 + u2 * u2);
-    q[1] = 2.0 * (beta * u1);
-    q[2] = 2.0 * (beta * u2);
-    q[3] = -2.0 * beta;
-    double ub[4];
+    for (int k = 0; k < 4; ++k) qb[k] = to_f64(qt[k]);
     ld4(Ub_acc, p, ub);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        double s = 0.0;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) s += qb[c] * q[c].d[k];
-        ub[k] += s;
-    }
+    const double g = P.inv_gm1, gm1 = 1.0 / g;
+    const double ir = 1.0 / u[0], m1 = u[1] * ir, m2 = u[2] * ir;            // velocities
+    const double ke = 0.5 * (u[1] * m1 + u[2] * m2);                          // m^2/(2 rho)
+    const double pr = gm1 * (u[3] - ke), ip = 1.0 / pr;
+    const double kp = ke * ip;                                                // m^2/(2 rho p)
+    // cotangents at fixed p, and that of p
+    const double rb = qb[0] * ir * (1.0 + g + kp) - qb[3] * ip;
+    const double ab = ip * (qb[1] - qb[0] * m1), bb = ip * (qb[2] - qb[0] * m2);
+    const double pb = ip * (qb[0] * (kp - g) - ip * (qb[1] * u[1] + qb[2] * u[2] - qb[3] * u[0]));
+    // p through rho, m and E
+    const double c = gm1 * pb;
+    ub[0] += rb + c * (0.5 * (m1 * m1 + m2 * m2));
+    ub[1] += ab - c * m1;
+    ub[2] += bb - c * m2;
+    ub[3] += c;
     st4(Ub_acc, p, ub);
 }
 
@@ -1002,6 +1269,44 @@ __global__ void k_tsrc(int64_t nnz, const int32_t *__restrict__ tedge, const int
     if (t < nnz) tsrc[t] = esrc[tedge[t]];
 }
 
+// weights and half offset of incoming edge t (edge tedge[t] of point tsrc[t])
+__global__ void k_incoming(int64_t nnz, DevGeom g, const int32_t *__restrict__ tedge, const int32_t *__restrict__ tsrc,
+                           double2 *__restrict__ tlsw, double2 *__restrict__ thd)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nnz) return;
+    const int e = tedge[t];
+    tlsw[t] = g.lsw[e];
+    if (g.hd) {
+        thd[t] = g.hd[e];
+    } else {
+        const double2 a = g.xy[tsrc[t]], b = g.xy[g.idx[e]];
+        thd[t] = make_double2(0.5 * (b.x - a.x), 0.5 * (b.y - a.y));
+    }
+}
+
+// the FP32 product's copies: the FP64 offsets and weights rounded once
+__global__ void k_float_edges(DevGeom g, float4 *__restrict__ ef, float2 *__restrict__ ea)
+{
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= g.n) return;
+    const double2 P0 = g.xy[p];
+    for (int e = g.off[p]; e < g.off[p + 1]; ++e) {
+        const double2 Pi = g.xy[g.idx[e]], w = g.fxw[e], a = g.lsw[e];
+        ef[e] = make_float4((float)(Pi.x - P0.x), (float)(Pi.y - P0.y), (float)w.x, (float)w.y);
+        ea[e] = make_float2((float)a.x, (float)a.y);
+    }
+}
+
+__global__ void k_float_incoming(int64_t nnz, const double2 *__restrict__ tlsw, const double2 *__restrict__ thd,
+                                 float4 *__restrict__ tf)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nnz) return;
+    const double2 a = tlsw[t], h = thd[t];
+    tf[t] = make_float4((float)a.x, (float)a.y, (float)(2.0 * h.x), (float)(2.0 * h.y));
+}
+
 unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
@@ -1040,20 +1345,50 @@ cudaError_t build_transpose_csr(int64_t n, int64_t nnz, const int32_t *off, cons
     return err;
 }
 
-template <class T>
-cudaError_t launch_adj_flux(const AdjParamsT<T> &P, cudaStream_t s)
+cudaError_t build_incoming(const DevGeom &g, int64_t nnz, const int32_t *tedge, const int32_t *tsrc, double2 *tlsw,
+                           double2 *thd, cudaStream_t s)
 {
-    k_adj_flux<T><<<blocks(P.g.n, 128), 128, 0, s>>>(P);
+    if (nnz <= 0) return cudaSuccess;
+    k_incoming<<<blocks(nnz, 256), 256, 0, s>>>(nnz, g, tedge, tsrc, tlsw, thd);
+    return cudaGetLastError();
+}
+
+cudaError_t build_float_geometry(const DevGeom &g, int64_t nnz, const double2 *tlsw, const double2 *thd, float4 *ef,
+                                 float2 *ea, float4 *tf, cudaStream_t s)
+{
+    if (nnz <= 0) return cudaSuccess;
+    k_float_edges<<<blocks(g.n, 128), 128, 0, s>>>(g, ef, ea);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    k_adj_flux_gather<T><<<blocks(P.g.n, 128), 128, 0, s>>>(P);
+    k_float_incoming<<<blocks(nnz, 256), 256, 0, s>>>(nnz, tlsw, thd, tf);
     return cudaGetLastError();
 }
 
 template <class T>
-cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gbar_in, T *gbar_out, cudaStream_t s)
+cudaError_t launch_adj_flux(const AdjParamsT<T> &P, bool geom, cudaStream_t s)
 {
-    k_adj_grad<T><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out);
+    const unsigned nb = blocks(P.g.n, 128);
+    bool pair = false;
+    if constexpr (std::is_same<T, double>::value) {
+        pair = P.g14 != 0;
+        if (pair && geom) k_adj_flux_pair<true><<<blocks(P.g.n, 64), 128, 0, s>>>(P);
+        if (pair && !geom) k_adj_flux_pair<false><<<blocks(P.g.n, 64), 128, 0, s>>>(P);
+    }
+    if (!pair && geom) k_adj_flux<T, true><<<nb, 128, 0, s>>>(P);
+    if (!pair && !geom) k_adj_flux<T, false><<<nb, 128, 0, s>>>(P);
+    cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+    if (geom) k_adj_flux_gather<T, true><<<nb, 128, 0, s>>>(P);
+    else k_adj_flux_gather<T, false><<<nb, 128, 0, s>>>(P);
+    return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gbar_in, T *gbar_out, bool geom,
+                            cudaStream_t s)
+{
+    if (geom) k_adj_grad<T, true><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out);
+    else k_adj_grad<T, false><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out);
     return cudaGetLastError();
 }
 
@@ -1100,11 +1435,11 @@ cudaError_t launch_to_float(int64_t m, const double *a, float *b, cudaStream_t s
     return cudaGetLastError();
 }
 
-template cudaError_t launch_adj_flux<double>(const AdjParamsT<double> &, cudaStream_t);
-template cudaError_t launch_adj_flux<float>(const AdjParamsT<float> &, cudaStream_t);
-template cudaError_t launch_adj_grad<double>(const AdjParamsT<double> &, const double *, const double *, double *,
+template cudaError_t launch_adj_flux<double>(const AdjParamsT<double> &, bool, cudaStream_t);
+template cudaError_t launch_adj_flux<float>(const AdjParamsT<float> &, bool, cudaStream_t);
+template cudaError_t launch_adj_grad<double>(const AdjParamsT<double> &, const double *, const double *, double *, bool,
                                              cudaStream_t);
-template cudaError_t launch_adj_grad<float>(const AdjParamsT<float> &, const float *, const float *, float *,
+template cudaError_t launch_adj_grad<float>(const AdjParamsT<float> &, const float *, const float *, float *, bool,
                                             cudaStream_t);
 template cudaError_t launch_adj_state<double>(const AdjParamsT<double> &, const double *, double *, cudaStream_t);
 template cudaError_t launch_adj_state<float>(const AdjParamsT<float> &, const double *, double *, cudaStream_t);

@@ -25,6 +25,13 @@ struct AdjParamsT {
     const int32_t *toff;   // [n+1] transpose CSR: incoming edges of each point
     const int32_t *tedge;  // [nnz] edge ids, grouped by destination, in edge order
     const int32_t *tsrc;   // [nnz] owner point of each incoming edge
+    const double2 *tlsw;   // [nnz] lsw of each incoming edge, in the transpose's order
+    const double2 *thd;    // [nnz] half offset of each incoming edge, likewise
+    // FP32 product: geometry rounded once, per edge (dx, dy, w_s, w_n) and
+    // (a_x, a_y), per incoming edge (a_x, a_y, dx, dy); nullptr in the FP64 one
+    const float4 *ef;
+    const float2 *ea;
+    const float4 *tf;
     const int32_t *perm;   // internal point -> input point
     double inv_gm1;
     int g14;               // gamma == 1.4: beta^(-1/(gamma-1)) = beta^-2.5 (as the forward kernels)
@@ -34,19 +41,29 @@ using AdjParams = AdjParamsT<double>;
 
 cudaError_t build_transpose_csr(int64_t n, int64_t nnz, const int32_t *off, const int32_t *idx, int32_t *toff,
                                 int32_t *tedge, int32_t *tsrc, cudaStream_t s);
+// the incoming edges' weights and half offsets in the transpose's order (tlsw, thd)
+cudaError_t build_incoming(const DevGeom &g, int64_t nnz, const int32_t *tedge, const int32_t *tsrc, double2 *tlsw,
+                           double2 *thd, cudaStream_t s);
+// the FP32 product's geometry (ef, ea, tf)
+cudaError_t build_float_geometry(const DevGeom &g, int64_t nnz, const double2 *tlsw, const double2 *thd, float4 *ef,
+                                 float2 *ea, float4 *tf, cudaStream_t s);
+// geom (here and below): the cotangents of the weights and offsets are wanted
+// too (wbar, abar, dbar); without it they are left alone.
 // flux adjoint: owner pass, then the neighbour-side gather (initialises qbar, gbar, ebar, wbar; adds into
 // dbar, which the caller zeroes once per product)
 template <class T>
-cudaError_t launch_adj_flux(const AdjParamsT<T> &P, cudaStream_t s);
+cudaError_t launch_adj_flux(const AdjParamsT<T> &P, bool geom, cudaStream_t s);
 // one E15 pass in reverse: gbar_in is the cotangent of this pass's output,
 // gbar_out receives that of its input iterate gprev (nullptr for the first-order pass)
 template <class T>
-cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gbar_in, T *gbar_out, cudaStream_t s);
+cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gbar_in, T *gbar_out, bool geom,
+                            cudaStream_t s);
 // the limiter (limiter_K > 0) in reverse, between the flux adjoint and the
 // last pass's: gbar_in is the cotangent of the limited last iterate, graw the
 // unlimited one; gbar_out receives the unlimited iterate's cotangent; adds
 // into qbar (the point and, through lidx/lval ([n][4] scratch), its extreme
-// neighbours) and into dbar (the largest-shift and nearest-neighbour edges)
+// neighbours) and into dbar (the largest-shift and nearest-neighbour edges;
+// always: a few entries per point)
 cudaError_t launch_adj_limit(const AdjParams &P, const double *graw, const double *gbar_in, double *gbar_out,
                              int32_t *lidx, double *lval, double limK, cudaStream_t s);
 // least-squares weight cotangents (abar, wbar) into the offset cotangents dbar

@@ -122,6 +122,7 @@ struct lskum_ctx {
     double *vebar = nullptr;
     double2 *vwbar = nullptr, *vabar = nullptr, *vdbar = nullptr;
     int32_t *toff = nullptr, *tedge = nullptr, *tsrc = nullptr;
+    double2 *tlsw = nullptr, *thd = nullptr;  // weights and half offsets of the incoming edges
     double *vGlim = nullptr;      // [n][8] the limited last iterate (limiter_K > 0)
     double *vext = nullptr;       // [n][4] the limiter's extremum measure (limiter_K > 0)
     int32_t *vlidx = nullptr;     // [n][4] limiter reverse: the extreme neighbour's edge
@@ -136,6 +137,8 @@ struct lskum_ctx {
     // FP32 residual VJP (mixed contexts; allocated on the first such call)
     bool fvjp_ready = false;
     float *fq = nullptr, *fG = nullptr, *fRb = nullptr, *fqb = nullptr, *fgb = nullptr, *fgb2 = nullptr, *febar = nullptr;
+    float4 *fef = nullptr, *ftf = nullptr;    // FP32 edge and incoming-edge geometry
+    float2 *fea = nullptr;
     double *fbuf = nullptr;
 
     // kernel timing (lskum_profile): event pairs per kernel class, reused
@@ -1320,6 +1323,8 @@ static lskum_status vjp_workspace(lskum_ctx *c)
     CK(c, dalloc(c, &c->toff, n + 1));
     CK(c, dalloc(c, &c->tedge, m));
     CK(c, dalloc(c, &c->tsrc, m));
+    CK(c, dalloc(c, &c->tlsw, m));
+    CK(c, dalloc(c, &c->thd, m));
     CK(c, dalloc(c, &c->vUacc, 4 * n));
     CK(c, dalloc(c, &c->vpxy, n));
     CK(c, dalloc(c, &c->fdsb, std::max<int64_t>(c->n_wall, 1)));
@@ -1331,14 +1336,13 @@ static lskum_status vjp_workspace(lskum_ctx *c)
     }
     c->launches += 4;
     LAUNCH(c, build_transpose_csr(n, c->nnz, c->off, c->idx, c->toff, c->tedge, c->tsrc, c->stream));
+    LAUNCH(c, build_incoming(c->geom(), c->nnz, c->tedge, c->tsrc, c->tlsw, c->thd, c->stream));
     c->vjp_ready = true;
     return LSKUM_OK;
 }
 
 static AdjParams adj_params(lskum_ctx *c)
 {
-    const int64_t n = c->n;
-    const int K = c->cfg.order == 2 ? c->cfg.inner_iters : 0;
     AdjParams P{};
     P.g = c->geom();
     P.q = c->vq;
@@ -1353,6 +1357,8 @@ static AdjParams adj_params(lskum_ctx *c)
     P.toff = c->toff;
     P.tedge = c->tedge;
     P.tsrc = c->tsrc;
+    P.tlsw = c->tlsw;
+    P.thd = c->thd;
     P.perm = c->perm;
     P.inv_gm1 = c->gas.inv_gm1;
     P.g14 = c->gas.g14;
@@ -1421,6 +1427,11 @@ static lskum_status fvjp_workspace(lskum_ctx *c)
     CK(c, dalloc(c, &c->fRb, 4 * n));
     CK(c, dalloc(c, &c->fqb, 4 * n));
     CK(c, dalloc(c, &c->febar, 4 * m));
+    CK(c, dalloc(c, &c->fef, m));
+    CK(c, dalloc(c, &c->fea, m));
+    CK(c, dalloc(c, &c->ftf, m));
+    c->launches++;
+    LAUNCH(c, build_float_geometry(c->geom(), c->nnz, c->tlsw, c->thd, c->fef, c->fea, c->ftf, c->stream));
     c->fvjp_ready = true;
     return LSKUM_OK;
 }
@@ -1458,21 +1469,24 @@ static lskum_status vjp_residual_fp32(lskum_ctx *c, const double *Ui, double *Ub
     P.toff = Pd.toff;
     P.tedge = Pd.tedge;
     P.tsrc = Pd.tsrc;
+    P.ef = c->fef;
+    P.ea = c->fea;
+    P.tf = c->ftf;
     P.perm = Pd.perm;
     P.inv_gm1 = Pd.inv_gm1;
     P.g14 = Pd.g14;
     P.order = Pd.order;
     c->launches++;
-    LAUNCH(c, launch_adj_flux(P, c->stream));
+    LAUNCH(c, launch_adj_flux(P, geom, c->stream));
     if (second) {
-        CK(c, cudaMemsetAsync(c->vabar, 0, std::max<int64_t>(c->nnz, 1) * sizeof(double2), c->stream));
+        if (geom) CK(c, cudaMemsetAsync(c->vabar, 0, std::max<int64_t>(c->nnz, 1) * sizeof(double2), c->stream));
         float *gin = c->fgb, *gout = c->fgb2;
         for (int k = K; k >= 1; --k) {
             LAUNCH(c, launch_adj_grad(P, (const float *)(c->fG + (int64_t)(k - 1) * 8 * n), (const float *)gin,
-                                      gout, c->stream));
+                                      gout, geom, c->stream));
             std::swap(gin, gout);
         }
-        LAUNCH(c, launch_adj_grad(P, (const float *)nullptr, (const float *)gin, (float *)nullptr, c->stream));
+        LAUNCH(c, launch_adj_grad(P, (const float *)nullptr, (const float *)gin, (float *)nullptr, geom, c->stream));
     }
     if (geom) LAUNCH(c, launch_adj_weights(Pd, c->stream));
     LAUNCH(c, launch_adj_state(P, Ui, Ub_acc, c->stream));
@@ -1491,9 +1505,9 @@ static lskum_status vjp_residual(lskum_ctx *c, const double *Ui, double *Ub_acc,
     if (!fwd_done && (st = vjp_forward(c, Ui)) != LSKUM_OK) return st;
     const AdjParams P = adj_params(c);
     c->launches++;
-    LAUNCH(c, launch_adj_flux(P, c->stream));
+    LAUNCH(c, launch_adj_flux(P, geom, c->stream));
     if (second) {
-        CK(c, cudaMemsetAsync(c->vabar, 0, std::max<int64_t>(c->nnz, 1) * sizeof(double2), c->stream));
+        if (geom) CK(c, cudaMemsetAsync(c->vabar, 0, std::max<int64_t>(c->nnz, 1) * sizeof(double2), c->stream));
         double *gin = c->vgb, *gout = c->vgb2;
         if (limited(c)) {
             // the limiter first: the flux saw the limited last iterate
@@ -1503,10 +1517,10 @@ static lskum_status vjp_residual(lskum_ctx *c, const double *Ui, double *Ub_acc,
             std::swap(gin, gout);
         }
         for (int k = K; k >= 1; --k) {
-            LAUNCH(c, launch_adj_grad(P, c->vG + (int64_t)(k - 1) * 8 * n, gin, gout, c->stream));
+            LAUNCH(c, launch_adj_grad(P, c->vG + (int64_t)(k - 1) * 8 * n, gin, gout, geom, c->stream));
             std::swap(gin, gout);
         }
-        LAUNCH(c, launch_adj_grad(P, (const double *)nullptr, (const double *)gin, (double *)nullptr, c->stream));
+        LAUNCH(c, launch_adj_grad(P, (const double *)nullptr, (const double *)gin, (double *)nullptr, geom, c->stream));
     }
     if (geom) LAUNCH(c, launch_adj_weights(P, c->stream));
     LAUNCH(c, launch_adj_state(P, Ui, Ub_acc, c->stream));

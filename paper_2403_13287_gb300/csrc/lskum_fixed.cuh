@@ -162,6 +162,7 @@ struct FixState {
     int64_t St, Sn;        // Q61, |.| < 4
     int64_t H;             // Q59, hc + (St^2 + Sn^2)/2 < 9.7
     int64_t c0, c1, c3;    // rho r, rho r^2, rho r^3: c 2^e, e from n and k (fix_e0 ...)
+    int64_t r;             // r 2^k in Q61, (0.7, 1.42)
     int n, k;              // exp(q1 + s2) = M 2^n, beta = b 4^k
 };
 LSKUM_FIX_FN int fix_e0(int n, int k) { return n - 6 * k - 58; }
@@ -260,6 +261,7 @@ LSKUM_FIX_FN bool fix_state(const double q[4], FixOp nx, FixOp ny, FixState &s)
     s.c0 = fix_mul_s<1>(M, r6);                                  // Q58, below 2^62 like the others
     s.c1 = fix_mul_s<1>(M, r7);                                  // Q57
     s.c3 = fix_mul_s<1>(M, r8);                                  // Q57
+    s.r = r;
     s.n = n;
     s.k = k;
     return ok;
@@ -276,9 +278,8 @@ LSKUM_FIX_FN int64_t fix_align_half(int64_t c, int e, int eo, int &es)
 // high word hi) into [2^61, 2^62)
 LSKUM_FIX_FN int fix_top(int64_t c, uint32_t hi) { return fix_clz((uint32_t)((uint64_t)c >> 32) | hi) - 2; }
 
-// the bounded parts of one state's split flux with z = sgn S_d, So the
-// transverse S: P in Q61, Phi/2 + z P in Q58, So P in Q58, H P - E/4 in Q57
-LSKUM_FIX_FN void fix_parts(int64_t Sd, int64_t sgn, int64_t So, int64_t H, int64_t F[4])
+// Phi (Q62), E (Q62) and P (Q61) of z = sgn S_d, returned with z (Q61) as an operand
+LSKUM_FIX_FN FixOp fix_phi_e(int64_t Sd, int64_t sgn, int64_t &Phi, int64_t &E, int64_t &P)
 {
     const int64_t a = fix_flip(Sd, Sd >> 63);
     const int kr = (int)((a + (1ll << 49)) >> 50);
@@ -308,11 +309,20 @@ LSKUM_FIX_FN void fix_parts(int64_t Sd, int64_t sgn, int64_t So, int64_t H, int6
     t1 += ((int64_t)t2 * uh) >> 12;
     e1 += ((int64_t)e2 * uh) >> 12;
     const int64_t T = t0 + (fix_mul(fix_op(t1), uo) >> 11);   // erf|z|/2, Q62
-    const int64_t E = e0 + (fix_mul(fix_op(e1), uo) >> 11);   // exp(-z^2)/(2 sqrt(pi)), Q62
+    E = e0 + (fix_mul(fix_op(e1), uo) >> 11);                 // exp(-z^2)/(2 sqrt(pi)), Q62
     const int64_t z = fix_flip(Sd, sgn);                      // Q61
-    const int64_t Phi = (1ll << 61) + fix_flip(T, z >> 63);   // Q62
+    Phi = (1ll << 61) + fix_flip(T, z >> 63);                 // Q62
     const FixOp zo = fix_op(z);
-    const int64_t P = (E >> 1) + fix_shl(fix_mul(zo, fix_op(Phi)), 2);
+    P = (E >> 1) + fix_shl(fix_mul(zo, fix_op(Phi)), 2);
+    return zo;
+}
+
+// the bounded parts of one state's split flux with z = sgn S_d, So the
+// transverse S: P in Q61, Phi/2 + z P in Q58, So P in Q58, H P - E/4 in Q57
+LSKUM_FIX_FN void fix_parts(int64_t Sd, int64_t sgn, int64_t So, int64_t H, int64_t F[4])
+{
+    int64_t Phi, E, P;
+    const FixOp zo = fix_phi_e(Sd, sgn, Phi, E, P);
     const FixOp Po = fix_op(P);
     F[0] = P;
     F[1] = (Phi >> 5) + fix_mul(zo, Po);

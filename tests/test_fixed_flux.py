@@ -323,3 +323,58 @@ def test_every_launch_form_gives_the_same_bits(order, limiter, boundary):
     Ro, S = oracle.residual(mid, oracle.split_stencils(mid), U0[id(mid)], order=order, inner=3, limiter=limiter,
                             want_scale=True, boundary=boundary, mach=0.85, aoa_deg=1.0)
     assert np.all(np.abs(got[3][0] - Ro) <= 1e-12 * S + 1e-300)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("gamma,mach", [(1.4, 7.0), (1.3, 2.0)])
+def test_vjp_across_the_range_matches_the_oracle(gamma, mach):
+    """The two-lane flux adjoint with states on both sides of the fixed-point
+    range, and the one-lane FP64 one (gamma = 1.3): sampled entries against
+    complex-step derivatives, at the VJP tests' 1e-10 of the largest."""
+    import torch
+
+    import oracle
+    from oracle import lskum_jvp
+    from paper_2403_13287_gb300.cloudgen import naca0012_cloud
+    from paper_2403_13287_gb300.lskum import Solver
+    c = naca0012_cloud(130, 24, seed=11)
+    rng = np.random.default_rng(4)
+    n = c["n"]
+    rho, p = 1 + 0.2 * rng.uniform(-1, 1, n), (1 + 0.2 * rng.uniform(-1, 1, n)) / gamma
+    m, a = mach * rng.uniform(0, 1, n), rng.uniform(0, 2 * np.pi, n)
+    u, v = m * np.sqrt(gamma * p / rho) * np.cos(a), m * np.sqrt(gamma * p / rho) * np.sin(a)
+    U = np.ascontiguousarray(np.stack([rho, rho * u, rho * v, p / (gamma - 1) + 0.5 * rho * (u * u + v * v)]))
+    Rb = rng.standard_normal((4, n))
+    s = Solver(c, order=1, inner_iters=0, mach=0.8, aoa_deg=1.0, gamma=gamma, reorder=1)
+    Ub, xb, yb = (t.cpu().numpy() for t in s.residual_vjp(torch.from_numpy(Rb).cuda(), torch.from_numpy(U).cuda()))
+    s.close()
+    ent = [("U", int(rng.integers(4)), int(k)) for k in rng.choice(n, 40, replace=False)]
+    ent += [(d, int(k)) for d in "xy" for k in rng.choice(n, 20, replace=False)]
+    want = lskum_jvp.vjp_entries(c, oracle.split_stencils(c), U, Rb, ent, order=1, inner=0, gamma=gamma)
+    got = np.array([Ub[e[1], e[2]] if e[0] == "U" else (xb if e[0] == "x" else yb)[e[1]] for e in ent])
+    for kind in "Uxy":
+        k = [i for i, e in enumerate(ent) if e[0] == kind]
+        assert np.all(np.abs(got - want)[k] <= 1e-10 * np.abs(want).max())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision,fp32,limiter", [(0, False, 0.0), (0, False, 1.0), (1, True, 0.0)])
+def test_state_cotangent_alone_is_that_of_the_full_product(precision, fp32, limiter):
+    """Without coordinate cotangents the reverse pass skips the weights' and
+    offsets' ones: U_bar is the same. (FP64 bitwise; FP32 to 1e-6 of its
+    largest entry: the two instantiations may contract differently.)"""
+    import torch
+
+    from paper_2403_13287_gb300.cloudgen import naca0012_cloud, smooth_state
+    from paper_2403_13287_gb300.lskum import Solver
+    c = naca0012_cloud(180, 99, seed=3, shuffle=True)
+    U = torch.from_numpy(smooth_state(c, 0.85, 1.0, amp=0.05, seed=9)).cuda()
+    Rb = torch.from_numpy(np.random.default_rng(1).standard_normal((4, c["n"]))).cuda()
+    s = Solver(c, order=2, inner_iters=3, limiter_K=limiter, precision=precision, reorder=1)
+    full = s.residual_vjp(Rb, U, fp32=fp32)[0].cpu().numpy()
+    only = s.residual_vjp(Rb, U, want_xy=False, fp32=fp32)[0].cpu().numpy()
+    s.close()
+    if fp32:
+        assert np.abs(full - only).max() <= 1e-6 * np.abs(full).max()
+    else:
+        assert np.array_equal(full, only)
