@@ -16,6 +16,11 @@ d^n/ds^n exp(-s^2) = (-1)^n H_n(s) exp(-s^2), erf' = 2/sqrt(pi) exp(-s^2).
 2. 2^(j/4096) 2^62, j = 0..4095, for the table-driven exp (P. T. P. Tang,
 ACM Trans. Math. Software 15 (1989) 144-157).
 
+3. log2 of a mantissa m in [1, 2): for the interval j of 1024, r_j is the
+reciprocal of its middle rounded to 32 bits (r_j 2^32) and the table holds
+-log2(r_j) 2^60; log2(m) = -log2(r_j) + log2(m r_j) with m r_j - 1 = z,
+|z| < 1.0005 2^-11, by the series of log2(1 + z) to z^5 in u = 2^11 z.
+
 The values are computed with mpmath at 50 significant digits and rounded to
 the nearest integer.
 
@@ -31,6 +36,7 @@ KMAX = 4 * STEP      # s_k up to 4
 DEG = 4
 SCALE = [62, 75, 56, 57, 58]
 EXP_N = 4096
+LOG_N = 1024
 
 
 def hermite(n, x):
@@ -90,6 +96,17 @@ def main():
         "#define LSKUM_FIX_A3 %d" % int(mp.nint(mp.ldexp(a1 ** 3 / 6, 59))),
         "#define LSKUM_FIX_LOG2E %dll" % int(mp.nint(mp.ldexp(1 / mp.log(2), 62))),
     ]
+    lines += ["", "// r_j 2^32 and -log2(r_j) 2^60", "struct FixLogRow {", "    int64_t log2c;", "    uint32_t r, pad;", "};",
+              "LSKUM_FIX_TABLE FixLogRow kFixLog2[%d] = {" % LOG_N]
+    for j in range(LOG_N):
+        r = int(mp.nint(mp.ldexp(1 / (1 + (mp.mpf(j) + mp.mpf(1) / 2) / LOG_N), 32)))
+        lines.append("    {%dll, %du, 0}," % (int(mp.nint(mp.ldexp(-mp.log(mp.ldexp(mp.mpf(r), -32)) / mp.log(2), 60))), r))
+    lines.append("};")
+    c = [(-1) ** (n + 1) / (n * mp.log(2)) * mp.mpf(2) ** (-11 * n) for n in range(1, 6)]
+    lines.append("// log2(1 + z) = u (c_1 + u (c_2 + u (c_3 + u (c_4 + u c_5)))): c_1 2^72, c_2 2^84, c_3 2^64, c_4 2^65, c_5 2^66; ln2 2^63")
+    for n, q in zip(range(1, 6), (72, 84, 64, 66, 68)):
+        lines.append("#define LSKUM_FIX_LOG_C%d %d%s" % (n, int(mp.nint(mp.ldexp(c[n - 1], q))), "ll" if n < 3 else ""))
+    lines.append("#define LSKUM_FIX_LN2 %dll" % int(mp.nint(mp.ldexp(mp.log(2), 63))))
     with open(os.path.join(here, "fix_tables.h"), "w") as f:
         f.write("\n".join(lines) + "\n")
 

@@ -607,7 +607,7 @@ __device__ __noinline__ StateCotangent state_cotangent_fp64(double q0, double q1
 }
 
 template <bool GEOM>
-__global__ void __launch_bounds__(128) k_adj_flux_pair(AdjParams P)
+__global__ void __launch_bounds__(128, 5) k_adj_flux_pair(AdjParams P)
 {
     const DevGeom &g = P.g;
     const int64_t pp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 1;
@@ -794,36 +794,6 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather(AdjParamsT<T> P)
     if (second) st8(P.gbar, p, gb);
 }
 
-// full-stencil weights and half offset of edge e of point p (neighbour i)
-__device__ __forceinline__ void outgoing(const AdjParamsT<double> &P, int e, int i, double2 xyp, bool inner, double &hx,
-                                         double &hy, double &ax, double &ay)
-{
-    const double2 a = P.g.lsw[e];
-    ax = a.x;
-    ay = a.y;
-    if (!inner) return;
-    if (P.g.hd) {
-        const double2 hh = P.g.hd[e];
-        hx = hh.x;
-        hy = hh.y;
-    } else {
-        const double2 xyi = P.g.xy[i];
-        hx = 0.5 * (xyi.x - xyp.x);
-        hy = 0.5 * (xyi.y - xyp.y);
-    }
-}
-__device__ __forceinline__ void outgoing(const AdjParamsT<float> &P, int e, int, double2, bool inner, float &hx,
-                                         float &hy, float &ax, float &ay)
-{
-    const float2 a = __ldg(P.ea + e);
-    ax = a.x;
-    ay = a.y;
-    if (!inner) return;
-    const float4 v = __ldg(P.ef + e);
-    hx = 0.5f * v.x;
-    hy = 0.5f * v.y;
-}
-
 // ---------------------------------------------------------------------------
 // one least-squares pass of E15 in reverse. Forward (per component c):
 //   g_p = sum_e a_e s_e,  s_e = (q_i - q_p) - [dx (gx'_i - gx'_p) + dy (gy'_i - gy'_p)]/2
@@ -833,62 +803,62 @@ __device__ __forceinline__ void outgoing(const AdjParamsT<float> &P, int e, int,
 // 640k points: 228 -> 58 us a pass, half of it from the geometry's FP32 copies,
 // which spare the FP64 pipe the conversions).
 // ---------------------------------------------------------------------------
-template <class T, bool GEOM>
-__global__ void __launch_bounds__(128) k_adj_grad(AdjParamsT<T> P, const T *__restrict__ gprev,
-                                                  const T *__restrict__ gbar_in, T *__restrict__ gbar_out)
+template <bool GEOM>
+__global__ void __launch_bounds__(128) k_adj_grad_fp32(AdjParamsT<float> P, const float *__restrict__ gprev,
+                                                       const float *__restrict__ gbar_in,
+                                                       float *__restrict__ gbar_out, int first)
 {
     const DevGeom &g = P.g;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= g.n) return;
     const bool inner = gprev != nullptr;
-    T qb[4], gb[8], qp[4], gbo[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    float qb[4], gb[8], qp[4], gbo[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     ld4(P.qbar, p, qb);
     ld8(gbar_in, p, gb);
-    double2 xyp = make_double2(0.0, 0.0);
-    if constexpr (GEOM) {
-        ld4(P.q, p, qp);
-        if (!g.hd) xyp = g.xy[p];
-    }
+    if constexpr (GEOM) ld4(P.q, p, qp);
     // an inner pass is sum_e a_e (q_i - q_0 - h_e.grad q_i) + grad q_0 / 2
     // (h_e the half offset; the terms in grad q_0 add up to grad q_0 / 2 since
     // sum_e a_e d_e^T = I, and the forward passes take them so), so grad q_0
     // gets gb / 2 and neither the weights nor the offsets see grad q_0
     if (inner) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) gbo[k] = T(0.5) * gb[k];
+        for (int k = 0; k < 8; ++k) gbo[k] = 0.5f * gb[k];
     }
     // outgoing edges: owner terms, and the cotangents of a_e and of the offsets
     for (int e = g.off[p]; e < g.off[p + 1]; ++e) {
-        T hx = T(0), hy = T(0), ax, ay;
+        const float2 a = __ldg(P.ea + e);
         if constexpr (!GEOM) {
-            outgoing(P, e, 0, xyp, false, hx, hy, ax, ay);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const T sb = ax * gb[k] + ay * gb[4 + k];
+                const float sb = a.x * gb[k] + a.y * gb[4 + k];
                 qb[k] -= sb;
             }
         } else {
             const int i = g.idx[e];
-            outgoing(P, e, i, xyp, inner, hx, hy, ax, ay);
-            T qi[4], gi[8];
+            float qi[4], gi[8], hx = 0.0f, hy = 0.0f;
             ld4(P.q, i, qi);
-            if (inner) ld8(gprev, i, gi);
-            T abx = T(0), aby = T(0), dbx = T(0), dby = T(0);
+            if (inner) {
+                const float4 v = __ldg(P.ef + e);
+                hx = 0.5f * v.x;
+                hy = 0.5f * v.y;
+                ld8(gprev, i, gi);
+            }
+            float abx = 0.0f, aby = 0.0f, dbx = 0.0f, dby = 0.0f;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const T sb = ax * gb[k] + ay * gb[4 + k];
-                T s = qi[k] - qp[k];
+                const float sb = a.x * gb[k] + a.y * gb[4 + k];
+                float s = qi[k] - qp[k];
                 if (inner) {
                     s = s - (hx * gi[k] + hy * gi[4 + k]);
                     // d_e = 2 h_e: d_bar = -(sb/2) grad q_i
-                    dbx -= T(0.5) * sb * gi[k];
-                    dby -= T(0.5) * sb * gi[4 + k];
+                    dbx -= 0.5f * sb * gi[k];
+                    dby -= 0.5f * sb * gi[4 + k];
                 }
                 qb[k] -= sb;
                 abx += s * gb[k];
                 aby += s * gb[4 + k];
             }
-            double2 ab = P.abar[e];
+            double2 ab = first ? make_double2(0.0, 0.0) : P.abar[e];
             ab.x += to_f64(abx);
             ab.y += to_f64(aby);
             P.abar[e] = ab;
@@ -904,13 +874,13 @@ __global__ void __launch_bounds__(128) k_adj_grad(AdjParamsT<T> P, const T *__re
     const int t1 = P.toff[p + 1];
     for (int t = P.toff[p]; t < t1; ++t) {
         const int src = P.tsrc[t];
-        T hx, hy, ax, ay;
+        float hx, hy, ax, ay;
         incoming(P, t, hx, hy, ax, ay);
-        T gs[8];
+        float gs[8];
         ld8(gbar_in, src, gs);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const T sb = ax * gs[k] + ay * gs[4 + k];
+            const float sb = ax * gs[k] + ay * gs[4 + k];
             qb[k] += sb;
             if (inner) {
                 gbo[k] -= hx * sb;
@@ -920,6 +890,122 @@ __global__ void __launch_bounds__(128) k_adj_grad(AdjParamsT<T> P, const T *__re
     }
     st4(P.qbar, p, qb);
     if (inner) st8(gbar_out, p, gbo);
+}
+
+// The FP64 pass: the outgoing and the incoming edges of a point go to blocks of
+// their own (blockIdx.y; twice the warps in flight, half the serial chain),
+// which keep the q cotangent apart (qbar2: the owner's share, summed with qbar
+// by k_adj_state), and the two-term products run on the integer pipes
+// (fix_dot): 40 FP64 instructions per edge of 68. 87 -> 62 us a pass at 40k points.
+__device__ __forceinline__ double dot2(const FixPair &a, const FixPair &b, double ax, double ay, double bx, double by)
+{
+    if (fix_dot_in_range(a, b)) return fix_dot(a, b);
+    return b.e ? fma(ay, by, ax * bx) : 0.0;   // both terms zero (or subnormal): nothing to add
+}
+
+template <bool GEOM>
+__global__ void __launch_bounds__(128, 5) k_adj_grad_fp64(AdjParams P, const double *__restrict__ gprev,
+                                                          const double *__restrict__ gbar_in,
+                                                          double *__restrict__ gbar_out, int first)
+{
+    const DevGeom &g = P.g;
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= g.n) return;
+    const bool inner = gprev != nullptr;
+    double qb[4] = {0.0, 0.0, 0.0, 0.0}, gb[8];
+    ld8(gbar_in, p, gb);
+    if (blockIdx.y == 0) {
+        // outgoing edges: owner terms, and the cotangents of a_e and of the offsets
+        if (!first) ld4(P.qbar2, p, qb);
+        FixPair gbp[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) gbp[k] = fix_pair(gb[k], gb[4 + k]);
+        double qp[4];
+        double2 xyp = make_double2(0.0, 0.0);
+        if constexpr (GEOM) {
+            ld4(P.q, p, qp);
+            if (!g.hd) xyp = g.xy[p];
+        }
+        const int e1 = g.off[p + 1];
+#pragma unroll 1
+        for (int e = g.off[p]; e < e1; ++e) {
+            const double2 a = g.lsw[e];
+            const FixPair ap = fix_pair(a.x, a.y);
+            double sb[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                sb[k] = dot2(ap, gbp[k], a.x, a.y, gb[k], gb[4 + k]);
+                qb[k] -= sb[k];
+            }
+            if constexpr (GEOM) {
+                const int64_t i = g.idx[e];
+                double qi[4], gi[8], s[4];
+                gather4(P.q, i, qi);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) s[k] = qi[k] - qp[k];
+                if (inner) {
+                    double2 h;
+                    if (g.hd) {
+                        h = g.hd[e];
+                    } else {
+                        const double2 xyi = g.xy[i];
+                        h = make_double2(0.5 * (xyi.x - xyp.x), 0.5 * (xyi.y - xyp.y));
+                    }
+                    const FixPair hp = fix_pair(h.x, h.y);
+                    gather8(gprev, i, gi);
+                    double dbx = 0.0, dby = 0.0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        s[k] -= dot2(hp, fix_pair(gi[k], gi[4 + k]), h.x, h.y, gi[k], gi[4 + k]);
+                        // d_e = 2 h_e: d_bar = -(sb/2) grad q_i
+                        dbx = fma(sb[k], gi[k], dbx);
+                        dby = fma(sb[k], gi[4 + k], dby);
+                    }
+                    double2 db = P.dbar[e];
+                    db.x = fma(-0.5, dbx, db.x);
+                    db.y = fma(-0.5, dby, db.y);
+                    P.dbar[e] = db;
+                }
+                double2 ab = first ? make_double2(0.0, 0.0) : P.abar[e];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    ab.x = fma(s[k], gb[k], ab.x);
+                    ab.y = fma(s[k], gb[4 + k], ab.y);
+                }
+                P.abar[e] = ab;
+            }
+        }
+        st4(P.qbar2, p, qb);
+    } else {
+        // incoming edges: the terms of this point as a neighbour; an inner pass
+        // gives grad q_0 the cotangent gb / 2 (see k_adj_grad_fp32)
+        ld4(P.qbar, p, qb);
+        double gbo[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) gbo[k] = 0.5 * gb[k];
+        const int t1 = P.toff[p + 1];
+#pragma unroll 1
+        for (int t = P.toff[p]; t < t1; ++t) {
+            const int64_t src = P.tsrc[t];
+            const double2 a = __ldg(P.tlsw + t);
+            const FixPair ap = fix_pair(a.x, a.y);
+            double gs[8];
+            gather8(gbar_in, src, gs);
+            double2 h = make_double2(0.0, 0.0);
+            if (inner) h = __ldg(P.thd + t);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const double sb = dot2(ap, fix_pair(gs[k], gs[4 + k]), a.x, a.y, gs[k], gs[4 + k]);
+                qb[k] += sb;
+                if (inner) {
+                    gbo[k] = fma(-h.x, sb, gbo[k]);
+                    gbo[4 + k] = fma(-h.y, sb, gbo[4 + k]);
+                }
+            }
+        }
+        st4(P.qbar, p, qb);
+        if (inner) st8(gbar_out, p, gbo);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1075,11 +1161,58 @@ __global__ void __launch_bounds__(128) k_adj_limit_gather(AdjParams P, const int
 }
 
 // ---------------------------------------------------------------------------
-// least-squares weights back to edge offsets (owner side)
+// least-squares weights back to edge offsets (owner side). A system with
+// M = sum d d^T and weights a = M^-1 d gives
+//   d_bar_k = b_k - B d_k,  b = M^-1 a_bar,  B = sum (b a^T + a b^T)
+//           = M^-1 [sum (a_bar d^T + d a_bar^T)] M^-1.
+// Full stencil (global frame): a_bar = abar. A sub-stencil (frame (s, n)) takes
+// one row of M^-1 d as its weight, so a_bar is the weight's cotangent wb along
+// that row, b = wb beta with beta the row of M^-1, and the bracket needs only
+// D = sum wb d. One pass over the edges forms all sums, a second the offsets'
+// cotangents: 53 FP64 instructions per edge and no indexed local arrays, where
+// three passes with b and a per edge took 125 (141 -> 94 us at 40k points).
 // ---------------------------------------------------------------------------
 struct Sym2 {
     double xx, xy, yy;
 };
+__device__ __forceinline__ Sym2 inverse2(const Sym2 &A)
+{
+    const double r = 1.0 / (A.xx * A.yy - A.xy * A.xy);
+    return Sym2{A.yy * r, -A.xy * r, A.xx * r};
+}
+__device__ __forceinline__ double2 times(const Sym2 &A, double2 v)
+{
+    return make_double2(fma(A.xx, v.x, A.xy * v.y), fma(A.xy, v.x, A.yy * v.y));
+}
+struct SubSums {   // one sub-stencil: M and D
+    Sym2 M;
+    double2 D;
+    __device__ __forceinline__ void add(bool in, double ds, double dn, double wb)
+    {
+        if (!in) return;
+        M.xx = fma(ds, ds, M.xx);
+        M.xy = fma(ds, dn, M.xy);
+        M.yy = fma(dn, dn, M.yy);
+        D.x = fma(wb, ds, D.x);
+        D.y = fma(wb, dn, D.y);
+    }
+};
+struct SubBack {   // beta and B = beta A^T + A beta^T, A = M^-1 D
+    double2 beta;
+    Sym2 B;
+};
+__device__ __forceinline__ SubBack sub_back(const SubSums &s, bool need, bool row1)
+{
+    SubBack o = {make_double2(0.0, 0.0), Sym2{0.0, 0.0, 0.0}};
+    if (!need) return o;
+    const Sym2 Mi = inverse2(s.M);
+    o.beta = row1 ? make_double2(Mi.xy, Mi.yy) : make_double2(Mi.xx, Mi.xy);
+    const double2 A = times(Mi, s.D);
+    o.B.xx = 2.0 * o.beta.x * A.x;
+    o.B.xy = fma(o.beta.x, A.y, o.beta.y * A.x);
+    o.B.yy = 2.0 * o.beta.y * A.y;
+    return o;
+}
 
 __global__ void __launch_bounds__(128) k_adj_weights(AdjParams P)
 {
@@ -1092,78 +1225,68 @@ __global__ void __launch_bounds__(128) k_adj_weights(AdjParams P)
     const double2 n0 = g.nrm[p];
     const double tx = n0.y, ty = -n0.x;
     const int e0 = g.off[p], e1 = g.off[p + 1];
-    // normal-equation sums: full stencil (global frame) and the sub-stencils (s, n)
-    Sym2 M = {0, 0, 0}, Ms[4] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+    Sym2 M = {0, 0, 0}, S = {0, 0, 0};
+    SubSums s0 = {}, s1 = {}, s2 = {}, s3 = {};
     for (int e = e0; e < e1; ++e) {
         const double2 xyi = g.xy[g.idx[e]];
         const double dx = xyi.x - xy0.x, dy = xyi.y - xy0.y;
         const double ds = dx * tx + dy * ty, dn = dx * n0.x + dy * n0.y;
-        M.xx += dx * dx; M.xy += dx * dy; M.yy += dy * dy;
         const uint8_t m = g.mask[e];
-        const int ks = xsub(m), kn = ysub(m);
-        if (ks >= 0) { Ms[ks].xx += ds * ds; Ms[ks].xy += ds * dn; Ms[ks].yy += dn * dn; }
-        if (kn >= 0) { Ms[kn].xx += ds * ds; Ms[kn].xy += ds * dn; Ms[kn].yy += dn * dn; }
-    }
-    // inverses (M^-1 = [[yy, -xy], [-xy, xx]] / det)
-    auto inv = [](const Sym2 &A) {
-        const double det = A.xx * A.yy - A.xy * A.xy;
-        Sym2 r = {A.yy / det, -A.xy / det, A.xx / det};
-        return r;
-    };
-    const Sym2 Mi = inv(M);
-    Sym2 Msi[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) Msi[k] = sub_needed(f, k) ? inv(Ms[k]) : Sym2{0, 0, 0};
-    // B = sum (b a^T + a b^T) per system, with a = M^-1 d and b = M^-1 a_bar
-    Sym2 B = {0, 0, 0}, Bs[4] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int e = e0; e < e1; ++e) {
-            const double2 xyi = g.xy[g.idx[e]];
-            const double dx = xyi.x - xy0.x, dy = xyi.y - xy0.y;
-            const double ds = dx * tx + dy * ty, dn = dx * n0.x + dy * n0.y;
-            const uint8_t m = g.mask[e];
-            const int ks = xsub(m), kn = ysub(m);
-            double gx = 0.0, gy = 0.0;   // offset cotangent, global frame
-            double gs = 0.0, gn = 0.0;   // offset cotangent, (s, n) frame
-            if (full) {
-                const double2 ab = P.abar[e];
-                const double ax = Mi.xx * dx + Mi.xy * dy, ay = Mi.xy * dx + Mi.yy * dy;
-                const double bx = Mi.xx * ab.x + Mi.xy * ab.y, by = Mi.xy * ab.x + Mi.yy * ab.y;
-                if (pass == 0) {
-                    B.xx += 2.0 * bx * ax;
-                    B.xy += bx * ay + ax * by;
-                    B.yy += 2.0 * by * ay;
-                } else {
-                    gx += bx - (B.xx * dx + B.xy * dy);
-                    gy += by - (B.xy * dx + B.yy * dy);
-                }
-            }
-            const double2 wb = P.wbar[e];
-            // x-sub weight = row 0 of M_s^-1 d, y-sub weight = row 1
-            for (int h = 0; h < 2; ++h) {
-                const int k = h == 0 ? ks : kn;
-                if (!sub_needed(f, k)) continue;
-                const Sym2 &Ai = Msi[k];
-                const double as = Ai.xx * ds + Ai.xy * dn, an = Ai.xy * ds + Ai.yy * dn;
-                const double abs_ = h == 0 ? wb.x : 0.0, abn = h == 0 ? 0.0 : wb.y;
-                const double bs = Ai.xx * abs_ + Ai.xy * abn, bn = Ai.xy * abs_ + Ai.yy * abn;
-                if (pass == 0) {
-                    Bs[k].xx += 2.0 * bs * as;
-                    Bs[k].xy += bs * an + as * bn;
-                    Bs[k].yy += 2.0 * bn * an;
-                } else {
-                    gs += bs - (Bs[k].xx * ds + Bs[k].xy * dn);
-                    gn += bn - (Bs[k].xy * ds + Bs[k].yy * dn);
-                }
-            }
-            if (pass == 1) {
-                // ds = dx tx + dy ty, dn = dx nx + dy ny
-                double2 d = P.dbar[e];
-                d.x += gx + gs * tx + gn * n0.x;
-                d.y += gy + gs * ty + gn * n0.y;
-                P.dbar[e] = d;
-            }
+        const double2 wb = P.wbar[e];
+        if (full) {
+            const double2 ab = P.abar[e];
+            M.xx = fma(dx, dx, M.xx);
+            M.xy = fma(dx, dy, M.xy);
+            M.yy = fma(dy, dy, M.yy);
+            S.xx = fma(ab.x, dx, S.xx);                          // half the diagonal
+            S.xy = fma(ab.x, dy, fma(ab.y, dx, S.xy));
+            S.yy = fma(ab.y, dy, S.yy);
         }
+        s0.add(xsub(m) == 0, ds, dn, wb.x);
+        s1.add(xsub(m) == 1, ds, dn, wb.x);
+        s2.add(ysub(m) == 2, ds, dn, wb.y);
+        s3.add(ysub(m) == 3, ds, dn, wb.y);
+    }
+    Sym2 Mi = {0, 0, 0}, B = {0, 0, 0};
+    if (full) {
+        Mi = inverse2(M);
+        // B = Mi S Mi, S with its diagonal doubled
+        const double2 c0 = times(Mi, make_double2(2.0 * S.xx, S.xy)), c1 = times(Mi, make_double2(S.xy, 2.0 * S.yy));
+        const double2 b0 = times(Mi, make_double2(c0.x, c1.x)), b1 = times(Mi, make_double2(c0.y, c1.y));
+        B = Sym2{b0.x, b0.y, b1.y};
+    }
+    const SubBack k0 = sub_back(s0, sub_needed(f, 0), false), k1 = sub_back(s1, sub_needed(f, 1), false);
+    const SubBack k2 = sub_back(s2, sub_needed(f, 2), true), k3 = sub_back(s3, sub_needed(f, 3), true);
+    for (int e = e0; e < e1; ++e) {
+        const double2 xyi = g.xy[g.idx[e]];
+        const double dx = xyi.x - xy0.x, dy = xyi.y - xy0.y;
+        const double ds = dx * tx + dy * ty, dn = dx * n0.x + dy * n0.y;
+        const uint8_t m = g.mask[e];
+        const double2 wb = P.wbar[e];
+        double2 d = P.dbar[e];
+        if (full) {
+            const double2 b = times(Mi, P.abar[e]), c = times(B, make_double2(dx, dy));
+            d.x += b.x - c.x;
+            d.y += b.y - c.y;
+        }
+        double gs = 0.0, gn = 0.0;   // (s, n) frame
+        const int ks = xsub(m), kn = ysub(m);
+        if (sub_needed(f, ks)) {
+            const SubBack &k = ks == 0 ? k0 : k1;
+            const double2 c = times(k.B, make_double2(ds, dn));
+            gs += fma(wb.x, k.beta.x, -c.x);
+            gn += fma(wb.x, k.beta.y, -c.y);
+        }
+        if (sub_needed(f, kn)) {
+            const SubBack &k = kn == 2 ? k2 : k3;
+            const double2 c = times(k.B, make_double2(ds, dn));
+            gs += fma(wb.y, k.beta.x, -c.x);
+            gn += fma(wb.y, k.beta.y, -c.y);
+        }
+        // ds = dx tx + dy ty, dn = dx nx + dy ny
+        d.x += gs * tx + gn * n0.x;
+        d.y += gs * ty + gn * n0.y;
+        P.dbar[e] = d;
     }
 }
 
@@ -1213,6 +1336,11 @@ __global__ void __launch_bounds__(256) k_adj_state(AdjParamsT<T> P, const double
     ld4(P.qbar, p, qt);
 #pragma unroll
     for (int k = 0; k < 4; ++k) qb[k] = to_f64(qt[k]);
+    if (P.qbar2) {
+        ld4(P.qbar2, p, qt);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) qb[k] += to_f64(qt[k]);
+    }
     ld4(Ub_acc, p, ub);
     const double g = P.inv_gm1, gm1 = 1.0 / g;
     const double ir = 1.0 / u[0], m1 = u[1] * ir, m2 = u[2] * ir;            // velocities
@@ -1385,10 +1513,16 @@ cudaError_t launch_adj_flux(const AdjParamsT<T> &P, bool geom, cudaStream_t s)
 
 template <class T>
 cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gbar_in, T *gbar_out, bool geom,
-                            cudaStream_t s)
+                            bool first, cudaStream_t s)
 {
-    if (geom) k_adj_grad<T, true><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out);
-    else k_adj_grad<T, false><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out);
+    if constexpr (std::is_same<T, double>::value) {
+        const dim3 nb(blocks(P.g.n, 128), 2);
+        if (geom) k_adj_grad_fp64<true><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+        else k_adj_grad_fp64<false><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+    } else {
+        if (geom) k_adj_grad_fp32<true><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+        else k_adj_grad_fp32<false><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+    }
     return cudaGetLastError();
 }
 
@@ -1438,9 +1572,9 @@ cudaError_t launch_to_float(int64_t m, const double *a, float *b, cudaStream_t s
 template cudaError_t launch_adj_flux<double>(const AdjParamsT<double> &, bool, cudaStream_t);
 template cudaError_t launch_adj_flux<float>(const AdjParamsT<float> &, bool, cudaStream_t);
 template cudaError_t launch_adj_grad<double>(const AdjParamsT<double> &, const double *, const double *, double *, bool,
-                                             cudaStream_t);
+                                             bool, cudaStream_t);
 template cudaError_t launch_adj_grad<float>(const AdjParamsT<float> &, const float *, const float *, float *, bool,
-                                            cudaStream_t);
+                                            bool, cudaStream_t);
 template cudaError_t launch_adj_state<double>(const AdjParamsT<double> &, const double *, double *, cudaStream_t);
 template cudaError_t launch_adj_state<float>(const AdjParamsT<float> &, const double *, double *, cudaStream_t);
 

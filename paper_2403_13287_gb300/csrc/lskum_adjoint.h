@@ -17,6 +17,7 @@ struct AdjParamsT {
     const T *qg;           // [n][8] final q-derivative iterate (order 2)
     const T *Rbar;         // [n][4] residual cotangent
     T *qbar;               // [n][4] q cotangent (accumulated)
+    T *qbar2;              // [n][4] the gradient passes' owner-side share of it (FP64, order 2), or nullptr
     T *gbar;               // [n][8] cotangent of the final q-derivative iterate
     T *ebar;               // [nnz][4] cotangent of the neighbour's reconstructed state, per edge
     double2 *wbar;         // [nnz] cotangents of the sub-stencil weights (w_s, w_n)
@@ -54,10 +55,12 @@ cudaError_t build_float_geometry(const DevGeom &g, int64_t nnz, const double2 *t
 template <class T>
 cudaError_t launch_adj_flux(const AdjParamsT<T> &P, bool geom, cudaStream_t s);
 // one E15 pass in reverse: gbar_in is the cotangent of this pass's output,
-// gbar_out receives that of its input iterate gprev (nullptr for the first-order pass)
+// gbar_out receives that of its input iterate gprev (nullptr for the first-order
+// pass). The product's first such call (the last forward pass) starts abar and
+// qbar2, the others add.
 template <class T>
 cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gbar_in, T *gbar_out, bool geom,
-                            cudaStream_t s);
+                            bool first, cudaStream_t s);
 // the limiter (limiter_K > 0) in reverse, between the flux adjoint and the
 // last pass's: gbar_in is the cotangent of the limited last iterate, graw the
 // unlimited one; gbar_out receives the unlimited iterate's cotangent; adds

@@ -118,12 +118,19 @@ struct lskum_ctx {
 
     // residual VJP workspace (FP64, allocated on the first lskum_residual_vjp)
     bool vjp_ready = false;
-    double *vq = nullptr, *vG = nullptr, *vRb = nullptr, *vqb = nullptr, *vgb = nullptr, *vgb2 = nullptr;
+    // FP64 forward of a state: q, the K + 1 q-derivative iterates, the limited last
+    // one ([n][8], limiter_K > 0). The iteration VJP keeps one per RK stage
+    struct Forward {
+        double *q = nullptr, *G = nullptr, *Glim = nullptr;
+    };
+    Forward fw[4];
+    bool stage_forwards = false;  // fw[1..3] are there (else a stage's forward is run again)
+    double *vRb = nullptr, *vqb = nullptr, *vgb = nullptr, *vgb2 = nullptr;
     double *vebar = nullptr;
     double2 *vwbar = nullptr, *vabar = nullptr, *vdbar = nullptr;
     int32_t *toff = nullptr, *tedge = nullptr, *tsrc = nullptr;
     double2 *tlsw = nullptr, *thd = nullptr;  // weights and half offsets of the incoming edges
-    double *vGlim = nullptr;      // [n][8] the limited last iterate (limiter_K > 0)
+    double *vqb2 = nullptr;       // [n][4] owner-side share of the q cotangent (order 2)
     double *vext = nullptr;       // [n][4] the limiter's extremum measure (limiter_K > 0)
     int32_t *vlidx = nullptr;     // [n][4] limiter reverse: the extreme neighbour's edge
     double *vlval = nullptr;      // [n][4] limiter reverse: its q cotangent
@@ -1297,22 +1304,30 @@ extern "C" lskum_status lskum_residual(lskum_ctx *c, const double *U, double *R)
 static bool limited(const lskum_ctx *c) { return c->cfg.order == 2 && c->cfg.limiter_K > 0.0; }
 
 // the final q-derivative iterate of the FP64 forward recomputation (vjp_forward)
-static const double *vjp_final_gradient(const lskum_ctx *c)
+static const double *vjp_final_gradient(const lskum_ctx *c, const lskum_ctx::Forward &f)
 {
     if (c->cfg.order != 2) return nullptr;
-    return limited(c) ? c->vGlim : c->vG + (int64_t)c->cfg.inner_iters * 8 * c->n;
+    return limited(c) ? f.Glim : f.G + (int64_t)c->cfg.inner_iters * 8 * c->n;
+}
+
+static cudaError_t alloc_forward(lskum_ctx *c, lskum_ctx::Forward &f)
+{
+    const int64_t n = c->n;
+    cudaError_t e = dalloc(c, &f.q, 4 * n);
+    if (e == cudaSuccess && c->cfg.order == 2) e = dalloc(c, &f.G, (int64_t)(c->cfg.inner_iters + 1) * 8 * n);
+    if (e == cudaSuccess && limited(c)) e = dalloc(c, &f.Glim, 8 * n);
+    return e;
 }
 
 static lskum_status vjp_workspace(lskum_ctx *c)
 {
     if (c->vjp_ready) return LSKUM_OK;
     const int64_t n = c->n, m = std::max<int64_t>(c->nnz, 1);
-    const int K = c->cfg.order == 2 ? c->cfg.inner_iters : 0;
-    CK(c, dalloc(c, &c->vq, 4 * n));
+    CK(c, alloc_forward(c, c->fw[0]));
     if (c->cfg.order == 2) {
-        CK(c, dalloc(c, &c->vG, (int64_t)(K + 1) * 8 * n));
         CK(c, dalloc(c, &c->vgb, 8 * n));
         CK(c, dalloc(c, &c->vgb2, 8 * n));
+        CK(c, dalloc(c, &c->vqb2, 4 * n));
     }
     CK(c, dalloc(c, &c->vRb, 4 * n));
     CK(c, dalloc(c, &c->vqb, 4 * n));
@@ -1329,7 +1344,6 @@ static lskum_status vjp_workspace(lskum_ctx *c)
     CK(c, dalloc(c, &c->vpxy, n));
     CK(c, dalloc(c, &c->fdsb, std::max<int64_t>(c->n_wall, 1)));
     if (limited(c)) {
-        CK(c, dalloc(c, &c->vGlim, 8 * n));
         CK(c, dalloc(c, &c->vext, 4 * n));
         CK(c, dalloc(c, &c->vlidx, 4 * n));
         CK(c, dalloc(c, &c->vlval, 4 * n));
@@ -1341,14 +1355,15 @@ static lskum_status vjp_workspace(lskum_ctx *c)
     return LSKUM_OK;
 }
 
-static AdjParams adj_params(lskum_ctx *c)
+static AdjParams adj_params(lskum_ctx *c, const lskum_ctx::Forward &f)
 {
     AdjParams P{};
     P.g = c->geom();
-    P.q = c->vq;
-    P.qg = vjp_final_gradient(c);
+    P.q = f.q;
+    P.qg = vjp_final_gradient(c, f);
     P.Rbar = c->vRb;
     P.qbar = c->vqb;
+    P.qbar2 = c->vqb2;
     P.gbar = c->vgb;
     P.ebar = c->vebar;
     P.wbar = c->vwbar;
@@ -1366,40 +1381,40 @@ static AdjParams adj_params(lskum_ctx *c)
     return P;
 }
 
-// FP64 q and q-derivative iterates of an internal state (vq, vG; with the
-// limiter also the limited last iterate vGlim, the forward's last pass run
-// again with the limiter)
-static lskum_status vjp_forward(lskum_ctx *c, const double *Ui)
+// FP64 q and q-derivative iterates of an internal state into f; with the
+// limiter the last pass writes its iterate both before and after it
+static lskum_status vjp_forward(lskum_ctx *c, const double *Ui, const lskum_ctx::Forward &f)
 {
     const int64_t n = c->n;
     const int K = c->cfg.inner_iters;
     const DevGeom g = c->geom();
-    LAUNCH(c, launch_q_from_U(n, c->gas, Ui, c->vq, c->status, c->stream));
+    LAUNCH(c, launch_q_from_U(n, c->gas, Ui, f.q, c->status, c->stream));
     if (c->cfg.order == 2) {
+        const bool lim = limited(c);
         const double limK = c->cfg.limiter_K;
-        double *ext = limited(c) && K > 0 ? c->vext : nullptr;
-        LAUNCH(c, launch_qgrad(g, c->vq, nullptr, nullptr, c->vG, ext, 0.0, c->stream));
-        for (int k = 1; k <= K; ++k)
-            LAUNCH(c, launch_qgrad(g, c->vq, c->vG + (int64_t)(k - 1) * 8 * n, c->vG, c->vG + (int64_t)k * 8 * n,
-                                   nullptr, 0.0, c->stream));
-        if (limited(c)) {
-            if (K == 0) LAUNCH(c, launch_qgrad(g, c->vq, nullptr, nullptr, c->vGlim, nullptr, limK, c->stream));
-            else
-                LAUNCH(c, launch_qgrad(g, c->vq, c->vG + (int64_t)(K - 1) * 8 * n, c->vG, c->vGlim, ext, limK,
-                                       c->stream));
+        double *ext = lim && K > 0 ? c->vext : nullptr;
+        if (lim && K == 0)
+            LAUNCH(c, launch_qgrad(g, f.q, nullptr, nullptr, f.Glim, nullptr, limK, c->stream, f.G));
+        else
+            LAUNCH(c, launch_qgrad(g, f.q, nullptr, nullptr, f.G, ext, 0.0, c->stream));
+        for (int k = 1; k <= K; ++k) {
+            const double *old = f.G + (int64_t)(k - 1) * 8 * n;
+            double *out = f.G + (int64_t)k * 8 * n;
+            if (lim && k == K) LAUNCH(c, launch_qgrad(g, f.q, old, f.G, f.Glim, ext, limK, c->stream, out));
+            else LAUNCH(c, launch_qgrad(g, f.q, old, f.G, out, nullptr, 0.0, c->stream));
         }
     }
     return LSKUM_OK;
 }
 
-// FP64 residual of an internal state (Rout internal [n][4]); leaves vq, vG at that state
-static lskum_status residual_fp64(lskum_ctx *c, const double *Ui, double *Rout)
+// FP64 residual of an internal state (Rout internal [n][4]); leaves its forward in f
+static lskum_status residual_fp64(lskum_ctx *c, const double *Ui, double *Rout, const lskum_ctx::Forward &f)
 {
-    lskum_status st = vjp_forward(c, Ui);
+    lskum_status st = vjp_forward(c, Ui, f);
     if (st != LSKUM_OK) return st;
     FluxLaunch L{};
-    L.q = c->vq;
-    L.qg = vjp_final_gradient(c);
+    L.q = f.q;
+    L.qg = vjp_final_gradient(c, f);
     L.R = Rout;
     L.norm_part = c->norm_part;
     L.status = c->status;
@@ -1454,7 +1469,7 @@ static lskum_status vjp_residual_fp32(lskum_ctx *c, const double *Ui, double *Ub
                                          c->fG + (int64_t)k * 8 * n, nullptr, 0.0, c->stream, c->var_qgrad));
     }
     LAUNCH(c, launch_to_float(4 * n, c->vRb, c->fRb, c->stream));
-    const AdjParams Pd = adj_params(c);
+    const AdjParams Pd = adj_params(c, c->fw[0]);
     AdjParamsT<float> P{};
     P.g = Pd.g;
     P.q = c->fq;
@@ -1479,14 +1494,13 @@ static lskum_status vjp_residual_fp32(lskum_ctx *c, const double *Ui, double *Ub
     c->launches++;
     LAUNCH(c, launch_adj_flux(P, geom, c->stream));
     if (second) {
-        if (geom) CK(c, cudaMemsetAsync(c->vabar, 0, std::max<int64_t>(c->nnz, 1) * sizeof(double2), c->stream));
         float *gin = c->fgb, *gout = c->fgb2;
         for (int k = K; k >= 1; --k) {
             LAUNCH(c, launch_adj_grad(P, (const float *)(c->fG + (int64_t)(k - 1) * 8 * n), (const float *)gin,
-                                      gout, geom, c->stream));
+                                      gout, geom, k == K, c->stream));
             std::swap(gin, gout);
         }
-        LAUNCH(c, launch_adj_grad(P, (const float *)nullptr, (const float *)gin, (float *)nullptr, geom, c->stream));
+        LAUNCH(c, launch_adj_grad(P, (const float *)nullptr, (const float *)gin, (float *)nullptr, geom, K == 0, c->stream));
     }
     if (geom) LAUNCH(c, launch_adj_weights(Pd, c->stream));
     LAUNCH(c, launch_adj_state(P, Ui, Ub_acc, c->stream));
@@ -1496,31 +1510,32 @@ static lskum_status vjp_residual_fp32(lskum_ctx *c, const double *Ui, double *Ub
 // one residual VJP at the internal state Ui for the internal cotangent vRb:
 // Ub_acc ([n][4], internal) += (dR/dU)^T R_bar; vdbar += the offset
 // cotangents (the caller zeroes vdbar once per product)
-static lskum_status vjp_residual(lskum_ctx *c, const double *Ui, double *Ub_acc, bool geom, bool fwd_done)
+static lskum_status vjp_residual(lskum_ctx *c, const double *Ui, double *Ub_acc, bool geom,
+                                 const lskum_ctx::Forward &f, bool fwd_done)
 {
     const int64_t n = c->n;
     const bool second = c->cfg.order == 2;
     const int K = second ? c->cfg.inner_iters : 0;
     lskum_status st;
-    if (!fwd_done && (st = vjp_forward(c, Ui)) != LSKUM_OK) return st;
-    const AdjParams P = adj_params(c);
+    if (!fwd_done && (st = vjp_forward(c, Ui, f)) != LSKUM_OK) return st;
+    const AdjParams P = adj_params(c, f);
     c->launches++;
     LAUNCH(c, launch_adj_flux(P, geom, c->stream));
     if (second) {
-        if (geom) CK(c, cudaMemsetAsync(c->vabar, 0, std::max<int64_t>(c->nnz, 1) * sizeof(double2), c->stream));
         double *gin = c->vgb, *gout = c->vgb2;
         if (limited(c)) {
             // the limiter first: the flux saw the limited last iterate
             c->launches++;
-            LAUNCH(c, launch_adj_limit(P, c->vG + (int64_t)K * 8 * n, gin, gout, c->vlidx, c->vlval,
+            LAUNCH(c, launch_adj_limit(P, f.G + (int64_t)K * 8 * n, gin, gout, c->vlidx, c->vlval,
                                        c->cfg.limiter_K, c->stream));
             std::swap(gin, gout);
         }
         for (int k = K; k >= 1; --k) {
-            LAUNCH(c, launch_adj_grad(P, c->vG + (int64_t)(k - 1) * 8 * n, gin, gout, geom, c->stream));
+            LAUNCH(c, launch_adj_grad(P, f.G + (int64_t)(k - 1) * 8 * n, gin, gout, geom, k == K, c->stream));
             std::swap(gin, gout);
         }
-        LAUNCH(c, launch_adj_grad(P, (const double *)nullptr, (const double *)gin, (double *)nullptr, geom, c->stream));
+        LAUNCH(c, launch_adj_grad(P, (const double *)nullptr, (const double *)gin, (double *)nullptr, geom, K == 0,
+                                  c->stream));
     }
     if (geom) LAUNCH(c, launch_adj_weights(P, c->stream));
     LAUNCH(c, launch_adj_state(P, Ui, Ub_acc, c->stream));
@@ -1545,7 +1560,7 @@ static lskum_status vjp_end(lskum_ctx *c, double *U_bar, double *x_bar, double *
 {
     if (flags & ~LSKUM_VJP_ACCUMULATE_XY) return fail(c, LSKUM_ERR_ARG, "unknown flags 0x%x", flags);
     if (x_bar || y_bar)
-        LAUNCH(c, launch_adj_points(adj_params(c), c->vpxy, x_bar, y_bar, (flags & LSKUM_VJP_ACCUMULATE_XY) != 0,
+        LAUNCH(c, launch_adj_points(adj_params(c, c->fw[0]), c->vpxy, x_bar, y_bar, (flags & LSKUM_VJP_ACCUMULATE_XY) != 0,
                                     c->stream));
     if (U_bar) LAUNCH(c, launch_state_out(c->n, c->perm, c->vUacc, U_bar, c->stream));
     return check_nonphysical(c);
@@ -1572,7 +1587,7 @@ extern "C" lskum_status lskum_residual_vjp(lskum_ctx *c, const double *U, const 
         if (limited(c))
             return fail(c, LSKUM_ERR_ARG, "the FP32 product needs limiter_K = 0 (the FP64 product covers the limiter)");
         if ((st = vjp_residual_fp32(c, Ui, c->vUacc, x_bar || y_bar)) != LSKUM_OK) return st;
-    } else if ((st = vjp_residual(c, Ui, c->vUacc, x_bar || y_bar, false)) != LSKUM_OK) {
+    } else if ((st = vjp_residual(c, Ui, c->vUacc, x_bar || y_bar, c->fw[0], false)) != LSKUM_OK) {
         return st;
     }
     return vjp_end(c, U_bar, x_bar, y_bar, flags & ~LSKUM_VJP_FP32);
@@ -1589,6 +1604,21 @@ static lskum_status step_vjp_workspace(lskum_ctx *c)
     CK(c, dalloc(c, &c->sUin, 4 * n));
     CK(c, dalloc(c, &c->sdt, n));
     CK(c, dalloc(c, &c->sdtb, n));
+    if (c->cfg.time_scheme == 1) {
+        // a forward per RK stage spares running it again in the reverse sweep;
+        // without the memory for them that is what happens
+        cudaError_t e = cudaSuccess;
+        const size_t kept = c->allocs.size();
+        for (int k = 1; k < 4 && e == cudaSuccess; ++k) e = alloc_forward(c, c->fw[k]);
+        if (e != cudaSuccess && e != cudaErrorMemoryAllocation) CK(c, e);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            for (size_t a = kept; a < c->allocs.size(); ++a) cudaFree(c->allocs[a]);
+            c->allocs.resize(kept);
+            for (int k = 1; k < 4; ++k) c->fw[k] = lskum_ctx::Forward{};
+        }
+        c->stage_forwards = e == cudaSuccess;
+    }
     c->svjp_ready = true;
     return LSKUM_OK;
 }
@@ -1622,17 +1652,18 @@ extern "C" lskum_status lskum_step_vjp(lskum_ctx *c, const double *U, const doub
     for (int k = 0; k < 4; ++k) S.Uinf[k] = c->gas.Uinf[k];
     // forward: dt frozen at U^n, the stage states and residuals (FP64)
     LAUNCH(c, launch_timestep(n, c->gas, c->cfg.cfl, c->dmin, Un, c->sdt, c->stream));
-    if ((st = residual_fp64(c, Un, c->sR[0])) != LSKUM_OK) return st;
+    if ((st = residual_fp64(c, Un, c->sR[0], c->fw[0])) != LSKUM_OK) return st;
     if (c->cfg.time_scheme == 0) {
         // U^{n+1} = P(U^n - dt R(U^n))
         LAUNCH(c, launch_stage_adj(S, c->sUb, c->sR[0], 1.0, true, c->vUacc, c->sdtb, c->vRb, c->stream));
-        if ((st = vjp_residual(c, Un, c->vUacc, geom, true)) != LSKUM_OK) return st;
+        if ((st = vjp_residual(c, Un, c->vUacc, geom, c->fw[0], true)) != LSKUM_OK) return st;
     } else {
         // U_{k+1} = P(U^n - c_k dt R_k), R_{k+1} = R(U_{k+1}); U_{k+1} is kept in sU[k]
         const double cst[3] = {0.5, 0.5, 1.0};
+        const bool kept = c->stage_forwards;
         for (int k = 0; k < 3; ++k) {
             LAUNCH(c, launch_stage_fwd(S, Un, c->sR[k], cst[k], c->sU[k], c->stream));
-            if ((st = residual_fp64(c, c->sU[k], c->sR[k + 1])) != LSKUM_OK) return st;
+            if ((st = residual_fp64(c, c->sU[k], c->sR[k + 1], c->fw[kept ? k + 1 : 0])) != LSKUM_OK) return st;
         }
         // reverse: the last stage, then stages 2, 1, 0 (their residuals R3, R2, R1, R0)
         const double *Rs[4] = {c->sR[0], c->sR[1], c->sR[2], c->sR[3]};
@@ -1641,13 +1672,14 @@ extern "C" lskum_status lskum_step_vjp(lskum_ctx *c, const double *U, const doub
             // the cotangent of the stage state U_k from R_k = R(U_k)
             CK(c, cudaMemsetAsync(c->sUb, 0, 4 * n * sizeof(double), c->stream));
             CK(c, cudaMemcpyAsync(c->vRb, c->sRb[k], 4 * n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-            if ((st = vjp_residual(c, c->sU[k - 1], c->sUb, geom, false)) != LSKUM_OK) return st;
+            // (without the other forwards the last stage's is still the current one)
+            if ((st = vjp_residual(c, c->sU[k - 1], c->sUb, geom, c->fw[kept ? k : 0], kept || k == 3)) != LSKUM_OK) return st;
             // U_k = P(U^n - c_k dt R_{k-1})
             LAUNCH(c, launch_stage_adj(S, c->sUb, c->sR[k - 1], cst[k - 1], false, c->vUacc, c->sdtb,
                                        c->sRb[k - 1], c->stream));
         }
         CK(c, cudaMemcpyAsync(c->vRb, c->sRb[0], 4 * n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-        if ((st = vjp_residual(c, Un, c->vUacc, geom, false)) != LSKUM_OK) return st;
+        if ((st = vjp_residual(c, Un, c->vUacc, geom, c->fw[0], kept)) != LSKUM_OK) return st;
     }
     LAUNCH(c, launch_dt_adj(S, c->geom(), c->cfg.cfl, c->gas.inv_gm1, Un, c->sdtb, c->vUacc, c->vdbar, c->stream));
     return vjp_end(c, U_bar, x_bar, y_bar, flags);

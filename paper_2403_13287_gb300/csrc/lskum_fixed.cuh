@@ -252,15 +252,12 @@ LSKUM_FIX_FN bool fix_state(const double q[4], FixOp nx, FixOp ny, FixState &s)
     x = fix_flip(x, b1 >> 63) + s2;
     int n;
     const FixOp M = fix_op(fix_exp(x, n));
-    // powers of r: r^2 <= 2 in Q61, r^4 <= 4 in Q60, r^6 <= 8 in Q59, r^7 < 11.4 and r^8 <= 16 in Q58
+    // r^2 <= 2 in Q61, r^4 <= 4 in Q60, r^6 <= 8 in Q59; the factors below 16, 22.7 and 32
     const FixOp r2 = fix_op(fix_sqr_s<3>(R));
     const FixOp r4 = fix_op(fix_sqr_s<2>(r2));
-    const FixOp r6 = fix_op(fix_mul_s<2>(r4, r2));
-    const FixOp r7 = fix_op(fix_mul_s<2>(r6, R));
-    const FixOp r8 = fix_op(fix_sqr_s<2>(r4));
-    s.c0 = fix_mul_s<1>(M, r6);                                  // Q58, below 2^62 like the others
-    s.c1 = fix_mul_s<1>(M, r7);                                  // Q57
-    s.c3 = fix_mul_s<1>(M, r8);                                  // Q57
+    s.c0 = fix_mul_s<1>(M, fix_op(fix_mul_s<2>(r4, r2)));        // Q58, below 2^62 like the others
+    s.c1 = fix_mul_s<2>(fix_op(s.c0), R);                        // Q57
+    s.c3 = fix_mul_s<3>(fix_op(s.c1), R);                        // Q57
     s.r = r;
     s.n = n;
     s.k = k;
@@ -473,6 +470,55 @@ LSKUM_FIX_FN double fix_difference(double a, double b)
     const int64_t ba = fix_bits(a), bb = fix_bits(b);
     return fix_to_double(fix_flip((ba & 0xfffffffffffffll) - (bb & 0xfffffffffffffll), ba >> 63),
                          ((int)(ba >> 52) & 0x7ff) - 1075);
+}
+
+// --- q-variables of a state ------------------------------------------------
+// positive and of an exponent for which the forms below stay normal
+LSKUM_FIX_FN bool fix_moderate(double x) { return (uint64_t)fix_bits(x) - (700ull << 52) < (700ull << 52); }
+
+// 1/x of a moderate x, within 2^-59 before the final rounding
+LSKUM_FIX_FN double fix_reciprocal(double x)
+{
+    const int64_t b = fix_bits(x);
+    return fix_to_double(fix_rcp(fix_mantissa<61>(b, 0)), 1023 - 62 - (int)(b >> 52));
+}
+
+// log2 of a positive normal x's mantissa in Q60, [0, 1)
+LSKUM_FIX_FN int64_t fix_log2_mantissa(double x)
+{
+    const int64_t b = fix_bits(x);
+    const int j = (int)(b >> 42) & 1023;
+#ifdef __CUDACC__
+    const int4 w = __ldg(reinterpret_cast<const int4 *>(kFixLog2 + j));
+    const int64_t lc = (int64_t)(((uint64_t)(uint32_t)w.y << 32) | (uint32_t)w.x);
+    const uint32_t r = (uint32_t)w.z;
+#else
+    const int64_t lc = kFixLog2[j].log2c;
+    const uint32_t r = kFixLog2[j].r;
+#endif
+    // u = 2^11 (m r - 1) in Q62, |u| < 1.001: the 1's 2^73 is 0 modulo 2^64
+    const uint64_t m = (uint64_t)((b & 0xfffffffffffffll) | 0x10000000000000ll);
+    const int64_t u = (int64_t)((((uint64_t)(uint32_t)m * r) >> 11) + (((m >> 32) * r) << 21));
+    const int32_t uh = (int32_t)(u >> 32);                                        // Q30
+    const FixOp uo = fix_op(u);
+    const int32_t t4 = LSKUM_FIX_LOG_C4 + fix_mulhi32(LSKUM_FIX_LOG_C5, uh);      // Q66
+    const int32_t t3 = LSKUM_FIX_LOG_C3 + fix_mulhi32(t4, uh);                    // Q64
+    const int64_t t2 = LSKUM_FIX_LOG_C2 + (((int64_t)t3 * uh) >> 10);             // Q84
+    const int64_t t1 = LSKUM_FIX_LOG_C1 + (fix_mul(fix_op(t2), uo) >> 10);        // Q72
+    return lc + (fix_mul(fix_op(t1), uo) >> 10);                                  // Q60
+}
+
+// ln(rho) + 2.5 ln(beta), beta = rho/(2p), of moderate rho and p, which is
+// (7 log2 rho - 5 log2 p - 5) ln2/2: within 2^-54 before the final rounding
+// while the bracket is below 117, beyond that to about a unit in the last place
+LSKUM_FIX_FN double fix_log_state(double rho, double p)
+{
+    const int n = 7 * ((int)(fix_bits(rho) >> 52) - 1023) - 5 * ((int)(fix_bits(p) >> 52) - 1023) - 5;
+    const int64_t f = 7 * fix_log2_mantissa(rho) - 5 * fix_log2_mantissa(p);      // Q60, (-5, 7)
+    const bool small = n >= -110 && n <= 110;
+    const int64_t l = (small ? fix_shl(n, 56) : 0) + (f >> 4);                    // the bracket in Q56, half of it in Q57
+    const double v = fix_to_double(fix_mul(fix_op(l), fix_op(LSKUM_FIX_LN2)), -56);
+    return small ? v : v + (double)n * 0.34657359027997264;
 }
 
 }  // namespace lskum

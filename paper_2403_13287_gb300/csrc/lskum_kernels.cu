@@ -206,7 +206,8 @@ __device__ __forceinline__ void largest_shift_screened(const DevGeom &g, int e0,
 template <bool KIN, int PASS, int LANES>
 __global__ void __launch_bounds__(128) k_qgrad(DevGeom g, const double *__restrict__ q,
                                                const double *__restrict__ qg_old, const double *__restrict__ g1,
-                                               double *__restrict__ qg_new, double *__restrict__ ext, double limK)
+                                               double *__restrict__ qg_new, double *__restrict__ ext, double limK,
+                                               double *__restrict__ raw)
 {
     constexpr bool INNER = (PASS & QG_INNER) != 0, LIMIT = (PASS & QG_LIMIT) != 0;
     constexpr bool EXTR = !INNER && (PASS & (QG_LIMIT | QG_EXTREMA)) != 0;   // extrema found here
@@ -347,6 +348,10 @@ __global__ void __launch_bounds__(128) k_qgrad(DevGeom g, const double *__restri
     }
     if constexpr (LIMIT) {
         if constexpr (INNER) gather_c<C>(ext + 4 * p + k0, xm);
+        if (raw) {   // the iterate before the limiter (a reverse pass needs both)
+            store_c<C>(raw + 8 * p + k0, sx);
+            store_c<C>(raw + 8 * p + 4 + k0, sy);
+        }
         unsigned long long dm[C];   // bits of d_m (non-negative doubles order as integers)
 #pragma unroll
         for (int k = 0; k < C; ++k) dm[k] = 0;
@@ -1003,20 +1008,20 @@ static inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t -
 
 template <bool KIN, int LANES>
 static void qgrad_pass(int pass, const DevGeom &g, const double *q, const double *qg_old, const double *g1,
-                       double *qg_new, double *ext, double limK, cudaStream_t s)
+                       double *qg_new, double *ext, double limK, double *raw, cudaStream_t s)
 {
     const unsigned nb = blocks_for(LANES * g.n, 128);
     switch (pass) {
-    case 0: k_qgrad<KIN, 0, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
-    case QG_EXTREMA: k_qgrad<KIN, QG_EXTREMA, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
-    case QG_LIMIT: k_qgrad<KIN, QG_LIMIT, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
-    case QG_INNER: k_qgrad<KIN, QG_INNER, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
-    default: k_qgrad<KIN, QG_INNER | QG_LIMIT, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK); break;
+    case 0: k_qgrad<KIN, 0, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK, raw); break;
+    case QG_EXTREMA: k_qgrad<KIN, QG_EXTREMA, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK, raw); break;
+    case QG_LIMIT: k_qgrad<KIN, QG_LIMIT, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK, raw); break;
+    case QG_INNER: k_qgrad<KIN, QG_INNER, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK, raw); break;
+    default: k_qgrad<KIN, QG_INNER | QG_LIMIT, LANES><<<nb, 128, 0, s>>>(g, q, qg_old, g1, qg_new, ext, limK, raw); break;
     }
 }
 
 cudaError_t launch_qgrad(const DevGeom &g, const double *q, const double *qg_old, const double *g1,
-                         double *qg_new, double *ext, double limiter_K, cudaStream_t s)
+                         double *qg_new, double *ext, double limiter_K, cudaStream_t s, double *raw)
 {
     const bool inner = qg_old != nullptr, limit = limiter_K > 0.0;
     if (inner && (!g1 || (limit && !ext))) return cudaErrorInvalidValue;
@@ -1029,12 +1034,12 @@ cudaError_t launch_qgrad(const DevGeom &g, const double *q, const double *qg_old
     // more. One lane with all four components: 27 us at 3k, 0.450 ms at 2.5M.
     const bool four = g.n < 60000;
     if (g.ioff) {
-        if (four) qgrad_pass<true, 4>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, s);
-        else qgrad_pass<true, 2>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, s);
+        if (four) qgrad_pass<true, 4>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, raw, s);
+        else qgrad_pass<true, 2>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, raw, s);
     } else if (four) {
-        qgrad_pass<false, 4>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, s);
+        qgrad_pass<false, 4>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, raw, s);
     } else {
-        qgrad_pass<false, 2>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, s);
+        qgrad_pass<false, 2>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, raw, s);
     }
     return cudaGetLastError();
 }

@@ -105,3 +105,13 @@ extern "C" void fixed_difference(long n, const double *a, double *d, int *ok)
         d[e] = ok[e] ? fix_difference(a[2 * e], a[2 * e + 1]) : 0.0;
     }
 }
+
+// rows [rho, p]: ln(rho) + 2.5 ln(rho/(2p)) and 1/rho; ok: both moderate
+extern "C" void fixed_log(long n, const double *a, double *l, double *r, int *ok)
+{
+    for (long e = 0; e < n; ++e) {
+        ok[e] = fix_moderate(a[2 * e]) && fix_moderate(a[2 * e + 1]);
+        l[e] = ok[e] ? fix_log_state(a[2 * e], a[2 * e + 1]) : 0.0;
+        r[e] = ok[e] ? fix_reciprocal(a[2 * e]) : 0.0;
+    }
+}

@@ -235,6 +235,34 @@ def test_limiter_quotient(shim, eps, d):
         assert abs(Fraction(float(f[e])) - want) <= want * Fraction(2, 2 ** 53)
 
 
+def test_logarithm_and_reciprocal(shim):
+    """ln(rho) + 2.5 ln(beta) against multiple precision: each log2 within
+    2 units of 2^-60, times 7/2 and 5/2, their sum cut to 2^-57 and a product
+    within 1.25 units of 2^-56 (together below 2^-54), then one rounding; extreme
+    exponents to two units in the last place. 1/rho: within 2^-59, then one rounding."""
+    mp = pytest.importorskip("mpmath")
+    mp.mp.dps = 40
+    rng = np.random.default_rng(9)
+    n = 1500
+    a = np.exp(rng.uniform(-2, 2, (n, 2)))
+    a[:300] = 2.0 ** rng.integers(-1, 2, (300, 2)) * (1 + rng.choice([0, 2.0 ** -52, -(2.0 ** -53), 1 / 1024, 1 / 2048], (300, 2)))
+    a[300:500] = 2.0 ** rng.uniform(-300, 300, (200, 2))
+    l, r, ok = np.zeros(n), np.zeros(n), np.zeros(n, dtype=np.int32)
+    ptr = lambda v: v.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+    shim.lib.fixed_log(ctypes.c_long(n), ptr(a), ptr(l), ptr(r), ptr(ok))
+    assert ok.all()
+    for e in range(n):
+        rho, p = mp.mpf(float(a[e, 0])), mp.mpf(float(a[e, 1]))
+        want = mp.log(rho) + mp.mpf(2.5) * mp.log(rho / (2 * p))
+        assert abs(mp.mpf(float(l[e])) - want) <= mp.mpf(2) ** -54 + abs(want) * mp.mpf(2) ** (-51 if 300 <= e < 500 else -53)
+        assert abs(mp.mpf(float(r[e])) * rho - 1) <= mp.mpf(2) ** -53 + mp.mpf(2) ** -58
+    bad = np.array([[0.0, 1], [-1, 1], [np.inf, 1], [np.nan, 1], [1, 0], [1, -0.0], [1, np.nan], [1e-310, 1], [1e300, 1]])
+    m = len(bad)
+    l, r, ok = np.zeros(m), np.zeros(m), np.zeros(m, dtype=np.int32)
+    shim.lib.fixed_log(ctypes.c_long(m), ptr(bad), ptr(l), ptr(r), ptr(ok))
+    assert not ok.any()
+
+
 def test_differences_are_exact(shim):
     rng = np.random.default_rng(7)
     a = rng.uniform(-4, 4, 4000)
