@@ -223,7 +223,7 @@ lskum_status lskum_residual(lskum_ctx *ctx, const double *U, double *R);
  * product is that of the branch the forward takes, with the forward's
  * choices (the first stencil extremum, the first largest reconstruction
  * shift, the first nearest neighbour in row order). Its workspace (about
- * 0.53 KB per point plus 120 B per edge for K = 3: 1.0 GB at 640k points;
+ * 0.67 KB per point plus 120 B per edge for K = 3: 1.1 GB at 640k points;
  * 0.16 KB per point more with the limiter; the FP32 product adds 0.16 KB per
  * point and 56 B per edge) is allocated on the first call
  * and kept. The kinetic boundary mode is not differentiated (LSKUM_ERR_ARG).

@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(128) k_adj_flux(AdjParamsT<T> P)
         // R = 0 there: no cotangent flows from this point
         for (int e = e0; e < e1; ++e) {
             st4(P.ebar, e, qb0);
-            if constexpr (GEOM) P.wbar[e] = make_double2(0.0, 0.0);
+            if (GEOM && !P.add) P.wbar[e] = make_double2(0.0, 0.0);
         }
         st4(P.qbar, p, qb0);
         if (second) st8(P.gbar, p, gb0);
@@ -501,7 +501,10 @@ __global__ void __launch_bounds__(128) k_adj_flux(AdjParamsT<T> P)
                 wbx += Rl[k] * (Gsi[k] - Gs0[k]);
                 wby += Rl[k] * (Gni[k] - Gn0[k]);
             }
-            P.wbar[e] = make_double2(us_ ? to_f64(wbx) : 0.0, un_ ? to_f64(wby) : 0.0);
+            double2 wb = P.add ? P.wbar[e] : make_double2(0.0, 0.0);
+            if (us_) wb.x += to_f64(wbx);
+            if (un_) wb.y += to_f64(wby);
+            P.wbar[e] = wb;
         }
         st4(P.ebar, e, qbi);
         T dxb = T(0), dyb = T(0);
@@ -621,7 +624,7 @@ __global__ void __launch_bounds__(128, 5) k_adj_flux_pair(AdjParams P)
         // R = 0 there: no cotangent flows from this point
         for (int e = e0; e < e1; ++e) {
             st4(P.ebar, e, qb0);
-            if constexpr (GEOM) P.wbar[e] = make_double2(0.0, 0.0);
+            if (GEOM && !P.add) P.wbar[e] = make_double2(0.0, 0.0);
         }
     }
     const int deg = live && f != FLAG_FARFIELD ? e1 - e0 : 0;
@@ -691,7 +694,12 @@ __global__ void __launch_bounds__(128, 5) k_adj_flux_pair(AdjParams P)
         // R += w (G(q~_i) - G(q~_0)): + for the neighbour, - for the owner
         if constexpr (GEOM) {
             const double Jso = __shfl_xor_sync(0xffffffffu, Js, 1), Jno = __shfl_xor_sync(0xffffffffu, Jn, 1);
-            if (act && l == 0) P.wbar[e] = make_double2(us_ ? Js - Jso : 0.0, un_ ? Jn - Jno : 0.0);
+            if (act && l == 0) {
+                double2 wb = P.add ? P.wbar[e] : make_double2(0.0, 0.0);
+                if (us_) wb.x += Js - Jso;
+                if (un_) wb.y += Jn - Jno;
+                P.wbar[e] = wb;
+            }
         }
         if (act && l == 0) st4(P.ebar, e, qb);
         if (act && l == 1) {
@@ -858,7 +866,7 @@ __global__ void __launch_bounds__(128) k_adj_grad_fp32(AdjParamsT<float> P, cons
                 abx += s * gb[k];
                 aby += s * gb[4 + k];
             }
-            double2 ab = first ? make_double2(0.0, 0.0) : P.abar[e];
+            double2 ab = first && !P.add ? make_double2(0.0, 0.0) : P.abar[e];
             ab.x += to_f64(abx);
             ab.y += to_f64(aby);
             P.abar[e] = ab;
@@ -966,7 +974,7 @@ __global__ void __launch_bounds__(128, 5) k_adj_grad_fp64(AdjParams P, const dou
                     db.y = fma(-0.5, dby, db.y);
                     P.dbar[e] = db;
                 }
-                double2 ab = first ? make_double2(0.0, 0.0) : P.abar[e];
+                double2 ab = first && !P.add ? make_double2(0.0, 0.0) : P.abar[e];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     ab.x = fma(s[k], gb[k], ab.x);
@@ -1027,111 +1035,138 @@ __global__ void __launch_bounds__(128, 5) k_adj_grad_fp64(AdjParams P, const dou
 // row order, P_0's own 0 winning ties; the first largest |h . g_raw|; the
 // first nearest neighbour by squared distance. Where phi = 1 the limiter is
 // inactive and gbar passes through.
+//
+// With s = x + d and r = 1/M: f_x = (2 s - phi (x + s)) r, f_d = (2 x - phi (x + 4 d)) r,
+// f_eps = (1 - phi) r = d (2 d - x) r^2.
+//
+// Four lanes per point, a component each; what they share is exchanged by
+// shuffles: the offset of an edge that several components chose is written
+// once, by the lowest of them. The FP64 pipe bounds it, so the searches compare
+// bits (the extreme neighbours by q_i itself, the shifts by magnitude) and r
+// comes from the integer pipes: 76 -> 33 us at 40k points, 700 -> 389 us at 640k.
 // ---------------------------------------------------------------------------
+// doubles in their order as integers (both zeros equal), and back
+__device__ __forceinline__ long long ordered(double v)
+{
+    long long b = __double_as_longlong(v);
+    if (b == (long long)kSignBit) b = 0;
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double unordered(long long b)
+{
+    return __longlong_as_double(b ^ ((b >> 63) & 0x7fffffffffffffffll));
+}
+
 __global__ void __launch_bounds__(128) k_adj_limit(AdjParams P, const double *__restrict__ graw,
                                                    const double *__restrict__ gbar_in, double *__restrict__ gbar_out,
                                                    int32_t *__restrict__ lidx, double *__restrict__ lval,
                                                    double limK)
 {
     const DevGeom &g = P.g;
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= g.n) return;
-    double q0[4], gr[8], gb[8], qb[4];
-    ld4(P.q, p, q0);
-    ld8(graw, p, gr);
-    ld8(gbar_in, p, gb);
-    ld4(P.qbar, p, qb);
-    const double2 P0 = g.xy[p];
-    double dmx[4] = {0.0, 0.0, 0.0, 0.0}, dmn[4] = {0.0, 0.0, 0.0, 0.0}, hm[4] = {-1.0, -1.0, -1.0, -1.0};
-    int emx[4] = {-1, -1, -1, -1}, emn[4] = {-1, -1, -1, -1}, eh[4] = {-1, -1, -1, -1};
-    double sh[4] = {0.0, 0.0, 0.0, 0.0};
-    double2 hh[4];
-    int enear = -1;
-    double d2near = 0.0;
-    for (int e = g.off[p]; e < g.off[p + 1]; ++e) {
+    const int64_t pp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+    const int k = threadIdx.x & 3;
+    const bool live = pp < g.n;
+    const int64_t p = live ? pp : g.n - 1;   // (lanes past the end take part in the shuffles)
+    const double q0 = P.q[4 * p + k];
+    const double grx = graw[8 * p + k], gry = graw[8 * p + 4 + k];
+    const double gbx = gbar_in[8 * p + k], gby = gbar_in[8 * p + 4 + k];
+    double2 P0 = make_double2(0.0, 0.0);
+    if (!g.hd) P0 = g.xy[p];
+    const int e1 = g.off[p + 1];
+    long long mx = ordered(q0), mn = mx, hm = -1;   // largest and smallest q, bits of d_m (none yet)
+    unsigned long long sh = 0;
+    int emx = -1, emn = -1, eh = -1;
+    double2 hh = make_double2(0.0, 0.0);
+    for (int e = g.off[p]; e < e1; ++e) {
         const int i = g.idx[e];
-        double qi[4];
-        ld4(P.q, i, qi);
-        const double2 Pi = g.xy[i];
-        const double dx = Pi.x - P0.x, dy = Pi.y - P0.y;
-        const double2 h = g.hd ? g.hd[e] : make_double2(0.5 * dx, 0.5 * dy);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const double dq = qi[k] - q0[k];
-            if (dq > dmx[k]) {
-                dmx[k] = dq;
-                emx[k] = e;
-            }
-            if (dq < dmn[k]) {
-                dmn[k] = dq;
-                emn[k] = e;
-            }
-            const double c = fma(h.x, gr[k], h.y * gr[4 + k]);
-            if (fabs(c) > hm[k]) {
-                hm[k] = fabs(c);
-                eh[k] = e;
-                sh[k] = c < 0.0 ? -1.0 : 1.0;
-                hh[k] = h;
-            }
+        const long long qi = ordered(P.q[4 * (int64_t)i + k]);
+        double2 h;
+        if (g.hd) {
+            h = g.hd[e];
+        } else {
+            const double2 Pi = g.xy[i];
+            h = make_double2(0.5 * (Pi.x - P0.x), 0.5 * (Pi.y - P0.y));
         }
-        const double d2 = dx * dx + dy * dy;
-        if (enear < 0 || d2 < d2near) {
-            enear = e;
-            d2near = d2;
+        if (qi > mx) {
+            mx = qi;
+            emx = e;
+        }
+        if (qi < mn) {
+            mn = qi;
+            emn = e;
+        }
+        const unsigned long long c = (unsigned long long)__double_as_longlong(fma(h.x, grx, h.y * gry));
+        const long long ca = (long long)(c & ~kSignBit);
+        if (ca > hm) {
+            hm = ca;
+            eh = e;
+            sh = c & kSignBit;
+            hh = h;
         }
     }
-    const double dmin = g.dmin[p], hK = dmin * limK, eps2 = hK * hK * hK;
-    double go[8];
-    double dminb = 0.0;
-    int32_t li[4] = {-1, -1, -1, -1};
-    double lv[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        go[k] = gb[k];
-        go[4 + k] = gb[4 + k];
-        const bool plus = dmx[k] <= -dmn[k];
-        const double x = plus ? dmx[k] : -dmn[k], d = hm[k];
-        if (eh[k] < 0 || !(x < 2.0 * d)) continue;   // phi = 1
-        const double N = fma(x, x + 2.0 * d, eps2), M = fma(x, x + d, fma(2.0 * d, d, eps2));
-        const double phi = N / M, iM2 = 1.0 / (M * M);
-        const double fx = ((2.0 * x + 2.0 * d) * M - N * (2.0 * x + d)) * iM2;
-        const double fd = (2.0 * x * M - N * (x + 4.0 * d)) * iM2;
-        const double fe = (M - N) * iM2;
-        const double G = gb[k] * gr[k] + gb[4 + k] * gr[4 + k];
-        const double gd = G * fd * sh[k];
-        go[k] = phi * gb[k] + gd * hh[k].x;
-        go[4 + k] = phi * gb[4 + k] + gd * hh[k].y;
-        const double xb = G * fx;
-        if (plus && emx[k] >= 0) {
-            qb[k] -= xb;
-            li[k] = emx[k];
-            lv[k] = xb;
-        } else if (!plus && emn[k] >= 0) {
-            qb[k] += xb;
-            li[k] = emn[k];
-            lv[k] = -xb;
-        }
+    const double dmx = unordered(mx) - q0, dmn = q0 - unordered(mn);
+    const bool plus = dmx <= dmn;
+    const double x = plus ? dmx : dmn, d = __longlong_as_double(hm), d2 = 2.0 * d;
+    const bool on = live && eh >= 0 && x < d2;   // else phi = 1
+    const double hK = g.dmin[p] * limK, hK2 = hK * hK;
+    double gox = gbx, goy = gby, xb = 0.0, cx = 0.0, cy = 0.0, db = 0.0;
+    int li = -1;
+    if (on) {
+        const double eps2 = hK2 * hK, s = x + d;
+        const double N = fma(x, x + d2, eps2), M = fma(x, s, fma(d2, d, eps2));
+        const double r = fix_moderate(M) ? fix_reciprocal(M) : 1.0 / M;
+        double phi = N * r;
+        phi = fma(fma(-M, phi, N), r, phi);
+        const double G = r * fma(gbx, grx, gby * gry);
+        const double gd = flip_sign(G * fma(-phi, fma(4.0, d, x), x + x), sh);
+        gox = fma(phi, gbx, gd * hh.x);
+        goy = fma(phi, gby, gd * hh.y);
+        li = plus ? emx : emn;
+        xb = G * fma(-phi, x + s, s + s);
+        if (!plus) xb = -xb;
         // d* = 2 h*: its offset cotangent is half that of h*
-        double2 db = P.dbar[eh[k]];
-        db.x += 0.5 * gd * gr[k];
-        db.y += 0.5 * gd * gr[4 + k];
-        P.dbar[eh[k]] = db;
-        dminb += G * fe * 3.0 * limK * limK * limK * dmin * dmin;
+        cx = 0.5 * gd * grx;
+        cy = 0.5 * gd * gry;
+        db = G * (r * (d * (d2 - x)));
     }
-    if (dminb != 0.0 && enear >= 0 && dmin > 0.0) {
-        const double2 Pi = g.xy[g.idx[enear]];
-        double2 db = P.dbar[enear];
-        db.x += dminb * (Pi.x - P0.x) / dmin;
-        db.y += dminb * (Pi.y - P0.y) / dmin;
-        P.dbar[enear] = db;
-    }
-    st4(P.qbar, p, qb);
-    st8(gbar_out, p, go);
+    const int mine = on ? eh : -1;
+    bool lead = on;
+    double sx = cx, sy = cy;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        lidx[4 * p + k] = li[k];
-        lval[4 * p + k] = lv[k];
+    for (int m = 1; m < 4; ++m) {
+        const int eo = __shfl_xor_sync(0xffffffffu, mine, m);
+        const double ox = __shfl_xor_sync(0xffffffffu, cx, m), oy = __shfl_xor_sync(0xffffffffu, cy, m);
+        if (eo == mine) {
+            sx += ox;
+            sy += oy;
+            if ((k ^ m) < k) lead = false;
+        }
     }
+    db += __shfl_xor_sync(0xffffffffu, db, 1);
+    db += __shfl_xor_sync(0xffffffffu, db, 2);
+    if (lead) {
+        double2 o = P.dbar[eh];
+        o.x += sx;
+        o.y += sy;
+        P.dbar[eh] = o;
+    }
+    __syncwarp();   // the nearest edge may be one of those
+    if (live && k == 0 && db != 0.0) {
+        const int e = P.near_e[p];
+        const double2 u = P.near_u[p];
+        const double dminb = 3.0 * limK * hK2 * db;
+        double2 o = P.dbar[e];
+        o.x = fma(dminb, u.x, o.x);
+        o.y = fma(dminb, u.y, o.y);
+        P.dbar[e] = o;
+    }
+    if (!live) return;
+    if (li < 0) xb = 0.0;
+    P.qbar[4 * p + k] -= xb;
+    gbar_out[8 * p + k] = gox;
+    gbar_out[8 * p + 4 + k] = goy;
+    lidx[4 * p + k] = li;
+    lval[4 * p + k] = xb;
 }
 
 // the extreme neighbours' share of the limiter's q cotangent (k_adj_limit),
@@ -1165,12 +1200,17 @@ __global__ void __launch_bounds__(128) k_adj_limit_gather(AdjParams P, const int
 // M = sum d d^T and weights a = M^-1 d gives
 //   d_bar_k = b_k - B d_k,  b = M^-1 a_bar,  B = sum (b a^T + a b^T)
 //           = M^-1 [sum (a_bar d^T + d a_bar^T)] M^-1.
-// Full stencil (global frame): a_bar = abar. A sub-stencil (frame (s, n)) takes
-// one row of M^-1 d as its weight, so a_bar is the weight's cotangent wb along
-// that row, b = wb beta with beta the row of M^-1, and the bracket needs only
-// D = sum wb d. One pass over the edges forms all sums, a second the offsets'
-// cotangents: 53 FP64 instructions per edge and no indexed local arrays, where
-// three passes with b and a per edge took 125 (141 -> 94 us at 40k points).
+// Full stencil: a_bar = abar. A sub-stencil takes one row of M^-1 d (frame
+// (s, n)) as its weight, so a_bar is the weight's cotangent wb along that row,
+// b = wb beta with beta the row of M^-1, A = M^-1 sum wb d and B = beta A^T + A beta^T.
+//
+// All M^-1 depend on the points alone: k_adj_plan forms them once per context,
+// so a product needs one pass for S = sum a_bar d^T and the D = sum wb d, and
+// one for the offsets' cotangents, with the B of an edge's two sub-stencils
+// added up first: 39 FP64 instructions per edge (half offsets h where they are
+// stored: S and D take them, B is doubled instead). The sub-stencils stay in the
+// frame that their weights were solved in: b and B d nearly cancel for a thin
+// sub-stencil, and B turned to global axes lost seven digits there. 94 -> 63 us at 40k points, 823 -> 502 us at 640k.
 // ---------------------------------------------------------------------------
 struct Sym2 {
     double xx, xy, yy;
@@ -1184,34 +1224,90 @@ __device__ __forceinline__ double2 times(const Sym2 &A, double2 v)
 {
     return make_double2(fma(A.xx, v.x, A.xy * v.y), fma(A.xy, v.x, A.yy * v.y));
 }
-struct SubSums {   // one sub-stencil: M and D
-    Sym2 M;
-    double2 D;
-    __device__ __forceinline__ void add(bool in, double ds, double dn, double wb)
-    {
-        if (!in) return;
-        M.xx = fma(ds, ds, M.xx);
-        M.xy = fma(ds, dn, M.xy);
-        M.yy = fma(dn, dn, M.yy);
-        D.x = fma(wb, ds, D.x);
-        D.y = fma(wb, dn, D.y);
-    }
-};
-struct SubBack {   // beta and B = beta A^T + A beta^T, A = M^-1 D
-    double2 beta;
-    Sym2 B;
-};
-__device__ __forceinline__ SubBack sub_back(const SubSums &s, bool need, bool row1)
+
+// (s, n) of an offset; the same operations for d and for h = d/2
+__device__ __forceinline__ double2 in_frame(double2 d, double2 n0)
 {
-    SubBack o = {make_double2(0.0, 0.0), Sym2{0.0, 0.0, 0.0}};
-    if (!need) return o;
-    const Sym2 Mi = inverse2(s.M);
-    o.beta = row1 ? make_double2(Mi.xy, Mi.yy) : make_double2(Mi.xx, Mi.xy);
-    const double2 A = times(Mi, s.D);
-    o.B.xx = 2.0 * o.beta.x * A.x;
-    o.B.xy = fma(o.beta.x, A.y, o.beta.y * A.x);
-    o.B.yy = 2.0 * o.beta.y * A.y;
-    return o;
+    return make_double2(fma(d.x, n0.y, -(d.y * n0.x)), fma(d.x, n0.x, d.y * n0.y));
+}
+
+// plan [kAdjPlan][n]: M^-1 (xx, xy, yy) of the full stencil, then of each
+// sub-stencil, zero where the point needs none
+__global__ void __launch_bounds__(128) k_adj_plan(DevGeom g, double *__restrict__ plan, int32_t *__restrict__ near_e,
+                                                  double2 *__restrict__ near_u)
+{
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, n = g.n;
+    if (p >= n) return;
+    const uint8_t f = g.flag[p] & 3;
+    const double2 xy0 = g.xy[p], n0 = g.nrm[p];
+    Sym2 M = {0, 0, 0};
+    Sym2 Ms[4] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+    // the nearest neighbour: the first of equals in row order
+    int best = -1;
+    double d2best = 0.0;
+    double2 dbest = make_double2(0.0, 0.0);
+    for (int e = g.off[p]; e < g.off[p + 1]; ++e) {
+        const double2 xyi = g.xy[g.idx[e]];
+        const double dx = xyi.x - xy0.x, dy = xyi.y - xy0.y;
+        const double2 t = in_frame(make_double2(dx, dy), n0);
+        const uint8_t m = g.mask[e];
+        M.xx = fma(dx, dx, M.xx);
+        M.xy = fma(dx, dy, M.xy);
+        M.yy = fma(dy, dy, M.yy);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if ((k < 2 ? xsub(m) : ysub(m)) != k) continue;
+            Ms[k].xx = fma(t.x, t.x, Ms[k].xx);
+            Ms[k].xy = fma(t.x, t.y, Ms[k].xy);
+            Ms[k].yy = fma(t.y, t.y, Ms[k].yy);
+        }
+        const double d2 = dx * dx + dy * dy;
+        if (best < 0 || d2 < d2best) {
+            best = e;
+            d2best = d2;
+            dbest = make_double2(dx, dy);
+        }
+    }
+    const double dmin = g.dmin[p];
+    near_e[p] = best;
+    near_u[p] = dmin > 0.0 ? make_double2(dbest.x / dmin, dbest.y / dmin) : make_double2(0.0, 0.0);
+    const Sym2 Mi = inverse2(M);
+    plan[p] = Mi.xx;
+    plan[n + p] = Mi.xy;
+    plan[2 * n + p] = Mi.yy;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        Sym2 A = {0, 0, 0};
+        if (sub_needed(f, k)) A = inverse2(Ms[k]);
+        double *o = plan + (3 + 3 * k) * n + p;
+        o[0] = A.xx;
+        o[n] = A.xy;
+        o[2 * n] = A.yy;
+    }
+}
+
+__device__ __forceinline__ double2 half_offset(const DevGeom &g, int e, double2 xy0)
+{
+    if (g.hd) return g.hd[e];
+    const double2 xyi = g.xy[g.idx[e]];
+    return make_double2(0.5 * (xyi.x - xy0.x), 0.5 * (xyi.y - xy0.y));
+}
+// D += w h for the one of two sums the edge belongs to (selects instead of two predicated sums)
+__device__ __forceinline__ void add_to(bool first, bool second, double w, double2 h, double2 &D0, double2 &D1)
+{
+    double2 t = first ? D0 : D1;
+    t.x = fma(w, h.x, t.x);
+    t.y = fma(w, h.y, t.y);
+    if (first) D0 = t;
+    if (second) D1 = t;
+}
+// 2 B of a sub-stencil from D / 2, and its beta (row 0 or 1 of M^-1)
+__device__ __forceinline__ Sym2 sub_back(const double *__restrict__ plan, int64_t n, double2 D, int row, double2 &beta)
+{
+    const Sym2 Mi = {plan[0], plan[n], plan[2 * n]};
+    beta = row ? make_double2(Mi.xy, Mi.yy) : make_double2(Mi.xx, Mi.xy);
+    const double2 A = times(Mi, make_double2(4.0 * D.x, 4.0 * D.y));
+    return Sym2{2.0 * beta.x * A.x, fma(beta.x, A.y, beta.y * A.x), 2.0 * beta.y * A.y};
 }
 
 __global__ void __launch_bounds__(128) k_adj_weights(AdjParams P)
@@ -1219,73 +1315,59 @@ __global__ void __launch_bounds__(128) k_adj_weights(AdjParams P)
     const DevGeom &g = P.g;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= g.n) return;
-    const uint8_t f = g.flag[p] & 3;
     const bool full = P.order == 2;
-    const double2 xy0 = g.xy[p];
+    double2 xy0 = make_double2(0.0, 0.0);
+    if (!g.hd) xy0 = g.xy[p];
     const double2 n0 = g.nrm[p];
-    const double tx = n0.y, ty = -n0.x;
     const int e0 = g.off[p], e1 = g.off[p + 1];
-    Sym2 M = {0, 0, 0}, S = {0, 0, 0};
-    SubSums s0 = {}, s1 = {}, s2 = {}, s3 = {};
+    Sym2 S = {0, 0, 0};
+    double2 D0 = make_double2(0.0, 0.0), D1 = D0, D2 = D0, D3 = D0;
     for (int e = e0; e < e1; ++e) {
-        const double2 xyi = g.xy[g.idx[e]];
-        const double dx = xyi.x - xy0.x, dy = xyi.y - xy0.y;
-        const double ds = dx * tx + dy * ty, dn = dx * n0.x + dy * n0.y;
-        const uint8_t m = g.mask[e];
+        const double2 h = half_offset(g, e, xy0), t = in_frame(h, n0);
+        const int ks = xsub(g.mask[e]), kn = ysub(g.mask[e]);
         const double2 wb = P.wbar[e];
         if (full) {
             const double2 ab = P.abar[e];
-            M.xx = fma(dx, dx, M.xx);
-            M.xy = fma(dx, dy, M.xy);
-            M.yy = fma(dy, dy, M.yy);
-            S.xx = fma(ab.x, dx, S.xx);                          // half the diagonal
-            S.xy = fma(ab.x, dy, fma(ab.y, dx, S.xy));
-            S.yy = fma(ab.y, dy, S.yy);
+            S.xx = fma(ab.x, h.x, S.xx);                          // half the diagonal
+            S.xy = fma(ab.x, h.y, fma(ab.y, h.x, S.xy));
+            S.yy = fma(ab.y, h.y, S.yy);
         }
-        s0.add(xsub(m) == 0, ds, dn, wb.x);
-        s1.add(xsub(m) == 1, ds, dn, wb.x);
-        s2.add(ysub(m) == 2, ds, dn, wb.y);
-        s3.add(ysub(m) == 3, ds, dn, wb.y);
+        add_to(ks == 0, ks == 1, wb.x, t, D0, D1);
+        add_to(kn == 2, kn == 3, wb.y, t, D2, D3);
     }
+    const double *pl = P.plan + p;
+    const int64_t n = g.n;
     Sym2 Mi = {0, 0, 0}, B = {0, 0, 0};
     if (full) {
-        Mi = inverse2(M);
-        // B = Mi S Mi, S with its diagonal doubled
-        const double2 c0 = times(Mi, make_double2(2.0 * S.xx, S.xy)), c1 = times(Mi, make_double2(S.xy, 2.0 * S.yy));
+        Mi = Sym2{pl[0], pl[n], pl[2 * n]};
+        // B = Mi S Mi, S with its diagonal doubled; 2 B of S / 2
+        const double2 c0 = times(Mi, make_double2(8.0 * S.xx, 4.0 * S.xy)), c1 = times(Mi, make_double2(4.0 * S.xy, 8.0 * S.yy));
         const double2 b0 = times(Mi, make_double2(c0.x, c1.x)), b1 = times(Mi, make_double2(c0.y, c1.y));
         B = Sym2{b0.x, b0.y, b1.y};
     }
-    const SubBack k0 = sub_back(s0, sub_needed(f, 0), false), k1 = sub_back(s1, sub_needed(f, 1), false);
-    const SubBack k2 = sub_back(s2, sub_needed(f, 2), true), k3 = sub_back(s3, sub_needed(f, 3), true);
+    double2 beta0, beta1, beta2, beta3;
+    const Sym2 B0 = sub_back(pl + 3 * n, n, D0, 0, beta0), B1 = sub_back(pl + 6 * n, n, D1, 0, beta1);
+    const Sym2 B2 = sub_back(pl + 9 * n, n, D2, 1, beta2), B3 = sub_back(pl + 12 * n, n, D3, 1, beta3);
+    const Sym2 zero = {0.0, 0.0, 0.0};
     for (int e = e0; e < e1; ++e) {
-        const double2 xyi = g.xy[g.idx[e]];
-        const double dx = xyi.x - xy0.x, dy = xyi.y - xy0.y;
-        const double ds = dx * tx + dy * ty, dn = dx * n0.x + dy * n0.y;
-        const uint8_t m = g.mask[e];
+        const double2 h = half_offset(g, e, xy0), t = in_frame(h, n0);
+        const int ks = xsub(g.mask[e]), kn = ysub(g.mask[e]);
         const double2 wb = P.wbar[e];
         double2 d = P.dbar[e];
+        const Sym2 X = ks == 0 ? B0 : ks == 1 ? B1 : zero, Y = kn == 2 ? B2 : kn == 3 ? B3 : zero;
+        const Sym2 C = {X.xx + Y.xx, X.xy + Y.xy, X.yy + Y.yy};
+        const double wx = ks >= 0 ? wb.x : 0.0, wy = kn >= 0 ? wb.y : 0.0;
+        const double2 bx = ks == 0 ? beta0 : beta1, by = kn == 2 ? beta2 : beta3;
+        const double gs = fma(wx, bx.x, fma(wy, by.x, -fma(C.xx, t.x, C.xy * t.y)));
+        const double gn = fma(wx, bx.y, fma(wy, by.y, -fma(C.xy, t.x, C.yy * t.y)));
         if (full) {
-            const double2 b = times(Mi, P.abar[e]), c = times(B, make_double2(dx, dy));
+            const double2 ab = P.abar[e], b = times(Mi, ab), c = times(B, h);
             d.x += b.x - c.x;
             d.y += b.y - c.y;
         }
-        double gs = 0.0, gn = 0.0;   // (s, n) frame
-        const int ks = xsub(m), kn = ysub(m);
-        if (sub_needed(f, ks)) {
-            const SubBack &k = ks == 0 ? k0 : k1;
-            const double2 c = times(k.B, make_double2(ds, dn));
-            gs += fma(wb.x, k.beta.x, -c.x);
-            gn += fma(wb.x, k.beta.y, -c.y);
-        }
-        if (sub_needed(f, kn)) {
-            const SubBack &k = kn == 2 ? k2 : k3;
-            const double2 c = times(k.B, make_double2(ds, dn));
-            gs += fma(wb.y, k.beta.x, -c.x);
-            gn += fma(wb.y, k.beta.y, -c.y);
-        }
-        // ds = dx tx + dy ty, dn = dx nx + dy ny
-        d.x += gs * tx + gn * n0.x;
-        d.y += gs * ty + gn * n0.y;
+        // s = d.t, n = d.n with t = (n_y, -n_x)
+        d.x = fma(gs, n0.y, fma(gn, n0.x, d.x));
+        d.y = fma(-gs, n0.x, fma(gn, n0.y, d.y));
         P.dbar[e] = d;
     }
 }
@@ -1481,6 +1563,12 @@ cudaError_t build_incoming(const DevGeom &g, int64_t nnz, const int32_t *tedge, 
     return cudaGetLastError();
 }
 
+cudaError_t build_adj_plan(const DevGeom &g, double *plan, int32_t *near_e, double2 *near_u, cudaStream_t s)
+{
+    k_adj_plan<<<blocks(g.n, 128), 128, 0, s>>>(g, plan, near_e, near_u);
+    return cudaGetLastError();
+}
+
 cudaError_t build_float_geometry(const DevGeom &g, int64_t nnz, const double2 *tlsw, const double2 *thd, float4 *ef,
                                  float2 *ea, float4 *tf, cudaStream_t s)
 {
@@ -1529,7 +1617,7 @@ cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gba
 cudaError_t launch_adj_limit(const AdjParams &P, const double *graw, const double *gbar_in, double *gbar_out,
                              int32_t *lidx, double *lval, double limK, cudaStream_t s)
 {
-    k_adj_limit<<<blocks(P.g.n, 128), 128, 0, s>>>(P, graw, gbar_in, gbar_out, lidx, lval, limK);
+    k_adj_limit<<<blocks(P.g.n, 32), 128, 0, s>>>(P, graw, gbar_in, gbar_out, lidx, lval, limK);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     k_adj_limit_gather<<<blocks(P.g.n, 128), 128, 0, s>>>(P, lidx, lval);
@@ -1696,8 +1784,9 @@ __global__ void __launch_bounds__(256) k_stage_adj_rk4_final(StageParams S, cons
 
 // reverse of timestep(): dt = CFL dmin / (|u| + 3 sqrt(p/rho)), dmin the
 // distance to the nearest neighbour (the first of equals in row order)
-__global__ void __launch_bounds__(256) k_dt_adj(StageParams S, DevGeom g, double cfl, double inv_gm1,
-                                                const double *__restrict__ U, const double *__restrict__ dtbar,
+__global__ void __launch_bounds__(256) k_dt_adj(StageParams S, const double *__restrict__ dmin,
+                                                const int32_t *__restrict__ near_e, const double2 *__restrict__ near_u,
+                                                double cfl, double inv_gm1, const double *__restrict__ U, const double *__restrict__ dtbar,
                                                 double *__restrict__ Uacc, double2 *__restrict__ dbar)
 {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1716,33 +1805,19 @@ __global__ void __launch_bounds__(256) k_dt_adj(StageParams S, DevGeom g, double
     const D4 pr = (1.0 / inv_gm1) * (Ud[3] - 0.5 * (Ud[0] * (uu * uu + vv * vv)));
     const D4 speed = dsqrt(uu * uu + vv * vv) + 3.0 * dsqrt(pr * rinv);
     const D4 inv_speed = recip(speed);
-    const double dmin = g.dmin[p];
     double a[4];
     ld4(Uacc, p, a);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) a[k] += tb * cfl * dmin * inv_speed.d[k];
+    for (int k = 0; k < 4; ++k) a[k] += tb * cfl * dmin[p] * inv_speed.d[k];
     st4(Uacc, p, a);
     // dmin = |P_i - P_0| of the nearest neighbour
     const double db = tb * cfl * inv_speed.v;
-    const double2 P0 = g.xy[p];
-    int best = -1;
-    double d2best = 0.0;
-    for (int e = g.off[p]; e < g.off[p + 1]; ++e) {
-        const double2 Pi = g.xy[g.idx[e]];
-        const double dx = Pi.x - P0.x, dy = Pi.y - P0.y;
-        const double d2 = dx * dx + dy * dy;
-        if (best < 0 || d2 < d2best) {
-            best = e;
-            d2best = d2;
-        }
-    }
-    if (best >= 0 && dmin > 0.0) {
-        const double2 Pi = g.xy[g.idx[best]];
-        double2 d = dbar[best];
-        d.x += db * (Pi.x - P0.x) / dmin;
-        d.y += db * (Pi.y - P0.y) / dmin;
-        dbar[best] = d;
-    }
+    const int e = near_e[p];
+    const double2 dir = near_u[p];
+    double2 d = dbar[e];
+    d.x = fma(db, dir.x, d.x);
+    d.y = fma(db, dir.y, d.y);
+    dbar[e] = d;
 }
 
 // forces: Cp_w = (p_w - p_inf)/q_inf, (fx, fy) = -sum Cp n ds, Cl = fy cos a - fx sin a,
@@ -1820,10 +1895,11 @@ cudaError_t launch_stage_adj_rk4_final(const StageParams &S, const double *Ub_ou
     return cudaGetLastError();
 }
 
-cudaError_t launch_dt_adj(const StageParams &S, const DevGeom &g, double cfl, double inv_gm1, const double *U,
-                          const double *dtbar, double *Uacc, double2 *dbar, cudaStream_t s)
+cudaError_t launch_dt_adj(const StageParams &S, const AdjParams &P, double cfl, double inv_gm1, const double *U,
+                          const double *dtbar, double *Uacc, cudaStream_t s)
 {
-    k_dt_adj<<<blocks(S.n, 256), 256, 0, s>>>(S, g, cfl, inv_gm1, U, dtbar, Uacc, dbar);
+    k_dt_adj<<<blocks(S.n, 256), 256, 0, s>>>(S, P.g.dmin, P.near_e, P.near_u, cfl, inv_gm1, U, dtbar,
+                                                    Uacc, P.dbar);
     return cudaGetLastError();
 }
 

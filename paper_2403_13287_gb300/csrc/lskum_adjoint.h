@@ -28,6 +28,9 @@ struct AdjParamsT {
     const int32_t *tsrc;   // [nnz] owner point of each incoming edge
     const double2 *tlsw;   // [nnz] lsw of each incoming edge, in the transpose's order
     const double2 *thd;    // [nnz] half offset of each incoming edge, likewise
+    const double *plan;    // [kAdjPlan][n] inverse systems of each point's stencils (k_adj_plan)
+    const int32_t *near_e; // [n] edge of the nearest neighbour (the first of equals)
+    const double2 *near_u; // [n] (P_i - P_0) / dmin of that edge
     // FP32 product: geometry rounded once, per edge (dx, dy, w_s, w_n) and
     // (a_x, a_y), per incoming edge (a_x, a_y, dx, dy); nullptr in the FP64 one
     const float4 *ef;
@@ -37,27 +40,32 @@ struct AdjParamsT {
     double inv_gm1;
     int g14;               // gamma == 1.4: beta^(-1/(gamma-1)) = beta^-2.5 (as the forward kernels)
     int order;
+    int add;               // wbar and abar add to an earlier residual's of this product (else they start here)
 };
 using AdjParams = AdjParamsT<double>;
+constexpr int kAdjPlan = 15;
 
 cudaError_t build_transpose_csr(int64_t n, int64_t nnz, const int32_t *off, const int32_t *idx, int32_t *toff,
                                 int32_t *tedge, int32_t *tsrc, cudaStream_t s);
 // the incoming edges' weights and half offsets in the transpose's order (tlsw, thd)
 cudaError_t build_incoming(const DevGeom &g, int64_t nnz, const int32_t *tedge, const int32_t *tsrc, double2 *tlsw,
                            double2 *thd, cudaStream_t s);
+// what the reverse of the weights, the limiter and the time step need of the points alone
+cudaError_t build_adj_plan(const DevGeom &g, double *plan, int32_t *near_e, double2 *near_u, cudaStream_t s);
 // the FP32 product's geometry (ef, ea, tf)
 cudaError_t build_float_geometry(const DevGeom &g, int64_t nnz, const double2 *tlsw, const double2 *thd, float4 *ef,
                                  float2 *ea, float4 *tf, cudaStream_t s);
 // geom (here and below): the cotangents of the weights and offsets are wanted
-// too (wbar, abar, dbar); without it they are left alone.
+// too (wbar, abar, dbar); without it they are left alone. With P.add wbar and
+// abar add to what an earlier residual of the product left there.
 // flux adjoint: owner pass, then the neighbour-side gather (initialises qbar, gbar, ebar, wbar; adds into
 // dbar, which the caller zeroes once per product)
 template <class T>
 cudaError_t launch_adj_flux(const AdjParamsT<T> &P, bool geom, cudaStream_t s);
 // one E15 pass in reverse: gbar_in is the cotangent of this pass's output,
 // gbar_out receives that of its input iterate gprev (nullptr for the first-order
-// pass). The product's first such call (the last forward pass) starts abar and
-// qbar2, the others add.
+// pass). The residual's first such call (the last forward pass) starts qbar2
+// and, without P.add, abar; the others add.
 template <class T>
 cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gbar_in, T *gbar_out, bool geom,
                             bool first, cudaStream_t s);
@@ -101,8 +109,8 @@ cudaError_t launch_stage_adj(const StageParams &S, const double *Ub_out, const d
 cudaError_t launch_stage_adj_rk4_final(const StageParams &S, const double *Ub_out, const double *const R[4],
                                        double *Uacc, double *dtbar, double *const Rb[4], cudaStream_t s);
 // reverse of the local time step: Uacc += (ddt/dU)^T dtbar, dbar of the nearest-neighbour edge
-cudaError_t launch_dt_adj(const StageParams &S, const DevGeom &g, double cfl, double inv_gm1, const double *U,
-                          const double *dtbar, double *Uacc, double2 *dbar, cudaStream_t s);
+cudaError_t launch_dt_adj(const StageParams &S, const AdjParams &P, double cfl, double inv_gm1, const double *U,
+                          const double *dtbar, double *Uacc, cudaStream_t s);
 // reverse of the force integrals of one wall contour for the force cotangent (fxb, fyb)
 cudaError_t launch_forces_adj(int64_t nwall, double gamma, double qinf, const int32_t *wall, const double *ds,
                               const double2 *nrm, const double2 *xy, const double *U, double fxb, double fyb,

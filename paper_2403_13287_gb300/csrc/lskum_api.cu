@@ -134,6 +134,9 @@ struct lskum_ctx {
     double *vRb = nullptr, *vqb = nullptr, *vgb = nullptr, *vgb2 = nullptr;
     double *vebar = nullptr;
     double2 *vwbar = nullptr, *vabar = nullptr, *vdbar = nullptr;
+    double *vplan = nullptr;
+    int32_t *near_e = nullptr;
+    double2 *near_u = nullptr;
     int32_t *toff = nullptr, *tedge = nullptr, *tsrc = nullptr;
     double2 *tlsw = nullptr, *thd = nullptr;  // weights and half offsets of the incoming edges
     double *vqb2 = nullptr;       // [n][4] owner-side share of the q cotangent (order 2)
@@ -1381,6 +1384,9 @@ static lskum_status vjp_workspace(lskum_ctx *c)
     CK(c, dalloc(c, &c->tsrc, m));
     CK(c, dalloc(c, &c->tlsw, m));
     CK(c, dalloc(c, &c->thd, m));
+    CK(c, dalloc(c, &c->vplan, kAdjPlan * n));
+    CK(c, dalloc(c, &c->near_e, n));
+    CK(c, dalloc(c, &c->near_u, n));
     CK(c, dalloc(c, &c->vUacc, 4 * n));
     CK(c, dalloc(c, &c->vpxy, n));
     CK(c, dalloc(c, &c->fdsb, std::max<int64_t>(c->n_wall, 1)));
@@ -1389,7 +1395,8 @@ static lskum_status vjp_workspace(lskum_ctx *c)
         CK(c, dalloc(c, &c->vlidx, 4 * n));
         CK(c, dalloc(c, &c->vlval, 4 * n));
     }
-    c->launches += 4;
+    c->launches += 5;
+    LAUNCH(c, build_adj_plan(c->geom(), c->vplan, c->near_e, c->near_u, c->stream));
     LAUNCH(c, build_transpose_csr(n, c->nnz, c->off, c->idx, c->toff, c->tedge, c->tsrc, c->stream));
     LAUNCH(c, build_incoming(c->geom(), c->nnz, c->tedge, c->tsrc, c->tlsw, c->thd, c->stream));
     c->vjp_ready = true;
@@ -1415,6 +1422,9 @@ static AdjParams adj_params(lskum_ctx *c, const lskum_ctx::Forward &f)
     P.tsrc = c->tsrc;
     P.tlsw = c->tlsw;
     P.thd = c->thd;
+    P.plan = c->vplan;
+    P.near_e = c->near_e;
+    P.near_u = c->near_u;
     P.perm = c->perm;
     P.inv_gm1 = c->gas.inv_gm1;
     P.g14 = c->gas.g14;
@@ -1543,23 +1553,24 @@ static lskum_status vjp_residual_fp32(lskum_ctx *c, const double *Ui, double *Ub
         }
         LAUNCH(c, launch_adj_grad(P, (const float *)nullptr, (const float *)gin, (float *)nullptr, geom, K == 0, c->stream));
     }
-    if (geom) LAUNCH(c, launch_adj_weights(Pd, c->stream));
     LAUNCH(c, launch_adj_state(P, Ui, Ub_acc, c->stream));
     return LSKUM_OK;
 }
 
 // one residual VJP at the internal state Ui for the internal cotangent vRb:
 // Ub_acc ([n][4], internal) += (dR/dU)^T R_bar; vdbar += the offset
-// cotangents (the caller zeroes vdbar once per product)
+// cotangents (the caller zeroes vdbar once per product); add: the weights'
+// cotangents add to those of the product's earlier residuals
 static lskum_status vjp_residual(lskum_ctx *c, const double *Ui, double *Ub_acc, bool geom,
-                                 const lskum_ctx::Forward &f, bool fwd_done)
+                                 const lskum_ctx::Forward &f, bool fwd_done, bool add)
 {
     const int64_t n = c->n;
     const bool second = c->cfg.order == 2;
     const int K = second ? c->cfg.inner_iters : 0;
     lskum_status st;
     if (!fwd_done && (st = vjp_forward(c, Ui, f)) != LSKUM_OK) return st;
-    const AdjParams P = adj_params(c, f);
+    AdjParams P = adj_params(c, f);
+    P.add = add;
     c->launches++;
     LAUNCH(c, launch_adj_flux(P, geom, c->stream));
     if (second) {
@@ -1578,8 +1589,15 @@ static lskum_status vjp_residual(lskum_ctx *c, const double *Ui, double *Ub_acc,
         LAUNCH(c, launch_adj_grad(P, (const double *)nullptr, (const double *)gin, (double *)nullptr, geom, K == 0,
                                   c->stream));
     }
-    if (geom) LAUNCH(c, launch_adj_weights(P, c->stream));
     LAUNCH(c, launch_adj_state(P, Ui, Ub_acc, c->stream));
+    return LSKUM_OK;
+}
+
+// the weights' cotangents into the offsets', once per product: linear in
+// them, so the four residuals of an RK4 step share it (40k points: 94 us each)
+static lskum_status vjp_weights(lskum_ctx *c)
+{
+    LAUNCH(c, launch_adj_weights(adj_params(c, c->fw[0]), c->stream));
     return LSKUM_OK;
 }
 
@@ -1623,14 +1641,16 @@ extern "C" lskum_status lskum_residual_vjp(lskum_ctx *c, const double *U, const 
         Ui = c->Ut;
     }
     LAUNCH(c, launch_state_in(c->n, c->perm, R_bar, c->vRb, c->stream));
+    const bool geom = x_bar || y_bar;
     if (flags & LSKUM_VJP_FP32) {
         if (!c->mixed) return fail(c, LSKUM_ERR_ARG, "the FP32 product needs a mixed-precision context");
         if (limited(c))
             return fail(c, LSKUM_ERR_ARG, "the FP32 product needs limiter_K = 0 (the FP64 product covers the limiter)");
-        if ((st = vjp_residual_fp32(c, Ui, c->vUacc, x_bar || y_bar)) != LSKUM_OK) return st;
-    } else if ((st = vjp_residual(c, Ui, c->vUacc, x_bar || y_bar, c->fw[0], false)) != LSKUM_OK) {
+        if ((st = vjp_residual_fp32(c, Ui, c->vUacc, geom)) != LSKUM_OK) return st;
+    } else if ((st = vjp_residual(c, Ui, c->vUacc, geom, c->fw[0], false, false)) != LSKUM_OK) {
         return st;
     }
+    if (geom && (st = vjp_weights(c)) != LSKUM_OK) return st;
     return vjp_end(c, U_bar, x_bar, y_bar, flags & ~LSKUM_VJP_FP32);
 }
 
@@ -1697,7 +1717,7 @@ extern "C" lskum_status lskum_step_vjp(lskum_ctx *c, const double *U, const doub
     if (c->cfg.time_scheme == 0) {
         // U^{n+1} = P(U^n - dt R(U^n))
         LAUNCH(c, launch_stage_adj(S, c->sUb, c->sR[0], 1.0, true, c->vUacc, c->sdtb, c->vRb, c->stream));
-        if ((st = vjp_residual(c, Un, c->vUacc, geom, c->fw[0], true)) != LSKUM_OK) return st;
+        if ((st = vjp_residual(c, Un, c->vUacc, geom, c->fw[0], true, false)) != LSKUM_OK) return st;
     } else {
         // U_{k+1} = P(U^n - c_k dt R_k), R_{k+1} = R(U_{k+1}); U_{k+1} is kept in sU[k]
         const double cst[3] = {0.5, 0.5, 1.0};
@@ -1714,15 +1734,17 @@ extern "C" lskum_status lskum_step_vjp(lskum_ctx *c, const double *U, const doub
             CK(c, cudaMemsetAsync(c->sUb, 0, 4 * n * sizeof(double), c->stream));
             CK(c, cudaMemcpyAsync(c->vRb, c->sRb[k], 4 * n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
             // (without the other forwards the last stage's is still the current one)
-            if ((st = vjp_residual(c, c->sU[k - 1], c->sUb, geom, c->fw[kept ? k : 0], kept || k == 3)) != LSKUM_OK) return st;
+            st = vjp_residual(c, c->sU[k - 1], c->sUb, geom, c->fw[kept ? k : 0], kept || k == 3, k != 3);
+            if (st != LSKUM_OK) return st;
             // U_k = P(U^n - c_k dt R_{k-1})
             LAUNCH(c, launch_stage_adj(S, c->sUb, c->sR[k - 1], cst[k - 1], false, c->vUacc, c->sdtb,
                                        c->sRb[k - 1], c->stream));
         }
         CK(c, cudaMemcpyAsync(c->vRb, c->sRb[0], 4 * n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-        if ((st = vjp_residual(c, Un, c->vUacc, geom, c->fw[0], kept)) != LSKUM_OK) return st;
+        if ((st = vjp_residual(c, Un, c->vUacc, geom, c->fw[0], kept, true)) != LSKUM_OK) return st;
     }
-    LAUNCH(c, launch_dt_adj(S, c->geom(), c->cfg.cfl, c->gas.inv_gm1, Un, c->sdtb, c->vUacc, c->vdbar, c->stream));
+    if (geom && (st = vjp_weights(c)) != LSKUM_OK) return st;
+    LAUNCH(c, launch_dt_adj(S, adj_params(c, c->fw[0]), c->cfg.cfl, c->gas.inv_gm1, Un, c->sdtb, c->vUacc, c->stream));
     return vjp_end(c, U_bar, x_bar, y_bar, flags);
 }
 

@@ -406,3 +406,54 @@ def test_state_cotangent_alone_is_that_of_the_full_product(precision, fp32, limi
         assert np.abs(full - only).max() <= 1e-6 * np.abs(full).max()
     else:
         assert np.array_equal(full, only)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("W,L,K", [(34, 12, 1.0), (50, 14, 0.3)])
+def test_limited_vjp_at_the_last_points_matches_the_oracle(W, L, K):
+    """The limiter's reverse takes four lanes per point: clouds that end inside
+    a warp, entries at the last points and the wall, against complex-step
+    derivatives at the VJP tests' 1e-10 of the largest."""
+    import torch
+
+    import oracle
+    from oracle import lskum_jvp
+    from paper_2403_13287_gb300.cloudgen import naca0012_cloud, smooth_state
+    from paper_2403_13287_gb300.lskum import Solver
+    c = naca0012_cloud(W, L, seed=5)
+    n = c["n"]
+    assert n % 32 and n % 8
+    rng = np.random.default_rng(W)
+    U = smooth_state(c, 0.85, 1.0, amp=0.05, seed=4)
+    Rb = rng.standard_normal((4, n))
+    s = Solver(c, order=2, inner_iters=2, mach=0.85, aoa_deg=1.0, limiter_K=K, reorder=0)
+    Ub, xb, yb = (t.cpu().numpy() for t in s.residual_vjp(torch.from_numpy(Rb).cuda(), torch.from_numpy(U).cuda()))
+    s.close()
+    pts = list(range(n - 8, n)) + [int(k) for k in rng.choice(n - 8, 8, replace=False)]
+    ent = [("U", int(rng.integers(4)), k) for k in pts] + [(d, k) for d in "xy" for k in pts]
+    want = lskum_jvp.vjp_entries(c, oracle.split_stencils(c), U, Rb, ent, order=2, inner=2, limiter=K)
+    got = np.array([Ub[e[1], e[2]] if e[0] == "U" else (xb if e[0] == "x" else yb)[e[1]] for e in ent])
+    assert np.all(np.abs(got - want) <= 1e-10 * np.abs(want).max())
+
+
+@pytest.mark.gpu
+def test_the_sign_of_zero_does_not_matter_to_the_limiter_reverse():
+    """The search for the extreme neighbours orders bit patterns: momenta of
+    +0 and -0 are the same state and give the same cotangents."""
+    import torch
+
+    from paper_2403_13287_gb300.cloudgen import naca0012_cloud, smooth_state
+    from paper_2403_13287_gb300.lskum import Solver
+    c = naca0012_cloud(50, 14, seed=5)
+    rng = np.random.default_rng(0)
+    U = smooth_state(c, 0.85, 1.0, amp=0.05, seed=4)
+    U[3] -= 0.5 * U[2] ** 2 / U[0]
+    U[2] = 0.0
+    Rb = torch.from_numpy(rng.standard_normal((4, c["n"]))).cuda()
+    V = U.copy()
+    V[2] = np.where(rng.random(c["n"]) < 0.5, -0.0, 0.0)
+    s = Solver(c, order=2, inner_iters=2, mach=0.85, aoa_deg=1.0, limiter_K=1.0)
+    a, b = (s.residual_vjp(Rb, torch.from_numpy(x).cuda()) for x in (U, V))
+    s.close()
+    for p, q in zip(a, b):
+        assert torch.equal(p, q)
