@@ -666,34 +666,73 @@ __device__ __forceinline__ void member_difference(bool act, int l, const double 
     }
 }
 
-// A[k] += w d[k] of the group's members in row order: the own one (PAIRS = 1),
-// or those that the PAIRS pairs of a point hold, one each
+// The sums over a point's members, in row order whatever PAIRS: A[k] += w d[k].
+// One pair of lanes takes its own members (all four components). Several pairs
+// hand their differences over through shared memory, and pair p sums component
+// p of all of them (2 pairs: 2p and 2p + 1), so that no addition is done
+// twice: by shuffles each lane summed everything, PAIRS times the FP64 work (4
+// pairs 29.1 -> 25.6 us at 3k points, 38.1 -> 34.1 at 10k; 2 pairs 71.8 -> 69.4 at 40k).
 template <int PAIRS>
-__device__ __forceinline__ void add_members(double w, const double d[4], double A[4])
-{
-    if constexpr (PAIRS == 1) {
+struct Members {
+    static constexpr int C = PAIRS == 1 ? 4 : PAIRS == 2 ? 2 : 1;   // components a lane sums
+    static constexpr int kStride = 34;                              // doubles: the reads of a component meet no bank twice
+    double A[C];
+    __device__ __forceinline__ Members()
+    {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) A[k] = fma(w, d[k], A[k]);
-    } else {
-        const int l = threadIdx.x & 1;
+        for (int k = 0; k < C; ++k) A[k] = 0.0;
+    }
+    static __device__ __forceinline__ int first() { return C * ((threadIdx.x >> 1) % PAIRS); }
+    // called by whole warps; x: 5 kStride doubles of the warp's own
+    __device__ __forceinline__ void add(double w, const double d[4], double *x)
+    {
+        if constexpr (PAIRS == 1) {
 #pragma unroll
-        for (int j = 0; j < PAIRS; ++j) {
-            const double wj = __shfl_sync(0xffffffffu, w, 2 * j + l, 2 * PAIRS);
+            for (int k = 0; k < 4; ++k) A[k] = fma(w, d[k], A[k]);
+        } else {
+            const int t = threadIdx.x & 31, base = (t & ~(2 * PAIRS - 1)) | (t & 1);
+            __syncwarp();   // the last round's reads are done
 #pragma unroll
-            for (int k = 0; k < 4; ++k) A[k] = fma(wj, __shfl_sync(0xffffffffu, d[k], 2 * j + l, 2 * PAIRS), A[k]);
+            for (int k = 0; k < 4; ++k) x[k * kStride + t] = d[k];
+            x[4 * kStride + t] = w;
+            __syncwarp();
+            const double *row = x + first() * kStride + base;
+#pragma unroll
+            for (int j = 0; j < PAIRS; ++j) {
+                const double wj = x[4 * kStride + base + 2 * j];
+#pragma unroll
+                for (int k = 0; k < C; ++k) A[k] = fma(wj, row[k * kStride + 2 * j], A[k]);
+            }
         }
     }
-}
+    // all four sums of a lane's direction, in every lane
+    __device__ __forceinline__ void all(double *x, double S[4]) const
+    {
+        if constexpr (PAIRS == 1) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) S[k] = A[k];
+        } else {
+            const int t = threadIdx.x & 31, base = (t & ~(2 * PAIRS - 1)) | (t & 1);
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < C; ++k) x[(first() + k) * kStride + base] = A[k];
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < 4; ++k) S[k] = x[k * kStride + base];
+        }
+    }
+};
 
-// What bounds it: the FP64 pipe (76 % busy: the reconstruction, the sums, the
-// state update) and the integer ALUs (52 %), 62 % of the issue slots. 64
-// registers and a few spills, for 32 warps per SM, beat 80 (24 warps) and 128
-// (16): 2.30 / 2.48 / 2.67 ms at 2.5 million points. One lane per member with
-// both states took 2.58 ms and a chain twice as long.
+// What bounds it at large sizes: the FP64 pipe (65 % busy: the reconstruction,
+// the sums, the state update), the integer multipliers (63 %) and ALUs (57 %),
+// 66 % of the issue slots; at a few thousand points one warp's chain of rounds.
+// 64 registers and a few spills, for 32 warps per SM, beat 80 (24 warps) and 128
+// (16): 2.22 ms at 2.5 million points, before the last changes 2.30 / 2.48 / 2.67.
+// One lane per member with both states took 2.58 ms and a chain twice as long.
 // Two lanes per member (member_difference), PAIRS pairs of lanes per point. With
 // one pair the members of a row follow one another; with 2 or 4 each pair takes
 // every second or fourth, and the differences are added in row order all the
-// same (add_members), so that a small cloud spreads over more warps with a
+// same (Members), so that a small cloud spreads over more warps with a
 // fraction of the serial chain and every launch gives the same bits. The state
 // update runs afterwards with one lane per point (R through shared memory).
 template <int PAIRS>
@@ -706,6 +745,9 @@ __global__ void __launch_bounds__(FluxShape<PAIRS>::kThreads, PAIRS == 1 ? 8 : P
 {
     constexpr int POINTS = FluxShape<PAIRS>::kPoints;
     __shared__ double2 s_R[POINTS][2];
+    constexpr int kWarps = PAIRS == 1 ? 0 : FluxShape<PAIRS>::kThreads / 32, kRow = 5 * Members<PAIRS>::kStride;
+    __shared__ double s_members[kWarps * kRow + 1];
+    double *const xw = s_members + (PAIRS == 1 ? 0 : (threadIdx.x >> 5) * kRow);
     const DevGeom &g = P.g;
     {
         const int l = threadIdx.x & 1, pair = (threadIdx.x >> 1) % PAIRS, pt = threadIdx.x / (2 * PAIRS);
@@ -719,7 +761,7 @@ __global__ void __launch_bounds__(FluxShape<PAIRS>::kThreads, PAIRS == 1 ? 8 : P
         const int e0 = g.off[p], deg = work ? g.off[p + 1] - e0 : 0;
         double2 xy0 = make_double2(0.0, 0.0);
         if (second && !g.hd) xy0 = g.xy[p];
-        double A[4] = {0.0, 0.0, 0.0, 0.0};
+        Members<PAIRS> sums;
         bool ok = true;
         // whole warps go through the longest row's rounds: the members exchange by shuffles
         const int most = __reduce_max_sync(0xffffffffu, (deg + PAIRS - 1) / PAIRS);
@@ -748,7 +790,7 @@ __global__ void __launch_bounds__(FluxShape<PAIRS>::kThreads, PAIRS == 1 ? 8 : P
                 for (int k = 0; k < 4; ++k) qt[k] = fma(-h.y, gr[4 + k], fma(-h.x, gr[k], qt[k]));
             }
             member_difference(act, l, qt, g.mask[e], w, n0, fnx, fny, P.gas, d, ok);
-            add_members<PAIRS>(l ? w.y : w.x, d, A);
+            sums.add(l ? w.y : w.x, d, xw);
         }
         if constexpr (KIN) {
             // kinetic boundary mode: the mirror images of the neighbours
@@ -778,13 +820,14 @@ __global__ void __launch_bounds__(FluxShape<PAIRS>::kThreads, PAIRS == 1 ? 8 : P
                     }
                 }
                 member_difference(act, l, qt, m, w, n0, fnx, fny, P.gas, d, ok);
-                add_members<PAIRS>(l ? w.y : w.x, d, A);
+                sums.add(l ? w.y : w.x, d, xw);
             }
         }
         if (!ok) flag_nonphysical(P.status, p);
         // lane 0 holds the sums along t, lane 1 those along n: R in the order
         // [mass, s-momentum, n-momentum, energy]
-        double N[4];
+        double A[4], N[4];
+        sums.all(xw, A);
 #pragma unroll
         for (int k = 0; k < 4; ++k) N[k] = other_lane(A[k]);
         if (threadIdx.x % (2 * PAIRS) == 0) {
@@ -1065,16 +1108,17 @@ cudaError_t launch_flux(const DevGeom &g, const Gas &gas, const FluxLaunch &L, c
     P.pcase = L.pcase; P.case_uinf = L.case_uinf;
     P.cfl = L.cfl; P.order = L.order; P.mode = L.mode; P.stage = L.stage;
     // Pairs of lanes per point (the same bits whichever): more while the cloud
-    // leaves SMs idle and the launch is one warp's serial chain. 4 / 2 / 1 pairs
-    // take 31 / 42 / 69 us at 3k points, 42 / 48 / 71 at 10k, 64 / 49 / 65 at
-    // 20k, 99 / 76 / 80 at 40k and 145 / 103 / 99 at 64k, where every pair adds
-    // all members' terms again.
+    // leaves SMs idle and the launch is one warp's serial chain. 4 / 2 pairs take
+    // 26 / 38 us at 3k points, 34 / 43 at 10k, 53 / 46 at 20k and 81 / 69 at 40k,
+    // 2 / 1 pairs 93 / 96 at 64k, 123 / 131 at 93k, 190 / 188 at 160k and 348 /
+    // 322 at 320k (lanes without a member in a point's last round). 8 pairs gain
+    // 1.4 us at 3k and lose above.
     if (!gas.g14) {
         if (g.ioff) k_flux_update_fp64<true><<<blocks_for(g.n, 128), 128, 0, s>>>(P);
         else k_flux_update_fp64<false><<<blocks_for(g.n, 128), 128, 0, s>>>(P);
     } else if (g.n < 14000) {
         flux_pairs<4>(P, s);
-    } else if (g.n < 50000) {
+    } else if (g.n < 120000) {
         flux_pairs<2>(P, s);
     } else {
         flux_pairs<1>(P, s);

@@ -321,7 +321,7 @@ def test_residual_across_the_range_matches_the_oracle(gamma, mach, boundary):
 def test_every_launch_form_gives_the_same_bits(order, limiter, boundary):
     """The FP64 kernels split a point over more lanes the smaller the cloud: 4,
     2 or 1 pairs in the flux kernel, 4 or 2 lanes in the q-derivative passes.
-    A 3250-point cloud alone, beside 18k points and beside 64k points in one
+    A 3250-point cloud alone, beside 18k points and beside 114k points in one
     batch (all three forms): bitwise the same states and residuals, and the
     18k cloud's residual at the oracle's bar."""
     import torch
@@ -329,7 +329,7 @@ def test_every_launch_form_gives_the_same_bits(order, limiter, boundary):
     import oracle
     from paper_2403_13287_gb300.cloudgen import naca0012_cloud, smooth_state
     from paper_2403_13287_gb300.lskum import Solver
-    a, mid, big = naca0012_cloud(130, 24, seed=11), naca0012_cloud(180, 99, seed=3, shuffle=True), naca0012_cloud(324, 197, seed=4)
+    a, mid, big = naca0012_cloud(130, 24, seed=11), naca0012_cloud(180, 99, seed=3, shuffle=True), naca0012_cloud(512, 221, seed=4)
     kw = dict(order=order, inner_iters=3, time_scheme=1, limiter_K=limiter, precision=0, reorder=1, boundary=boundary)
     U0 = {id(c): smooth_state(c, 0.85, 1.0, amp=0.05, seed=9) for c in (a, mid, big)}
     got = []
