@@ -905,52 +905,70 @@ __global__ void __launch_bounds__(128) k_adj_grad_fp32(AdjParamsT<float> P, cons
 // which keep the q cotangent apart (qbar2: the owner's share, summed with qbar
 // by k_adj_state), and the two-term products run on the integer pipes
 // (fix_dot): 40 FP64 instructions per edge of 68. 87 -> 62 us a pass at 40k points.
+// LANES 2: two lanes per point, two components each. Without the geometry's
+// cotangents that is the better form at all sizes (residual product 0.48 -> 0.46
+// ms at 40k points, 3.75 -> 3.71 at 640k); with them the lanes add up a_bar and
+// d_bar, one each, from both halves, which pays while the cloud leaves SMs idle
+// (0.50 -> 0.45 ms at 8k, 0.73 -> 0.69 at 40k; 1.14 -> 1.18 at 93k, 5.77 -> 5.94
+// at 640k). U_bar has the same bits in both forms, x_bar and y_bar differ in
+// rounding (a sum of two halves for one of four terms).
 __device__ __forceinline__ double dot2(const FixPair &a, const FixPair &b, double ax, double ay, double bx, double by)
 {
     if (fix_dot_in_range(a, b)) return fix_dot(a, b);
     return b.e ? fma(ay, by, ax * bx) : 0.0;   // both terms zero (or subnormal): nothing to add
 }
 
-template <bool GEOM>
-__global__ void __launch_bounds__(128, 5) k_adj_grad_fp64(AdjParams P, const double *__restrict__ gprev,
+template <bool GEOM, int LANES>
+__global__ void __launch_bounds__(128, LANES == 1 ? 5 : GEOM ? 5 : 8) k_adj_grad_fp64(AdjParams P, const double *__restrict__ gprev,
                                                           const double *__restrict__ gbar_in,
                                                           double *__restrict__ gbar_out, int first)
 {
+    constexpr int C = 4 / LANES;
     const DevGeom &g = P.g;
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= g.n) return;
+    const int64_t pp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+    const int l = threadIdx.x % LANES, k0 = C * l;
+    const bool live = pp < g.n;
+    if (LANES == 1 && !live) return;
+    const int64_t p = live ? pp : g.n - 1;   // (lanes past the end take part in the shuffles)
     const bool inner = gprev != nullptr;
-    double qb[4] = {0.0, 0.0, 0.0, 0.0}, gb[8];
-    ld8(gbar_in, p, gb);
+    double qb[C], gx[C], gy[C];
+    gather_c<C>(gbar_in + 8 * p + k0, gx);
+    gather_c<C>(gbar_in + 8 * p + 4 + k0, gy);
     if (blockIdx.y == 0) {
         // outgoing edges: owner terms, and the cotangents of a_e and of the offsets
-        if (!first) ld4(P.qbar2, p, qb);
-        FixPair gbp[4];
+        FixPair gbp[C];
+        double qp[C];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) gbp[k] = fix_pair(gb[k], gb[4 + k]);
-        double qp[4];
+        for (int k = 0; k < C; ++k) {
+            qb[k] = first ? 0.0 : P.qbar2[4 * p + k0 + k];
+            gbp[k] = fix_pair(gx[k], gy[k]);
+        }
         double2 xyp = make_double2(0.0, 0.0);
         if constexpr (GEOM) {
-            ld4(P.q, p, qp);
+            gather_c<C>(P.q + 4 * p + k0, qp);
             if (!g.hd) xyp = g.xy[p];
         }
-        const int e1 = g.off[p + 1];
+        const int e0 = g.off[p], deg = live ? g.off[p + 1] - e0 : 0;
+        // two lanes: whole warps go through the longest row, as the lanes exchange sums by shuffles
+        const int most = GEOM && LANES > 1 ? __reduce_max_sync(0xffffffffu, deg) : deg;
 #pragma unroll 1
-        for (int e = g.off[p]; e < e1; ++e) {
+        for (int j = 0; j < most; ++j) {
+            const bool act = j < deg;
+            const int e = act ? e0 + j : e0;
             const double2 a = g.lsw[e];
             const FixPair ap = fix_pair(a.x, a.y);
-            double sb[4];
+            double sb[C];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                sb[k] = dot2(ap, gbp[k], a.x, a.y, gb[k], gb[4 + k]);
-                qb[k] -= sb[k];
+            for (int k = 0; k < C; ++k) {
+                sb[k] = dot2(ap, gbp[k], a.x, a.y, gx[k], gy[k]);
+                if (act) qb[k] -= sb[k];
             }
             if constexpr (GEOM) {
                 const int64_t i = g.idx[e];
-                double qi[4], gi[8], s[4];
-                gather4(P.q, i, qi);
+                double qi[C], s[C], dbx = 0.0, dby = 0.0;
+                gather_c<C>(P.q + 4 * i + k0, qi);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) s[k] = qi[k] - qp[k];
+                for (int k = 0; k < C; ++k) s[k] = qi[k] - qp[k];
                 if (inner) {
                     double2 h;
                     if (g.hd) {
@@ -960,59 +978,85 @@ __global__ void __launch_bounds__(128, 5) k_adj_grad_fp64(AdjParams P, const dou
                         h = make_double2(0.5 * (xyi.x - xyp.x), 0.5 * (xyi.y - xyp.y));
                     }
                     const FixPair hp = fix_pair(h.x, h.y);
-                    gather8(gprev, i, gi);
-                    double dbx = 0.0, dby = 0.0;
+                    double ix[C], iy[C];
+                    gather_c<C>(gprev + 8 * i + k0, ix);
+                    gather_c<C>(gprev + 8 * i + 4 + k0, iy);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        s[k] -= dot2(hp, fix_pair(gi[k], gi[4 + k]), h.x, h.y, gi[k], gi[4 + k]);
+                    for (int k = 0; k < C; ++k) {
+                        s[k] -= dot2(hp, fix_pair(ix[k], iy[k]), h.x, h.y, ix[k], iy[k]);
                         // d_e = 2 h_e: d_bar = -(sb/2) grad q_i
-                        dbx = fma(sb[k], gi[k], dbx);
-                        dby = fma(sb[k], gi[4 + k], dby);
+                        dbx = fma(sb[k], ix[k], dbx);
+                        dby = fma(sb[k], iy[k], dby);
                     }
-                    double2 db = P.dbar[e];
-                    db.x = fma(-0.5, dbx, db.x);
-                    db.y = fma(-0.5, dby, db.y);
-                    P.dbar[e] = db;
                 }
-                double2 ab = first && !P.add ? make_double2(0.0, 0.0) : P.abar[e];
+                if constexpr (LANES == 1) {
+                    if (inner) {
+                        double2 db = P.dbar[e];
+                        db.x = fma(-0.5, dbx, db.x);
+                        db.y = fma(-0.5, dby, db.y);
+                        P.dbar[e] = db;
+                    }
+                    double2 ab = first && !P.add ? make_double2(0.0, 0.0) : P.abar[e];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    ab.x = fma(s[k], gb[k], ab.x);
-                    ab.y = fma(s[k], gb[4 + k], ab.y);
+                    for (int k = 0; k < C; ++k) {
+                        ab.x = fma(s[k], gx[k], ab.x);
+                        ab.y = fma(s[k], gy[k], ab.y);
+                    }
+                    P.abar[e] = ab;
+                } else {
+                    // lane 0 completes a_bar, lane 1 d_bar
+                    const double abx = fma(s[1], gx[1], s[0] * gx[0]), aby = fma(s[1], gy[1], s[0] * gy[0]);
+                    const double tx = (l ? dbx : abx) + __shfl_xor_sync(0xffffffffu, l ? abx : dbx, 1);
+                    const double ty = (l ? dby : aby) + __shfl_xor_sync(0xffffffffu, l ? aby : dby, 1);
+                    if (act && (l == 0 || inner)) {
+                        double2 *o = (l ? P.dbar : P.abar) + e;
+                        const double f = l ? -0.5 : 1.0;
+                        double2 v = l == 0 && first && !P.add ? make_double2(0.0, 0.0) : *o;
+                        v.x = fma(f, tx, v.x);
+                        v.y = fma(f, ty, v.y);
+                        *o = v;
+                    }
                 }
-                P.abar[e] = ab;
             }
         }
-        st4(P.qbar2, p, qb);
+        if (live) store_c<C>(P.qbar2 + 4 * p + k0, qb);
     } else {
         // incoming edges: the terms of this point as a neighbour; an inner pass
         // gives grad q_0 the cotangent gb / 2 (see k_adj_grad_fp32)
-        ld4(P.qbar, p, qb);
-        double gbo[8];
+        if (!live) return;
+        double ox[C], oy[C];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) gbo[k] = 0.5 * gb[k];
+        for (int k = 0; k < C; ++k) {
+            qb[k] = P.qbar[4 * p + k0 + k];
+            ox[k] = 0.5 * gx[k];
+            oy[k] = 0.5 * gy[k];
+        }
         const int t1 = P.toff[p + 1];
 #pragma unroll 1
         for (int t = P.toff[p]; t < t1; ++t) {
             const int64_t src = P.tsrc[t];
             const double2 a = __ldg(P.tlsw + t);
             const FixPair ap = fix_pair(a.x, a.y);
-            double gs[8];
-            gather8(gbar_in, src, gs);
+            double sx[C], sy[C];
+            gather_c<C>(gbar_in + 8 * src + k0, sx);
+            gather_c<C>(gbar_in + 8 * src + 4 + k0, sy);
             double2 h = make_double2(0.0, 0.0);
             if (inner) h = __ldg(P.thd + t);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const double sb = dot2(ap, fix_pair(gs[k], gs[4 + k]), a.x, a.y, gs[k], gs[4 + k]);
+            for (int k = 0; k < C; ++k) {
+                const double sb = dot2(ap, fix_pair(sx[k], sy[k]), a.x, a.y, sx[k], sy[k]);
                 qb[k] += sb;
                 if (inner) {
-                    gbo[k] = fma(-h.x, sb, gbo[k]);
-                    gbo[4 + k] = fma(-h.y, sb, gbo[4 + k]);
+                    ox[k] = fma(-h.x, sb, ox[k]);
+                    oy[k] = fma(-h.y, sb, oy[k]);
                 }
             }
         }
-        st4(P.qbar, p, qb);
-        if (inner) st8(gbar_out, p, gbo);
+        store_c<C>(P.qbar + 4 * p + k0, qb);
+        if (inner) {
+            store_c<C>(gbar_out + 8 * p + k0, ox);
+            store_c<C>(gbar_out + 8 * p + 4 + k0, oy);
+        }
     }
 }
 
@@ -1604,9 +1648,12 @@ cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gba
                             bool first, cudaStream_t s)
 {
     if constexpr (std::is_same<T, double>::value) {
-        const dim3 nb(blocks(P.g.n, 128), 2);
-        if (geom) k_adj_grad_fp64<true><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
-        else k_adj_grad_fp64<false><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+        // (lanes per point: see the kernel)
+        const bool two = !geom || P.g.n < 60000;
+        const dim3 nb(blocks(P.g.n, two ? 64 : 128), 2);
+        if (!geom) k_adj_grad_fp64<false, 2><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+        else if (two) k_adj_grad_fp64<true, 2><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+        else k_adj_grad_fp64<true, 1><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
     } else {
         if (geom) k_adj_grad_fp32<true><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
         else k_adj_grad_fp32<false><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);

@@ -338,6 +338,33 @@ __device__ __forceinline__ void gather8(const double *a, int64_t p, double v[8])
     gather4(a, 2 * p + 1, v + 4);
 }
 
+// C consecutive values of a row (aligned to C values): read-only load, store
+template <int C>
+__device__ __forceinline__ void gather_c(const double *a, double v[C])
+{
+    if constexpr (C == 4) {
+        gather4(a, 0, v);
+    } else if constexpr (C == 2) {
+        const double2 w = __ldg(reinterpret_cast<const double2 *>(a));
+        v[0] = w.x;
+        v[1] = w.y;
+    } else {
+        v[0] = __ldg(a);
+    }
+}
+template <int C>
+__device__ __forceinline__ void store_c(double *a, const double v[C])
+{
+    if constexpr (C == 4) {
+        store4(a, 0, v);
+    } else if constexpr (C == 2) {
+        *reinterpret_cast<double2 *>(a) = make_double2(v[0], v[1]);
+    } else {
+        *a = v[0];
+    }
+}
+// components k0 .. k0 + C - 1 (k0 a multiple of C) without an indexed array in memory
+
 // double -> float, round to nearest (ties away), on the integer pipe for
 // magnitudes of 2^-100 to 2^100 and for 0; the conversion instruction (FP64
 // pipe) elsewhere

@@ -66,32 +66,6 @@ __device__ __forceinline__ void image_q(const DevGeom &g, int e, uint8_t m, doub
 // 1/64 of the integer ALU rate, so the stencil extrema take this form.
 __device__ __forceinline__ long long order_key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffLL); }
 
-// C consecutive values of a row (aligned to C values): read-only load, store
-template <int C>
-__device__ __forceinline__ void gather_c(const double *a, double v[C])
-{
-    if constexpr (C == 4) {
-        gather4(a, 0, v);
-    } else if constexpr (C == 2) {
-        const double2 w = __ldg(reinterpret_cast<const double2 *>(a));
-        v[0] = w.x;
-        v[1] = w.y;
-    } else {
-        v[0] = __ldg(a);
-    }
-}
-template <int C>
-__device__ __forceinline__ void store_c(double *a, const double v[C])
-{
-    if constexpr (C == 4) {
-        store4(a, 0, v);
-    } else if constexpr (C == 2) {
-        *reinterpret_cast<double2 *>(a) = make_double2(v[0], v[1]);
-    } else {
-        *a = v[0];
-    }
-}
-// components k0 .. k0 + C - 1 (k0 a multiple of C) without an indexed array in memory
 template <int C>
 __device__ __forceinline__ void components(const double v[4], int k0, double o[C])
 {

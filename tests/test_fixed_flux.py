@@ -457,3 +457,34 @@ def test_the_sign_of_zero_does_not_matter_to_the_limiter_reverse():
     s.close()
     for p, q in zip(a, b):
         assert torch.equal(p, q)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("limiter", [0.0, 1.0])
+def test_both_lane_forms_of_the_reverse_gradient_passes(limiter):
+    """One or two lanes per point by the size of the cloud: a 3250-point cloud
+    alone and beside 64k points in one batch. U_bar bitwise; x_bar and y_bar,
+    whose sums take their four terms in another order, to 1e-13 of the largest
+    (2^-53 per addition of at most 20 edges' terms that cancel by up to 10)."""
+    import torch
+
+    from paper_2403_13287_gb300.cloudgen import naca0012_cloud, smooth_state
+    from paper_2403_13287_gb300.lskum import Solver
+    a, big = naca0012_cloud(130, 24, seed=11), naca0012_cloud(324, 197, seed=4)
+    n = a["n"]
+    kw = dict(order=2, inner_iters=3, time_scheme=1, limiter_K=limiter, precision=0, reorder=1)
+    U0 = [smooth_state(c, 0.85, 1.0, amp=0.05, seed=9) for c in (a, big)]
+    Rb = np.random.default_rng(2).standard_normal((4, n + big["n"]))
+    got = []
+    for clouds in ([a], [a, big]):
+        m = sum(c["n"] for c in clouds)
+        s = Solver.batch([(c, 0.85, 1.0) for c in clouds], **kw) if len(clouds) > 1 else Solver(a, mach=0.85, aoa_deg=1.0, **kw)
+        U = np.ascontiguousarray(np.concatenate(U0[:len(clouds)], axis=1))
+        out = s.residual_vjp(torch.from_numpy(np.ascontiguousarray(Rb[:, :m])).cuda(), torch.from_numpy(U).cuda())
+        only = s.residual_vjp(torch.from_numpy(np.ascontiguousarray(Rb[:, :m])).cuda(), torch.from_numpy(U).cuda(), want_xy=False)[0]
+        assert torch.equal(out[0], only)
+        got.append([t.cpu().numpy()[..., :n] for t in out])
+        s.close()
+    assert np.array_equal(got[0][0], got[1][0])
+    for p, q in zip(got[0][1:], got[1][1:]):
+        assert np.abs(p - q).max() <= 1e-13 * np.abs(p).max()
