@@ -1354,47 +1354,71 @@ static const double *vjp_final_gradient(const lskum_ctx *c, const lskum_ctx::For
     return limited(c) ? f.Glim : f.G + (int64_t)c->cfg.inner_iters * 8 * c->n;
 }
 
-static cudaError_t alloc_forward(lskum_ctx *c, lskum_ctx::Forward &f)
+// arrays that are allocated together, in one piece of device memory: an
+// allocation costs tens of microseconds, and a product's first call made some
+// thirty (first FP32 product at 8k points 1.02 -> 0.58 ms, first RK4 step
+// product at 40k 4.4 -> 2.9 ms). None of them is set unless all are there.
+struct Workspace {
+    std::vector<std::pair<void **, size_t>> parts;
+    size_t bytes = 0;
+    template <class T>
+    void add(T **p, int64_t count)
+    {
+        parts.push_back({reinterpret_cast<void **>(p), bytes});
+        bytes += ((size_t)std::max<int64_t>(count, 1) * sizeof(T) + 255) / 256 * 256;
+    }
+    cudaError_t alloc(lskum_ctx *c) const
+    {
+        char *base = nullptr;
+        const cudaError_t e = dalloc(c, &base, bytes);
+        if (e != cudaSuccess) return e;
+        for (const auto &p : parts) *p.first = base + p.second;
+        return e;
+    }
+};
+
+static void add_forward(lskum_ctx *c, Workspace &w, lskum_ctx::Forward &f)
 {
     const int64_t n = c->n;
-    cudaError_t e = dalloc(c, &f.q, 4 * n);
-    if (e == cudaSuccess && c->cfg.order == 2) e = dalloc(c, &f.G, (int64_t)(c->cfg.inner_iters + 1) * 8 * n);
-    if (e == cudaSuccess && limited(c)) e = dalloc(c, &f.Glim, 8 * n);
-    return e;
+    w.add(&f.q, 4 * n);
+    if (c->cfg.order == 2) w.add(&f.G, (int64_t)(c->cfg.inner_iters + 1) * 8 * n);
+    if (limited(c)) w.add(&f.Glim, 8 * n);
 }
 
 static lskum_status vjp_workspace(lskum_ctx *c)
 {
     if (c->vjp_ready) return LSKUM_OK;
     const int64_t n = c->n, m = std::max<int64_t>(c->nnz, 1);
-    CK(c, alloc_forward(c, c->fw[0]));
+    Workspace w;
+    add_forward(c, w, c->fw[0]);
     if (c->cfg.order == 2) {
-        CK(c, dalloc(c, &c->vgb, 8 * n));
-        CK(c, dalloc(c, &c->vgb2, 8 * n));
-        CK(c, dalloc(c, &c->vqb2, 4 * n));
+        w.add(&c->vgb, 8 * n);
+        w.add(&c->vgb2, 8 * n);
+        w.add(&c->vqb2, 4 * n);
     }
-    CK(c, dalloc(c, &c->vRb, 4 * n));
-    CK(c, dalloc(c, &c->vqb, 4 * n));
-    CK(c, dalloc(c, &c->vebar, 4 * m));
-    CK(c, dalloc(c, &c->vwbar, m));
-    CK(c, dalloc(c, &c->vabar, m));
-    CK(c, dalloc(c, &c->vdbar, m));
-    CK(c, dalloc(c, &c->toff, n + 1));
-    CK(c, dalloc(c, &c->tedge, m));
-    CK(c, dalloc(c, &c->tsrc, m));
-    CK(c, dalloc(c, &c->tlsw, m));
-    CK(c, dalloc(c, &c->thd, m));
-    CK(c, dalloc(c, &c->vplan, kAdjPlan * n));
-    CK(c, dalloc(c, &c->near_e, n));
-    CK(c, dalloc(c, &c->near_u, n));
-    CK(c, dalloc(c, &c->vUacc, 4 * n));
-    CK(c, dalloc(c, &c->vpxy, n));
-    CK(c, dalloc(c, &c->fdsb, std::max<int64_t>(c->n_wall, 1)));
+    w.add(&c->vRb, 4 * n);
+    w.add(&c->vqb, 4 * n);
+    w.add(&c->vebar, 4 * m);
+    w.add(&c->vwbar, m);
+    w.add(&c->vabar, m);
+    w.add(&c->vdbar, m);
+    w.add(&c->toff, n + 1);
+    w.add(&c->tedge, m);
+    w.add(&c->tsrc, m);
+    w.add(&c->tlsw, m);
+    w.add(&c->thd, m);
+    w.add(&c->vplan, kAdjPlan * n);
+    w.add(&c->near_e, n);
+    w.add(&c->near_u, n);
+    w.add(&c->vUacc, 4 * n);
+    w.add(&c->vpxy, n);
+    w.add(&c->fdsb, std::max<int64_t>(c->n_wall, 1));
     if (limited(c)) {
-        CK(c, dalloc(c, &c->vext, 4 * n));
-        CK(c, dalloc(c, &c->vlidx, 4 * n));
-        CK(c, dalloc(c, &c->vlval, 4 * n));
+        w.add(&c->vext, 4 * n);
+        w.add(&c->vlidx, 4 * n);
+        w.add(&c->vlval, 4 * n);
     }
+    CK(c, w.alloc(c));
     c->launches += 5;
     LAUNCH(c, build_adj_plan(c->geom(), c->vplan, c->near_e, c->near_u, c->stream));
     LAUNCH(c, build_transpose_csr(n, c->nnz, c->off, c->idx, c->toff, c->tedge, c->tsrc, c->stream));
@@ -1484,18 +1508,20 @@ static lskum_status fvjp_workspace(lskum_ctx *c)
     if (c->fvjp_ready) return LSKUM_OK;
     const int64_t n = c->n, m = std::max<int64_t>(c->nnz, 1);
     const int K = c->cfg.order == 2 ? c->cfg.inner_iters : 0;
-    CK(c, dalloc(c, &c->fq, 4 * n));
+    Workspace w;
+    w.add(&c->fq, 4 * n);
     if (c->cfg.order == 2) {
-        CK(c, dalloc(c, &c->fG, (int64_t)(K + 1) * 8 * n));
-        CK(c, dalloc(c, &c->fgb, 8 * n));
-        CK(c, dalloc(c, &c->fgb2, 8 * n));
+        w.add(&c->fG, (int64_t)(K + 1) * 8 * n);
+        w.add(&c->fgb, 8 * n);
+        w.add(&c->fgb2, 8 * n);
     }
-    CK(c, dalloc(c, &c->fRb, 4 * n));
-    CK(c, dalloc(c, &c->fqb, 4 * n));
-    CK(c, dalloc(c, &c->febar, 4 * m));
-    CK(c, dalloc(c, &c->fef, m));
-    CK(c, dalloc(c, &c->fea, m));
-    CK(c, dalloc(c, &c->ftf, m));
+    w.add(&c->fRb, 4 * n);
+    w.add(&c->fqb, 4 * n);
+    w.add(&c->febar, 4 * m);
+    w.add(&c->fef, m);
+    w.add(&c->fea, m);
+    w.add(&c->ftf, m);
+    CK(c, w.alloc(c));
     c->launches++;
     LAUNCH(c, build_float_geometry(c->geom(), c->nnz, c->tlsw, c->thd, c->fef, c->fea, c->ftf, c->stream));
     c->fvjp_ready = true;
@@ -1658,26 +1684,23 @@ static lskum_status step_vjp_workspace(lskum_ctx *c)
 {
     if (c->svjp_ready) return LSKUM_OK;
     const int64_t n = c->n;
-    for (auto &b : c->sR) CK(c, dalloc(c, &b, 4 * n));
-    for (auto &b : c->sRb) CK(c, dalloc(c, &b, 4 * n));
-    for (auto &b : c->sU) CK(c, dalloc(c, &b, 4 * n));
-    CK(c, dalloc(c, &c->sUb, 4 * n));
-    CK(c, dalloc(c, &c->sUin, 4 * n));
-    CK(c, dalloc(c, &c->sdt, n));
-    CK(c, dalloc(c, &c->sdtb, n));
+    Workspace w;
+    for (auto &b : c->sR) w.add(&b, 4 * n);
+    for (auto &b : c->sRb) w.add(&b, 4 * n);
+    for (auto &b : c->sU) w.add(&b, 4 * n);
+    w.add(&c->sUb, 4 * n);
+    w.add(&c->sUin, 4 * n);
+    w.add(&c->sdt, n);
+    w.add(&c->sdtb, n);
+    CK(c, w.alloc(c));
     if (c->cfg.time_scheme == 1) {
         // a forward per RK stage spares running it again in the reverse sweep;
         // without the memory for them that is what happens
-        cudaError_t e = cudaSuccess;
-        const size_t kept = c->allocs.size();
-        for (int k = 1; k < 4 && e == cudaSuccess; ++k) e = alloc_forward(c, c->fw[k]);
+        Workspace stages;
+        for (int k = 1; k < 4; ++k) add_forward(c, stages, c->fw[k]);
+        const cudaError_t e = stages.alloc(c);
         if (e != cudaSuccess && e != cudaErrorMemoryAllocation) CK(c, e);
-        if (e == cudaErrorMemoryAllocation) {
-            cudaGetLastError();
-            for (size_t a = kept; a < c->allocs.size(); ++a) cudaFree(c->allocs[a]);
-            c->allocs.resize(kept);
-            for (int k = 1; k < 4; ++k) c->fw[k] = lskum_ctx::Forward{};
-        }
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();
         c->stage_forwards = e == cudaSuccess;
     }
     c->svjp_ready = true;
