@@ -144,12 +144,12 @@ def measured_peaks():
 
 def algorithmic_bytes_per_point(kernel, dbar, order, scheme, stage_avg=True):
     """Bytes each array contributes once per launch, per point (FP64 layout):
-    q 32, q-derivatives 64, coordinates 16, normals 16, flag 1, dmin 8, CSR
+    q 32, q-derivatives 64, normals 16, flag 1, dmin 8, CSR
     offset 4, and per edge: index 4, mask 1, LS weights 16 (fused kernel:
     flux weights 16), half offsets (P_i - P_0)/2 16 (second order).
     Neighbour gathers are assumed served from cache."""
     if kernel == "flux":
-        b = 32 + 16 + 16 + 1 + 4 + dbar * (4 + 1 + 16)       # q, xy, nrm, flag, off, edges
+        b = 32 + 16 + 1 + 4 + dbar * (4 + 1 + 16)            # q, nrm, flag, off, edges
         if order == 2:
             b += 64 + dbar * 16                               # own q-derivatives, half offsets
         b += 32 + 32 + 32                                     # U^n read, U_out and q_out written
@@ -205,14 +205,15 @@ def algorithmic_bytes_per_point_mixed(kernel, dbar, order, scheme):
 
 
 # Per-unit figures of the FP64 fused flux kernel (ncu counters, 640k-point
-# capture, profiles/k_flux_update_fp64_naca0012_640k.md): executed FP64
-# instructions per stencil edge (every FP64 instruction, of which DFMA + DMUL +
-# DADD are 176.0) and the flops they carry (2 DFMA + DMUL + DADD); DRAM bytes
-# per point of one full-size 2.5M launch (single-pass capture,
-# profiles/launch_list_naca0012_2p5m_fp64.md).
-FP64_INSTR_PER_EDGE_FLUX = 178.34
-FP64_FLOPS_PER_EDGE_FLUX = 285.05
-FLUX_DRAM_BYTES_PER_POINT = 598.0
+# capture, profiles/k_flux_update_fp64_naca0012_640k.md): instructions that the
+# FP64 pipe executes per stencil edge (arithmetic and 64-bit conversions, lanes
+# of its warp instructions), the flops among them (2 DFMA + DMUL + DADD) and all
+# warp instructions issued per edge; DRAM bytes per point of one full-size 2.5M
+# launch (single-pass capture, profiles/launch_list_naca0012_2p5m_fp64.md).
+FP64_INSTR_PER_EDGE_FLUX = 39.91
+FP64_FLOPS_PER_EDGE_FLUX = 54.72
+FP64_FLUX_WARP_INSTR_PER_EDGE = 91.66
+FLUX_DRAM_BYTES_PER_POINT = 692.4
 # FP64 peak: ncu's DFMA unit count, 304 FP64 thread-instructions per cycle
 # (each DFMA 2 flops), at the 2070 MHz maximum SM clock
 FP64_PEAK_GINSTR = 304 * 2.070
@@ -220,15 +221,18 @@ FP64_PEAK_GFLOPS = 2 * FP64_PEAK_GINSTR
 
 
 def roofline_fp64(flux_avg_s, n, dbar, fb, achieved_gbs, peaks, peak_src, fp64_measured=None):
-    """The FP64 flux kernel is bound by the FP64 pipe: its issue rate of FP64
-    instructions (a DMUL or DADD takes a slot as a DFMA does) against the
-    pipe's 304 per cycle; the same rate against the FP64 multiply-add rate
-    measured on this GPU (lskum_probe_peak, GFLOP/s / 2); the flop rate and
-    the HBM view beside it, the latter also as flat keys."""
+    """The FP64 flux kernel splits its arithmetic between the FP64 pipe and the
+    integer pipes (64-bit fixed point), each about two thirds busy: the FP64
+    pipe's rate (a DMUL, a DADD or a conversion takes a slot as a DFMA does)
+    against its 304 per cycle and against the FP64 multiply-add rate measured
+    on this GPU (lskum_probe_peak, GFLOP/s / 2); the rate of all warp
+    instructions against the issue slots; the flop rate and the HBM view beside
+    it, the latter also as flat keys."""
     instr = FP64_INSTR_PER_EDGE_FLUX * dbar * n
     flops = FP64_FLOPS_PER_EDGE_FLUX * dbar * n
     achieved = instr / flux_avg_s / 1e9
     gflops = flops / flux_avg_s / 1e9
+    issued = FP64_FLUX_WARP_INSTR_PER_EDGE * dbar * n / flux_avg_s / 1e9
     r = {"bound": "alu", "kernel": "k_flux_update", "achieved": achieved,
          "peak": FP64_PEAK_GINSTR, "unit": "G FP64 instructions/s", "frac": achieved / FP64_PEAK_GINSTR,
          "traffic": FLUX_DRAM_BYTES_PER_POINT * n,
@@ -236,6 +240,8 @@ def roofline_fp64(flux_avg_s, n, dbar, fb, achieved_gbs, peaks, peak_src, fp64_m
          "gflops": gflops, "gflops_peak": FP64_PEAK_GFLOPS, "gflops_frac": gflops / FP64_PEAK_GFLOPS,
          "avg_launch_ms": flux_avg_s * 1e3,
          "peak_source": "derived: 304 FP64 instructions/cycle x 2.07 GHz (ncu unit count, max SM clock)",
+         "issue": {"achieved": issued, "peak": ISSUE_PEAK_GINSTR, "unit": "G warp instructions/s",
+                   "frac": issued / ISSUE_PEAK_GINSTR},
          "hbm_achieved_gbs": achieved_gbs, "hbm_peak_gbs": peaks["hbm_gbs"],
          "hbm_frac": achieved_gbs / peaks["hbm_gbs"], "hbm_algorithmic_bytes_per_launch": fb,
          "hbm_traffic_bytes_per_launch": FLUX_DRAM_BYTES_PER_POINT * n, "hbm_peak_source": peak_src,

@@ -1,25 +1,28 @@
 // Vector-Jacobian product of the q-LSKUM residual (E10 with E11, E13-E15):
 // U_bar = (dR/dU)^T R_bar and (x_bar, y_bar) = (dR/dx, dR/dy)^T R_bar, in
-// FP64, for the unlimited scheme of order 1 or 2.
+// FP64 or (mixed contexts, unlimited) FP32, for order 1 or 2.
 //
 // Reverse pass, every sum a gather (no atomics, bitwise reproducible):
 //   flux      per point (owner of its edges): the transposed split-flux
 //             Jacobians at both reconstructed states applied to the
-//             cotangents (FP64: reverse mode through the regrouped split
-//             fluxes; FP32: forward-mode duals, 4 tangents), giving
+//             cotangents (FP64: in the variables of the fixed-point fluxes,
+//             k_adj_flux_pair, or through the regrouped split fluxes for
+//             gamma != 1.4; FP32: forward-mode duals, 4 tangents), giving
 //             cotangents of the owner's q~_0, of each neighbour's q~_i (kept
 //             per edge) and of the sub-stencil weights;
 //   gather    per point over its incoming edges (transpose CSR): the
 //             neighbour-side cotangents;
+//   limiter   (limiter_K > 0) back to the unlimited last iterate;
 //   gradient  the K+1 least-squares passes of E15 in reverse (saved forward
 //             iterates), each pass one kernel with an outgoing-edge loop
 //             (owner terms, weight and offset cotangents) and an incoming-
-//             edge loop (neighbour terms);
-//   geometry  least-squares weight cotangents back to edge offsets
+//             edge loop (neighbour terms; FP64: in blocks of their own);
+//   state     q_bar to U_bar through the E13 Jacobian;
+//   geometry  once per product, and only if coordinate cotangents are asked
+//             for: least-squares weight cotangents back to edge offsets
 //             (a = M^-1 d with M = sum d d^T gives d_bar_k = b_k - B d_k,
 //             b = M^-1 a_bar, B = sum (b a^T + a b^T)), then offsets to
-//             points by one more gather;
-//   state     q_bar to U_bar through the E13 Jacobian.
+//             points by one more gather.
 #include <cub/cub.cuh>
 #include <type_traits>
 

@@ -8,7 +8,7 @@
 // and two adds, 3-4 cycles instead of 16, and keeps 60 bits where a double
 // keeps 53. The result is rounded to a double once per component. The flux
 // launch went from 178 to 50 FP64 warp instructions per edge and from 6.82 to
-// 2.26 ms at 2.5 million points (second order, RK4), its error against multiple
+// 2.22 ms at 2.5 million points (second order, RK4), its error against multiple
 // precision is 2-8 times below that of the FP64 chain.
 //
 // With r = beta^(-1/2), S_t = u.t sqrt(beta), S_n likewise, every flux is a
@@ -25,8 +25,8 @@
 //
 // Taken when fix_state says so: beta in [2^-40, 2^40), S_t^2 + S_n^2 < 15.875
 // with each component of sqrt(beta) (u, v) below 3.9375 (Mach 4.7), |q1| < 32,
-// i.e. every state such flows meet; the FP64 form takes the others. The same code compiles on the host, where it is tested against
-// multiple precision.
+// i.e. every state such flows meet; the FP64 form takes the others. The same
+// code compiles on the host, where it is tested against multiple precision.
 #pragma once
 
 #include <cstdint>
