@@ -805,6 +805,58 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather(AdjParamsT<T> P)
     if (second) st8(P.gbar, p, gb);
 }
 
+// the same in FP64 for small clouds (order 2, with the offsets' cotangents): two
+// lanes per point, two components each, of which one adds to the offset's x and
+// one to its y. A point's incoming edges are a serial chain of dependent loads
+// and FP64 sums: 37 -> 28 us at 40k points. At 640k the one-lane form's 0.27 ms
+// is already bound by the FP64 pipe (87 %).
+__global__ void __launch_bounds__(128) k_adj_flux_gather_pair(AdjParams P)
+{
+    const int64_t n = P.g.n, pp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 1;
+    const int l = threadIdx.x & 1, k0 = 2 * l;
+    const bool live = pp < n;
+    const int64_t p = live ? pp : n - 1;   // (lanes past the end take part in the shuffles)
+    double qb[2], gx[2], gy[2], px[2], py[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        qb[k] = P.qbar[4 * p + k0 + k];
+        gx[k] = P.gbar[8 * p + k0 + k];
+        gy[k] = P.gbar[8 * p + 4 + k0 + k];
+    }
+    gather_c<2>(P.qg + 8 * p + k0, px);
+    gather_c<2>(P.qg + 8 * p + 4 + k0, py);
+    const int t0 = P.toff[p], deg = live ? P.toff[p + 1] - t0 : 0;
+    const int most = __reduce_max_sync(0xffffffffu, deg);
+#pragma unroll 1
+    for (int j = 0; j < most; ++j) {
+        double dx = 0.0, dy = 0.0;
+        int e = 0;
+        if (j < deg) {
+            e = P.tedge[t0 + j];
+            const double2 h = __ldg(P.thd + t0 + j);
+            const double2 eb = *reinterpret_cast<const double2 *>(P.ebar + 4 * (int64_t)e + k0);
+            qb[0] += eb.x;
+            qb[1] += eb.y;
+            // q~_p = q_p - h.grad q_p on this edge
+            gx[0] = fma(-h.x, eb.x, gx[0]);
+            gx[1] = fma(-h.x, eb.y, gx[1]);
+            gy[0] = fma(-h.y, eb.x, gy[0]);
+            gy[1] = fma(-h.y, eb.y, gy[1]);
+            dx = fma(eb.y, px[1], eb.x * px[0]);
+            dy = fma(eb.y, py[1], eb.x * py[0]);
+        }
+        const double d = (l ? dy : dx) + __shfl_xor_sync(0xffffffffu, l ? dx : dy, 1);
+        if (j < deg) {
+            double *o = reinterpret_cast<double *>(P.dbar + e) + l;
+            *o = fma(-0.5, d, *o);
+        }
+    }
+    if (!live) return;
+    store_c<2>(P.qbar + 4 * p + k0, qb);
+    store_c<2>(P.gbar + 8 * p + k0, gx);
+    store_c<2>(P.gbar + 8 * p + 4 + k0, gy);
+}
+
 // ---------------------------------------------------------------------------
 // one least-squares pass of E15 in reverse. Forward (per component c):
 //   g_p = sum_e a_e s_e,  s_e = (q_i - q_p) - [dx (gx'_i - gx'_p) + dy (gy'_i - gy'_p)]/2
@@ -1451,7 +1503,12 @@ __global__ void __launch_bounds__(256) k_adj_points(AdjParams P, const double2 *
 // q_bar to U_bar through E13, adds into Ub_acc ([n][4], internal order). With
 // p = (gamma-1) (E - m^2/(2 rho)), m^2 = m1^2 + m2^2 and g = 1/(gamma-1):
 //   q1 = ln rho + g ln(rho/(2p)) - m^2/(2 rho p), q2 = m1/p, q3 = m2/p, q4 = -rho/p,
-// in reverse by hand (40 FP64 operations and two quotients per point)
+// in reverse by hand (45 FP64 operations and two reciprocals per point)
+// 1/x by the integer pipes, within 2^-59 before the rounding; extreme x divide.
+// (k_adj_state, bound by the FP64 pipe, with two of them and 1/inv_gm1 from the
+// host: 71 -> 52 us at 640k points)
+__device__ __forceinline__ double reciprocal(double x) { return fix_moderate(x) ? fix_reciprocal(x) : 1.0 / x; }
+
 template <class T>
 __global__ void __launch_bounds__(256) k_adj_state(AdjParamsT<T> P, const double *__restrict__ U,
                                                    double *__restrict__ Ub_acc)
@@ -1471,10 +1528,10 @@ __global__ void __launch_bounds__(256) k_adj_state(AdjParamsT<T> P, const double
         for (int k = 0; k < 4; ++k) qb[k] += to_f64(qt[k]);
     }
     ld4(Ub_acc, p, ub);
-    const double g = P.inv_gm1, gm1 = 1.0 / g;
-    const double ir = 1.0 / u[0], m1 = u[1] * ir, m2 = u[2] * ir;            // velocities
+    const double g = P.inv_gm1, gm1 = P.gm1;
+    const double ir = reciprocal(u[0]), m1 = u[1] * ir, m2 = u[2] * ir;            // velocities
     const double ke = 0.5 * (u[1] * m1 + u[2] * m2);                          // m^2/(2 rho)
-    const double pr = gm1 * (u[3] - ke), ip = 1.0 / pr;
+    const double pr = gm1 * (u[3] - ke), ip = reciprocal(pr);
     const double kp = ke * ip;                                                // m^2/(2 rho p)
     // cotangents at fixed p, and that of p
     const double rb = qb[0] * ir * (1.0 + g + kp) - qb[3] * ip;
@@ -1641,6 +1698,12 @@ cudaError_t launch_adj_flux(const AdjParamsT<T> &P, bool geom, cudaStream_t s)
     if (!pair && !geom) k_adj_flux<T, false><<<nb, 128, 0, s>>>(P);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
+    if constexpr (std::is_same<T, double>::value) {
+        if (geom && P.order == 2 && P.g.n < 60000) {
+            k_adj_flux_gather_pair<<<blocks(P.g.n, 64), 128, 0, s>>>(P);
+            return cudaGetLastError();
+        }
+    }
     if (geom) k_adj_flux_gather<T, true><<<nb, 128, 0, s>>>(P);
     else k_adj_flux_gather<T, false><<<nb, 128, 0, s>>>(P);
     return cudaGetLastError();

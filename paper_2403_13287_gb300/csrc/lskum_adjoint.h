@@ -37,7 +37,7 @@ struct AdjParamsT {
     const float2 *ea;
     const float4 *tf;
     const int32_t *perm;   // internal point -> input point
-    double inv_gm1;
+    double inv_gm1, gm1;
     int g14;               // gamma == 1.4: beta^(-1/(gamma-1)) = beta^-2.5 (as the forward kernels)
     int order;
     int add;               // wbar and abar add to an earlier residual's of this product (else they start here)

@@ -1451,6 +1451,7 @@ static AdjParams adj_params(lskum_ctx *c, const lskum_ctx::Forward &f)
     P.near_u = c->near_u;
     P.perm = c->perm;
     P.inv_gm1 = c->gas.inv_gm1;
+    P.gm1 = 1.0 / c->gas.inv_gm1;
     P.g14 = c->gas.g14;
     P.order = c->cfg.order;
     return P;
@@ -1566,6 +1567,7 @@ static lskum_status vjp_residual_fp32(lskum_ctx *c, const double *Ui, double *Ub
     P.tf = c->ftf;
     P.perm = Pd.perm;
     P.inv_gm1 = Pd.inv_gm1;
+    P.gm1 = Pd.gm1;
     P.g14 = Pd.g14;
     P.order = Pd.order;
     c->launches++;
