@@ -7,8 +7,8 @@
 // full. A 64 x 64 product keeping the high word costs three wide multiply-adds
 // and two adds, 3-4 cycles instead of 16, and keeps 60 bits where a double
 // keeps 53. The result is rounded to a double once per component. The flux
-// launch went from 178 to 50 FP64 warp instructions per edge and from 6.82 to
-// 2.22 ms at 2.5 million points (second order, RK4), its error against multiple
+// launch went from 178 to 40 FP64 instructions per edge and from 6.82 to
+// 2.14 ms at 2.5 million points (second order, RK4), its error against multiple
 // precision is 2-8 times below that of the FP64 chain.
 //
 // With r = beta^(-1/2), S_t = u.t sqrt(beta), S_n likewise, every flux is a

@@ -484,28 +484,24 @@ __device__ __forceinline__ void state_update(const FluxParams &P, int64_t p, boo
 struct Vec4 {
     double v[4];
 };
-struct FluxDifference {
-    double d[4];
+struct StateFluxes {
+    double t[4], n[4];   // [mass, along, transverse, energy]
     bool ok;
 };
 
-// G(q~_i) - G(q~_0) along t or n, [mass, along, transverse, energy], in FP64:
-// for states outside the fixed-point form's ranges. Not inlined: it keeps its
-// registers out of the loop that hardly ever calls it. The difference is an
-// unfused subtraction of the two rounded fluxes, so equal states give exactly
-// zero (a contracted fma(rho_i, m_i, -rho_0 m_0) would leave a product's rounding).
-__device__ __noinline__ FluxDifference flux_difference_fp64(Vec4 qi, Vec4 q0, bool along_t, unsigned long long sbit,
-                                                            double2 n0, Gas gas)
+// both directions' split fluxes of one state in FP64, for members outside the
+// fixed-point form's ranges: each lane of a pair takes its own state, as there
+// (a residual of 160k points all at Mach 7: 0.88 ms with both states in each
+// lane, 0.71 ms so). Not inlined: it keeps its registers out of the loop that
+// hardly ever calls it.
+__device__ __noinline__ StateFluxes state_fluxes_fp64(Vec4 q, unsigned long long st, unsigned long long sn, double2 n0,
+                                                      Gas gas)
 {
-    FluxDifference o = {{0.0, 0.0, 0.0, 0.0}, true};
-    Prim si, s0;
-    o.ok &= prim_from_q(qi.v, gas, n0.y, -n0.x, n0, si);
-    o.ok &= prim_from_q(q0.v, gas, n0.y, -n0.x, n0, s0);
-    double Gi[4], G0[4];
-    split_flux(sbit, si, along_t ? si.us : si.un, along_t ? si.un : si.us, along_t ? si.Ss : si.Sn, Gi);
-    split_flux(sbit, s0, along_t ? s0.us : s0.un, along_t ? s0.un : s0.us, along_t ? s0.Ss : s0.Sn, G0);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) o.d[k] = __dsub_rn(Gi[k], G0[k]);
+    StateFluxes o;
+    Prim s;
+    o.ok = prim_from_q(q.v, gas, n0.y, -n0.x, n0, s);
+    split_flux(st, s, s.us, s.un, s.Ss, o.t);
+    split_flux(sn, s, s.un, s.us, s.Sn, o.n);
     return o;
 }
 
@@ -621,21 +617,26 @@ __device__ __forceinline__ void member_difference(bool act, int l, const double 
     }
     const bool slow = differ && !fixed;
     if (__any_sync(0xffffffffu, slow)) {
-        Vec4 qi, q0;
+        StateFluxes f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) f.t[k] = f.n[k] = 0.0;
+        if (slow) {
+            Vec4 q;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) q.v[k] = qt[k];
+            f = state_fluxes_fp64(q, xp ? 0ull : kSignBit, yp ? 0ull : kSignBit, n0, gas);
+            ok &= f.ok;
+        }
+        // an unfused subtraction of the two rounded fluxes, so equal states give
+        // exactly zero (a contracted fma(rho_i, m_i, -rho_0 m_0) would leave a
+        // product's rounding); a direction of weight zero adds nothing, whatever
+        // its difference
+        const bool use = slow && (__double_as_longlong(l ? w.y : w.x) & ~(long long)kSignBit) != 0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const double r = other_lane(qt[k]);
-            qi.v[k] = l ? r : qt[k];
-            q0.v[k] = l ? qt[k] : r;
-        }
-        if (slow) {
-            const FluxDifference f = flux_difference_fp64(qi, q0, l == 0, sbit, n0, gas);
-            // (a direction of weight zero adds nothing, whatever its difference)
-            if ((__double_as_longlong(l ? w.y : w.x) & ~(long long)kSignBit) != 0) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) d[k] = f.d[k];
-            }
-            ok &= f.ok;
+            const double r = other_lane(l ? f.t[k] : f.n[k]);
+            const double v = l ? __dsub_rn(r, f.n[k]) : __dsub_rn(f.t[k], r);
+            if (use) d[k] = v;
         }
     }
 }
@@ -701,7 +702,7 @@ struct Members {
 // the sums, the state update), the integer multipliers (63 %) and ALUs (57 %),
 // 66 % of the issue slots; at a few thousand points one warp's chain of rounds.
 // 64 registers and a few spills, for 32 warps per SM, beat 80 (24 warps) and 128
-// (16): 2.22 ms at 2.5 million points, before the last changes 2.30 / 2.48 / 2.67.
+// (16): 2.14 ms at 2.5 million points, before the last changes 2.30 / 2.48 / 2.67.
 // One lane per member with both states took 2.58 ms and a chain twice as long.
 // Two lanes per member (member_difference), PAIRS pairs of lanes per point. With
 // one pair the members of a row follow one another; with 2 or 4 each pair takes
