@@ -698,8 +698,8 @@ struct Members {
     }
 };
 
-// What bounds it at large sizes: the FP64 pipe (65 % busy: the reconstruction,
-// the sums, the state update), the integer multipliers (63 %) and ALUs (57 %),
+// What bounds it at large sizes: the FP64 pipe (68 % busy: the reconstruction,
+// the sums, the state update), the integer multipliers (62 %) and ALUs (58 %),
 // 66 % of the issue slots; at a few thousand points one warp's chain of rounds.
 // 64 registers and a few spills, for 32 warps per SM, beat 80 (24 warps) and 128
 // (16): 2.14 ms at 2.5 million points, before the last changes 2.30 / 2.48 / 2.67.
