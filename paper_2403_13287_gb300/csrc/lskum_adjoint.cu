@@ -970,7 +970,7 @@ __global__ void __launch_bounds__(128) k_adj_grad_fp32(AdjParamsT<float> P, cons
 __device__ __forceinline__ double dot2(const FixPair &a, const FixPair &b, double ax, double ay, double bx, double by)
 {
     if (fix_dot_in_range(a, b)) return fix_dot(a, b);
-    return b.e ? fma(ay, by, ax * bx) : 0.0;   // both terms zero (or subnormal): nothing to add
+    return fix_pair_zero(b) ? 0.0 : fma(ay, by, ax * bx);   // both terms zero (or subnormal): nothing to add
 }
 
 template <bool GEOM, int LANES>

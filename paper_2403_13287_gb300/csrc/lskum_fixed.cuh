@@ -338,65 +338,73 @@ LSKUM_FIX_FN void fix_scale(FixOp c0, FixOp c1, FixOp c3, int64_t F[4])
 }
 
 // --- the q-derivative passes' parts ------------------------------------------
-// Two doubles with one exponent: x = X 2^(e-1084), X the op's value, |X| < 2^62.
+// Two doubles, each with an exponent of its own: x = X 2^(ex-1084), 2^61 <= |X| <
+// 2^62 the op's value; a zero (or subnormal) component is X = 0 with an exponent
+// below all others, so that the other one alone sets a product's scale. (One
+// exponent for both, the larger one's, was 60 bits of the vector's size but not of
+// a small component: a stencil stretched A : 1 lost log2(A) bits of h . g where the
+// gradient runs across it, 8.8e-14 of |h.x g.x| + |h.y g.y| at 1000 : 1.)
+constexpr int kFixZeroExponent = -8192;
 struct FixPair {
     FixOp x, y;
-    int e;   // the larger biased exponent (0: both zero or subnormal, 0x7ff: not finite)
+    int ex, ey;   // biased exponents (0x7ff: not finite)
 };
 template <int Q>
-LSKUM_FIX_FN int64_t fix_mantissa(int64_t b, int drop)   // 1.xx in Q60 or Q61, signed, shifted right
+LSKUM_FIX_FN int64_t fix_mantissa(int64_t b)   // 1.xx in Q<Q>, signed
 {
-    const int64_t m = (((b & 0xfffffffffffffll) | 0x10000000000000ll) << (Q - 52)) >> fix_min(drop, 63);
-    return fix_flip(m, b >> 63);
+    return fix_flip(((b & 0xfffffffffffffll) | 0x10000000000000ll) << (Q - 52), b >> 63);
 }
 LSKUM_FIX_FN FixPair fix_pair(double x, double y)
 {
     const int64_t bx = fix_bits(x), by = fix_bits(y);
     const int ex = (int)(bx >> 52) & 0x7ff, ey = (int)(by >> 52) & 0x7ff;
     FixPair p;
-    p.e = fix_max(ex, ey);
-    // a zero beside a finite number is shifted out: its exponent field is 0
-    p.x = fix_op(ex ? fix_mantissa<61>(bx, p.e - ex) : 0);
-    p.y = fix_op(ey ? fix_mantissa<61>(by, p.e - ey) : 0);
+    p.ex = ex ? ex : kFixZeroExponent;
+    p.ey = ey ? ey : kFixZeroExponent;
+    p.x = fix_op(ex ? fix_mantissa<61>(bx) : 0);
+    p.y = fix_op(ey ? fix_mantissa<61>(by) : 0);
     return p;
 }
-// A pair with its exponent in the low bits of the two words, 4 each: e - 895
-// (1..255, |x|, |y| up to 2^127 and the larger at least 2^-127); 0 where it
-// does not fit. The bits given up are below 2^-57 of the larger.
+// both components zero (or subnormal)
+LSKUM_FIX_FN bool fix_pair_zero(const FixPair &p) { return fix_max(p.ex, p.ey) < 0; }
+// A pair without loss in two words: a component's 53 bits leave the word's low 9
+// to its exponent, e - 639 (1..511; 0 beside a zero). Both words 0 where the pair
+// does not fit: the larger component outside 2^-127..2^128, the smaller one not
+// zero and below 2^-383.
 LSKUM_FIX_FN void fix_pack_pair(double x, double y, int64_t &wx, int64_t &wy)
 {
     const FixPair p = fix_pair(x, y);
-    const int e = p.e - 895;
-    const bool fits = e >= 1 && e <= 255;
-    wx = fits ? (fix_value(p.x) & ~15ll) | (e & 15) : 0;
-    wy = fits ? (fix_value(p.y) & ~15ll) | (e >> 4) : 0;
+    const int e = fix_max(p.ex, p.ey) - 895;
+    const int cx = p.ex < 0 ? 0 : p.ex - 639, cy = p.ey < 0 ? 0 : p.ey - 639;
+    const bool fits = e >= 1 && e <= 255 && (cx > 0 || p.ex < 0) && (cy > 0 || p.ey < 0);
+    wx = fits ? fix_value(p.x) | cx : 0;
+    wy = fits ? fix_value(p.y) | cy : 0;
 }
 LSKUM_FIX_FN FixPair fix_unpack_pair(int64_t wx, int64_t wy)
 {
     FixPair p;
-    const int e = ((int)wx & 15) | (((int)wy & 15) << 4);
-    p.e = e ? e + 895 : 0x7ff;   // 0x7ff: fix_dot_in_range refuses it
-    p.x = fix_op(wx & ~15ll);
-    p.y = fix_op(wy & ~15ll);
+    const int cx = (int)wx & 511, cy = (int)wy & 511;
+    p.ex = cx ? cx + 639 : kFixZeroExponent;
+    p.ey = cy ? cy + 639 : kFixZeroExponent;
+    p.x = fix_op(wx & ~511ll);
+    p.y = fix_op(wy & ~511ll);
     return p;
 }
 // the exponents of h and g for which fix_dot's result is a normal number: away
 // from both ends by the 60 bits that a cancelling sum may lose
 LSKUM_FIX_FN bool fix_dot_in_range(const FixPair &h, const FixPair &g)
 {
-    return (unsigned)(h.e + g.e - 1100) < 1900u && fix_max(h.e, g.e) < 0x7ff;
+    const int e = fix_max(h.ex + g.ex, h.ey + g.ey);
+    return (unsigned)(e - 1100) < 1900u && fix_max(fix_max(h.ex, h.ey), fix_max(g.ex, g.ey)) < 0x7ff;
 }
-// h.x g.x + h.y g.y, rounded once (2^-56 of |h||g| before the rounding; the
-// cross sum stays below 2^63: four times (2^30 - 1) 2^31)
+// h.x g.x + h.y g.y, rounded once: each product within 1.25 units of 2^-58 of
+// itself, the smaller one shifted to the larger one's exponent (a unit more), so
+// 2^-56 of the larger product before the rounding
 LSKUM_FIX_FN double fix_dot(const FixPair &h, const FixPair &g)
 {
-    int64_t m = (int64_t)h.x.hi * g.x.lo;
-    m += (int64_t)h.x.lo * g.x.hi;
-    m += (int64_t)h.y.hi * g.y.lo;
-    m += (int64_t)h.y.lo * g.y.hi;
-    int64_t c = (int64_t)h.x.hi * g.x.hi + (m >> 32);
-    c += (int64_t)h.y.hi * g.y.hi;
-    return fix_to_double(c, h.e + g.e - 2104);
+    const int a = h.ex + g.ex, b = h.ey + g.ey, e = fix_max(a, b);
+    const int64_t c = (fix_mul(h.x, g.x) >> fix_min(e - a, 63)) + (fix_mul(h.y, g.y) >> fix_min(e - b, 63));
+    return fix_to_double(c, e - 2104);
 }
 
 // round(2^22 / f) within a unit or so, f the float with these bits in [1, 2)
@@ -443,11 +451,11 @@ LSKUM_FIX_FN double fix_phi(double x, double d, double eps2)
     const int64_t bx = fix_bits(x), bd = fix_bits(d), be = fix_bits(eps2);
     const int ex = (int)(bx >> 52), ed = (int)(bd >> 52), ee = (int)(be >> 52);
     const int p = fix_max(ed, 1023 + ((ee - 1022) >> 1));          // biased exponent of the scale
-    const int64_t X = ex ? fix_mantissa<60>(bx, 0) : 0;             // x = X 2^(ex - p), 1.xx in Q60
+    const int64_t X = ex ? fix_mantissa<60>(bx) : 0;             // x = X 2^(ex - p), 1.xx in Q60
     const int ux = ex ? ex - p : -4096, ue = ee ? ee + 1023 - 2 * p : -4096;   // ux <= 1, ue <= 0
     const int64_t xs = X >> fix_min(1 - ux, 63);                    // x < 4 in Q59
-    const int64_t ds = fix_mantissa<60>(bd, p - ed + 1);            // d < 2 in Q59
-    const int64_t E = ee ? fix_mantissa<57>(be, 0) : 0;             // eps2 = E 2^ue, 1.xx in Q57
+    const int64_t ds = fix_mantissa<60>(bd) >> fix_min(p - ed + 1, 63);            // d < 2 in Q59
+    const int64_t E = ee ? fix_mantissa<57>(be) : 0;             // eps2 = E 2^ue, 1.xx in Q57
     const int64_t T = fix_mul_s<2>(fix_op(X), fix_op(xs + 2 * ds)); // x (x + 2d) = T 2^ux, T < 16 in Q57
     const int un = fix_max(ux, ue);
     const int64_t N = (T >> fix_min(un - ux, 63)) + (E >> fix_min(un - ue, 63));   // Q57, times 2^un
@@ -480,7 +488,7 @@ LSKUM_FIX_FN bool fix_moderate(double x) { return (uint64_t)fix_bits(x) - (700ul
 LSKUM_FIX_FN double fix_reciprocal(double x)
 {
     const int64_t b = fix_bits(x);
-    return fix_to_double(fix_rcp(fix_mantissa<61>(b, 0)), 1023 - 62 - (int)(b >> 52));
+    return fix_to_double(fix_rcp(fix_mantissa<61>(b)), 1023 - 62 - (int)(b >> 52));
 }
 
 // log2 of a positive normal x's mantissa in Q60, [0, 1)

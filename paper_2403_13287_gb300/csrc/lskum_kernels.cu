@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(128) k_qgrad(DevGeom g, const double *__restri
                 double c = 0.0;
                 if (fix_dot_in_range(hp, gp)) {
                     c = fix_dot(hp, gp);
-                } else if (gp.e) {
+                } else if (!fix_pair_zero(gp)) {
                     const double2 h = half_offset(e, i);
                     c = fma(h.y, gy[k], h.x * gx[k]);
                 }
