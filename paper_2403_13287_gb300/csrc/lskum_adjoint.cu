@@ -1297,19 +1297,22 @@ __global__ void __launch_bounds__(128) k_adj_limit_gather(AdjParams P, const int
 // ---------------------------------------------------------------------------
 // least-squares weights back to edge offsets (owner side). A system with
 // M = sum d d^T and weights a = M^-1 d gives
-//   d_bar_k = b_k - B d_k,  b = M^-1 a_bar,  B = sum (b a^T + a b^T)
-//           = M^-1 [sum (a_bar d^T + d a_bar^T)] M^-1.
-// Full stencil: a_bar = abar. A sub-stencil takes one row of M^-1 d (frame
-// (s, n)) as its weight, so a_bar is the weight's cotangent wb along that row,
-// b = wb beta with beta the row of M^-1, A = M^-1 sum wb d and B = beta A^T + A beta^T.
+//   d_bar_k = b_k - B d_k,  b = M^-1 a_bar,  B = sum (b a^T + a b^T).
+// Full stencil: a_bar = abar, and with C = sum a_bar a^T over the forward's own
+// weights B = M^-1 C + (M^-1 C)^T. (S = sum (a_bar d^T + d a_bar^T) and B = M^-1 S M^-1
+// has the same count of operations but takes S through M^-1 twice: on a stencil
+// stretched 1000 : 1 across both axes y_bar was 3e-9 off where the forward's
+// conditioning gives 4e-11.) A sub-stencil takes one row of M^-1 d (frame (s, n)) as
+// its weight, so a_bar is the weight's cotangent wb along that row, b = wb beta
+// with beta the row of M^-1, A = M^-1 sum wb d and B = beta A^T + A beta^T.
 //
 // All M^-1 depend on the points alone: k_adj_plan forms them once per context,
-// so a product needs one pass for S = sum a_bar d^T and the D = sum wb d, and
-// one for the offsets' cotangents, with the B of an edge's two sub-stencils
-// added up first: 39 FP64 instructions per edge (half offsets h where they are
-// stored: S and D take them, B is doubled instead). The sub-stencils stay in the
-// frame that their weights were solved in: b and B d nearly cancel for a thin
-// sub-stencil, and B turned to global axes lost seven digits there. 94 -> 63 us at 40k points, 823 -> 502 us at 640k.
+// so a product needs one pass for C and the D = sum wb d, and one for the
+// offsets' cotangents, with the B of an edge's two sub-stencils added up first:
+// 39 FP64 instructions per edge (half offsets h where they are stored: D takes
+// them, B is doubled instead). The sub-stencils stay in the frame that their
+// weights were solved in: b and B d nearly cancel for a thin sub-stencil, and B
+// turned to global axes lost seven digits there. 94 -> 63 us at 40k points, 823 -> 502 us at 640k.
 // ---------------------------------------------------------------------------
 struct Sym2 {
     double xx, xy, yy;
@@ -1419,17 +1422,18 @@ __global__ void __launch_bounds__(128) k_adj_weights(AdjParams P)
     if (!g.hd) xy0 = g.xy[p];
     const double2 n0 = g.nrm[p];
     const int e0 = g.off[p], e1 = g.off[p + 1];
-    Sym2 S = {0, 0, 0};
-    double2 D0 = make_double2(0.0, 0.0), D1 = D0, D2 = D0, D3 = D0;
+    double2 C0 = make_double2(0.0, 0.0), C1 = C0;   // rows of C = sum a_bar a^T
+    double2 D0 = C0, D1 = C0, D2 = C0, D3 = C0;
     for (int e = e0; e < e1; ++e) {
         const double2 h = half_offset(g, e, xy0), t = in_frame(h, n0);
         const int ks = xsub(g.mask[e]), kn = ysub(g.mask[e]);
         const double2 wb = P.wbar[e];
         if (full) {
-            const double2 ab = P.abar[e];
-            S.xx = fma(ab.x, h.x, S.xx);                          // half the diagonal
-            S.xy = fma(ab.x, h.y, fma(ab.y, h.x, S.xy));
-            S.yy = fma(ab.y, h.y, S.yy);
+            const double2 ab = P.abar[e], a = g.lsw[e];
+            C0.x = fma(ab.x, a.x, C0.x);
+            C0.y = fma(ab.x, a.y, C0.y);
+            C1.x = fma(ab.y, a.x, C1.x);
+            C1.y = fma(ab.y, a.y, C1.y);
         }
         add_to(ks == 0, ks == 1, wb.x, t, D0, D1);
         add_to(kn == 2, kn == 3, wb.y, t, D2, D3);
@@ -1439,10 +1443,9 @@ __global__ void __launch_bounds__(128) k_adj_weights(AdjParams P)
     Sym2 Mi = {0, 0, 0}, B = {0, 0, 0};
     if (full) {
         Mi = Sym2{pl[0], pl[n], pl[2 * n]};
-        // B = Mi S Mi, S with its diagonal doubled; 2 B of S / 2
-        const double2 c0 = times(Mi, make_double2(8.0 * S.xx, 4.0 * S.xy)), c1 = times(Mi, make_double2(4.0 * S.xy, 8.0 * S.yy));
-        const double2 b0 = times(Mi, make_double2(c0.x, c1.x)), b1 = times(Mi, make_double2(c0.y, c1.y));
-        B = Sym2{b0.x, b0.y, b1.y};
+        // 2 B = 2 (Mi C + (Mi C)^T), for half offsets
+        const double2 b0 = times(Mi, make_double2(C0.x, C1.x)), b1 = times(Mi, make_double2(C0.y, C1.y));   // columns of Mi C
+        B = Sym2{4.0 * b0.x, 2.0 * (b0.y + b1.x), 4.0 * b1.y};
     }
     double2 beta0, beta1, beta2, beta3;
     const Sym2 B0 = sub_back(pl + 3 * n, n, D0, 0, beta0), B1 = sub_back(pl + 6 * n, n, D1, 0, beta1);

@@ -97,6 +97,15 @@ def thin_state(cloud, stretch, seed, amp=0.1):
     return np.ascontiguousarray(np.stack([rho, rho * u, rho * v, p / 0.4 + 0.5 * rho * (u * u + v * v)]))
 
 
+def turned(cloud, U, angle):
+    """The cloud with its normals and the state's momentum turned by -angle."""
+    c, s = np.cos(angle), np.sin(angle)
+    out = dict(cloud)
+    out["x"], out["y"] = cloud["x"] * c + cloud["y"] * s, cloud["y"] * c - cloud["x"] * s
+    out["nx"], out["ny"] = cloud["nx"] * c + cloud["ny"] * s, cloud["ny"] * c - cloud["nx"] * s
+    return out, np.ascontiguousarray(np.stack([U[0], U[1] * c + U[2] * s, U[2] * c - U[1] * s, U[3]]))
+
+
 def extended_q_derivatives(cloud, U, inner):
     """E13-E15 in numpy's extended precision, and the size of the summands."""
     T = np.longdouble
@@ -172,3 +181,32 @@ def test_products_of_a_stretched_cloud(limiter):
     for kind in "Uy":
         k = [i for i, e in enumerate(ent) if e[0] == kind]
         assert np.all(np.abs(got - want)[k] <= 1e-10 * np.abs(want[k]).max())
+
+
+@pytest.mark.gpu
+def test_products_of_a_stretched_cloud_across_both_axes():
+    """Stretched A = 4096 : 1 at half a radian to the axes. The determinants of the
+    closed 2 x 2 solves cancel to A^-2 of their products, so weights, and sums of
+    them, carry a few units of 2^-53 A^2 on either side: 16 of them of the largest
+    entry."""
+    import torch
+
+    import oracle
+    from oracle import lskum_jvp
+    from paper_2403_13287_gb300.lskum import Solver
+    A = 4096.0
+    c = thin_cloud(31, 29, A, seed=3)
+    c, U = turned(c, thin_state(c, A, seed=5), 0.5)
+    n = c["n"]
+    rng = np.random.default_rng(2)
+    Rb = rng.standard_normal((4, n))
+    s = Solver(c, order=2, inner_iters=2, mach=0.5, aoa_deg=0.0)
+    Ub, xb, yb = (t.cpu().numpy() for t in s.residual_vjp(torch.from_numpy(Rb).cuda(), torch.from_numpy(U).cuda()))
+    s.close()
+    ent = [("U", int(rng.integers(4)), int(k)) for k in rng.choice(n, 20, replace=False)]
+    ent += [(d, int(k)) for d in "xy" for k in rng.choice(n, 30, replace=False)]
+    want = lskum_jvp.vjp_entries(c, oracle.split_stencils(c), U, Rb, ent, order=2, inner=2)
+    got = np.array([Ub[e[1], e[2]] if e[0] == "U" else (xb if e[0] == "x" else yb)[e[1]] for e in ent])
+    for kind in "Uxy":
+        k = [i for i, e in enumerate(ent) if e[0] == kind]
+        assert np.all(np.abs(got - want)[k] <= 16 * A * A * 2.0 ** -53 * np.abs(want[k]).max()), kind
