@@ -668,9 +668,13 @@ __global__ void __launch_bounds__(128, 5) k_adj_flux_pair(AdjParams P)
         }
         FixState s;
         if (fix_state(qt, fnx, fny, s)) {
-            const double St = fix_to_double(s.St, -61), Sn = fix_to_double(s.Sn, -61), H = fix_to_double(s.H, -59);
+            double St = fix_to_double(s.St, -61), Sn = fix_to_double(s.Sn, -61);
+            const double H = fix_to_double(s.H, -59);
             const double C0 = fix_to_double(s.c0, fix_e0(s.n, s.k)), C1 = fix_to_double(s.c1, fix_e1(s.n, s.k)),
                          C3 = fix_to_double(s.c3, fix_e3(s.n, s.k)), hr = fix_to_double(s.r, -62 - s.k);
+            // (as in the forward: a small one in FP64)
+            if (fix_slow(s.St)) St = fma(qt[1], tx, qt[2] * ty) * hr;
+            if (fix_slow(s.Sn)) Sn = fma(qt[1], n0.x, qt[2] * n0.y) * hr;
             const DirCotangent a = direction_cotangent(s, true, (m & M_XPOS) ? 0ull : kSignBit, St, Sn, H, C0, C1, C3,
                                                        Rb[0], Rs, Rn, Rb[3], w.x);
             const DirCotangent b = direction_cotangent(s, false, (m & M_YPOS) ? 0ull : kSignBit, Sn, St, H, C0, C1, C3,

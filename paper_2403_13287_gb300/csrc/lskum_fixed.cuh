@@ -264,6 +264,12 @@ LSKUM_FIX_FN bool fix_state(const double q[4], FixOp nx, FixOp ny, FixState &s)
     return ok;
 }
 
+// |S| below 2^-7, S in Q61. The formats leave S, and with it a transverse momentum
+// flux, 2^-57.6 of the flux's scale rho r^2 (rms, measured); products in FP64
+// carry about 2^-52.5 |S_o| instead, less from here on, which counts where one
+// direction's weights are far above the other's (slow gas in a thin stencil).
+LSKUM_FIX_FN bool fix_slow(int64_t S) { return (uint32_t)((int32_t)(S >> 32) + (1 << 22)) < (1u << 23); }
+
 // c 2^e, c below 2^62, against another factor's exponent eo: c at the larger of
 // the two (es)
 LSKUM_FIX_FN int64_t fix_align_half(int64_t c, int e, int eo, int &es)

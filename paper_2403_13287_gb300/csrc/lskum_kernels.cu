@@ -554,6 +554,14 @@ __device__ __forceinline__ double other_lane(double v)
     return __longlong_as_double(other_lane((int64_t)__double_as_longlong(v)));
 }
 
+// (u.t, u.n) of a q-vector, u = -(q2, q3)/q4. Not inlined: hardly ever needed, and
+// the loop that calls it has no registers to spare
+__device__ __noinline__ double2 frame_velocity(double q2, double q3, double q4, double2 n0)
+{
+    const double r = -1.0 / q4;
+    return make_double2(fma(q2, n0.y, -(q3 * n0.x)) * r, fma(q2, n0.x, q3 * n0.y) * r);
+}
+
 // One member of a point's stencil, evaluated by two neighbouring lanes: lane 0
 // holds the neighbour's reconstructed state, lane 1 the point's own one (qt).
 // Each turns its state into fixed point and forms the products c F of both
@@ -585,8 +593,10 @@ __device__ __forceinline__ void member_difference(bool act, int l, const double 
     const unsigned long long sbit = (l ? yp : xp) ? 0ull : kSignBit;   // of this lane's direction
     FixState s;
     bool fixed = fix_state(qt, nx, ny, s);
-    const uint32_t other_fixed = other_lane((uint32_t)fixed);
-    fixed = fixed && other_fixed != 0;
+    // (bit 0: in range; bits 1 and 2: slow along t and along n)
+    const uint32_t mine = (fixed ? 1u : 0u) | (fix_slow(s.St) ? 2u : 0u) | (fix_slow(s.Sn) ? 4u : 0u);
+    const uint32_t both = mine & other_lane(mine);
+    fixed = (both & 1u) != 0;
     if (__any_sync(0xffffffffu, differ && fixed)) {
         if (!fixed) s.St = s.Sn = 0;   // an index of the tables; the result is not used
         // the two states' factors at common exponents
@@ -607,12 +617,23 @@ __device__ __forceinline__ void member_difference(bool act, int l, const double 
         // lane 0: G_t(neighbour) - G_t(own), lane 1: G_n(neighbour) - G_n(own);
         // the products lack the factor sgn of components 0, 2 and 3
         const bool use = differ && fixed;
+        // both transverse velocities small: that momentum's flux as velocity times
+        // mass flux in FP64 (fix_slow says why; a step of 2.5 million points 16.10 ->
+        // 16.27 ms, and 16.41 with this after the loop, which spills more)
+        const bool slow_o = use && (both & (l ? 2u : 4u)) != 0;
+        double d2 = 0.0;
+        if (__any_sync(0xffffffffu, slow_o)) {
+            const double2 u = frame_velocity(qt[1], qt[2], qt[3], n0);
+            const double gt = fix_to_double(Ft[0], e0 - z0 + 2) * u.y, gn = fix_to_double(Fn[0], e0 - z0 + 2) * u.x;
+            const double r = other_lane(l ? gt : gn);
+            d2 = l ? __dsub_rn(r, gn) : __dsub_rn(gt, r);
+        }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int64_t r = other_lane(l ? Ft[k] : Fn[k]);
             const double v =
                 fix_to_double(l ? r - Fn[k] : Ft[k] - r, k == 0 ? e0 - z0 + 2 : k == 3 ? e3 - z3 + 5 : e1 - z1 + 4);
-            if (use) d[k] = k == 1 ? v : flip_sign(v, sbit);
+            if (use) d[k] = k == 1 ? v : flip_sign(k == 2 && slow_o ? d2 : v, sbit);
         }
     }
     const bool slow = differ && !fixed;

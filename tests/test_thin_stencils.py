@@ -210,3 +210,45 @@ def test_products_of_a_stretched_cloud_across_both_axes():
     for kind in "Uxy":
         k = [i for i, e in enumerate(ent) if e[0] == kind]
         assert np.all(np.abs(got - want)[k] <= 16 * A * A * 2.0 ** -53 * np.abs(want[k]).max()), kind
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("axis", [0, 1])
+def test_slow_gas_in_thin_stencils(axis):
+    """Velocities of 1e-8 in a cloud stretched 2^30 : 1, either way: the momentum
+    across the weak direction is carried by the transverse fluxes, rho u_t u_n P
+    with a small u, times the strong direction's weights. First-order residual at
+    1e-12 of each component's largest entry (the parity tests' bar), and its product
+    with a cotangent of that component, at the VJP tests' 1e-10."""
+    import torch
+
+    import oracle
+    from oracle import lskum_jvp
+    from paper_2403_13287_gb300.lskum import Solver
+    A = 2.0 ** 30 if axis == 0 else 2.0 ** -30
+    c = thin_cloud(23, 21, A, seed=3)
+    n = c["n"]
+    U = thin_state(c, A, seed=5)
+    u = U[1:3] / U[0]
+    U[3] += 0.5 * U[0] * ((1e-16 - 1) * (u * u).sum(0))
+    U[1:3] *= 1e-8
+    s = Solver(c, order=1, inner_iters=0, mach=0.5, aoa_deg=0.0)
+    R = s.residual(torch.from_numpy(U).cuda()).cpu().numpy()
+    m = oracle.split_stencils(c)
+    Ro = oracle.residual(c, m, U, order=1, inner=0)
+    k = 1 + axis
+    for j in range(4):
+        assert np.abs(R[j] - Ro[j]).max() <= 1e-12 * np.abs(Ro[j]).max(), j
+    rng = np.random.default_rng(1)
+    Rb = np.zeros((4, n))
+    Rb[k] = rng.standard_normal(n)
+    Ub, xb, yb = (t.cpu().numpy() for t in s.residual_vjp(torch.from_numpy(Rb).cuda(), torch.from_numpy(U).cuda()))
+    s.close()
+    ent = [("U", int(rng.integers(4)), int(e)) for e in rng.choice(n, 20, replace=False)]
+    ent += [("y" if axis == 0 else "x", int(e)) for e in rng.choice(n, 20, replace=False)]
+    want = lskum_jvp.vjp_entries(c, m, U, Rb, ent, order=1, inner=0)
+    got = np.array([Ub[e[1], e[2]] if e[0] == "U" else (xb if e[0] == "x" else yb)[e[1]] for e in ent])
+    for kind in "Uxy":
+        i = [j for j, e in enumerate(ent) if e[0] == kind]
+        if i:
+            assert np.all(np.abs(got - want)[i] <= 1e-10 * np.abs(want[i]).max()), kind
