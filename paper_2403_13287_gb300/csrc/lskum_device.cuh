@@ -391,11 +391,12 @@ __device__ __forceinline__ bool q_from_U(const double U[4], const Gas &gas, doub
         const double t = fma(U[1], U[1], U[2] * U[2]) * fix_reciprocal(rho);   // |m|^2/rho
         const double p = (gas.gamma - 1.0) * fma(-0.5, t, U[3]);
         if (fix_moderate(p)) {
-            const double ip = fix_reciprocal(p);
+            double ip, rp;
+            fix_quotient(rho, p, ip, rp);
             q[0] = fma(-0.5 * t, ip, fix_log_state(rho, p));
             q[1] = U[1] * ip;
             q[2] = U[2] * ip;
-            q[3] = -rho * ip;
+            q[3] = -rp;
             return isfinite(q[0]);
         }
     }
