@@ -758,6 +758,24 @@ __device__ __forceinline__ void incoming(const AdjParamsT<float> &P, int t, floa
     hy = 0.5f * v.w;
 }
 
+// start + a0 b0 + a1 b1. An offset's or weight's cotangent sums four components:
+// its x in the order 0 1 2 3 and its y in the order 2 3 0 1, so that two lanes with
+// two components each go through both at once, handing the half-done sum over in
+// the middle (half_dot), and one lane with all four gets the same bits: a cloud's
+// x_bar and y_bar do not depend on what else is in its batch.
+__device__ __forceinline__ double dot_rest(const double *a, const double *b, double start)
+{
+    return fma(a[1], b[1], fma(a[0], b[0], start));
+}
+// lane l of a pair holds components 2l and 2l + 1 of a, of x and of y: lane 1
+// returns x0 + a.x, lane 0 y0 + a.y. start is this lane's part, x0 in lane 0 and y0
+// in lane 1. Called by whole warps.
+__device__ __forceinline__ double half_dot(int l, const double a[2], const double x[2], const double y[2], double start)
+{
+    const double mine[2] = {l ? y[0] : x[0], l ? y[1] : x[1]}, other[2] = {l ? x[0] : y[0], l ? x[1] : y[1]};
+    return dot_rest(a, other, __shfl_xor_sync(0xffffffffu, dot_rest(a, mine, start), 1));
+}
+
 // ---------------------------------------------------------------------------
 // flux adjoint, neighbour side: point p gathers the cotangents of q~_p over
 // the edges that reach it
@@ -786,21 +804,28 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather(AdjParamsT<T> P)
         if (second) {
             T hx, hy, ax, ay;
             incoming(P, t, hx, hy, ax, ay);
-            T dxb = T(0), dyb = T(0);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 // q~_p = q_p - (dx qx_p + dy qy_p)/2 on this edge
                 gb[k] -= hx * eb[k];
                 gb[4 + k] -= hy * eb[k];
-                if constexpr (GEOM) {
-                    dxb -= h * eb[k] * gp[k];
-                    dyb -= h * eb[k] * gp[4 + k];
-                }
             }
             if constexpr (GEOM) {
                 double2 d = P.dbar[e];
-                d.x += to_f64(dxb);
-                d.y += to_f64(dyb);
+                if constexpr (std::is_same<T, double>::value) {
+                    // (the two-lane form's order)
+                    d.x = fma(-0.5, dot_rest(eb + 2, gp + 2, dot_rest(eb, gp, 0.0)), d.x);
+                    d.y = fma(-0.5, dot_rest(eb, gp + 4, dot_rest(eb + 2, gp + 6, 0.0)), d.y);
+                } else {
+                    T dxb = T(0), dyb = T(0);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        dxb -= h * eb[k] * gp[k];
+                        dyb -= h * eb[k] * gp[4 + k];
+                    }
+                    d.x += to_f64(dxb);
+                    d.y += to_f64(dyb);
+                }
                 P.dbar[e] = d;
             }
         }
@@ -810,8 +835,7 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather(AdjParamsT<T> P)
 }
 
 // the same in FP64 for small clouds (order 2, with the offsets' cotangents): two
-// lanes per point, two components each, of which one adds to the offset's x and
-// one to its y. A point's incoming edges are a serial chain of dependent loads
+// lanes per point, two components each (half_dot). A point's incoming edges are a serial chain of dependent loads
 // and FP64 sums: 37 -> 28 us at 40k points. At 640k the one-lane form's 0.27 ms
 // is already bound by the FP64 pipe (87 %).
 __global__ void __launch_bounds__(128) k_adj_flux_gather_pair(AdjParams P)
@@ -833,25 +857,25 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather_pair(AdjParams P)
     const int most = __reduce_max_sync(0xffffffffu, deg);
 #pragma unroll 1
     for (int j = 0; j < most; ++j) {
-        double dx = 0.0, dy = 0.0;
+        double eb[2] = {0.0, 0.0};
         int e = 0;
         if (j < deg) {
             e = P.tedge[t0 + j];
             const double2 h = __ldg(P.thd + t0 + j);
-            const double2 eb = *reinterpret_cast<const double2 *>(P.ebar + 4 * (int64_t)e + k0);
-            qb[0] += eb.x;
-            qb[1] += eb.y;
-            // q~_p = q_p - h.grad q_p on this edge
-            gx[0] = fma(-h.x, eb.x, gx[0]);
-            gx[1] = fma(-h.x, eb.y, gx[1]);
-            gy[0] = fma(-h.y, eb.x, gy[0]);
-            gy[1] = fma(-h.y, eb.y, gy[1]);
-            dx = fma(eb.y, px[1], eb.x * px[0]);
-            dy = fma(eb.y, py[1], eb.x * py[0]);
+            const double2 v = *reinterpret_cast<const double2 *>(P.ebar + 4 * (int64_t)e + k0);
+            eb[0] = v.x;
+            eb[1] = v.y;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                qb[k] += eb[k];
+                // q~_p = q_p - h.grad q_p on this edge
+                gx[k] = fma(-h.x, eb[k], gx[k]);
+                gy[k] = fma(-h.y, eb[k], gy[k]);
+            }
         }
-        const double d = (l ? dy : dx) + __shfl_xor_sync(0xffffffffu, l ? dx : dy, 1);
+        const double d = half_dot(l, eb, px, py, 0.0);
         if (j < deg) {
-            double *o = reinterpret_cast<double *>(P.dbar + e) + l;
+            double *o = reinterpret_cast<double *>(P.dbar + e) + (1 - l);
             *o = fma(-0.5, d, *o);
         }
     }
@@ -967,10 +991,9 @@ __global__ void __launch_bounds__(128) k_adj_grad_fp32(AdjParamsT<float> P, cons
 // LANES 2: two lanes per point, two components each. Without the geometry's
 // cotangents that is the better form at all sizes (residual product 0.48 -> 0.46
 // ms at 40k points, 3.75 -> 3.71 at 640k); with them the lanes add up a_bar and
-// d_bar, one each, from both halves, which pays while the cloud leaves SMs idle
+// d_bar together (half_dot), which pays while the cloud leaves SMs idle
 // (0.50 -> 0.45 ms at 8k, 0.73 -> 0.69 at 40k; 1.14 -> 1.18 at 93k, 5.77 -> 5.94
-// at 640k). U_bar has the same bits in both forms, x_bar and y_bar differ in
-// rounding (a sum of two halves for one of four terms).
+// at 640k). Both forms give the same bits.
 __device__ __forceinline__ double dot2(const FixPair &a, const FixPair &b, double ax, double ay, double bx, double by)
 {
     if (fix_dot_in_range(a, b)) return fix_dot(a, b);
@@ -1024,7 +1047,7 @@ __global__ void __launch_bounds__(128, LANES == 1 ? 5 : GEOM ? 5 : 8) k_adj_grad
             }
             if constexpr (GEOM) {
                 const int64_t i = g.idx[e];
-                double qi[C], s[C], dbx = 0.0, dby = 0.0;
+                double qi[C], s[C], ix[C], iy[C];
                 gather_c<C>(P.q + 4 * i + k0, qi);
 #pragma unroll
                 for (int k = 0; k < C; ++k) s[k] = qi[k] - qp[k];
@@ -1037,43 +1060,32 @@ __global__ void __launch_bounds__(128, LANES == 1 ? 5 : GEOM ? 5 : 8) k_adj_grad
                         h = make_double2(0.5 * (xyi.x - xyp.x), 0.5 * (xyi.y - xyp.y));
                     }
                     const FixPair hp = fix_pair(h.x, h.y);
-                    double ix[C], iy[C];
                     gather_c<C>(gprev + 8 * i + k0, ix);
                     gather_c<C>(gprev + 8 * i + 4 + k0, iy);
 #pragma unroll
-                    for (int k = 0; k < C; ++k) {
-                        s[k] -= dot2(hp, fix_pair(ix[k], iy[k]), h.x, h.y, ix[k], iy[k]);
-                        // d_e = 2 h_e: d_bar = -(sb/2) grad q_i
-                        dbx = fma(sb[k], ix[k], dbx);
-                        dby = fma(sb[k], iy[k], dby);
-                    }
+                    for (int k = 0; k < C; ++k) s[k] -= dot2(hp, fix_pair(ix[k], iy[k]), h.x, h.y, ix[k], iy[k]);
                 }
+                // a_bar += s gb, and with d_e = 2 h_e: d_bar -= (sb/2) grad q_i
+                const bool start = first && !P.add;
                 if constexpr (LANES == 1) {
                     if (inner) {
                         double2 db = P.dbar[e];
-                        db.x = fma(-0.5, dbx, db.x);
-                        db.y = fma(-0.5, dby, db.y);
+                        db.x = fma(-0.5, dot_rest(sb + 2, ix + 2, dot_rest(sb, ix, 0.0)), db.x);
+                        db.y = fma(-0.5, dot_rest(sb, iy, dot_rest(sb + 2, iy + 2, 0.0)), db.y);
                         P.dbar[e] = db;
                     }
-                    double2 ab = first && !P.add ? make_double2(0.0, 0.0) : P.abar[e];
-#pragma unroll
-                    for (int k = 0; k < C; ++k) {
-                        ab.x = fma(s[k], gx[k], ab.x);
-                        ab.y = fma(s[k], gy[k], ab.y);
-                    }
+                    double2 ab = start ? make_double2(0.0, 0.0) : P.abar[e];
+                    ab.x = dot_rest(s + 2, gx + 2, dot_rest(s, gx, ab.x));
+                    ab.y = dot_rest(s, gy, dot_rest(s + 2, gy + 2, ab.y));
                     P.abar[e] = ab;
                 } else {
-                    // lane 0 completes a_bar, lane 1 d_bar
-                    const double abx = fma(s[1], gx[1], s[0] * gx[0]), aby = fma(s[1], gy[1], s[0] * gy[0]);
-                    const double tx = (l ? dbx : abx) + __shfl_xor_sync(0xffffffffu, l ? abx : dbx, 1);
-                    const double ty = (l ? dby : aby) + __shfl_xor_sync(0xffffffffu, l ? aby : dby, 1);
-                    if (act && (l == 0 || inner)) {
-                        double2 *o = (l ? P.dbar : P.abar) + e;
-                        const double f = l ? -0.5 : 1.0;
-                        double2 v = l == 0 && first && !P.add ? make_double2(0.0, 0.0) : *o;
-                        v.x = fma(f, tx, v.x);
-                        v.y = fma(f, ty, v.y);
-                        *o = v;
+                    // a lane starts one sum and ends, and stores, the other
+                    double *const ab = reinterpret_cast<double *>(P.abar + e), *const db = reinterpret_cast<double *>(P.dbar + e);
+                    const double a1 = half_dot(l, s, gx, gy, start ? 0.0 : ab[l]);
+                    if (act) ab[1 - l] = a1;
+                    if (inner) {   // (the same in every lane)
+                        const double d1 = half_dot(l, sb, ix, iy, 0.0);
+                        if (act) db[1 - l] = fma(-0.5, d1, db[1 - l]);
                     }
                 }
             }
