@@ -758,15 +758,15 @@ __device__ __forceinline__ void incoming(const AdjParamsT<float> &P, int t, floa
     hy = 0.5f * v.w;
 }
 
-// start + a0 b0 + a1 b1. An offset's or weight's cotangent sums four components:
-// its x in the order 0 1 2 3 and its y in the order 2 3 0 1, so that two lanes with
-// two components each go through both at once, handing the half-done sum over in
-// the middle (half_dot), and one lane with all four gets the same bits: a cloud's
-// x_bar and y_bar do not depend on what else is in its batch.
+// start + a0 b0 + a1 b1
 __device__ __forceinline__ double dot_rest(const double *a, const double *b, double start)
 {
     return fma(a[1], b[1], fma(a[0], b[0], start));
 }
+// An offset's or weight's cotangent sums four components over the two lanes of a
+// point: its x in the order 0 1 2 3 and its y in the order 2 3 0 1, so that the
+// lanes go through both at once and hand the half-done sum over in the middle
+// (half the FP64 additions of a lane for each sum).
 // lane l of a pair holds components 2l and 2l + 1 of a, of x and of y: lane 1
 // returns x0 + a.x, lane 0 y0 + a.y. start is this lane's part, x0 in lane 0 and y0
 // in lane 1. Called by whole warps.
@@ -811,21 +811,15 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather(AdjParamsT<T> P)
                 gb[4 + k] -= hy * eb[k];
             }
             if constexpr (GEOM) {
-                double2 d = P.dbar[e];
-                if constexpr (std::is_same<T, double>::value) {
-                    // (the two-lane form's order)
-                    d.x = fma(-0.5, dot_rest(eb + 2, gp + 2, dot_rest(eb, gp, 0.0)), d.x);
-                    d.y = fma(-0.5, dot_rest(eb, gp + 4, dot_rest(eb + 2, gp + 6, 0.0)), d.y);
-                } else {
-                    T dxb = T(0), dyb = T(0);
+                T dxb = T(0), dyb = T(0);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        dxb -= h * eb[k] * gp[k];
-                        dyb -= h * eb[k] * gp[4 + k];
-                    }
-                    d.x += to_f64(dxb);
-                    d.y += to_f64(dyb);
+                for (int k = 0; k < 4; ++k) {
+                    dxb -= h * eb[k] * gp[k];
+                    dyb -= h * eb[k] * gp[4 + k];
                 }
+                double2 d = P.dbar[e];
+                d.x += to_f64(dxb);
+                d.y += to_f64(dyb);
                 P.dbar[e] = d;
             }
         }
@@ -834,10 +828,10 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather(AdjParamsT<T> P)
     if (second) st8(P.gbar, p, gb);
 }
 
-// the same in FP64 for small clouds (order 2, with the offsets' cotangents): two
-// lanes per point, two components each (half_dot). A point's incoming edges are a serial chain of dependent loads
-// and FP64 sums: 37 -> 28 us at 40k points. At 640k the one-lane form's 0.27 ms
-// is already bound by the FP64 pipe (87 %).
+// the same in FP64 of order 2 with the offsets' cotangents: two lanes per point,
+// two components each (half_dot). A point's incoming edges are a serial chain of
+// dependent loads and FP64 sums: 37 -> 28 us at 40k points; at 640k (0.27 ms) the
+// FP64 pipe bounds both forms.
 __global__ void __launch_bounds__(128) k_adj_flux_gather_pair(AdjParams P)
 {
     const int64_t n = P.g.n, pp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 1;
@@ -988,29 +982,27 @@ __global__ void __launch_bounds__(128) k_adj_grad_fp32(AdjParamsT<float> P, cons
 // which keep the q cotangent apart (qbar2: the owner's share, summed with qbar
 // by k_adj_state), and the two-term products run on the integer pipes
 // (fix_dot): 40 FP64 instructions per edge of 68. 87 -> 62 us a pass at 40k points.
-// LANES 2: two lanes per point, two components each. Without the geometry's
-// cotangents that is the better form at all sizes (residual product 0.48 -> 0.46
-// ms at 40k points, 3.75 -> 3.71 at 640k); with them the lanes add up a_bar and
-// d_bar together (half_dot), which pays while the cloud leaves SMs idle
-// (0.50 -> 0.45 ms at 8k, 0.73 -> 0.69 at 40k; 1.14 -> 1.18 at 93k, 5.77 -> 5.94
-// at 640k). Both forms give the same bits.
+// Two lanes per point, two components each, which add up a_bar and d_bar together
+// (half_dot). One lane with all four: a residual product of 8k points 0.50 ms
+// against 0.45, 64k 0.857 / 0.806, 160k 1.64 / 1.57, 640k 5.46 / 5.28. Blocks per SM
+// (registers against warps) 5 / 6 / 7 / 8: 0.434 / 0.437 / 0.444 / 0.453 ms at 18k,
+// 1.608 / 1.588 / 1.570 / 1.582 at 160k, 5.43 / 5.34 / 5.28 / 5.28 at 640k.
 __device__ __forceinline__ double dot2(const FixPair &a, const FixPair &b, double ax, double ay, double bx, double by)
 {
     if (fix_dot_in_range(a, b)) return fix_dot(a, b);
     return fix_pair_zero(b) ? 0.0 : fma(ay, by, ax * bx);   // both terms zero (or subnormal): nothing to add
 }
 
-template <bool GEOM, int LANES>
-__global__ void __launch_bounds__(128, LANES == 1 ? 5 : GEOM ? 5 : 8) k_adj_grad_fp64(AdjParams P, const double *__restrict__ gprev,
-                                                          const double *__restrict__ gbar_in,
-                                                          double *__restrict__ gbar_out, int first)
+template <bool GEOM>
+__global__ void __launch_bounds__(128, GEOM ? 7 : 8) k_adj_grad_fp64(AdjParams P, const double *__restrict__ gprev,
+                                                                    const double *__restrict__ gbar_in,
+                                                                    double *__restrict__ gbar_out, int first)
 {
-    constexpr int C = 4 / LANES;
+    constexpr int C = 2;
     const DevGeom &g = P.g;
-    const int64_t pp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
-    const int l = threadIdx.x % LANES, k0 = C * l;
+    const int64_t pp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 1;
+    const int l = threadIdx.x & 1, k0 = C * l;
     const bool live = pp < g.n;
-    if (LANES == 1 && !live) return;
     const int64_t p = live ? pp : g.n - 1;   // (lanes past the end take part in the shuffles)
     const bool inner = gprev != nullptr;
     double qb[C], gx[C], gy[C];
@@ -1031,8 +1023,8 @@ __global__ void __launch_bounds__(128, LANES == 1 ? 5 : GEOM ? 5 : 8) k_adj_grad
             if (!g.hd) xyp = g.xy[p];
         }
         const int e0 = g.off[p], deg = live ? g.off[p + 1] - e0 : 0;
-        // two lanes: whole warps go through the longest row, as the lanes exchange sums by shuffles
-        const int most = GEOM && LANES > 1 ? __reduce_max_sync(0xffffffffu, deg) : deg;
+        // whole warps go through the longest row where the lanes exchange sums by shuffles
+        const int most = GEOM ? __reduce_max_sync(0xffffffffu, deg) : deg;
 #pragma unroll 1
         for (int j = 0; j < most; ++j) {
             const bool act = j < deg;
@@ -1067,26 +1059,13 @@ __global__ void __launch_bounds__(128, LANES == 1 ? 5 : GEOM ? 5 : 8) k_adj_grad
                 }
                 // a_bar += s gb, and with d_e = 2 h_e: d_bar -= (sb/2) grad q_i
                 const bool start = first && !P.add;
-                if constexpr (LANES == 1) {
-                    if (inner) {
-                        double2 db = P.dbar[e];
-                        db.x = fma(-0.5, dot_rest(sb + 2, ix + 2, dot_rest(sb, ix, 0.0)), db.x);
-                        db.y = fma(-0.5, dot_rest(sb, iy, dot_rest(sb + 2, iy + 2, 0.0)), db.y);
-                        P.dbar[e] = db;
-                    }
-                    double2 ab = start ? make_double2(0.0, 0.0) : P.abar[e];
-                    ab.x = dot_rest(s + 2, gx + 2, dot_rest(s, gx, ab.x));
-                    ab.y = dot_rest(s, gy, dot_rest(s + 2, gy + 2, ab.y));
-                    P.abar[e] = ab;
-                } else {
-                    // a lane starts one sum and ends, and stores, the other
-                    double *const ab = reinterpret_cast<double *>(P.abar + e), *const db = reinterpret_cast<double *>(P.dbar + e);
-                    const double a1 = half_dot(l, s, gx, gy, start ? 0.0 : ab[l]);
-                    if (act) ab[1 - l] = a1;
-                    if (inner) {   // (the same in every lane)
-                        const double d1 = half_dot(l, sb, ix, iy, 0.0);
-                        if (act) db[1 - l] = fma(-0.5, d1, db[1 - l]);
-                    }
+                // (a lane starts one sum and ends, and stores, the other)
+                double *const ab = reinterpret_cast<double *>(P.abar + e), *const db = reinterpret_cast<double *>(P.dbar + e);
+                const double a1 = half_dot(l, s, gx, gy, start ? 0.0 : ab[l]);
+                if (act) ab[1 - l] = a1;
+                if (inner) {   // (the same in every lane)
+                    const double d1 = half_dot(l, sb, ix, iy, 0.0);
+                    if (act) db[1 - l] = fma(-0.5, d1, db[1 - l]);
                 }
             }
         }
@@ -1717,14 +1696,10 @@ cudaError_t launch_adj_flux(const AdjParamsT<T> &P, bool geom, cudaStream_t s)
     if (!pair && !geom) k_adj_flux<T, false><<<nb, 128, 0, s>>>(P);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    if constexpr (std::is_same<T, double>::value) {
-        if (geom && P.order == 2 && P.g.n < 60000) {
-            k_adj_flux_gather_pair<<<blocks(P.g.n, 64), 128, 0, s>>>(P);
-            return cudaGetLastError();
-        }
-    }
-    if (geom) k_adj_flux_gather<T, true><<<nb, 128, 0, s>>>(P);
-    else k_adj_flux_gather<T, false><<<nb, 128, 0, s>>>(P);
+    const bool offsets = geom && P.order == 2;   // (order 1 has none)
+    if (!offsets) k_adj_flux_gather<T, false><<<nb, 128, 0, s>>>(P);
+    else if constexpr (std::is_same<T, double>::value) k_adj_flux_gather_pair<<<blocks(P.g.n, 64), 128, 0, s>>>(P);
+    else k_adj_flux_gather<T, true><<<nb, 128, 0, s>>>(P);
     return cudaGetLastError();
 }
 
@@ -1733,12 +1708,9 @@ cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gba
                             bool first, cudaStream_t s)
 {
     if constexpr (std::is_same<T, double>::value) {
-        // (lanes per point: see the kernel)
-        const bool two = !geom || P.g.n < 60000;
-        const dim3 nb(blocks(P.g.n, two ? 64 : 128), 2);
-        if (!geom) k_adj_grad_fp64<false, 2><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
-        else if (two) k_adj_grad_fp64<true, 2><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
-        else k_adj_grad_fp64<true, 1><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+        const dim3 nb(blocks(P.g.n, 64), 2);
+        if (geom) k_adj_grad_fp64<true><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+        else k_adj_grad_fp64<false><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
     } else {
         if (geom) k_adj_grad_fp32<true><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
         else k_adj_grad_fp32<false><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);

@@ -1,6 +1,5 @@
-"""A cloud's products are the same bits alone and inside a batch: the reverse
-kernels choose lanes per point by the batch's size, and every form adds the same
-terms in the same order (needs a GPU)."""
+"""A cloud's products are the same bits alone and inside a batch: no reverse
+kernel adds in an order that depends on the number of points (needs a GPU)."""
 import numpy as np
 import pytest
 
@@ -11,8 +10,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("order,limiter,gamma,reorder", [(2, 0.0, 1.4, 1), (2, 1.0, 1.4, 0), (2, 0.0, 1.3, 1), (1, 0.0, 1.4, 1)])
 def test_products_of_a_cloud_do_not_depend_on_the_batch(order, limiter, gamma, reorder):
-    """3250 points alone (two lanes) and beside 64k points (one lane): residual and
-    step products, all of U_bar, x_bar and y_bar."""
+    """3250 points alone and beside 64k points: residual and step products, all of
+    U_bar, x_bar and y_bar."""
     import torch
 
     from paper_2403_13287_gb300.lskum import Solver
