@@ -1125,9 +1125,10 @@ __global__ void __launch_bounds__(128, GEOM ? 7 : 8) k_adj_grad_fp64(AdjParams P
 //         and added by k_adj_limit_gather
 //   the offsets: d* = 2 h* gets G f_d s g_raw / 2, the nearest neighbour's
 //         offset gets 3 K^3 dmin^2 G f_eps d/|d| (through eps^2)
-// The choices are the forward's: the first largest (smallest) q_i - q_0 in
-// row order, P_0's own 0 winning ties; the first largest |h . g_raw|; the
-// first nearest neighbour by squared distance. Where phi = 1 the limiter is
+// The choices: the first largest (smallest) q_i in row order, P_0's own winning
+// ties (the forward takes the value of the largest rounded q_i - q_0 alone; where
+// several differences round alike, q_i still tells which is the extreme one); the
+// first largest |h . g_raw|; the first nearest neighbour by squared distance. Where phi = 1 the limiter is
 // inactive and gbar passes through.
 //
 // With s = x + d and r = 1/M: f_x = (2 s - phi (x + s)) r, f_d = (2 x - phi (x + 4 d)) r,
