@@ -393,6 +393,16 @@ lskum_status lskum_autotune(lskum_ctx *ctx, int reps, lskum_tuning *out);
 lskum_status lskum_set_tuning(lskum_ctx *ctx, int flux_variant, int qgrad_variant);
 
 /*
+ * Memory against time (not in the paper). Some of a context's device arrays only
+ * save time: an FP64 context's half offsets in the form its passes read (16 B per
+ * edge), taken when it is created. Where the device has no memory for one, the
+ * context does without it. lean = 1 gives them back to the device and takes none
+ * any more, lean = 0 (how a context starts) takes them again. Results are the same
+ * bits either way. Synchronises. LSKUM_ERR_ARG on another value.
+ */
+lskum_status lskum_set_lean(lskum_ctx *ctx, int lean);
+
+/*
  * Mixed contexts: *count receives the number of points whose least-squares
  * closures run in FP64 because FP32 would lose bits there (a sub-stencil
  * with sum |w_i||P_i - P_0| > 16; not in the paper, a property of the mixed

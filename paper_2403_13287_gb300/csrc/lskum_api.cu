@@ -34,6 +34,8 @@ struct lskum_ctx {
     Gas gas{};
     std::vector<int32_t> perm_h;
     std::vector<void *> allocs;
+    std::vector<void *> optional;  // arrays that only save time (optional_alloc)
+    bool lean = false;             // without them
 
     double2 *xy = nullptr, *nrm = nullptr;
     uint8_t *flag = nullptr, *mask = nullptr;
@@ -41,7 +43,7 @@ struct lskum_ctx {
     int32_t *off = nullptr, *idx = nullptr, *off_in = nullptr;
     double2 *lsw = nullptr, *fxw = nullptr, *hd = nullptr;
     float2 *hd_f = nullptr;  // FP64 contexts: hd in FP32, for the limiter's screening of d_m
-    longlong2 *hfx = nullptr;  // FP64 contexts: hd in fixed point, for the inner passes
+    longlong2 *hfx = nullptr;  // FP64 contexts: hd in fixed point, for the inner passes (optional)
     // kinetic boundary mode: mirror images of the neighbours of wall and
     // far-field points (CSR per internal point) and each case's free-stream q
     bool kinetic = false;
@@ -272,10 +274,47 @@ static cudaError_t dalloc(lskum_ctx *c, T **p, size_t count)
     return e;
 }
 
+// an array that only saves time: *p is nullptr where the device has no memory for
+// it or the context is lean. Results do not depend on it.
+template <typename T>
+static cudaError_t optional_alloc(lskum_ctx *c, T **p, size_t count)
+{
+    *p = nullptr;
+    if (c->lean) return cudaSuccess;
+    void *v = nullptr;
+    const cudaError_t e = cudaMalloc(&v, std::max<size_t>(count, 1) * sizeof(T));
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        return cudaSuccess;
+    }
+    if (e == cudaSuccess) {
+        c->optional.push_back(v);
+        *p = static_cast<T *>(v);
+    }
+    return e;
+}
+
+static void free_optional(lskum_ctx *c)
+{
+    for (void *p : c->optional) cudaFree(p);
+    c->optional.clear();
+    c->hfx = nullptr;
+}
+
 static void free_all(lskum_ctx *c)
 {
+    free_optional(c);
     for (void *p : c->allocs) cudaFree(p);
     c->allocs.clear();
+}
+
+// 16 B per edge: the inner passes otherwise form it from hd in the loop
+static lskum_status fixed_offsets(lskum_ctx *c)
+{
+    if (c->mixed) return LSKUM_OK;
+    CK(c, optional_alloc(c, &c->hfx, c->nnz));
+    if (c->hfx) LAUNCH(c, launch_fixed_offsets(c->nnz, c->hd, c->hfx, c->stream));
+    return LSKUM_OK;
 }
 
 static void freestream(double gamma, double mach, double aoa_deg, double U[4])
@@ -668,8 +707,7 @@ static lskum_status create_impl(lskum_ctx *c, const double *x, const double *y, 
     if (!c->mixed) {
         CK(c, dalloc(c, &c->hd, std::max<int64_t>(nnz, 1)));
         CK(c, dalloc(c, &c->hd_f, std::max<int64_t>(nnz, 1)));
-        CK(c, dalloc(c, &c->hfx, std::max<int64_t>(nnz, 1)));
-        LAUNCH(c, launch_half_offsets(n, c->xy, c->off, c->idx, c->hd, c->hd_f, c->hfx, s));
+        LAUNCH(c, launch_half_offsets(n, c->xy, c->off, c->idx, c->hd, c->hd_f, s));
     }
     int bad_h[2];
     CK(c, cudaMemcpyAsync(bad_h, bad, sizeof bad_h, cudaMemcpyDeviceToHost, s));
@@ -831,7 +869,7 @@ static lskum_status create_impl(lskum_ctx *c, const double *x, const double *y, 
     if (c->ncases > 1) LAUNCH(c, launch_fill_state_cases(n, c->pcase, c->case_uinf, c->U, s));
     else LAUNCH(c, launch_fill_state(n, c->gas.Uinf, c->U, s));
     lskum_status st = refresh_q(c, c->U, c->q_cur);
-    if (st != LSKUM_OK) return st;
+    if (st != LSKUM_OK || (st = fixed_offsets(c)) != LSKUM_OK) return st;
     CK(c, cudaStreamSynchronize(s));
     return LSKUM_OK;
 }
@@ -1841,6 +1879,19 @@ static void drop_graphs(lskum_ctx *c)
         if (g.exec) cudaGraphExecDestroy(g.exec);
         g = lskum_ctx::StepGraph{};
     }
+}
+
+extern "C" lskum_status lskum_set_lean(lskum_ctx *c, int lean)
+{
+    if (!c) return LSKUM_ERR_ARG;
+    c->err.clear();
+    if (lean != 0 && lean != 1) return fail(c, LSKUM_ERR_ARG, "lean must be 0 or 1");
+    if (c->lean == (lean == 1)) return LSKUM_OK;
+    CK(c, cudaStreamSynchronize(c->stream));
+    drop_graphs(c);   // captured launches hold the arrays' addresses
+    free_optional(c);
+    c->lean = lean == 1;
+    return fixed_offsets(c);
 }
 
 extern "C" lskum_status lskum_set_tuning(lskum_ctx *c, int flux_variant, int qgrad_variant)

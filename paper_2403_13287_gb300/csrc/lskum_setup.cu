@@ -147,10 +147,9 @@ cudaError_t launch_geometry(int64_t n, const double2 *xy, const double2 *nrm, co
 
 // per edge (P_i - P_0)/2 (FP64 contexts): the E14 reconstruction and correction
 // terms use it directly, two fused multiply-adds per component; hd_f (if not
-// null) receives it rounded to FP32, hfx in fixed point
+// null) receives it rounded to FP32
 __global__ void k_half_offsets(int64_t n, const double2 *__restrict__ xy, const int32_t *__restrict__ off,
-                               const int32_t *__restrict__ idx, double2 *__restrict__ hd, float2 *__restrict__ hd_f,
-                               longlong2 *__restrict__ hfx)
+                               const int32_t *__restrict__ idx, double2 *__restrict__ hd, float2 *__restrict__ hd_f)
 {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
@@ -160,16 +159,31 @@ __global__ void k_half_offsets(int64_t n, const double2 *__restrict__ xy, const 
         const double2 h = make_double2(0.5 * (Pi.x - P0.x), 0.5 * (Pi.y - P0.y));
         hd[e] = h;
         if (hd_f) hd_f[e] = make_float2(__double2float_rn(h.x), __double2float_rn(h.y));
-        int64_t wx, wy;
-        fix_pack_pair(h.x, h.y, wx, wy);
-        hfx[e] = make_longlong2(wx, wy);
     }
 }
 
-cudaError_t launch_half_offsets(int64_t n, const double2 *xy, const int32_t *off, const int32_t *idx, double2 *hd,
-                                float2 *hd_f, longlong2 *hfx, cudaStream_t s)
+// hfx[e]: hd[e] in fixed point
+__global__ void k_fixed_offsets(int64_t nnz, const double2 *__restrict__ hd, longlong2 *__restrict__ hfx)
 {
-    k_half_offsets<<<nblk(n, 128), 128, 0, s>>>(n, xy, off, idx, hd, hd_f, hfx);
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= nnz) return;
+    const double2 h = hd[e];
+    int64_t wx, wy;
+    fix_pack_pair(h.x, h.y, wx, wy);
+    hfx[e] = make_longlong2(wx, wy);
+}
+
+cudaError_t launch_half_offsets(int64_t n, const double2 *xy, const int32_t *off, const int32_t *idx, double2 *hd,
+                                float2 *hd_f, cudaStream_t s)
+{
+    k_half_offsets<<<nblk(n, 128), 128, 0, s>>>(n, xy, off, idx, hd, hd_f);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fixed_offsets(int64_t nnz, const double2 *hd, longlong2 *hfx, cudaStream_t s)
+{
+    if (nnz <= 0) return cudaSuccess;
+    k_fixed_offsets<<<nblk(nnz, 256), 256, 0, s>>>(nnz, hd, hfx);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,66 @@
+"""Contexts without the arrays that only save time (lskum_set_lean): the same bits,
+and the memory is given back (needs a GPU)."""
+import numpy as np
+import pytest
+
+from paper_2403_13287_gb300.cloudgen import naca0012_cloud, smooth_state
+
+pytestmark = pytest.mark.gpu
+
+
+def _everything(s, U):
+    import torch
+    out = {"R": s.residual(U)}
+    out["qx"], out["qy"] = s.q_derivatives(U)
+    s.set_state(U)
+    out["history"] = torch.from_numpy(s.step(3))
+    out["state"] = torch.from_numpy(s.get_state())
+    return {k: v.cpu().numpy() for k, v in out.items()}
+
+
+@pytest.mark.parametrize("order,limiter,boundary,time_scheme", [(2, 0.0, 0, 1), (2, 1.0, 0, 0), (2, 1.0, 1, 1), (1, 0.0, 0, 1)])
+def test_forward_is_the_same_without_optional_arrays(order, limiter, boundary, time_scheme):
+    """Before, lean, and back again on one context, the step graphs replayed in
+    between."""
+    import torch
+
+    from paper_2403_13287_gb300.lskum import Solver
+    c = naca0012_cloud(180, 99, seed=3, shuffle=True)
+    U = torch.from_numpy(smooth_state(c, 0.85, 1.0, amp=0.05, seed=9)).cuda()
+    s = Solver(c, order=order, inner_iters=3 if order == 2 else 0, time_scheme=time_scheme, limiter_K=limiter, mach=0.85,
+               aoa_deg=1.0, reorder=1, boundary=boundary)
+    got = []
+    for lean in (None, True, False):
+        if lean is not None:
+            s.set_lean(lean)
+        got.append(_everything(s, U))
+    s.close()
+    for other in got[1:]:
+        for k in got[0]:
+            assert np.array_equal(got[0][k], other[k]), k
+
+
+def test_memory_is_given_back():
+    """16 B per edge of an FP64 context (21 MB here; the device hands out pieces of
+    2 MB), none of a mixed one."""
+    import torch
+
+    from paper_2403_13287_gb300.lskum import Solver
+    c = naca0012_cloud(512, 311, seed=3)
+    for precision, want in ((0, 16 * c["nbr_idx"].size), (1, 0)):
+        s = Solver(c, order=2, inner_iters=3, mach=0.85, aoa_deg=1.0, precision=precision, reorder=1)
+        free0 = torch.cuda.mem_get_info()[0]
+        s.set_lean()
+        free1 = torch.cuda.mem_get_info()[0]
+        s.set_lean(False)
+        free2 = torch.cuda.mem_get_info()[0]
+        s.close()
+        assert abs((free1 - free0) - want) <= 4 << 20 and free2 == free0
+
+
+def test_lean_takes_0_or_1():
+    from paper_2403_13287_gb300.lskum import LSKUM_ERR_ARG, Solver
+    s = Solver(naca0012_cloud(34, 12, seed=1), order=2, mach=0.5, aoa_deg=0.0)
+    assert s._L.lskum_set_lean(s._ctx, 2) == LSKUM_ERR_ARG and s._L.lskum_set_lean(s._ctx, -1) == LSKUM_ERR_ARG
+    assert s._L.lskum_set_lean(None, 1) == LSKUM_ERR_ARG
+    s.close()
