@@ -222,11 +222,12 @@ lskum_status lskum_residual(lskum_ctx *ctx, const double *U, double *R);
  * LSKUM_ERR_ARG with LSKUM_VJP_FP32): it is piecewise smooth, and the
  * product is that of the branch the forward takes, with the forward's
  * choices (the first stencil extremum, the first largest reconstruction
- * shift, the first nearest neighbour in row order). Its workspace (about
- * 0.67 KB per point plus 120 B per edge for K = 3: 1.1 GB at 640k points;
- * 0.16 KB per point more with the limiter; the FP32 product adds 0.16 KB per
- * point and 56 B per edge) is allocated on the first call
- * and kept. The kinetic boundary mode is not differentiated (LSKUM_ERR_ARG).
+ * shift, the first nearest neighbour in row order). Its workspace (0.52 KB per
+ * point plus 88 B per edge for K = 3: 0.8 GB at 640k points; 0.14 KB per point
+ * more with the limiter; the FP32 product adds 0.24 KB per point and 16 B per
+ * edge) is allocated on the first call and kept, with 120 B per point and 32 B
+ * per edge (FP32: 40 B per edge more) that only save time (lskum_set_lean).
+ * The kinetic boundary mode is not differentiated (LSKUM_ERR_ARG).
  * Does not change the context's state.
  */
 #define LSKUM_VJP_ACCUMULATE_XY 1 /* flags: add into x_bar, y_bar instead of overwriting them */
@@ -395,8 +396,9 @@ lskum_status lskum_set_tuning(lskum_ctx *ctx, int flux_variant, int qgrad_varian
 /*
  * Memory against time (not in the paper). Some of a context's device arrays only
  * save time: an FP64 context's half offsets in the form its passes read (16 B per
- * edge), taken when it is created. Where the device has no memory for one, the
- * context does without it. lean = 1 gives them back to the device and takes none
+ * edge), taken when it is created, and part of the products' workspaces. Where the
+ * device has no memory for one, the context does without it, and it gives them back
+ * when another of its allocations needs the room. lean = 1 gives them back to the device and takes none
  * any more, lean = 0 (how a context starts) takes them again. Results are the same
  * bits either way. Synchronises. LSKUM_ERR_ARG on another value.
  */

@@ -396,6 +396,9 @@ __device__ __forceinline__ void state_adjoint_rev(const double qt[4], double tx,
 // gamma != 1.4. GEOM: with the cotangents of weights and offsets.
 // ---------------------------------------------------------------------------
 // weights (w_s, w_n) and offset of an edge: the FP64 geometry, or its FP32 copy
+// COPIES: the FP32 product's copies of the geometry are there (a kernel for each
+// case: the choice inside the loops cost the product 13 %)
+template <bool COPIES>
 __device__ __forceinline__ void edge_geometry(const AdjParamsT<double> &P, int e, int i, double2 xy0, bool second,
                                               double &wx, double &wy, double &dx, double &dy)
 {
@@ -408,10 +411,30 @@ __device__ __forceinline__ void edge_geometry(const AdjParamsT<double> &P, int e
         dy = xyi.y - xy0.y;
     }
 }
-__device__ __forceinline__ void edge_geometry(const AdjParamsT<float> &P, int e, int, double2, bool, float &wx,
+// (dx, dy, w_s, w_n) and (a_x, a_y) of an edge in FP32: the copies, or made here
+__device__ __forceinline__ float4 float_edge(const DevGeom &g, int e, int i, double2 xy0)
+{
+    const double2 Pi = g.xy[i], w = g.fxw[e];
+    return make_float4((float)(Pi.x - xy0.x), (float)(Pi.y - xy0.y), (float)w.x, (float)w.y);
+}
+template <bool COPIES>
+__device__ __forceinline__ float2 float_weights(const AdjParamsT<float> &P, int e)
+{
+    if constexpr (COPIES) return __ldg(P.ea + e);
+    const double2 a = P.g.lsw[e];
+    return make_float2((float)a.x, (float)a.y);
+}
+template <bool COPIES>
+__device__ __forceinline__ float4 float_offsets(const AdjParamsT<float> &P, int e, int i, double2 xy0)
+{
+    if constexpr (COPIES) return __ldg(P.ef + e);
+    return float_edge(P.g, e, i, xy0);
+}
+template <bool COPIES>
+__device__ __forceinline__ void edge_geometry(const AdjParamsT<float> &P, int e, int i, double2 xy0, bool, float &wx,
                                               float &wy, float &dx, float &dy)
 {
-    const float4 v = __ldg(P.ef + e);
+    const float4 v = float_offsets<COPIES>(P, e, i, xy0);
     dx = v.x;
     dy = v.y;
     wx = v.z;
@@ -423,7 +446,7 @@ __device__ __forceinline__ void edge_geometry(const AdjParamsT<float> &P, int e,
 __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return f32_to_f64_ip(v); }
 
-template <class T, bool GEOM>
+template <class T, bool GEOM, bool COPIES>
 __global__ void __launch_bounds__(128) k_adj_flux(AdjParamsT<T> P)
 {
     const DevGeom &g = P.g;
@@ -461,7 +484,7 @@ __global__ void __launch_bounds__(128) k_adj_flux(AdjParamsT<T> P)
         const int ks = xsub(m), kn = ysub(m);
         const bool us_ = sub_needed(f, ks), un_ = sub_needed(f, kn);
         T wx, wy, dx = T(0), dy = T(0);
-        edge_geometry(P, e, i, xy0, second, wx, wy, dx, dy);
+        edge_geometry<COPIES>(P, e, i, xy0, second, wx, wy, dx, dy);
         T qti[4], qt0[4];
         ld4(P.q, i, qti);
         T gi[8];
@@ -740,18 +763,46 @@ __global__ void __launch_bounds__(128, 5) k_adj_flux_pair(AdjParams P)
     }
 }
 
-// half offset and full-stencil weights of incoming edge t
+// half offset and full-stencil weights of incoming edge t: the copies in the order
+// that they are read in, or the edge's own
+__device__ __forceinline__ double2 edge_half_offset(const DevGeom &g, int e, int64_t src)
+{
+    if (g.hd) return g.hd[e];
+    const double2 a = g.xy[src], b = g.xy[g.idx[e]];
+    return make_double2(0.5 * (b.x - a.x), 0.5 * (b.y - a.y));
+}
+__device__ __forceinline__ double2 incoming_offset(const AdjParamsT<double> &P, int t)
+{
+    return P.thd ? __ldg(P.thd + t) : edge_half_offset(P.g, P.tedge[t], P.tsrc[t]);
+}
+__device__ __forceinline__ double2 incoming_weights(const AdjParamsT<double> &P, int t)
+{
+    return P.tlsw ? __ldg(P.tlsw + t) : P.g.lsw[P.tedge[t]];
+}
+__device__ __forceinline__ float4 float_incoming(const DevGeom &g, int e, int src)
+{
+    const double2 a = g.lsw[e], A = g.xy[src], B = g.xy[g.idx[e]];
+    return make_float4((float)a.x, (float)a.y, (float)(B.x - A.x), (float)(B.y - A.y));
+}
+template <bool COPIES>
 __device__ __forceinline__ void incoming(const AdjParamsT<double> &P, int t, double &hx, double &hy, double &ax, double &ay)
 {
-    const double2 hh = __ldg(P.thd + t), a = __ldg(P.tlsw + t);
+    const double2 hh = incoming_offset(P, t), a = incoming_weights(P, t);
     hx = hh.x;
     hy = hh.y;
     ax = a.x;
     ay = a.y;
 }
+template <bool COPIES>
+__device__ __forceinline__ float4 float_incoming_edge(const AdjParamsT<float> &P, int t)
+{
+    if constexpr (COPIES) return __ldg(P.tf + t);
+    return float_incoming(P.g, P.tedge[t], P.tsrc[t]);
+}
+template <bool COPIES>
 __device__ __forceinline__ void incoming(const AdjParamsT<float> &P, int t, float &hx, float &hy, float &ax, float &ay)
 {
-    const float4 v = __ldg(P.tf + t);
+    const float4 v = float_incoming_edge<COPIES>(P, t);
     ax = v.x;
     ay = v.y;
     hx = 0.5f * v.z;
@@ -780,7 +831,7 @@ __device__ __forceinline__ double half_dot(int l, const double a[2], const doubl
 // flux adjoint, neighbour side: point p gathers the cotangents of q~_p over
 // the edges that reach it
 // ---------------------------------------------------------------------------
-template <class T, bool GEOM>
+template <class T, bool GEOM, bool COPIES>
 __global__ void __launch_bounds__(128) k_adj_flux_gather(AdjParamsT<T> P)
 {
     const DevGeom &g = P.g;
@@ -803,7 +854,7 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather(AdjParamsT<T> P)
         for (int k = 0; k < 4; ++k) qb[k] += eb[k];
         if (second) {
             T hx, hy, ax, ay;
-            incoming(P, t, hx, hy, ax, ay);
+            incoming<COPIES>(P, t, hx, hy, ax, ay);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 // q~_p = q_p - (dx qx_p + dy qy_p)/2 on this edge
@@ -855,7 +906,7 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather_pair(AdjParams P)
         int e = 0;
         if (j < deg) {
             e = P.tedge[t0 + j];
-            const double2 h = __ldg(P.thd + t0 + j);
+            const double2 h = incoming_offset(P, t0 + j);
             const double2 v = *reinterpret_cast<const double2 *>(P.ebar + 4 * (int64_t)e + k0);
             eb[0] = v.x;
             eb[1] = v.y;
@@ -888,7 +939,7 @@ __global__ void __launch_bounds__(128) k_adj_flux_gather_pair(AdjParams P)
 // 640k points: 228 -> 58 us a pass, half of it from the geometry's FP32 copies,
 // which spare the FP64 pipe the conversions).
 // ---------------------------------------------------------------------------
-template <bool GEOM>
+template <bool GEOM, bool COPIES>
 __global__ void __launch_bounds__(128) k_adj_grad_fp32(AdjParamsT<float> P, const float *__restrict__ gprev,
                                                        const float *__restrict__ gbar_in,
                                                        float *__restrict__ gbar_out, int first)
@@ -911,7 +962,7 @@ __global__ void __launch_bounds__(128) k_adj_grad_fp32(AdjParamsT<float> P, cons
     }
     // outgoing edges: owner terms, and the cotangents of a_e and of the offsets
     for (int e = g.off[p]; e < g.off[p + 1]; ++e) {
-        const float2 a = __ldg(P.ea + e);
+        const float2 a = float_weights<COPIES>(P, e);
         if constexpr (!GEOM) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -923,7 +974,7 @@ __global__ void __launch_bounds__(128) k_adj_grad_fp32(AdjParamsT<float> P, cons
             float qi[4], gi[8], hx = 0.0f, hy = 0.0f;
             ld4(P.q, i, qi);
             if (inner) {
-                const float4 v = __ldg(P.ef + e);
+                const float4 v = float_offsets<COPIES>(P, e, i, g.xy[p]);
                 hx = 0.5f * v.x;
                 hy = 0.5f * v.y;
                 ld8(gprev, i, gi);
@@ -960,7 +1011,7 @@ __global__ void __launch_bounds__(128) k_adj_grad_fp32(AdjParamsT<float> P, cons
     for (int t = P.toff[p]; t < t1; ++t) {
         const int src = P.tsrc[t];
         float hx, hy, ax, ay;
-        incoming(P, t, hx, hy, ax, ay);
+        incoming<COPIES>(P, t, hx, hy, ax, ay);
         float gs[8];
         ld8(gbar_in, src, gs);
 #pragma unroll
@@ -1085,13 +1136,13 @@ __global__ void __launch_bounds__(128, GEOM ? 7 : 8) k_adj_grad_fp64(AdjParams P
 #pragma unroll 1
         for (int t = P.toff[p]; t < t1; ++t) {
             const int64_t src = P.tsrc[t];
-            const double2 a = __ldg(P.tlsw + t);
+            const double2 a = incoming_weights(P, t);
             const FixPair ap = fix_pair(a.x, a.y);
             double sx[C], sy[C];
             gather_c<C>(gbar_in + 8 * src + k0, sx);
             gather_c<C>(gbar_in + 8 * src + 4 + k0, sy);
             double2 h = make_double2(0.0, 0.0);
-            if (inner) h = __ldg(P.thd + t);
+            if (inner) h = incoming_offset(P, t);
 #pragma unroll
             for (int k = 0; k < C; ++k) {
                 const double sb = dot2(ap, fix_pair(sx[k], sy[k]), a.x, a.y, sx[k], sy[k]);
@@ -1590,12 +1641,7 @@ __global__ void k_incoming(int64_t nnz, DevGeom g, const int32_t *__restrict__ t
     if (t >= nnz) return;
     const int e = tedge[t];
     tlsw[t] = g.lsw[e];
-    if (g.hd) {
-        thd[t] = g.hd[e];
-    } else {
-        const double2 a = g.xy[tsrc[t]], b = g.xy[g.idx[e]];
-        thd[t] = make_double2(0.5 * (b.x - a.x), 0.5 * (b.y - a.y));
-    }
+    thd[t] = edge_half_offset(g, e, tsrc[t]);
 }
 
 // the FP32 product's copies: the FP64 offsets and weights rounded once
@@ -1605,19 +1651,17 @@ __global__ void k_float_edges(DevGeom g, float4 *__restrict__ ef, float2 *__rest
     if (p >= g.n) return;
     const double2 P0 = g.xy[p];
     for (int e = g.off[p]; e < g.off[p + 1]; ++e) {
-        const double2 Pi = g.xy[g.idx[e]], w = g.fxw[e], a = g.lsw[e];
-        ef[e] = make_float4((float)(Pi.x - P0.x), (float)(Pi.y - P0.y), (float)w.x, (float)w.y);
+        const double2 a = g.lsw[e];
+        ef[e] = float_edge(g, e, g.idx[e], P0);
         ea[e] = make_float2((float)a.x, (float)a.y);
     }
 }
 
-__global__ void k_float_incoming(int64_t nnz, const double2 *__restrict__ tlsw, const double2 *__restrict__ thd,
-                                 float4 *__restrict__ tf)
+__global__ void k_float_incoming(int64_t nnz, DevGeom g, const int32_t *__restrict__ tedge,
+                                 const int32_t *__restrict__ tsrc, float4 *__restrict__ tf)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nnz) return;
-    const double2 a = tlsw[t], h = thd[t];
-    tf[t] = make_float4((float)a.x, (float)a.y, (float)(2.0 * h.x), (float)(2.0 * h.y));
+    if (t < nnz) tf[t] = float_incoming(g, tedge[t], tsrc[t]);
 }
 
 unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -1672,49 +1716,72 @@ cudaError_t build_adj_plan(const DevGeom &g, double *plan, int32_t *near_e, doub
     return cudaGetLastError();
 }
 
-cudaError_t build_float_geometry(const DevGeom &g, int64_t nnz, const double2 *tlsw, const double2 *thd, float4 *ef,
+cudaError_t build_float_geometry(const DevGeom &g, int64_t nnz, const int32_t *tedge, const int32_t *tsrc, float4 *ef,
                                  float2 *ea, float4 *tf, cudaStream_t s)
 {
     if (nnz <= 0) return cudaSuccess;
     k_float_edges<<<blocks(g.n, 128), 128, 0, s>>>(g, ef, ea);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    k_float_incoming<<<blocks(nnz, 256), 256, 0, s>>>(nnz, tlsw, thd, tf);
+    k_float_incoming<<<blocks(nnz, 256), 256, 0, s>>>(nnz, g, tedge, tsrc, tf);
+    return cudaGetLastError();
+}
+
+// launches the kernel of T that fits: with the FP32 copies or without
+template <class T, bool GEOM, bool COPIES>
+static void adj_flux_owner(const AdjParamsT<T> &P, cudaStream_t s)
+{
+    if constexpr (std::is_same<T, double>::value) {
+        if (P.g14) {
+            k_adj_flux_pair<GEOM><<<blocks(P.g.n, 64), 128, 0, s>>>(P);
+            return;
+        }
+    }
+    k_adj_flux<T, GEOM, COPIES><<<blocks(P.g.n, 128), 128, 0, s>>>(P);
+}
+template <class T, bool GEOM, bool COPIES>
+static void adj_flux_gather(const AdjParamsT<T> &P, cudaStream_t s)
+{
+    if constexpr (GEOM && std::is_same<T, double>::value) k_adj_flux_gather_pair<<<blocks(P.g.n, 64), 128, 0, s>>>(P);
+    else k_adj_flux_gather<T, GEOM, COPIES><<<blocks(P.g.n, 128), 128, 0, s>>>(P);
+}
+template <class T, bool COPIES>
+static cudaError_t adj_flux(const AdjParamsT<T> &P, bool geom, cudaStream_t s)
+{
+    if (geom) adj_flux_owner<T, true, COPIES>(P, s);
+    else adj_flux_owner<T, false, COPIES>(P, s);
+    const cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+    if (geom && P.order == 2) adj_flux_gather<T, true, COPIES>(P, s);   // (order 1 has no offsets)
+    else adj_flux_gather<T, false, COPIES>(P, s);
     return cudaGetLastError();
 }
 
 template <class T>
 cudaError_t launch_adj_flux(const AdjParamsT<T> &P, bool geom, cudaStream_t s)
 {
-    const unsigned nb = blocks(P.g.n, 128);
-    bool pair = false;
-    if constexpr (std::is_same<T, double>::value) {
-        pair = P.g14 != 0;
-        if (pair && geom) k_adj_flux_pair<true><<<blocks(P.g.n, 64), 128, 0, s>>>(P);
-        if (pair && !geom) k_adj_flux_pair<false><<<blocks(P.g.n, 64), 128, 0, s>>>(P);
+    if constexpr (std::is_same<T, float>::value) {
+        if (!P.ef) return adj_flux<T, false>(P, geom, s);
     }
-    if (!pair && geom) k_adj_flux<T, true><<<nb, 128, 0, s>>>(P);
-    if (!pair && !geom) k_adj_flux<T, false><<<nb, 128, 0, s>>>(P);
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
-    const bool offsets = geom && P.order == 2;   // (order 1 has none)
-    if (!offsets) k_adj_flux_gather<T, false><<<nb, 128, 0, s>>>(P);
-    else if constexpr (std::is_same<T, double>::value) k_adj_flux_gather_pair<<<blocks(P.g.n, 64), 128, 0, s>>>(P);
-    else k_adj_flux_gather<T, true><<<nb, 128, 0, s>>>(P);
-    return cudaGetLastError();
+    return adj_flux<T, true>(P, geom, s);
 }
 
 template <class T>
 cudaError_t launch_adj_grad(const AdjParamsT<T> &P, const T *gprev, const T *gbar_in, T *gbar_out, bool geom,
                             bool first, cudaStream_t s)
 {
+    const int f = first ? 1 : 0;
+    const unsigned nb = blocks(P.g.n, 128);
     if constexpr (std::is_same<T, double>::value) {
-        const dim3 nb(blocks(P.g.n, 64), 2);
-        if (geom) k_adj_grad_fp64<true><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
-        else k_adj_grad_fp64<false><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+        const dim3 pairs(blocks(P.g.n, 64), 2);
+        if (geom) k_adj_grad_fp64<true><<<pairs, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, f);
+        else k_adj_grad_fp64<false><<<pairs, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, f);
+    } else if (P.ef) {
+        if (geom) k_adj_grad_fp32<true, true><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, f);
+        else k_adj_grad_fp32<false, true><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, f);
     } else {
-        if (geom) k_adj_grad_fp32<true><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
-        else k_adj_grad_fp32<false><<<blocks(P.g.n, 128), 128, 0, s>>>(P, gprev, gbar_in, gbar_out, first ? 1 : 0);
+        if (geom) k_adj_grad_fp32<true, false><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, f);
+        else k_adj_grad_fp32<false, false><<<nb, 128, 0, s>>>(P, gprev, gbar_in, gbar_out, f);
     }
     return cudaGetLastError();
 }

@@ -26,13 +26,14 @@ struct AdjParamsT {
     const int32_t *toff;   // [n+1] transpose CSR: incoming edges of each point
     const int32_t *tedge;  // [nnz] edge ids, grouped by destination, in edge order
     const int32_t *tsrc;   // [nnz] owner point of each incoming edge
-    const double2 *tlsw;   // [nnz] lsw of each incoming edge, in the transpose's order
+    const double2 *tlsw;   // [nnz] lsw of each incoming edge, in the transpose's order (or nullptr, with thd)
     const double2 *thd;    // [nnz] half offset of each incoming edge, likewise
     const double *plan;    // [kAdjPlan][n] inverse systems of each point's stencils (k_adj_plan)
     const int32_t *near_e; // [n] edge of the nearest neighbour (the first of equals)
     const double2 *near_u; // [n] (P_i - P_0) / dmin of that edge
     // FP32 product: geometry rounded once, per edge (dx, dy, w_s, w_n) and
-    // (a_x, a_y), per incoming edge (a_x, a_y, dx, dy); nullptr in the FP64 one
+    // (a_x, a_y), per incoming edge (a_x, a_y, dx, dy); nullptr in the FP64 one, and
+    // where there is no memory for them
     const float4 *ef;
     const float2 *ea;
     const float4 *tf;
@@ -53,7 +54,7 @@ cudaError_t build_incoming(const DevGeom &g, int64_t nnz, const int32_t *tedge, 
 // what the reverse of the weights, the limiter and the time step need of the points alone
 cudaError_t build_adj_plan(const DevGeom &g, double *plan, int32_t *near_e, double2 *near_u, cudaStream_t s);
 // the FP32 product's geometry (ef, ea, tf)
-cudaError_t build_float_geometry(const DevGeom &g, int64_t nnz, const double2 *tlsw, const double2 *thd, float4 *ef,
+cudaError_t build_float_geometry(const DevGeom &g, int64_t nnz, const int32_t *tedge, const int32_t *tsrc, float4 *ef,
                                  float2 *ea, float4 *tf, cudaStream_t s);
 // geom (here and below): the cotangents of the weights and offsets are wanted
 // too (wbar, abar, dbar); without it they are left alone. With P.add wbar and

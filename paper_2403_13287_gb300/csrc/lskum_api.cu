@@ -136,12 +136,13 @@ struct lskum_ctx {
     double *vRb = nullptr, *vqb = nullptr, *vgb = nullptr, *vgb2 = nullptr;
     double *vebar = nullptr;
     double2 *vwbar = nullptr, *vabar = nullptr, *vdbar = nullptr;
-    double *vplan = nullptr;
+    double *vplan = nullptr;      // optional: else made in vebar for each product
+    bool extras_tried = false;    // tlsw, thd, vplan and (FP32) fef, fea, ftf: taken once, if there is memory
+    bool fextras_tried = false;
     int32_t *near_e = nullptr;
     double2 *near_u = nullptr;
     int32_t *toff = nullptr, *tedge = nullptr, *tsrc = nullptr;
-    double2 *tlsw = nullptr, *thd = nullptr;  // weights and half offsets of the incoming edges
-    double *vqb2 = nullptr;       // [n][4] owner-side share of the q cotangent (order 2)
+    double2 *tlsw = nullptr, *thd = nullptr;  // weights and half offsets of the incoming edges (optional)
     double *vext = nullptr;       // [n][4] the limiter's extremum measure (limiter_K > 0)
     int32_t *vlidx = nullptr;     // [n][4] limiter reverse: the extreme neighbour's edge
     double *vlval = nullptr;      // [n][4] limiter reverse: its q cotangent
@@ -155,7 +156,7 @@ struct lskum_ctx {
     // FP32 residual VJP (mixed contexts; allocated on the first such call)
     bool fvjp_ready = false;
     float *fq = nullptr, *fG = nullptr, *fRb = nullptr, *fqb = nullptr, *fgb = nullptr, *fgb2 = nullptr, *febar = nullptr;
-    float4 *fef = nullptr, *ftf = nullptr;    // FP32 edge and incoming-edge geometry
+    float4 *fef = nullptr, *ftf = nullptr;    // FP32 edge and incoming-edge geometry (optional)
     float2 *fea = nullptr;
     double *fbuf = nullptr;
 
@@ -262,11 +263,20 @@ static cudaError_t next_event(lskum_ctx *c, cudaEvent_t *ev)
         }                                                                                       \
     } while (0)
 
+static void give_back(lskum_ctx *c);
+
+// an array that the context needs; where memory runs out, the ones that only save
+// time go first
 template <typename T>
 static cudaError_t dalloc(lskum_ctx *c, T **p, size_t count)
 {
     void *v = nullptr;
     cudaError_t e = cudaMalloc(&v, std::max<size_t>(count, 1) * sizeof(T));
+    if (e == cudaErrorMemoryAllocation && !c->optional.empty()) {
+        cudaGetLastError();
+        give_back(c);
+        e = cudaMalloc(&v, std::max<size_t>(count, 1) * sizeof(T));
+    }
     if (e == cudaSuccess) {
         c->allocs.push_back(v);
         *p = static_cast<T *>(v);
@@ -299,6 +309,22 @@ static void free_optional(lskum_ctx *c)
     for (void *p : c->optional) cudaFree(p);
     c->optional.clear();
     c->hfx = nullptr;
+    c->tlsw = c->thd = nullptr;
+    c->vplan = nullptr;
+    c->fef = c->ftf = nullptr;
+    c->fea = nullptr;
+    c->extras_tried = c->fextras_tried = false;
+}
+
+// (captured launches hold the arrays' addresses; a call allocates before it launches)
+static void give_back(lskum_ctx *c)
+{
+    cudaStreamSynchronize(c->stream);
+    for (auto &g : c->graphs) {
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+        g = lskum_ctx::StepGraph{};
+    }
+    free_optional(c);
 }
 
 static void free_all(lskum_ctx *c)
@@ -1413,6 +1439,14 @@ struct Workspace {
         for (const auto &p : parts) *p.first = base + p.second;
         return e;
     }
+    // arrays that only save time: all nullptr where there is no memory for them
+    cudaError_t alloc_optional(lskum_ctx *c) const
+    {
+        char *base = nullptr;
+        const cudaError_t e = optional_alloc(c, &base, bytes);
+        for (const auto &p : parts) *p.first = base ? base + p.second : nullptr;
+        return e;
+    }
 };
 
 static void add_forward(lskum_ctx *c, Workspace &w, lskum_ctx::Forward &f)
@@ -1432,20 +1466,16 @@ static lskum_status vjp_workspace(lskum_ctx *c)
     if (c->cfg.order == 2) {
         w.add(&c->vgb, 8 * n);
         w.add(&c->vgb2, 8 * n);
-        w.add(&c->vqb2, 4 * n);
     }
-    w.add(&c->vRb, 4 * n);
     w.add(&c->vqb, 4 * n);
-    w.add(&c->vebar, 4 * m);
+    // (also the scratch of the plan, 15 values per point, where that is not kept)
+    w.add(&c->vebar, std::max(4 * m, kAdjPlan * n));
     w.add(&c->vwbar, m);
     w.add(&c->vabar, m);
     w.add(&c->vdbar, m);
     w.add(&c->toff, n + 1);
     w.add(&c->tedge, m);
     w.add(&c->tsrc, m);
-    w.add(&c->tlsw, m);
-    w.add(&c->thd, m);
-    w.add(&c->vplan, kAdjPlan * n);
     w.add(&c->near_e, n);
     w.add(&c->near_u, n);
     w.add(&c->vUacc, 4 * n);
@@ -1457,11 +1487,28 @@ static lskum_status vjp_workspace(lskum_ctx *c)
         w.add(&c->vlval, 4 * n);
     }
     CK(c, w.alloc(c));
-    c->launches += 5;
-    LAUNCH(c, build_adj_plan(c->geom(), c->vplan, c->near_e, c->near_u, c->stream));
+    c->vRb = c->Rt;   // (lskum_residual's, which no product uses)
+    c->launches += 4;
     LAUNCH(c, build_transpose_csr(n, c->nnz, c->off, c->idx, c->toff, c->tedge, c->tsrc, c->stream));
-    LAUNCH(c, build_incoming(c->geom(), c->nnz, c->tedge, c->tsrc, c->tlsw, c->thd, c->stream));
     c->vjp_ready = true;
+    return LSKUM_OK;
+}
+
+// what a product needs of the points alone: the nearest neighbours, and (120 B per
+// point and 32 B per edge, where there is memory) the plan of the weights' reverse
+// and the incoming edges' geometry in the order they are read in
+static lskum_status vjp_extras(lskum_ctx *c)
+{
+    if (c->extras_tried) return LSKUM_OK;
+    const int64_t n = c->n, m = std::max<int64_t>(c->nnz, 1);
+    Workspace w;
+    w.add(&c->tlsw, m);
+    w.add(&c->thd, m);
+    w.add(&c->vplan, kAdjPlan * n);
+    CK(c, w.alloc_optional(c));
+    LAUNCH(c, build_adj_plan(c->geom(), c->vplan ? c->vplan : c->vebar, c->near_e, c->near_u, c->stream));
+    if (c->thd) LAUNCH(c, build_incoming(c->geom(), c->nnz, c->tedge, c->tsrc, c->tlsw, c->thd, c->stream));
+    c->extras_tried = true;
     return LSKUM_OK;
 }
 
@@ -1473,7 +1520,9 @@ static AdjParams adj_params(lskum_ctx *c, const lskum_ctx::Forward &f)
     P.qg = vjp_final_gradient(c, f);
     P.Rbar = c->vRb;
     P.qbar = c->vqb;
-    P.qbar2 = c->vqb2;
+    // (ebar is read for the last time before the gradient passes start qbar2; every
+    // point has an edge)
+    P.qbar2 = c->cfg.order == 2 ? c->vebar : nullptr;
     P.gbar = c->vgb;
     P.ebar = c->vebar;
     P.wbar = c->vwbar;
@@ -1484,7 +1533,7 @@ static AdjParams adj_params(lskum_ctx *c, const lskum_ctx::Forward &f)
     P.tsrc = c->tsrc;
     P.tlsw = c->tlsw;
     P.thd = c->thd;
-    P.plan = c->vplan;
+    P.plan = c->vplan ? c->vplan : c->vebar;
     P.near_e = c->near_e;
     P.near_u = c->near_u;
     P.perm = c->perm;
@@ -1557,13 +1606,26 @@ static lskum_status fvjp_workspace(lskum_ctx *c)
     w.add(&c->fRb, 4 * n);
     w.add(&c->fqb, 4 * n);
     w.add(&c->febar, 4 * m);
+    CK(c, w.alloc(c));
+    c->fvjp_ready = true;
+    return LSKUM_OK;
+}
+
+// the FP32 copies of the geometry (40 B per edge, where there is memory)
+static lskum_status fvjp_extras(lskum_ctx *c)
+{
+    if (c->fextras_tried) return LSKUM_OK;
+    const int64_t m = std::max<int64_t>(c->nnz, 1);
+    Workspace w;
     w.add(&c->fef, m);
     w.add(&c->fea, m);
     w.add(&c->ftf, m);
-    CK(c, w.alloc(c));
-    c->launches++;
-    LAUNCH(c, build_float_geometry(c->geom(), c->nnz, c->tlsw, c->thd, c->fef, c->fea, c->ftf, c->stream));
-    c->fvjp_ready = true;
+    CK(c, w.alloc_optional(c));
+    if (c->fef) {
+        c->launches++;
+        LAUNCH(c, build_float_geometry(c->geom(), c->nnz, c->tedge, c->tsrc, c->fef, c->fea, c->ftf, c->stream));
+    }
+    c->fextras_tried = true;
     return LSKUM_OK;
 }
 
@@ -1575,7 +1637,7 @@ static lskum_status vjp_residual_fp32(lskum_ctx *c, const double *Ui, double *Ub
     const bool second = c->cfg.order == 2;
     const int K = second ? c->cfg.inner_iters : 0;
     lskum_status st = fvjp_workspace(c);
-    if (st != LSKUM_OK) return st;
+    if (st != LSKUM_OK || (st = fvjp_extras(c)) != LSKUM_OK) return st;
     const MixedGeom mg = c->mgeom();
     LAUNCH(c, launch_q_from_U_mixed(n, c->gas, Ui, c->fq, c->status, c->stream));
     if (second) {
@@ -1663,6 +1725,7 @@ static lskum_status vjp_residual(lskum_ctx *c, const double *Ui, double *Ub_acc,
 // them, so the four residuals of an RK4 step share it (40k points: 94 us each)
 static lskum_status vjp_weights(lskum_ctx *c)
 {
+    if (!c->vplan) LAUNCH(c, build_adj_plan(c->geom(), c->vebar, c->near_e, c->near_u, c->stream));
     LAUNCH(c, launch_adj_weights(adj_params(c, c->fw[0]), c->stream));
     return LSKUM_OK;
 }
@@ -1673,7 +1736,7 @@ static lskum_status vjp_begin(lskum_ctx *c)
         return fail(c, LSKUM_ERR_ARG, "derivatives need boundary = 0 (the mirror images are not differentiated)");
     lskum_status st = vjp_workspace(c);
     if (st != LSKUM_OK) return st;
-    if ((st = reset_status(c)) != LSKUM_OK) return st;
+    if ((st = vjp_extras(c)) != LSKUM_OK || (st = reset_status(c)) != LSKUM_OK) return st;
     CK(c, cudaMemsetAsync(c->vdbar, 0, std::max<int64_t>(c->nnz, 1) * sizeof(double2), c->stream));
     CK(c, cudaMemsetAsync(c->vpxy, 0, c->n * sizeof(double2), c->stream));
     CK(c, cudaMemsetAsync(c->vUacc, 0, 4 * c->n * sizeof(double), c->stream));
@@ -1888,8 +1951,7 @@ extern "C" lskum_status lskum_set_lean(lskum_ctx *c, int lean)
     if (lean != 0 && lean != 1) return fail(c, LSKUM_ERR_ARG, "lean must be 0 or 1");
     if (c->lean == (lean == 1)) return LSKUM_OK;
     CK(c, cudaStreamSynchronize(c->stream));
-    drop_graphs(c);   // captured launches hold the arrays' addresses
-    free_optional(c);
+    give_back(c);
     c->lean = lean == 1;
     return fixed_offsets(c);
 }

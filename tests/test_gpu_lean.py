@@ -64,3 +64,30 @@ def test_lean_takes_0_or_1():
     assert s._L.lskum_set_lean(s._ctx, 2) == LSKUM_ERR_ARG and s._L.lskum_set_lean(s._ctx, -1) == LSKUM_ERR_ARG
     assert s._L.lskum_set_lean(None, 1) == LSKUM_ERR_ARG
     s.close()
+
+
+@pytest.mark.parametrize("precision,fp32,limiter,order,gamma", [(0, False, 1.0, 2, 1.4), (0, False, 0.0, 1, 1.4),
+                                                                (0, False, 0.0, 2, 1.3), (1, True, 0.0, 2, 1.4), (1, False, 0.0, 2, 1.4)])
+def test_products_are_the_same_without_optional_arrays(precision, fp32, limiter, order, gamma):
+    """Residual product (FP64 of both contexts, FP32), U alone and with coordinates:
+    with the arrays, without, and with them again on one context."""
+    import torch
+
+    from paper_2403_13287_gb300.lskum import Solver
+    c = naca0012_cloud(180, 99, seed=3, shuffle=True)
+    U = torch.from_numpy(smooth_state(c, 0.85, 1.0, amp=0.05, seed=9, gamma=gamma)).cuda()
+    Rb = torch.from_numpy(np.random.default_rng(1).standard_normal((4, c["n"]))).cuda()
+    s = Solver(c, order=order, inner_iters=3 if order == 2 else 0, limiter_K=limiter, mach=0.85, aoa_deg=1.0, gamma=gamma,
+               reorder=1, precision=precision)
+    got = []
+    for lean in (None, True, False):
+        if lean is not None:
+            s.set_lean(lean)
+        for _ in range(2):
+            out = s.residual_vjp(Rb, U, fp32=fp32)
+            got.append([t.cpu().numpy() for t in out] + [s.residual_vjp(Rb, U, want_xy=False, fp32=fp32)[0].cpu().numpy()])
+            s.residual(U)
+    s.close()
+    for other in got[1:]:
+        for p, q in zip(got[0], other):
+            assert np.array_equal(p, q)
