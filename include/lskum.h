@@ -258,9 +258,9 @@ lskum_status lskum_residual_vjp(lskum_ctx *ctx, const double *U, const double *R
  *   U_bar       device float64[4*n] in input order (written), or NULL
  *   x_bar, y_bar  device float64[n] in input order (written, or added into with
  *                 flags = LSKUM_VJP_ACCUMULATE_XY), or NULL
- * Workspace: about 0.45 KB per point more than lskum_residual_vjp, and for RK4
- * 0.9 KB (K = 3; 1.1 KB with the limiter) for the stages' forward iterates where
- * the device has it, allocated on the first call. Does not change the context's state.
+ * Workspace: 0.43 KB per point more than lskum_residual_vjp, allocated on the first
+ * call, and for RK4 0.86 KB (K = 3; 1.06 KB with the limiter) for the stages' forward
+ * iterates, which only save time (lskum_set_lean). Does not change the context's state.
  */
 lskum_status lskum_step_vjp(lskum_ctx *ctx, const double *U, const double *U_bar_next, double *U_bar,
                             double *x_bar, double *y_bar, int flags);

@@ -132,7 +132,7 @@ struct lskum_ctx {
         double *q = nullptr, *G = nullptr, *Glim = nullptr;
     };
     Forward fw[4];
-    bool stage_forwards = false;  // fw[1..3] are there (else a stage's forward is run again)
+    bool forwards_tried = false;  // fw[1..3] are optional: without them a stage's forward is run again
     double *vRb = nullptr, *vqb = nullptr, *vgb = nullptr, *vgb2 = nullptr;
     double *vebar = nullptr;
     double2 *vwbar = nullptr, *vabar = nullptr, *vdbar = nullptr;
@@ -313,7 +313,8 @@ static void free_optional(lskum_ctx *c)
     c->vplan = nullptr;
     c->fef = c->ftf = nullptr;
     c->fea = nullptr;
-    c->extras_tried = c->fextras_tried = false;
+    for (int k = 1; k < 4; ++k) c->fw[k] = lskum_ctx::Forward{};
+    c->extras_tried = c->fextras_tried = c->forwards_tried = false;
 }
 
 // (captured launches hold the arrays' addresses; a call allocates before it launches)
@@ -1796,17 +1797,19 @@ static lskum_status step_vjp_workspace(lskum_ctx *c)
     w.add(&c->sdt, n);
     w.add(&c->sdtb, n);
     CK(c, w.alloc(c));
-    if (c->cfg.time_scheme == 1) {
-        // a forward per RK stage spares running it again in the reverse sweep;
-        // without the memory for them that is what happens
-        Workspace stages;
-        for (int k = 1; k < 4; ++k) add_forward(c, stages, c->fw[k]);
-        const cudaError_t e = stages.alloc(c);
-        if (e != cudaSuccess && e != cudaErrorMemoryAllocation) CK(c, e);
-        if (e == cudaErrorMemoryAllocation) cudaGetLastError();
-        c->stage_forwards = e == cudaSuccess;
-    }
     c->svjp_ready = true;
+    return LSKUM_OK;
+}
+
+// a forward per RK stage (where there is memory) spares running it again in the
+// reverse sweep
+static lskum_status stage_forwards(lskum_ctx *c)
+{
+    if (c->forwards_tried || c->cfg.time_scheme != 1) return LSKUM_OK;
+    Workspace w;
+    for (int k = 1; k < 4; ++k) add_forward(c, w, c->fw[k]);
+    CK(c, w.alloc_optional(c));
+    c->forwards_tried = true;
     return LSKUM_OK;
 }
 
@@ -1820,7 +1823,7 @@ extern "C" lskum_status lskum_step_vjp(lskum_ctx *c, const double *U, const doub
     if (!U_bar && !x_bar && !y_bar) return LSKUM_OK;
     lskum_status st = vjp_begin(c);
     if (st != LSKUM_OK) return st;
-    if ((st = step_vjp_workspace(c)) != LSKUM_OK) return st;
+    if ((st = step_vjp_workspace(c)) != LSKUM_OK || (st = stage_forwards(c)) != LSKUM_OK) return st;
     const int64_t n = c->n;
     const bool geom = x_bar || y_bar;
     const double *Un = c->U;
@@ -1847,7 +1850,7 @@ extern "C" lskum_status lskum_step_vjp(lskum_ctx *c, const double *U, const doub
     } else {
         // U_{k+1} = P(U^n - c_k dt R_k), R_{k+1} = R(U_{k+1}); U_{k+1} is kept in sU[k]
         const double cst[3] = {0.5, 0.5, 1.0};
-        const bool kept = c->stage_forwards;
+        const bool kept = c->fw[1].q != nullptr;
         for (int k = 0; k < 3; ++k) {
             LAUNCH(c, launch_stage_fwd(S, Un, c->sR[k], cst[k], c->sU[k], c->stream));
             if ((st = residual_fp64(c, c->sU[k], c->sR[k + 1], c->fw[kept ? k + 1 : 0])) != LSKUM_OK) return st;

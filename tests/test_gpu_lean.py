@@ -91,3 +91,51 @@ def test_products_are_the_same_without_optional_arrays(precision, fp32, limiter,
     for other in got[1:]:
         for p, q in zip(got[0], other):
             assert np.array_equal(p, q)
+
+
+@pytest.mark.parametrize("limiter,order,time_scheme,want_xy", [(0.0, 2, 1, True), (1.0, 2, 1, True), (1.0, 2, 1, False),
+                                                               (0.0, 1, 1, True), (1.0, 2, 0, True)])
+def test_step_products_are_the_same_without_optional_arrays(limiter, order, time_scheme, want_xy):
+    """With every RK stage's forward kept, and with each run again in the reverse
+    sweep: the same bits, first product and repeated ones, another state in between."""
+    import torch
+
+    from paper_2403_13287_gb300.lskum import Solver
+    c = naca0012_cloud(130, 24, seed=11, shuffle=True)
+    U = [torch.from_numpy(smooth_state(c, 0.85, 1.0, amp=0.05, seed=k)).cuda() for k in (9, 10)]
+    bar = torch.from_numpy(np.random.default_rng(1).standard_normal((4, c["n"]))).cuda()
+    kw = dict(order=order, inner_iters=3 if order == 2 else 0, time_scheme=time_scheme, limiter_K=limiter, mach=0.85,
+              aoa_deg=1.0, reorder=1)
+    got = []
+    kept, lean = Solver(c, **kw), Solver(c, **kw)
+    lean.set_lean()
+    for s in (kept, lean):
+        got.append([t.cpu().numpy() for u in (U[0], U[1], U[0]) for t in s.step_vjp(bar, U=u, want_xy=want_xy) if t is not None])
+    kept.set_lean()
+    got.append([t.cpu().numpy() for u in (U[0], U[1], U[0]) for t in kept.step_vjp(bar, U=u, want_xy=want_xy) if t is not None])
+    kept.close()
+    lean.close()
+    for other in got[1:]:
+        assert len(other) == len(got[0])
+        for p, q in zip(got[0], other):
+            assert np.array_equal(p, q)
+
+
+def test_products_give_their_memory_back():
+    """120 B per point and 32 B per edge of the plan and the incoming edges, 1056 B per
+    point of the stages' forwards (limited, K = 3), 16 B per edge of the context."""
+    import torch
+
+    from paper_2403_13287_gb300.lskum import Solver
+    c = naca0012_cloud(512, 311, seed=3)
+    U = torch.from_numpy(smooth_state(c, 0.85, 1.0, amp=0.05, seed=9)).cuda()
+    bar = torch.ones_like(U)
+    s = Solver(c, order=2, inner_iters=3, time_scheme=1, limiter_K=1.0, mach=0.85, aoa_deg=1.0, reorder=1)
+    s.step_vjp(bar, U=U)
+    torch.cuda.empty_cache()
+    free0 = torch.cuda.mem_get_info()[0]
+    s.set_lean()
+    given = torch.cuda.mem_get_info()[0] - free0
+    s.close()
+    want = (120 + 1056) * c["n"] + (32 + 16) * c["nbr_idx"].size
+    assert abs(given - want) <= 8 << 20, (given, want)
