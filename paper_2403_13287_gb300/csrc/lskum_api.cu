@@ -214,6 +214,7 @@ static lskum_status fail(lskum_ctx *c, lskum_status st, const char *fmt, ...)
 #define CK(c, call)                                                                             \
     do {                                                                                        \
         cudaError_t e_ = (call);                                                                \
+        if (e_ == cudaErrorMemoryAllocation) cudaGetLastError(); /* not the next call's error */ \
         if (e_ != cudaSuccess)                                                                  \
             return fail((c), e_ == cudaErrorMemoryAllocation ? LSKUM_ERR_OOM : LSKUM_ERR_CUDA,  \
                         "%s failed: %s", #call, cudaGetErrorString(e_));                         \
@@ -1487,10 +1488,16 @@ static lskum_status vjp_workspace(lskum_ctx *c)
         w.add(&c->vlidx, 4 * n);
         w.add(&c->vlval, 4 * n);
     }
-    CK(c, w.alloc(c));
+    if (!c->vRb) CK(c, w.alloc(c));
     c->vRb = c->Rt;   // (lskum_residual's, which no product uses)
     c->launches += 4;
-    LAUNCH(c, build_transpose_csr(n, c->nnz, c->off, c->idx, c->toff, c->tedge, c->tsrc, c->stream));
+    cudaError_t transpose_csr = build_transpose_csr(n, c->nnz, c->off, c->idx, c->toff, c->tedge, c->tsrc, c->stream);
+    if (transpose_csr == cudaErrorMemoryAllocation && !c->optional.empty()) {   // (its sort takes memory for a moment)
+        cudaGetLastError();
+        give_back(c);
+        transpose_csr = build_transpose_csr(n, c->nnz, c->off, c->idx, c->toff, c->tedge, c->tsrc, c->stream);
+    }
+    LAUNCH(c, transpose_csr);
     c->vjp_ready = true;
     return LSKUM_OK;
 }
