@@ -23,7 +23,7 @@
 // the range that each n leaves room for. A product's high word drops less than
 // 1.25 units of its Qn.
 //
-// Taken when fix_state says so: beta in [2^-40, 2^40), S_t^2 + S_n^2 < 15.875
+// Taken when fix_state says so: beta in [2^-80, 2^80), S_t^2 + S_n^2 < 15.875
 // with each component of sqrt(beta) (u, v) below 3.9375 (Mach 4.7), |q1| < 32,
 // i.e. every state such flows meet; the FP64 form takes the others. The same
 // code compiles on the host, where it is tested against multiple precision.

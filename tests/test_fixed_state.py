@@ -46,3 +46,44 @@ def test_quotient_rounds_once(lib):
     lib.fixed_quotient(ctypes.c_long(m), _ptr(bad), _ptr(r), _ptr(q), _ptr(ok))
     assert not ok.any()
 
+
+
+def test_ends_of_the_accepted_range(tmp_path):
+    """States at the ends of what fix_state takes: beta = -q4/2 from 2^-80 up to (not
+    including) 2^80, |q1| just below 32, |S|^2 up to 15.4. Against multiple precision
+    at the bound of the flux tests; one step outside is left to the FP64 form."""
+    mp = pytest.importorskip("mpmath")
+    import test_fixed_flux as flux
+    mp.mp.dps = 40
+    out = str(tmp_path / "libfixed.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC, "-o", out,
+                    os.path.join(HERE, "fixed_flux_shim.cpp")], check=True)
+    so = ctypes.CDLL(out)
+
+    def shim(qi, q0, nx, ny, along, sgn):
+        n = len(nx)
+        a = [np.ascontiguousarray(v, dtype=np.float64) for v in (qi, q0, nx, ny)]
+        b = [np.ascontiguousarray(v, dtype=np.int32) for v in (along, sgn)]
+        dG, ok = np.zeros((n, 4)), np.zeros(n, dtype=np.int32)
+        so.fixed_flux(ctypes.c_long(n), *[_ptr(v) for v in a + b + [dG, ok]])
+        return dG, ok.astype(bool)
+
+    rng = np.random.default_rng(12)
+
+    def states(beta, n):
+        a, S = rng.uniform(0, 2 * np.pi, n), np.sqrt(rng.uniform(0, 15.4, n))
+        q1 = rng.choice([-31.99, 31.99, 0.3], n) + 0.005 * rng.uniform(-1, 1, n)
+        return np.stack([q1, 2 * S * np.cos(a) * np.sqrt(beta), 2 * S * np.sin(a) * np.sqrt(beta), -2 * beta], axis=-1)
+
+    n = 96
+    ends = [2.0 ** -80, np.nextafter(2.0 ** -79, 0), 2.0 ** -79 * 1.5, 2.0 ** 79, np.nextafter(2.0 ** 80, 0), 2.0 ** 78 * 1.25, 1.0]
+    for beta in ends:
+        q = states(np.full(n, beta), n)
+        near = q * np.array([1, 1 + 1e-5, 1 - 1e-5, 1])
+        flux._check(shim, q, near, rng)
+    flux._check(shim, states(rng.choice(ends[:3], n), n), states(rng.choice(ends[3:6], n), n), rng)   # one state at each end
+    good = states(np.ones(4), 4)
+    one = np.ones(4)
+    for beta in (np.nextafter(2.0 ** -80, 0), 2.0 ** 80):
+        q = states(np.full(4, beta), 4)
+        assert not shim(q, good, one, 0 * one, one, one)[1].any() and not shim(good, q, one, 0 * one, one, one)[1].any()
