@@ -103,7 +103,7 @@ def main():
         lines.append("    {%dll, %du, 0}," % (int(mp.nint(mp.ldexp(-mp.log(mp.ldexp(mp.mpf(r), -32)) / mp.log(2), 60))), r))
     lines.append("};")
     c = [(-1) ** (n + 1) / (n * mp.log(2)) * mp.mpf(2) ** (-11 * n) for n in range(1, 6)]
-    lines.append("// log2(1 + z) = u (c_1 + u (c_2 + u (c_3 + u (c_4 + u c_5)))): c_1 2^72, c_2 2^84, c_3 2^64, c_4 2^65, c_5 2^66; ln2 2^63")
+    lines.append("// log2(1 + z) = u (c_1 + u (c_2 + u (c_3 + u (c_4 + u c_5)))): c_1 2^72, c_2 2^84, c_3 2^64, c_4 2^66, c_5 2^68; ln2 2^63")
     for n, q in zip(range(1, 6), (72, 84, 64, 66, 68)):
         lines.append("#define LSKUM_FIX_LOG_C%d %d%s" % (n, int(mp.nint(mp.ldexp(c[n - 1], q))), "ll" if n < 3 else ""))
     lines.append("#define LSKUM_FIX_LN2 %dll" % int(mp.nint(mp.ldexp(mp.log(2), 63))))

@@ -363,7 +363,6 @@ __device__ __forceinline__ void store_c(double *a, const double v[C])
         *a = v[0];
     }
 }
-// components k0 .. k0 + C - 1 (k0 a multiple of C) without an indexed array in memory
 
 // double -> float, round to nearest (ties away), on the integer pipe for
 // magnitudes of 2^-100 to 2^100 and for 0; the conversion instruction (FP64

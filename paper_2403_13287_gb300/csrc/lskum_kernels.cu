@@ -1,7 +1,8 @@
 // Hot-path kernels of q-LSKUM (arXiv 2403.13287): q-derivatives (E14, E15),
 // the fused flux residual + state update (E10-E12, E16 / RK4) and the
-// reductions (residue, forces). One thread per point; the neighbour loop
-// gathers q, q-derivatives and coordinates of the stencil.
+// reductions (residue, forces). One to four pairs of lanes per point in the flux
+// kernel, two or four lanes in the q-derivative passes; the neighbour loop gathers
+// q, q-derivatives and offsets of the stencil.
 #include "lskum_device.cuh"
 #include "lskum_fixed.cuh"
 #include "lskum_kernels.h"
@@ -66,6 +67,7 @@ __device__ __forceinline__ void image_q(const DevGeom &g, int e, uint8_t m, doub
 // 1/64 of the integer ALU rate, so the stencil extrema take this form.
 __device__ __forceinline__ long long order_key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffLL); }
 
+// components k0 .. k0 + C - 1 (k0 a multiple of C) without an indexed array in memory
 template <int C>
 __device__ __forceinline__ void components(const double v[4], int k0, double o[C])
 {

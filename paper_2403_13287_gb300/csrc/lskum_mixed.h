@@ -82,7 +82,7 @@ cudaError_t launch_sell_fill(int64_t n, const int32_t *off, const int32_t *slice
                              const uint8_t *mask, const float2 *dxy, const float2 *lsw, const float2 *fxw,
                              const double2 *fxw64, const MixedGeom &m, cudaStream_t s);
 // launch-shape variants (threads per block, minimum resident blocks per SM);
-// kernel_class 0 = flux, 1 = q-derivatives; variant 0 is the default
+// kernel_class 0 = flux, 1 = q-derivatives (whose default is variant 0)
 int mixed_variants(int kernel_class);
 int mixed_default_flux(int64_t n, bool kinetic);  // flux variant of an untuned context
 void mixed_variant_shape(int kernel_class, int variant, int *threads, int *min_blocks);
