@@ -646,6 +646,31 @@ def summary_of(line, forms):
     return out
 
 
+LINE_LIMIT = 2900   # characters: readers that keep the last 3000 of the output get the whole line
+
+
+def _rounded(v):
+    if isinstance(v, dict):
+        return {k: _rounded(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [_rounded(x) for x in v]
+    return float("%.6g" % v) if isinstance(v, float) else v
+
+
+def split_line(line):
+    """(the line for standard output, the details for standard error): what the run
+    measured in full is in the details; the line keeps its own form, with side
+    figures to six digits, and the other forms' headline figures (summary)."""
+    out = {k: v for k, v in line.items() if k not in ("forms", "kernels", "tuning", "measured_fma_peaks_gflops")}
+    exact = {k: out[k] for k in ("value", "ms_per_step") if k in out}
+    keep = ("bound", "kernel", "achieved", "peak", "unit", "frac", "hbm_frac")
+    if "roofline" in out:
+        out["roofline"] = {k: out["roofline"][k] for k in keep if k in out["roofline"]}
+    if "cpu_baseline" in out:
+        out["cpu_baseline"] = {k: out["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind") if k in out["cpu_baseline"]}
+    return dict(_rounded(out), **exact), {"details": line}
+
+
 def measure_mixed_error(args, cloud, tuning, stream):
     """The error of the mixed form beside its speedup: on the bench cloud
     after the warm-up plus timed iterations from the timed start state, and
@@ -1111,7 +1136,9 @@ def run_ours(args, rank, world, local):
         m = oracle.split_stencils(cloud)
         line["cpu_baseline"] = cpu_baseline_sample(cloud, m, args)
     line["summary"] = summary_of(line, forms)
-    print(json.dumps(line), flush=True)
+    short, details = split_line(line)
+    print(json.dumps(details), file=sys.stderr, flush=True)
+    print(json.dumps(short), flush=True)
     if dist:
         dist.destroy_process_group()
     return 0
