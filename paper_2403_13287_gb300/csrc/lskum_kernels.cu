@@ -174,7 +174,7 @@ __device__ __forceinline__ void largest_shift_screened(const DevGeom &g, int e0,
 // and component the inner pass keeps two FP64 fused multiply-adds (s -= a c);
 // c = h . grad q_i comes from the integer pipes (fix_dot), q_i - q_0 of the
 // first pass too where it is exact, and the limiter's quotient (fix_phi): pass
-// average 0.700 -> 0.444 ms at 2.5 million points.
+// average 0.700 -> 0.456 ms at 2.5 million points.
 // LANES lanes per point, 4 / LANES components each: every lane runs the point's
 // whole edge loop in row order, so the arithmetic of a component is the same
 // bit for bit whatever LANES is, and a small cloud spreads over more warps with
@@ -725,7 +725,7 @@ struct Members {
 // the sums, the state update), the integer multipliers (62 %) and ALUs (58 %),
 // 66 % of the issue slots; at a few thousand points one warp's chain of rounds.
 // 64 registers and a few spills, for 32 warps per SM, beat 80 (24 warps) and 128
-// (16): 2.14 ms at 2.5 million points, before the last changes 2.30 / 2.48 / 2.67.
+// (16): 2.30 / 2.48 / 2.67 ms at 2.5 million points when they were compared, 2.20 now.
 // One lane per member with both states took 2.58 ms and a chain twice as long.
 // Two lanes per member (member_difference), PAIRS pairs of lanes per point. With
 // one pair the members of a row follow one another; with 2 or 4 each pair takes
@@ -1069,11 +1069,11 @@ cudaError_t launch_qgrad(const DevGeom &g, const double *q, const double *qg_old
     const int pass = inner ? (QG_INNER | (limit ? QG_LIMIT : 0)) : limit ? QG_LIMIT : ext ? QG_EXTREMA : 0;
     // Lanes per point (the same bits either way). A small cloud is bound by the
     // serial chain of a warp and by idle SMs, and 4 lanes shorten the one and
-    // fill the other: pass average 14.8 against 18.9 us at 3k points, 18.4
-    // against 19.4 at 40k. From 64k on (23.8 against 23.3 us; 0.497 against 0.444 ms at
-    // 2.5M) the index, weight and offset work that every lane repeats counts
-    // more. One lane with all four components: 27 us at 3k, 0.450 ms at 2.5M.
-    const bool four = g.n < 60000;
+    // fill the other: pass average 14.4 against 18.8 us at 3k points, 18.0
+    // against 19.7 at 40k, 28.8 against 30.3 at 93k. From there on (both 42.0 us at
+    // 160k, 74.8 against 72.8 at 320k) the index, weight and offset work that every
+    // lane repeats counts more. One lane with all four components: 27 us at 3k.
+    const bool four = g.n < 120000;
     if (g.ioff) {
         if (four) qgrad_pass<true, 4>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, raw, s);
         else qgrad_pass<true, 2>(pass, g, q, qg_old, g1, qg_new, ext, limiter_K, raw, s);
@@ -1107,9 +1107,9 @@ cudaError_t launch_flux(const DevGeom &g, const Gas &gas, const FluxLaunch &L, c
     P.cfl = L.cfl; P.order = L.order; P.mode = L.mode; P.stage = L.stage;
     // Pairs of lanes per point (the same bits whichever): more while the cloud
     // leaves SMs idle and the launch is one warp's serial chain. 4 / 2 pairs take
-    // 26 / 38 us at 3k points, 34 / 43 at 10k, 53 / 46 at 20k and 81 / 69 at 40k,
-    // 2 / 1 pairs 93 / 96 at 64k, 123 / 131 at 93k, 190 / 188 at 160k and 348 /
-    // 322 at 320k (lanes without a member in a point's last round). 8 pairs gain
+    // 25 / 38 us at 3k points, 33 / 42 at 10k, 53 / 46 at 20k and 81 / 70 at 40k,
+    // 2 / 1 pairs 96 / 95 at 64k, 127 / 130 at 93k, 194 / 187 at 160k and 357 /
+    // 323 at 320k (lanes without a member in a point's last round). 8 pairs gain
     // 1.4 us at 3k and lose above.
     if (!gas.g14) {
         if (g.ioff) k_flux_update_fp64<true><<<blocks_for(g.n, 128), 128, 0, s>>>(P);
