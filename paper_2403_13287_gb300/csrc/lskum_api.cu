@@ -1738,13 +1738,15 @@ static lskum_status vjp_weights(lskum_ctx *c)
     return LSKUM_OK;
 }
 
-static lskum_status vjp_begin(lskum_ctx *c)
+// extras: the product reads the plan, the nearest neighbours or the FP64 copies
+static lskum_status vjp_begin(lskum_ctx *c, bool extras)
 {
     if (c->kinetic)
         return fail(c, LSKUM_ERR_ARG, "derivatives need boundary = 0 (the mirror images are not differentiated)");
     lskum_status st = vjp_workspace(c);
     if (st != LSKUM_OK) return st;
-    if ((st = vjp_extras(c)) != LSKUM_OK || (st = reset_status(c)) != LSKUM_OK) return st;
+    if (extras && (st = vjp_extras(c)) != LSKUM_OK) return st;
+    if ((st = reset_status(c)) != LSKUM_OK) return st;
     CK(c, cudaMemsetAsync(c->vdbar, 0, std::max<int64_t>(c->nnz, 1) * sizeof(double2), c->stream));
     CK(c, cudaMemsetAsync(c->vpxy, 0, c->n * sizeof(double2), c->stream));
     CK(c, cudaMemsetAsync(c->vUacc, 0, 4 * c->n * sizeof(double), c->stream));
@@ -1770,7 +1772,8 @@ extern "C" lskum_status lskum_residual_vjp(lskum_ctx *c, const double *U, const 
     c->err.clear();
     if (!R_bar) return fail(c, LSKUM_ERR_ARG, "R_bar is NULL");
     if (!U_bar && !x_bar && !y_bar) return LSKUM_OK;
-    lskum_status st = vjp_begin(c);
+    const bool geom = x_bar || y_bar;
+    lskum_status st = vjp_begin(c, geom || !(flags & LSKUM_VJP_FP32));
     if (st != LSKUM_OK) return st;
     const double *Ui = c->U;
     if (U) {
@@ -1778,7 +1781,6 @@ extern "C" lskum_status lskum_residual_vjp(lskum_ctx *c, const double *U, const 
         Ui = c->Ut;
     }
     LAUNCH(c, launch_state_in(c->n, c->perm, R_bar, c->vRb, c->stream));
-    const bool geom = x_bar || y_bar;
     if (flags & LSKUM_VJP_FP32) {
         if (!c->mixed) return fail(c, LSKUM_ERR_ARG, "the FP32 product needs a mixed-precision context");
         if (limited(c))
@@ -1828,7 +1830,7 @@ extern "C" lskum_status lskum_step_vjp(lskum_ctx *c, const double *U, const doub
     c->err.clear();
     if (!U_bar_next) return fail(c, LSKUM_ERR_ARG, "U_bar_next is NULL");
     if (!U_bar && !x_bar && !y_bar) return LSKUM_OK;
-    lskum_status st = vjp_begin(c);
+    lskum_status st = vjp_begin(c, true);
     if (st != LSKUM_OK) return st;
     if ((st = step_vjp_workspace(c)) != LSKUM_OK || (st = stage_forwards(c)) != LSKUM_OK) return st;
     const int64_t n = c->n;
