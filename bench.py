@@ -210,10 +210,10 @@ def algorithmic_bytes_per_point_mixed(kernel, dbar, order, scheme):
 # of its warp instructions), the flops among them (2 DFMA + DMUL + DADD) and all
 # warp instructions issued per edge; DRAM bytes per point of one full-size 2.5M
 # launch (single-pass capture, profiles/launch_list_naca0012_2p5m_fp64.md).
-FP64_INSTR_PER_EDGE_FLUX = 39.91
-FP64_FLOPS_PER_EDGE_FLUX = 54.72
-FP64_FLUX_WARP_INSTR_PER_EDGE = 90.68
-FLUX_DRAM_BYTES_PER_POINT = 626.2
+FP64_INSTR_PER_EDGE_FLUX = 44.90
+FP64_FLOPS_PER_EDGE_FLUX = 58.49
+FP64_FLUX_WARP_INSTR_PER_EDGE = 91.73
+FLUX_DRAM_BYTES_PER_POINT = 613.9
 # FP64 peak: ncu's DFMA unit count, 304 FP64 thread-instructions per cycle
 # (each DFMA 2 flops), at the 2070 MHz maximum SM clock
 FP64_PEAK_GINSTR = 304 * 2.070

@@ -221,7 +221,7 @@ lskum_status lskum_residual(lskum_ctx *ctx, const double *U, double *R);
  * With limiter_K > 0 the limiter is differentiated too (FP64 product only;
  * LSKUM_ERR_ARG with LSKUM_VJP_FP32): it is piecewise smooth, and the
  * product is that of the branch the forward takes, with the forward's
- * choices (the first stencil extremum, the first largest reconstruction
+ * choices (the first extreme q of the stencil, the first largest reconstruction
  * shift, the first nearest neighbour in row order). Its workspace (0.52 KB per
  * point plus 88 B per edge for K = 3: 0.8 GB at 640k points; 0.14 KB per point
  * more with the limiter; the FP32 product adds 0.24 KB per point and 16 B per

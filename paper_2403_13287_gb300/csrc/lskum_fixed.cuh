@@ -5,11 +5,12 @@
 // SM, measured; FP32 and logic 128, 32 x 32 -> 64 multiply-add 41-64), so the
 // FP64 split fluxes left 90 % of the issue slots empty while the FP64 pipe was
 // full. A 64 x 64 product keeping the high word costs three wide multiply-adds
-// and two adds, 3-4 cycles instead of 16, and keeps 60 bits where a double
-// keeps 53. The result is rounded to a double once per component. The flux
-// launch went from 178 to 40 FP64 instructions per edge and from 6.82 to
-// 2.14 ms at 2.5 million points (second order, RK4), its error against multiple
-// precision is 2-8 times below that of the FP64 chain.
+// and two adds, 3-4 cycles instead of 16, and keeps 60 bits of its format's range
+// where a double keeps 53 of its own size. The result is rounded to a double once
+// per component. The flux launch went from 178 to 45 FP64 instructions per edge and
+// from 6.82 to 2.20 ms at 2.5 million points (second order, RK4), its error against
+// multiple precision is 2-8 times below that of the FP64 chain (slow transverse
+// momenta, where it would not be, are left to FP64: fix_slow).
 //
 // With r = beta^(-1/2), S_t = u.t sqrt(beta), S_n likewise, every flux is a
 // bounded function of (S_t, S_n) times a power of r times rho. For a direction
