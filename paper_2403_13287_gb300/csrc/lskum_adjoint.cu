@@ -1112,7 +1112,7 @@ __global__ void __launch_bounds__(128, GEOM ? 7 : 8) k_adj_grad_fp64(AdjParams P
                 const bool start = first && !P.add;
                 // (a lane starts one sum and ends, and stores, the other)
                 double *const ab = reinterpret_cast<double *>(P.abar + e), *const db = reinterpret_cast<double *>(P.dbar + e);
-                const double a1 = half_dot(l, s, gx, gy, start ? 0.0 : ab[l]);
+                const double a1 = half_dot(l, s, gx, gy, start || !act ? 0.0 : ab[l]);
                 if (act) ab[1 - l] = a1;
                 if (inner) {   // (the same in every lane)
                     const double d1 = half_dot(l, sb, ix, iy, 0.0);
